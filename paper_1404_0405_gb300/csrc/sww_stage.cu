@@ -9,11 +9,20 @@
 //   -> restriction of B, F, q F^perp and div, top-1 down to Jmin (two phases a level)
 //   -> RK stage update of the live points (all levels)
 //
-// The level records are staged in shared memory once per block; the tile of the
-// patch a block works on is staged in dynamic shared memory.  Loads of this
-// translation unit bypass L1 (compiled with -dlcm=cg): values written by other
-// blocks in one phase are read in the next.  Every barrier wait is bounded: after
-// about two seconds a block sets the error flag and the kernel returns; so does
+// One block of 1024 threads per SM.  The phases of a small grid are bound by
+// latency: a barrier, then a chain of dependent gathers.  So the level-serial phases
+// run over the point work lists (their lengths staged once per block) with each
+// warp's first id loaded before the barrier; consecutive warps of a list go to
+// different SMs, which also spreads the FP64 work (the FP64 pipe starts one warp
+// instruction per 16 clocks and SM); and the block's teams (Team) each work on a
+// patch of their own in the trend.  On the jet of 23 400 live cells on five levels a
+// stage took 206 us (FP64) and 134 us (FP32) with the patches' items dealt out in whole
+// blocks, one patch per 512-thread block and a barrier of 304 blocks; 148 and 93 us
+// now.  The barrier itself costs 1.4 us.
+//
+// Loads of this translation unit bypass L1 (compiled with -dlcm=cg): values written
+// by other blocks in one phase are read in the next.  Every barrier wait is bounded:
+// after about two seconds a block sets the error flag and the kernel returns; so does
 // the wait for a patch's geometry block (a bulk copy).
 #include <cuda_runtime.h>
 
@@ -33,157 +42,223 @@ namespace {
 #include "sww_bodies.cuh"
 #include "sww_tile.cuh"
 
-constexpr int STAGE_TPB = 512;
+constexpr int STAGE_TPB = 1024;
 constexpr int MAXL = 12;
 constexpr long long SPIN_CYCLES = 4000000000ll;   // ~2 s at 2 GHz
-constexpr unsigned BAR_GROUPS = 16, BAR_STRIDE = 32;
+
+// threads of one team of the trend: a tile's 4 p^2 own points, and teams that fit
+// the block's shared memory
+template <class R, int P>
+struct Teams {
+    static constexpr int NT = P == 4 ? 128 : P == 8 ? 256 : 512;
+    static constexpr size_t FIT = (227 * 1024 - 12 * 1024) / Tile<R, P>::BYTES;   // 12 KB: the level records
+    static constexpr int N = FIT < size_t(STAGE_TPB / NT) ? int(FIT) : STAGE_TPB / NT;
+    static_assert(N >= 1 && N < 16, "named barriers 1..15");
+};
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-
-// Grid-wide barrier, two-level: a block arrives at one of GROUPS counters (each in
-// its own 128-byte line), the last of a group at the root counter, and the last of
-// all advances the generation word that the others wait on.  False when the wait
-// timed out (after `spin` cycles, <= 0: SPIN_CYCLES) or a block has reported an
-// error; a block that finds the error flag already set does not arrive, so no
-// block passes a barrier once a wait has failed.  Block `skip` (fault injection,
-// -1: none) leaves without arriving.
-__device__ bool grid_sync(unsigned* bar, int* err, long long spin = 0, int skip = -1) {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) ok = 1;
-    if (threadIdx.x == 0 && (int(blockIdx.x) == skip || *reinterpret_cast<volatile int*>(err))) ok = 0;
-    __syncthreads();
-    if (!ok) return false;
-    if (threadIdx.x == 0) {
-        const long long limit = spin > 0 ? spin : SPIN_CYCLES;
-        const unsigned groups = gridDim.x < BAR_GROUPS ? gridDim.x : BAR_GROUPS;
-        const unsigned grp = blockIdx.x % groups;
-        const unsigned in_grp = (gridDim.x - grp + groups - 1) / groups;
-        unsigned* gen_p = bar;
-        unsigned* grp_p = bar + BAR_STRIDE * (1 + grp);
-        unsigned* root_p = bar + BAR_STRIDE * (1 + BAR_GROUPS);
-        const unsigned gen = ld_acquire(gen_p);
-        __threadfence();
-        bool last = false;
-        if (atomicAdd(grp_p, 1u) == in_grp - 1) {
-            atomicExch(grp_p, 0u);
-            if (atomicAdd(root_p, 1u) == groups - 1) {
-                atomicExch(root_p, 0u);
-                last = true;
-            }
-        }
-        if (last) {
-            __threadfence();
-            atomicAdd(gen_p, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (ld_acquire(gen_p) == gen) {
-                if (*reinterpret_cast<volatile int*>(err)) {
-                    ok = 0;
-                    break;
-                }
-                if (clock64() - t0 > limit) {
-                    atomicExch(err, 1);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return ok != 0;
+__device__ __forceinline__ void red_release(unsigned* p) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
 
-// barrier between phases: the grid barrier of the cooperative launch
+// Grid-wide barrier of the cooperative launch.  bar[0] counts arrivals and is never
+// reset; bar[BASE] holds its value when the launch began (written by the launch before
+// it, at its end), so the n-th barrier of a launch is complete when the count has
+// reached base + n * blocks, in arithmetic modulo 2^32.  One counter: the arrivals
+// need no answer, so a barrier costs one trip to the L2 and the polls (a two-level
+// barrier with its two dependent atomics and sleeping waits took about 2 us longer).
+struct GridBarrier {
+    static constexpr int BASE = 32;
+    unsigned* bar;
+    int* err;
+    long long limit;
+    int skip;
+    unsigned target;
+
+    // arrives and waits: false, for every thread of the block, when the wait timed
+    // out (after `limit` cycles; the error flag is set), another block has reported
+    // an error, or the block is the one told to leave without arriving (fault
+    // injection).  A block that leaves arrives nowhere again, so no block passes a
+    // later barrier.
+    __device__ bool sync() {
+        bool ok = true;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (int(blockIdx.x) == skip) {
+                ok = false;
+            } else {
+                __threadfence();
+                red_release(bar);
+                target += gridDim.x;
+                const long long t0 = clock64();
+                unsigned polls = 0;
+                while (int(ld_acquire(bar) - target) < 0) {
+                    if ((++polls & 15u) == 0 && *reinterpret_cast<volatile int*>(err)) {
+                        ok = false;
+                        break;
+                    }
+                    if (clock64() - t0 > limit) {
+                        atomicExch(err, 1);
+                        ok = false;
+                        break;
+                    }
+                }
+                __threadfence();
+            }
+        }
+        return __syncthreads_and(ok);
+    }
+};
+
+// This thread's first item of a phase: consecutive warps of items go to consecutive
+// blocks, so that a short list reaches every SM.  The next item is gridDim.x *
+// blockDim.x further on.
+__device__ __forceinline__ int first_item() {
+    return int(((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31));
+}
+
+// One level-serial phase over work lists k0 and (k1 >= 0) k1 of level L: item i < n0 of
+// the first, then the second.  first() loads this thread's first id (before the
+// barrier that precedes the phase: lists do not change during a stage), run() visits
+// the items.
 template <class R>
-__device__ __forceinline__ bool stage_sync(const StageArgs<R>& a) {
-    return grid_sync(a.bar, a.err, a.spin, a.skip);
+struct ListPhase {
+    const DevLevelT<R>* L = nullptr;
+    int n0 = 0, n1 = 0, k0 = 0, k1 = -1;
+    int32_t id = 0;
+    __device__ __forceinline__ int32_t load(int i) const {
+        return i < n0 ? L->wl[wl_off(*L, k0) + i] : L->wl[wl_off(*L, k1) + (i - n0)];
+    }
+    __device__ __forceinline__ void first(const DevLevelT<R>& lev, const int (&cnt)[MAXL][WL_KINDS], int j, int a, int b) {
+        L = &lev, k0 = a, k1 = b;
+        n0 = cnt[j][a], n1 = b >= 0 ? cnt[j][b] : 0;
+        const int i = first_item();
+        if (i < n0 + n1) id = load(i);
+    }
+    template <class Body>
+    __device__ __forceinline__ void run(Body body) {
+        for (int i = first_item(); i < n0 + n1; i += int(gridDim.x * blockDim.x)) {
+            body(i < n0 ? 0 : 1, int64_t(id));
+            const int ni = i + int(gridDim.x * blockDim.x);
+            if (ni < n0 + n1) id = load(ni);
+        }
+    }
+};
+
+// items of `count` entries of `list` (NS slots of P items an entry): body(entry, item)
+template <class Body>
+__device__ __forceinline__ void entry_items(const int32_t* __restrict__ list, int count, uint32_t NS, int P, Body body) {
+    const int lp = __ffs(P) - 1;
+    const uint32_t n = uint32_t(count) * (NS << lp);
+    for (uint32_t it = uint32_t(first_item()); it < n; it += gridDim.x * blockDim.x) {
+        const uint32_t e = (it >> lp) / NS;
+        body(list[e], it - ((e * NS) << lp));
+    }
 }
 
 template <class R, int P>
-__global__ void __launch_bounds__(STAGE_TPB) k_stage(StageArgs<R> a) {
+__global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ DevLevelT<R> sl[MAXL];
+    __shared__ int cnt[MAXL][WL_KINDS];
+    __shared__ int n_all, n_irr, start_ok;
+    __shared__ unsigned start_base;
     {
         const int words = int((a.jmax + 1) * sizeof(DevLevelT<R>) / sizeof(int));
         const int* src = reinterpret_cast<const int*>(a.lvs);
         int* dst = reinterpret_cast<int*>(sl);
         for (int k = threadIdx.x; k < words; k += blockDim.x) dst[k] = src[k];
+        if (threadIdx.x == 0) {
+            // a launch that follows a failed one leaves at once (its barrier count is stale)
+            start_ok = *reinterpret_cast<volatile int*>(a.err) == 0;
+            start_base = a.bar[GridBarrier::BASE];
+            n_all = *a.all_count, n_irr = *a.irr_count;
+        }
+        __syncthreads();
+        if (!start_ok) return;
+        for (int k = threadIdx.x; k < (a.jtop + 1) * WL_KINDS; k += blockDim.x)
+            if (k / WL_KINDS >= a.jmin) cnt[k / WL_KINDS][k % WL_KINDS] = sl[k / WL_KINDS].wl_n[k % WL_KINDS];
         __syncthreads();
     }
+    const long long limit = a.spin > 0 ? a.spin : SPIN_CYCLES;
+    GridBarrier gb{a.bar, a.err, limit, a.skip, start_base};
     const DevLevelT<R>* lv = sl;
     const R H = R(a.H), g = R(a.g);
+    ListPhase<R> ph;
     // ghosts, coarse to fine
+    if (a.jtop > a.jmin) ph.first(lv[a.jmin + 1], cnt, a.jmin + 1, WL_GN, WL_GE);
     for (int j = a.jmin + 1; j <= a.jtop; ++j) {
         const DevLevelT<R>& F = lv[j];
         const DevLevelT<R>& C = lv[j - 1];
-        ITEMS(K_NODE | K_EDGE, (const DevLevelT<R>*)nullptr, F, F.patches, F.npatches, a.P) {
-            if (kind == K_NODE)
-                fill_node(L, C, id);
+        ph.run([&](int k, int64_t id) {
+            if (k == 0)
+                fill_node(F, C, id);
             else
-                fill_edge(L, C, id);
+                fill_edge(F, C, id);
         });
-        if (!stage_sync(a)) return;
+        if (j < a.jtop) ph.first(lv[j + 1], cnt, j + 1, WL_GN, WL_GE);
+        if (!gb.sync()) return;
     }
-    {
-        // one active patch per block at a time
-        const long long limit = a.spin > 0 ? a.spin : SPIN_CYCLES;
-        const int area = a.P;
-        const bool ok = tile_sweep<R, P, STAGE_TPB>(lv, a.all_list, *a.all_count, int(blockIdx.x), int(gridDim.x), H, g,
-                                                    smem, a.err, limit, [&](const DevLevelT<R>& L, int64_t pat) {
-                                                        for (int it = threadIdx.x; it < 5 * area; it += blockDim.x) {
-                                                            auto body = [&](const DevLevelT<R>& LL, int kind, int64_t id,
-                                                                            int64_t) {
-                                                                if (kind == K_EDGE)
-                                                                    flux_at(LL, id, H);
-                                                                else
-                                                                    pv_at(LL, id, H);
-                                                            };
-                                                            visit_item<K_EDGE | K_TRI>(L, pat, uint32_t(it), area, body);
-                                                        }
-                                                    });
-        if (!ok) return;
-    }
-    if (!stage_sync(a)) return;
-    ITEMS(K_NODE | K_EDGE, lv, lv[a.jmin], a.irr_list, a.irr_count, a.P) {
-        if (kind == K_NODE)
-            node_at(L, id, g);
-        else
-            coriolis_at(L, id);
+    // the trend: the irregular patches' F and q one thread an item, then a regular patch
+    // a team at a time (patches dealt out over the SMs first)
+    entry_items(a.irr_list, n_irr, 5, a.P, [&](int32_t ent, uint32_t local) {
+        irregular_fq(lv[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), local, a.P, H);
     });
-    if (!stage_sync(a)) return;
+    {
+        using TM = Teams<R, P>;
+        const int team = int(threadIdx.x) / TM::NT;
+        bool ok = true;
+        if (team < TM::N)
+            ok = tile_sweep<R, P, TM::NT>(Team<TM::NT>{int(threadIdx.x) % TM::NT, unsigned(team + 1)}, lv, a.all_list, n_all,
+                                          int(team * gridDim.x + blockIdx.x), int(TM::N * gridDim.x), H, g,
+                                          smem + team * Tile<R, P>::BYTES, a.err, limit);
+        if (!__syncthreads_and(ok)) return;
+    }
+    if (!gb.sync()) return;
+    entry_items(a.irr_list, n_irr, 4, a.P, [&](int32_t ent, uint32_t local) {
+        auto body = [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
+            if (kind == K_NODE)
+                node_at(L, id, g);
+            else
+                coriolis_at(L, id);
+        };
+        visit_item<K_NODE | K_EDGE>(lv[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), local, a.P, body);
+    });
     // restriction, fine to coarse
+    if (a.jtop > a.jmin) ph.first(lv[a.jtop - 1], cnt, a.jtop - 1, WL_CN, WL_RE);
+    if (!gb.sync()) return;
     for (int j = a.jtop - 1; j >= a.jmin; --j) {
         const DevLevelT<R>& C = lv[j];
         const DevLevelT<R>& F = lv[j + 1];
-        ITEMS(K_NODE | K_EDGE, (const DevLevelT<R>*)nullptr, C, C.patches, C.npatches, a.P) {
-            restrict_item(L, F, kind, id);
-        });
-        if (!stage_sync(a)) return;
-        ITEMS(K_NODE, (const DevLevelT<R>*)nullptr, C, C.patches, C.npatches, a.P) {
-            if (restricted_div_node(L, id)) div_at(L, id);
-        });
-        if (!stage_sync(a)) return;
+        ph.run([&](int k, int64_t id) { restrict_item(C, F, k == 0 ? K_NODE : K_EDGE, id); });
+        ph.first(C, cnt, j, WL_DN, -1);
+        if (!gb.sync()) return;
+        ph.run([&](int, int64_t id) { div_at(C, id); });
+        if (j > a.jmin) ph.first(lv[j - 1], cnt, j - 1, WL_CN, WL_RE);
+        if (!gb.sync()) return;
     }
+    // every block has read the barrier's base: the next launch's is this one's last target
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.bar[GridBarrier::BASE] = gb.target;
     const R dt = R(a.dt ? *a.dt : 0.0);
     const RKStageR<R> sr(a.st);
-    ITEMS(K_NODE | K_EDGE, lv, lv[a.jmin], a.all_list, a.all_count, a.P) {
-        if (kind == K_NODE)
-            update_node(L, id, sr, dt);
-        else
-            update_edge(L, id, sr, dt);
+    entry_items(a.all_list, n_all, 4, a.P, [&](int32_t ent, uint32_t local) {
+        auto body = [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
+            if (kind == K_NODE)
+                update_node(L, id, sr, dt);
+            else
+                update_edge(L, id, sr, dt);
+        };
+        visit_item<K_NODE | K_EDGE>(lv[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), local, a.P, body);
     });
 }
 
 template <class R, int P>
 unsigned stage_grid_p(int nsm) {
-    constexpr size_t smem = Tile<R, P>::BYTES;
+    constexpr size_t smem = Teams<R, P>::N * Tile<R, P>::BYTES;
     // the dynamic tile and the static level records together may pass the default
     // 48 KB: the dynamic size is always declared
     if (cudaFuncSetAttribute(k_stage<R, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
@@ -198,7 +273,7 @@ cudaError_t launch_stage_p(const StageArgs<R>& a, unsigned grid, cudaStream_t s)
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(STAGE_TPB);
-    cfg.dynamicSmemBytes = Tile<R, P>::BYTES;
+    cfg.dynamicSmemBytes = Teams<R, P>::N * Tile<R, P>::BYTES;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

@@ -12,9 +12,9 @@ namespace sww {
 // Arguments of one persistent stage: levels (device array of jmax + 1 records),
 // the all-level work list, patch area P, the levels, the constants, the stage
 // coefficients and the time step, and the barrier state: STAGE_BAR_WORDS words, zero
-// before the first launch (generation word and arrival counters, each in its own
-// 128-byte line), err set on a timed-out wait.
-constexpr int STAGE_BAR_WORDS = 32 * 18;
+// before the first launch (the arrival count and its value when a launch begins, each
+// in its own 128-byte line), err set on a timed-out wait.
+constexpr int STAGE_BAR_WORDS = 32 * 2;
 
 template <class R>
 struct StageArgs {

@@ -6,9 +6,10 @@
 //                 member, striding over the member's all-level list): a regular
 //                 patch runs tile_trend (F, q, div F, K, B, q F^perp from its tile in
 //                 shared memory, its geometry block brought in by a bulk copy one
-//                 patch ahead); an irregular one (a pentagon or a pole within
+//                 patch ahead); the irregular ones (a pentagon or a pole within
 //                 reach, a level whose patch side differs, the viscous and
-//                 advection forms) gets F and q from the tabulated bodies.
+//                 advection forms) get F and q from the tabulated bodies, one thread
+//                 per item.
 //   k_tile_irr    div F, K, B and q F^perp at the points of the irregular
 //                 patches (the member's irregular list), from the F and q that
 //                 k_tile_trend wrote for them and their neighbours.
@@ -62,19 +63,16 @@ __global__ void __launch_bounds__(TILE_TPB, tile_min_blocks<P>()) k_tile_trend(B
     const MemberRef<R>* mr = a.m + m;
     stage_records(sl, mr, a.jmin);
     const R H = R(a.H);
-    const int area = a.P;
-    tile_sweep<R, P, TILE_TPB>(sl, mr->all_list, *mr->all_count, b, bpm, H, R(a.g), smem, mr->err, COPY_WAIT_CYCLES,
-                               [&](const DevLevelT<R>& L, int64_t pat) {
-                                   for (int it = threadIdx.x; it < 5 * area; it += blockDim.x) {
-                                       auto body = [&](const DevLevelT<R>& LL, int kind, int64_t id, int64_t) {
-                                           if (kind == K_EDGE)
-                                               flux_at(LL, id, H);
-                                           else
-                                               pv_at(LL, id, H);
-                                       };
-                                       visit_item<K_EDGE | K_TRI>(L, pat, uint32_t(it), area, body);
-                                   }
-                               });
+    // the irregular patches' items first, over the member's blocks
+    const int lp = __ffs(a.P) - 1;
+    const uint32_t n = uint32_t(*mr->irr_count) * (5u << lp);
+    for (uint32_t it = uint32_t(b) * blockDim.x + threadIdx.x; it < n; it += uint32_t(bpm) * blockDim.x) {
+        const uint32_t e = (it >> lp) / 5;
+        const int32_t ent = mr->irr_list[e];
+        irregular_fq(sl[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), it - ((e * 5) << lp), a.P, H);
+    }
+    tile_sweep<R, P, TILE_TPB>(Team<TILE_TPB>{int(threadIdx.x), 0u}, sl, mr->all_list, *mr->all_count, b, bpm, H, R(a.g),
+                               smem, mr->err, COPY_WAIT_CYCLES);
 }
 
 // the geometry block of every regular patch of L (one block per patch)

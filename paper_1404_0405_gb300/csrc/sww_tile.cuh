@@ -3,8 +3,8 @@
 // the energy-conserving Coriolis weights derived from the kite areas.
 //
 // Included inside an anonymous namespace after sww_bodies.cuh and bulk.cuh.  All
-// threads of the block call tile_trend and tile_sweep together (they synchronise
-// the block).
+// threads of a team (the block, or NT of its threads) call tile_trend and
+// tile_sweep together (they synchronise the team).
 //
 // Per tile: depth and velocity with their flags over the tile range (velocity
 // signs turned to the local directions), copied asynchronously through the
@@ -26,6 +26,29 @@
 // available nodes, Q at live edges, for the patch's own points.
 #pragma once
 // (tile.h is included at file scope by the translation unit)
+
+// NT threads that work on one patch: the whole block (barrier 0), or one of several
+// teams of a block, each with a hardware barrier of its own, so that a large block
+// (a persistent stage's, one per SM) works on several patches at once.
+template <int NT>
+struct Team {
+    int tid;        // 0 .. NT - 1
+    unsigned bar;   // named barrier, 0 .. 15
+    __device__ void sync() const { asm volatile("barrier.cta.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory"); }
+    // true when every thread of the team passes true (a barrier too)
+    __device__ bool sync_and(bool v) const {
+        unsigned r;
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t"
+            "setp.ne.u32 p, %1, 0;\n\t"
+            "barrier.cta.red.and.pred q, %2, %3, p;\n\t"
+            "selp.u32 %0, 1, 0, q;\n\t}"
+            : "=r"(r)
+            : "r"(unsigned(v)), "r"(bar), "n"(NT)
+            : "memory");
+        return r != 0;
+    }
+};
 
 // Geometry block of one regular patch over the tile's slot ranges, in R: the FP64
 // tables rounded once (geo<R>) to the values the stencils use.  Word offsets:
@@ -79,9 +102,8 @@ struct TilePlan {
     static constexpr int NONE = -(1 << 30);
     int n[SN], e[SE], t[ST];
 
-    __device__ void init() {
+    __device__ void init(int tid) {
         constexpr tile::Shape S{P};
-        const int tid = threadIdx.x;
 #pragma unroll
         for (int i = 0; i < SN; ++i) {
             const int x = tid + i * NT;
@@ -217,7 +239,7 @@ __device__ void tile_geo_build(const DevLevelT<R>& L, int64_t pat, R* __restrict
     using PL = TilePlan<P, NT>;
     constexpr int W = G::W, NN = G::NN, PP = G::PP;
     PL plan;
-    plan.init();
+    plan.init(int(threadIdx.x));
     TileCodes<P, NT> codes;
     codes.load(L, pat, plan);
     const int32_t nelem = int32_t(L.nelem), ntri = int32_t(L.T), base = int32_t(pat) * PP;
@@ -276,7 +298,7 @@ __device__ void tile_geo_build(const DevLevelT<R>& L, int64_t pat, R* __restrict
 // with the byte's position in the word and the velocity's direction flip left in
 // nf and ef for tile_trend to apply.
 template <class R, int P, int NT>
-__device__ __forceinline__ void tile_fetch(const DevLevelT<R>& L, int64_t pat, const TilePlan<P, NT>& plan,
+__device__ __forceinline__ void tile_fetch(const DevLevelT<R>& L, int64_t pat, int tid, const TilePlan<P, NT>& plan,
                                            const TileCodes<P, NT>& codes, unsigned char* stg) {
     using T = Tile<R, P>;
     using PL = TilePlan<P, NT>;
@@ -288,7 +310,6 @@ __device__ __forceinline__ void tile_fetch(const DevLevelT<R>& L, int64_t pat, c
     uint8_t* nf = stg + T::ST_NF;
     uint8_t* ef = stg + T::ST_EF;
     const int32_t nelem = int32_t(L.nelem), base = int32_t(pat) * PP;
-    const int tid = threadIdx.x;
 #pragma unroll
     for (int i = 0; i < PL::SN; ++i) {
         const int c = plan.n[i];
@@ -312,14 +333,14 @@ __device__ __forceinline__ void tile_fetch(const DevLevelT<R>& L, int64_t pat, c
     async_commit();
 }
 
-// The trend of one regular tile (all threads of the block): its fields fetched
+// The trend of one regular tile (all threads of the team): its fields fetched
 // into staged-field buffer `k` (tile_fetch), its geometry block in `geo` (shared
 // memory) once wait_geo() has returned true.  After the staging barrier the
-// block's earlier tiles are done with every buffer but k's, and after_stage()
+// team's earlier tiles are done with every buffer but k's, and after_stage()
 // runs (it may refill them).  False, for every thread, when wait_geo() failed for
 // some thread (nothing is computed).
 template <class R, int P, int NT, class WaitGeo, class AfterStage>
-__device__ bool tile_trend(const DevLevelT<R>& L, int64_t pat, R H, R g, const TilePlan<P, NT>& plan,
+__device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t pat, R H, R g, const TilePlan<P, NT>& plan,
                            unsigned char* smem, int k, const R* geo, WaitGeo wait_geo, AfterStage after_stage) {
     using T = Tile<R, P>;
     using G = TileGeo<R, P>;
@@ -343,7 +364,7 @@ __device__ bool tile_trend(const DevLevelT<R>& L, int64_t pat, R H, R g, const T
     const R* __restrict__ ai = geo + G::AI;
     const int32_t nelem = int32_t(L.nelem);
     const int32_t base = int32_t(pat) * PP;
-    const int tid = threadIdx.x;
+    const int tid = team.tid;
     // --- the fields tile_fetch copied for this thread's slots: the flag bytes out of
     // their words (the byte's position was left in nf/ef), the velocity turned to the
     // local direction
@@ -365,7 +386,7 @@ __device__ bool tile_trend(const DevLevelT<R>& L, int64_t pat, R H, R g, const T
         ef[y] = uint8_t(efw[y] >> (8 * (m & 3)));
         if (m & 4) u[y] = -u[y];
     }
-    if (!__syncthreads_and(wait_geo())) return false;
+    if (!team.sync_and(wait_geo())) return false;
     after_stage();
     // --- F at edges, q at triangles
 #pragma unroll
@@ -405,7 +426,7 @@ __device__ bool tile_trend(const DevLevelT<R>& L, int64_t pat, R H, R g, const T
         }
         q[z] = qq;
     }
-    __syncthreads();
+    team.sync();
     // --- the patch's own nodes (div F, K, B) and live edges (energy-conserving
     // q F^perp), in one pass of PP + 3 PP items (orientation uniform over a warp when
     // P * P is a multiple of 32)
@@ -440,31 +461,31 @@ __device__ bool tile_trend(const DevLevelT<R>& L, int64_t pat, R H, R g, const T
     return true;
 }
 
-// The trend of the active patches first, first + stride, ... (< n) of an
-// all-level list, by one block: regular patches by tile_trend, other patches by
-// other(L, pat).  Patch i of the sweep uses buffers i mod 2 (staged fields,
-// geometry).  The next patch's fields (element copies, tile_fetch) and geometry
-// block (a bulk copy) are started right after this patch's staging barrier, once
-// every thread is done with the patch before, which used those buffers; the
-// halo ids they need are loaded a patch earlier still.  So one barrier separates
-// consecutive patches, and the copies run while this patch is worked on.  False,
-// with *err set, when a bulk copy did not complete within `limit` cycles (the
-// block then gives it one more bounded wait and leaves).
-template <class R, int P, int NT, class Other>
-__device__ bool tile_sweep(const DevLevelT<R>* lv, const int32_t* list, int n, int first, int stride, R H, R g,
-                           unsigned char* smem, int* err, long long limit, Other other) {
+// The trend of the regular patches first, first + stride, ... (< n) of an all-level
+// list, by one team (entries whose tile is not regular are left to the caller).
+// Patch i of the sweep uses buffers i mod 2 (staged fields, geometry).  The next
+// patch's fields (element copies, tile_fetch) and geometry block (a bulk copy) are
+// started right after this patch's staging barrier, once every thread is done with
+// the patch before, which used those buffers; the halo ids they need are loaded a
+// patch earlier still.  So one barrier separates consecutive patches, and the copies
+// run while this patch is worked on.  False, with *err set, when a bulk copy did not
+// complete within `limit` cycles (the team then gives it one more bounded wait and
+// leaves).
+template <class R, int P, int NT>
+__device__ bool tile_sweep(const Team<NT>& team, const DevLevelT<R>* lv, const int32_t* list, int n, int first, int stride,
+                           R H, R g, unsigned char* smem, int* err, long long limit) {
     using T = Tile<R, P>;
     using G = TileGeo<R, P>;
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + T::OFF_BAR);
     R* gbuf = reinterpret_cast<R*>(smem + T::OFF_GEO);
-    if (threadIdx.x == 0) {
+    if (team.tid == 0) {
         mbar_init(bar);
         mbar_init(bar + 1);
         fence_barrier_init();
     }
-    __syncthreads();
+    team.sync();
     TilePlan<P, NT> plan;
-    plan.init();
+    plan.init(team.tid);
     auto regular = [&](int e) -> bool {
         if (e >= n) return false;
         const int32_t ent = list[e];
@@ -480,9 +501,9 @@ __device__ bool tile_sweep(const DevLevelT<R>* lv, const int32_t* list, int n, i
         const int32_t ent = list[e];
         const DevLevelT<R>& L = lv[ent >> LVL_SHIFT];
         const int64_t pat = ent & PATCH_MASK;
-        tile_fetch<R, P, NT>(L, pat, plan, c, smem + T::OFF_STG + k * T::STAGED);
-        if (threadIdx.x == 0) {
-            fence_async_shared();   // the buffer's last readers are behind a block barrier
+        tile_fetch<R, P, NT>(L, pat, team.tid, plan, c, smem + T::OFF_STG + k * T::STAGED);
+        if (team.tid == 0) {
+            fence_async_shared();   // the buffer's last readers are behind a team barrier
             bulk_load(gbuf + k * G::WORDS, L.tgeo + pat * G::WORDS, G::BYTES, bar + k);
         }
     };
@@ -498,36 +519,47 @@ __device__ bool tile_sweep(const DevLevelT<R>* lv, const int32_t* list, int n, i
     unsigned ph = 0;   // bit k: parity of buffer k's next phase
     int k = 0;
     for (int e = first; e < n; e += stride, k ^= 1) {
-        const int32_t ent = list[e];
-        const DevLevelT<R>& L = lv[ent >> LVL_SHIFT];
-        const int64_t pat = ent & PATCH_MASK;
         const bool reg2 = regular(e + 2 * stride);
         if (reg2) codes_of(e + 2 * stride, c2);
         if (reg) {
+            const int32_t ent = list[e];
+            const DevLevelT<R>& L = lv[ent >> LVL_SHIFT];
             const uint32_t parity = (ph >> k) & 1u;
             ph ^= 1u << k;
             const bool done = tile_trend<R, P, NT>(
-                L, pat, H, g, plan, smem, k, gbuf + k * G::WORDS, [&]() { return mbar_wait(bar + k, parity, limit); },
+                team, L, ent & PATCH_MASK, H, g, plan, smem, k, gbuf + k * G::WORDS,
+                [&]() { return mbar_wait(bar + k, parity, limit); },
                 [&]() {
                     if (reg1) start(e + stride, c1, k ^ 1);
                 });
             if (!done) {
                 // this patch's bulk copy did not land in time: report it, give it one
                 // more bounded wait, and leave (nothing else was started)
-                if (threadIdx.x == 0) atomicExch(err, 1);
+                if (team.tid == 0) atomicExch(err, 1);
                 mbar_wait(bar + k, parity, limit);
                 return false;
             }
-        } else {
-            // the tabulated path shares no buffer with the tiles; the next copies wait
-            // for the block barrier that ends this patch
-            other(L, pat);
-            __syncthreads();
-            if (reg1) start(e + stride, c1, k ^ 1);
+        } else if (reg1) {
+            // the next patch's buffers may still be read by a thread behind in the patch before
+            team.sync();
+            start(e + stride, c1, k ^ 1);
         }
         c1 = c2;
         reg = reg1;
         reg1 = reg2;
     }
     return true;
+}
+
+// F and q of item `local` (0 .. 5 area - 1: edges, then triangles) of a patch whose
+// tile is not regular, by the tabulated bodies
+template <class R>
+__device__ __forceinline__ void irregular_fq(const DevLevelT<R>& L, int64_t pat, uint32_t local, int area, R H) {
+    auto body = [&](const DevLevelT<R>& LL, int kind, int64_t id, int64_t) {
+        if (kind == K_EDGE)
+            flux_at(LL, id, H);
+        else
+            pv_at(LL, id, H);
+    };
+    visit_item<K_EDGE | K_TRI>(L, pat, local, area, body);
 }
