@@ -244,10 +244,9 @@ struct sww_handle {
     std::vector<void*> allocs;
     unsigned long long *red = nullptr, *cnt = nullptr;
     double *thr = nullptr, *dt = nullptr, *part = nullptr, *sums = nullptr;
-    int32_t *all_list = nullptr, *all_count = nullptr, *d_counts = nullptr, *sig_any = nullptr;
-    // entries of all_list whose tile is not regular, and a bound on their number
-    int32_t *irr_list = nullptr, *irr_count = nullptr;
-    int64_t irr_bound = 0;
+    int32_t *d_counts = nullptr, *sig_any = nullptr;
+    GridLists lists{};              // all-level lists
+    int64_t irr_bound = 0;          // a bound on the entries whose tile is not regular
     uint8_t* self_ref = nullptr;    // device MemberRef of this handle (its own trend launches)
     // candidate lists of the list-based mask (all levels)
     int32_t *cand = nullptr, *cand_count = nullptr, *gcand = nullptr, *gcand_count = nullptr;
@@ -501,7 +500,9 @@ void alloc_state(sww_handle* h, int j) {
     for (auto p : bN) *p = h->alloc<uint8_t>(N16);
     D.eflag = h->alloc<uint8_t>(E16);
     D.pflag = h->alloc<uint8_t>(D.npatch);
+    D.kflag = h->alloc<uint8_t>(D.npatch + 1);
     ck(cudaMemset(D.pflag, 0, D.npatch), "memset");
+    ck(cudaMemset(D.kflag, 0, D.npatch + 1), "memset");
     D.pfeat = h->alloc<float>(NF * (D.npatch + 1));
     D.prop = h->alloc<uint8_t>(D.npatch + 1);
     D.prop_prev = h->alloc<uint8_t>(D.npatch + 1);
@@ -510,7 +511,9 @@ void alloc_state(sww_handle* h, int j) {
     for (uint8_t* p : pz) ck(cudaMemset(p, 0, D.npatch + 1), "memset");
     ck(cudaMemset(D.pfeat, 0, NF * (D.npatch + 1) * sizeof(float)), "memset");
     D.patches = h->alloc<int32_t>(D.npatch + 1);
-    D.npatches = h->alloc<int32_t>(1);
+    D.clist = h->alloc<int32_t>(D.npatch + 1);
+    D.ilist = h->alloc<int32_t>(D.npatch + 1);
+    D.npatches = h->alloc<int32_t>(LIST_COUNTS);
     D.wl = h->alloc<int32_t>(3 * N + 2 * E);
     D.wl_n = h->alloc<int32_t>(WL_WORDS);
     ck(cudaMemset(D.wl_n, 0, WL_WORDS * sizeof(int32_t)), "memset");
@@ -530,7 +533,7 @@ void alloc_state(sww_handle* h, int j) {
     for (auto p : bN) ck(cudaMemset(*p, 0, N16), "memset");
     ck(cudaMemset(D.eflag, 0, E16), "memset");
     ck(cudaMemset(D.ue, 0, coarse_E * sizeof(R)), "memset");
-    ck(cudaMemset(D.npatches, 0, sizeof(int32_t)), "memset");
+    ck(cudaMemset(D.npatches, 0, LIST_COUNTS * sizeof(int32_t)), "memset");
     lvl<R>(h)[j] = D;
 }
 
@@ -603,12 +606,22 @@ struct Trace {
 
 template <class R>
 WorkT<R> work_all(const sww_handle* h) {
-    return WorkT<R>{dlv<R>(h), h->all_list, h->all_count, h->S, h->grid_all};
+    return WorkT<R>{dlv<R>(h), h->lists.all, h->lists.count, h->S, h->grid_all};
+}
+// the patches that hold or border live points (CORE_HOPS), for passes over live points
+template <class R>
+WorkT<R> work_core(const sww_handle* h) {
+    return WorkT<R>{dlv<R>(h), h->lists.core, h->lists.count + 1, h->S, h->grid_all};
 }
 template <class R>
 WorkT<R> work_level(const sww_handle* h, int j) {
     const DevLevelT<R>& L = lvl<R>(h)[j];
     return WorkT<R>{nullptr, L.patches, L.npatches, h->S, h->grid_lv[j]};
+}
+template <class R>
+WorkT<R> work_level_core(const sww_handle* h, int j) {
+    const DevLevelT<R>& L = lvl<R>(h)[j];
+    return WorkT<R>{nullptr, L.clist, L.npatches + 1, h->S, h->grid_lv[j]};
 }
 
 // ------------------------------------------------------------------ sequences
@@ -647,7 +660,7 @@ void trend(sww_handle* h) {
 template <class R>
 void update(sww_handle* h, const RKStage& st) {
     Trace t(h, SWW_K_UPDATE);
-    launch_update(work_all<R>(h), st, h->dt, h->stream);
+    launch_update(work_core<R>(h), st, h->dt, h->stream);
 }
 
 // trend and RK stage: one persistent cooperative launch, or one launch per phase
@@ -659,8 +672,8 @@ void stage(sww_handle* h, const RKStage& st) {
         return;
     }
     Trace t(h, SWW_K_STAGE);
-    StageArgs<R> a{dlv<R>(h), h->all_list, h->all_count, h->irr_list, h->irr_count, h->S, h->cfg.jmin, h->jtop,
-                   h->cfg.jmax, h->cfg.H, h->cfg.g, st, h->dt, h->bar, h->err, h->spin_cycles, h->skip_block};
+    StageArgs<R> a{dlv<R>(h), h->lists, h->S, h->cfg.jmin, h->jtop, h->cfg.jmax, h->cfg.H, h->cfg.g, st, h->dt, h->bar,
+                   h->err, h->spin_cycles, h->skip_block};
     ck(launch_stage(a, h->stage_blocks, h->stream), "persistent stage launch");
 }
 
@@ -679,7 +692,7 @@ void compute_dt(sww_handle* h) {
     Trace t(h, SWW_K_DT);
     count_launch(1);
     k_reset_red<<<1, 32, 0, h->stream>>>(h->red);
-    launch_dt(work_all<R>(h), h->cfg.H, h->cfg.g, h->red, h->stream);
+    launch_dt(work_core<R>(h), h->cfg.H, h->cfg.g, h->red, h->stream);
     launch_dt_final<R>(dlv<R>(h), h->red, h->cfg.cfl, h->dt, h->stream);
 }
 
@@ -757,9 +770,8 @@ template <class R>
 MaskMember<R> mask_member(const sww_handle* h) {
     MaskMember<R> m{};
     m.lvs = dlv<R>(h);
-    m.active = h->all_list, m.active_count = h->all_count;
+    m.lists = h->lists;
     m.cand = h->cand, m.cand_count = h->cand_count, m.gcand = h->gcand, m.gcand_count = h->gcand_count;
-    m.all = h->all_list, m.all_count = h->all_count, m.irr = h->irr_list, m.irr_count = h->irr_count;
     m.thr = h->thr, m.sig_any = h->sig_any, m.lstat = h->lstat, m.net = h->d_net;
     m.logit_tau = std::log(h->tau / (1.f - h->tau));
     m.learn = h->learn_mode;
@@ -818,7 +830,7 @@ void mask_and_inverse(sww_handle* h) {
     mask_only<R>(h);
     // inverse transform of the retained coefficients, coarse to fine, ghosts per level
     for (int j = j0 + 1; j <= j1; ++j) {
-        { Trace t(h, SWW_K_INVERSE); launch_inverse(lv[j], lv[j - 1], work_level<R>(h, j), s); }
+        { Trace t(h, SWW_K_INVERSE); launch_inverse(lv[j], lv[j - 1], work_level_core<R>(h, j), s); }
         { Trace t(h, SWW_K_FILL); launch_fill(lv[j], lv[j - 1], work_level<R>(h, j), s); }
     }
 }
@@ -830,11 +842,11 @@ double eps_coeff(const sww_config& c) { return c.regime == 1 ? c.eps * std::sqrt
 template <class R>
 void adapt(sww_handle* h, double eh, double eu) {
     cudaStream_t s = h->stream;
-    { Trace t(h, SWW_K_COEFF); launch_details(work_all<R>(h), h->cfg.jmin, s); }
+    { Trace t(h, SWW_K_COEFF); launch_details(work_core<R>(h), h->cfg.jmin, s); }
     {
         Trace t(h, SWW_K_MASK);
         ck(cudaMemsetAsync(h->red + 2, 0, 2 * sizeof(unsigned long long), s), "memset red");
-        launch_maxabs(work_all<R>(h), h->red, s);
+        launch_maxabs(work_core<R>(h), h->red, s);
         launch_thresholds(h->red, eps_coeff(h->cfg), eh, eu, h->cfg.advect, h->thr, s);
     }
     mask_and_inverse<R>(h);
@@ -881,7 +893,7 @@ void one_step(sww_handle* h, double dt, bool do_adapt, int part = 0) {
         } else {
             compute_dt<R>(h);
         }
-        { Trace t(h, SWW_K_UPDATE); launch_save_base(work_all<R>(h), h->stream); }
+        { Trace t(h, SWW_K_UPDATE); launch_save_base(work_core<R>(h), h->stream); }
     }
     if (part == 0) {
         int ns;
@@ -949,8 +961,8 @@ void run_step(sww_handle* h, double dt, bool do_adapt, int part = 0) {
 template <class R>
 MemberRef<R> member_ref(const sww_handle* h) {
     const int j1 = std::min(h->jtop + 1, h->cfg.jmax);
-    return MemberRef<R>{dlv<R>(h), h->all_list, h->all_count, h->dt, h->jtop, h->red, h->cfg.cfl, h->thr,
-                        eps_coeff(h->cfg), h->cfg.advect, j1, h->cfg.jmax, h->err, h->irr_list, h->irr_count};
+    return MemberRef<R>{dlv<R>(h), h->lists, h->dt, h->jtop, h->red, h->cfg.cfl, h->thr, eps_coeff(h->cfg), h->cfg.advect,
+                        j1, h->cfg.jmax, h->err};
 }
 
 // Device buffers of ensemble steps led by `lead` (allocated on first use).
@@ -1172,11 +1184,9 @@ int create_handle(const sww_config* cfg, void* stream, std::shared_ptr<Geometry>
             ck(cudaMemcpy(h->d_lvs, h->lv.data(), sizeof(DevLevelT<double>) * (cfg->jmax + 1), cudaMemcpyHostToDevice),
                "levels");
         }
-        h->all_list = h->alloc<int32_t>(total);
-        h->all_count = h->alloc<int32_t>(1);
-        h->irr_list = h->alloc<int32_t>(total);
-        h->irr_count = h->alloc<int32_t>(1);
-        ck(cudaMemset(h->irr_count, 0, sizeof(int32_t)), "memset");
+        h->lists = GridLists{h->alloc<int32_t>(total), h->alloc<int32_t>(total), h->alloc<int32_t>(total),
+                             h->alloc<int32_t>(LIST_COUNTS)};
+        ck(cudaMemset(h->lists.count, 0, LIST_COUNTS * sizeof(int32_t)), "memset");
         h->total_entries = total;
         h->irr_bound = 0;
         for (int j = cfg->jmin; j <= cfg->jmax; ++j)
@@ -1220,7 +1230,6 @@ int create_handle(const sww_config* cfg, void* stream, std::shared_ptr<Geometry>
         h->part = h->alloc<double>(4 * size_t(sums_blocks(meta(h, cfg->jmin))));
         ck(cudaMemset(h->thr, 0, 2 * sizeof(double)), "memset");
         ck(cudaMemset(h->dt, 0, sizeof(double)), "memset");
-        ck(cudaMemset(h->all_count, 0, sizeof(int32_t)), "memset");
         h->jtop = cfg->jmax;
         // the handle's own member record (the fields its trend launches read are fixed)
         h->self_ref = h->alloc<uint8_t>(sizeof(MemberRef<double>));
@@ -1360,7 +1369,7 @@ static int set_state_at(sww_handle* h, const double* dh, const double* u, int J,
             if (J > j0) launch_covered_all(dlv<R>(h), a.nodes_c, s);
             MaskArgsT<R> b = mask_args<R>(h, j0, j1, false);
             launch_patches_all(dlv<R>(h), b.patches, s);
-            launch_concat(dlv<R>(h), j0, j1, h->all_list, h->all_count, h->irr_list, h->irr_count, h->S, h->grid_all, s);
+            launch_concat(dlv<R>(h), j0, j1, h->lists, h->S, h->grid_all, s);
             read_counts<R>(h);
             check_launch();
             return 0;
@@ -1657,7 +1666,7 @@ int sww_forward(sww_handle* h) {
             using R = decltype(r);
             Join jn(h);
             Trace t(h, SWW_K_COEFF);
-            launch_details(work_all<R>(h), h->cfg.jmin, h->stream);
+            launch_details(work_core<R>(h), h->cfg.jmin, h->stream);
             check_launch();
             return 0;
         });
@@ -1677,7 +1686,7 @@ int sww_inverse(sww_handle* h) {
             cudaStream_t s = h->stream;
             launch_mark_support(work_all<R>(h), s);
             for (int j = h->cfg.jmin + 1; j <= h->jtop; ++j) {
-                { Trace t(h, SWW_K_INVERSE); launch_inverse(lv[j], lv[j - 1], work_level<R>(h, j), s); }
+                { Trace t(h, SWW_K_INVERSE); launch_inverse(lv[j], lv[j - 1], work_level_core<R>(h, j), s); }
                 { Trace t(h, SWW_K_FILL); launch_fill(lv[j], lv[j - 1], work_level<R>(h, j), s); }
             }
             check_launch();
@@ -1874,7 +1883,7 @@ int sww_load(sww_handle* h, const char* path) {
                 ck(cudaMemcpyAsync(h->thr, thr, sizeof(thr), cudaMemcpyHostToDevice, s), "load thr");
                 MaskArgsT<R> a = mask_args<R>(h, j0, j1, false);
                 launch_patches_all(dlv<R>(h), a.patches, s);
-                launch_concat(dlv<R>(h), j0, j1, h->all_list, h->all_count, h->irr_list, h->irr_count, h->S, h->grid_all, s);
+                launch_concat(dlv<R>(h), j0, j1, h->lists, h->S, h->grid_all, s);
                 read_counts<R>(h);
                 check_launch();
                 ck(cudaStreamSynchronize(s), "load");   // host buffers live on this frame

@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(BATCH_TPB, 8) k_phase_batch(BatchArgs<R> a, in
                     for (int w = 0; w < RED_WORDS; ++w) mr->red[w] = 0ull;
                 }
             }
-            member_items<K_NODE | K_EDGE>(sl, mr->all_list, *mr->all_count, a.P, b, bpm,
+            member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
                                           [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
                                               if (kind == K_NODE) {
                                                   if (L.nflag[id] & LIVE) L.dh0[id] = L.dh[id];
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(BATCH_TPB, 8) k_phase_batch(BatchArgs<R> a, in
             __syncthreads();
             unsigned long long wmax = 0;
             LevelMax um;
-            member_items<K_NODE | K_EDGE>(sl, mr->all_list, *mr->all_count, a.P, b, bpm,
+            member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
                                           [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
                                               if (kind == K_NODE) {
                                                   if (L.advect || !(L.nflag[id] & LIVE)) return;
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(BATCH_TPB, 8) k_phase_batch(BatchArgs<R> a, in
             // read dh and u)
             __shared__ unsigned long long shm[BATCH_TPB / 32];
             unsigned long long hmax = 0, umax = 0;
-            member_items<K_NODE | K_EDGE | K_CEDGE>(sl, mr->all_list, *mr->all_count, a.P, b, bpm,
+            member_items<K_NODE | K_EDGE | K_CEDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
                                                     [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t el) {
                                                         if (kind == K_NODE) {
                                                             if (L.nflag[id] & LIVE) hmax = max(hmax, abs_key(L.dh[id]));
@@ -232,13 +232,13 @@ __global__ void __launch_bounds__(BATCH_TPB, 8) k_phase_batch(BatchArgs<R> a, in
             break;
         }
         case PH_INV_A:
-            member_items<K_NODE | K_EDGE>(sl, sl[j].patches, *sl[j].npatches, a.P, b, bpm,
+            member_items<K_NODE | K_EDGE>(sl, sl[j].clist, sl[j].npatches[1], a.P, b, bpm,
                                           [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
                                               inverse_a_item(L, (&L)[-1], kind, id);
                                           });
             break;
         case PH_INV_B:
-            member_items<K_NODE>(sl, sl[j].patches, *sl[j].npatches, a.P, b, bpm,
+            member_items<K_NODE>(sl, sl[j].clist, sl[j].npatches[1], a.P, b, bpm,
                                  [&](const DevLevelT<R>& L, int, int64_t id, int64_t) { inverse_b_item(L, id); });
             break;
         case PH_PARTIAL:
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(BATCH_TPB, 8) k_phase_batch(BatchArgs<R> a, in
         default: {
             const R dt = R(*mr->dt);
             const RKStageR<R> sr(a.st);
-            member_items<K_NODE | K_EDGE>(sl, mr->all_list, *mr->all_count, a.P, b, bpm,
+            member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
                                           [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
                                               if (kind == K_NODE)
                                                   update_node(L, id, sr, dt);

@@ -106,6 +106,12 @@ __device__ __forceinline__ double cfl_step(const DevLevelT<R>* lvs, const unsign
     return cfl * fmin(1.0 / w, r);
 }
 
+// patch of node x (the poles: npatch); the patch side is a power of two
+template <class Lv>
+__device__ __forceinline__ int64_t patch_of(const Lv& L, int64_t x) {
+    return x < L.nelem ? int64_t(uint32_t(x) >> (2 * (__ffs(int(L.p)) - 1))) : L.npatch;
+}
+
 // Item kinds of a work-list entry, in slot order.
 constexpr int K_NODE = 1, K_EDGE = 2, K_TRI = 4, K_CEDGE = 8;
 
@@ -557,7 +563,7 @@ __device__ __forceinline__ void adjacent_node(const DevLevelT<R>& F, const DevLe
                 if (cy[k] >= 0) t |= C.sig[cy[k]];
         }
     }
-    const int64_t P = x < F.nelem ? x / (F.p * F.p) : F.npatch;
+    const int64_t P = patch_of(F, x);
     if (t)
         F.pexact[P] = 1;
     else if (F.prop[P])
@@ -598,7 +604,7 @@ __device__ __forceinline__ void live_edge(const DevLevelT<R>& L, int64_t e) {
 // one neighbour hop of the ghost band: band1 <- dilate(band0) when `forward`,
 // band0 <- dilate(band1) otherwise
 template <class R>
-__device__ __forceinline__ void dilate_node(const DevLevelT<R>& L, int64_t x, bool forward) {
+__device__ __forceinline__ uint8_t dilate_node(const DevLevelT<R>& L, int64_t x, bool forward) {
     const uint8_t* __restrict__ in = forward ? L.band0 : L.band1;
     uint8_t* __restrict__ out = forward ? L.band1 : L.band0;
     // band bytes are 0 or 1; the neighbours' loads are issued together
@@ -610,6 +616,7 @@ __device__ __forceinline__ void dilate_node(const DevLevelT<R>& L, int64_t x, bo
             if (k < dg) t |= in[L.ring_n[k * L.N + x]];
     }
     out[x] = t;
+    return t;
 }
 
 template <class R>
@@ -637,6 +644,23 @@ __device__ __forceinline__ void covered_node(const DevLevelT<R>& C, const DevLev
 
 // ---------------------------------------------------------------------------- patch lists (Sec. 5.2)
 
+// the 32 bytes flag[i0..) (those below n) as bits; flag + i0 is 16-byte aligned
+__device__ __forceinline__ unsigned flag_bits(const uint8_t* __restrict__ flag, int64_t i0, int64_t n) {
+    unsigned bits = 0u;
+    if (i0 + 32 <= n) {
+        const uint4 a = *reinterpret_cast<const uint4*>(flag + i0);
+        const uint4 b = *reinterpret_cast<const uint4*>(flag + i0 + 16);
+        const unsigned words[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) bits |= (((words[q] >> (8 * k)) & 0xffu) ? 1u : 0u) << (4 * q + k);
+    } else {
+        for (int k = 0; k < 32 && i0 + k < n; ++k) bits |= (flag[i0 + k] ? 1u : 0u) << k;
+    }
+    return bits;
+}
+
 // The indices of the nonzero bytes of flag[0..n) into out (tag | index), in
 // ascending order, by one block: each thread takes 32 consecutive flags per pass
 // (two 16-byte loads), the block forms an exclusive prefix of the counts, and each
@@ -650,18 +674,7 @@ __device__ int compact_flags(const uint8_t* __restrict__ flag, int64_t n, int32_
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int64_t start = 0; start < n; start += 32 * int64_t(blockDim.x)) {
         const int64_t i0 = start + 32 * int64_t(threadIdx.x);
-        unsigned bits = 0u;
-        if (i0 + 32 <= n) {
-            const uint4 a = *reinterpret_cast<const uint4*>(flag + i0);
-            const uint4 b = *reinterpret_cast<const uint4*>(flag + i0 + 16);
-            const unsigned words[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) bits |= (((words[q] >> (8 * k)) & 0xffu) ? 1u : 0u) << (4 * q + k);
-        } else {
-            for (int k = 0; k < 32 && i0 + k < n; ++k) bits |= (flag[i0 + k] ? 1u : 0u) << k;
-        }
+        unsigned bits = flag_bits(flag, i0, n);
         const int cnt = __popc(bits);
         int incl = cnt;
 #pragma unroll
@@ -694,67 +707,97 @@ __device__ int compact_flags(const uint8_t* __restrict__ flag, int64_t n, int32_
     return total;
 }
 
-// The ascending list of level L's flagged patches (+ the pole entry when a pole is
-// live or ghost), one block of any width (ballot and a warp-total prefix).
+// Level L's three ascending lists from its patch flags, by one block of any width: the
+// active patches (pflag), of these the core (kflag; `whole`: every active patch, as on
+// Jmin, which is live in full), and of the core the patches whose tile is not regular;
+// each with the pole entry last when a pole is live or ghost.  A thread takes 32 flags
+// a pass, and the three counts are prefix-summed together.  The flag arrays are
+// 16-byte aligned.
 template <class R>
-__device__ void patch_scan_level(const DevLevelT<R>& L) {
+__device__ void patch_scan_level(const DevLevelT<R>& L, bool whole) {
+    using U64 = unsigned long long;
+    __shared__ U64 wsum[32], total;      // active patches in the low half, core in the high half
+    __shared__ unsigned wsum_i[32], total_i;
     const int32_t tag = int32_t(L.J) << LVL_SHIFT;
-    const int n = compact_flags(L.pflag, L.npatch, tag, L.patches);
+    const bool all_irr = viscous(L) || L.advect || L.thalo == nullptr;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (threadIdx.x == 0) total = 0, total_i = 0;
+    __syncthreads();
+    for (int64_t start = 0; start < L.npatch; start += 32 * int64_t(blockDim.x)) {
+        const int64_t i0 = start + 32 * int64_t(threadIdx.x);
+        const unsigned a = flag_bits(L.pflag, i0, L.npatch);
+        const unsigned c = a & (whole || !a ? ~0u : flag_bits(L.kflag, i0, L.npatch));
+        const unsigned r = c & (all_irr || !c ? ~0u : flag_bits(L.tirr, i0, L.npatch));
+        const U64 cnt = U64(__popc(a)) | U64(__popc(c)) << 32;
+        const unsigned cnt_i = __popc(r);
+        U64 incl = cnt;
+        unsigned incl_i = cnt_i;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const U64 v = __shfl_up_sync(0xffffffffu, incl, o);
+            const unsigned vi = __shfl_up_sync(0xffffffffu, incl_i, o);
+            if (lane >= o) incl += v, incl_i += vi;
+        }
+        if (lane == 31) wsum[w] = incl, wsum_i[w] = incl_i;
+        __syncthreads();
+        if (w == 0) {
+            const U64 v = lane < nw ? wsum[lane] : 0;
+            const unsigned vi = lane < nw ? wsum_i[lane] : 0;
+            U64 iv = v;
+            unsigned ii = vi;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const U64 t = __shfl_up_sync(0xffffffffu, iv, o);
+                const unsigned ti = __shfl_up_sync(0xffffffffu, ii, o);
+                if (lane >= o) iv += t, ii += ti;
+            }
+            if (lane < nw) wsum[lane] = iv - v, wsum_i[lane] = ii - vi;   // exclusive prefix over warps
+        }
+        __syncthreads();
+        const U64 before = total + wsum[w] + incl - cnt;
+        const unsigned before_i = total_i + wsum_i[w] + incl_i - cnt_i;
+        auto put = [&](unsigned bits, int32_t* __restrict__ out, unsigned pos) {
+            while (bits) {
+                out[pos++] = tag | int32_t(i0 + __ffs(bits) - 1);
+                bits &= bits - 1u;
+            }
+        };
+        put(a, L.patches, unsigned(before));
+        put(c, L.clist, unsigned(before >> 32));
+        put(r, L.ilist, before_i);
+        __syncthreads();
+        if (threadIdx.x == blockDim.x - 1) total = before + cnt, total_i = before_i + cnt_i;
+        __syncthreads();
+    }
     if (threadIdx.x == 0) {
-        int m = n;
-        if ((L.nflag[L.nelem] | L.nflag[L.nelem + 1]) & AVAIL) L.patches[m++] = tag | int32_t(L.npatch);
-        *L.npatches = m;
+        int n[LIST_COUNTS] = {int(unsigned(total)), int(total >> 32), int(total_i)};
+        if ((L.nflag[L.nelem] | L.nflag[L.nelem + 1]) & AVAIL) {
+            const int32_t pole = tag | int32_t(L.npatch);
+            L.patches[n[0]++] = pole, L.clist[n[1]++] = pole, L.ilist[n[2]++] = pole;
+        }
+        for (int q = 0; q < LIST_COUNTS; ++q) L.npatches[q] = n[q];
     }
 }
 
-// The all-level list of levels jmin..jmax from the levels' lists, and its entries
-// whose tile is not regular (the irregular list, same order); one block.
+// The all-level lists of levels jmin..jmax from the levels' lists (in level order):
+// block j - jmin copies level j's entries behind those of the levels below it, and
+// clears the level's work-list counts (the point work lists are rebuilt next).
 template <class R>
-__device__ void concat_lists(const DevLevelT<R>* __restrict__ lvs, int jmin, int jmax, int32_t* all, int32_t* count,
-                             int32_t* irr, int32_t* irr_count) {
-    __shared__ int base, ibase;
-    __shared__ int warp_tot[32];
-    if (threadIdx.x == 0) base = 0, ibase = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int j = jmin; j <= jmax; ++j) {
-        const DevLevelT<R>& L = lvs[j];
-        const int n = *L.npatches;
-        const bool all_irr = viscous(L) || L.advect || L.thalo == nullptr;
-        // all entries in level order; the entries whose tile is not regular (see
-        // tile_regular) also into the irregular list, in the same order
-        for (int start = 0; start < n; start += blockDim.x) {
-            const int i = start + threadIdx.x;
-            int32_t ent = 0;
-            int f = 0;
-            if (i < n) {
-                ent = L.patches[i];
-                all[base + i] = ent;
-                const int64_t pat = ent & PATCH_MASK;
-                f = (all_irr || pat >= L.npatch || L.tirr[pat]) ? 1 : 0;
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, f);
-            if (lane == 0) warp_tot[w] = __popc(bal);
-            __syncthreads();
-            int off = 0;
-            for (int k = 0; k < w; ++k) off += warp_tot[k];
-            if (f) irr[ibase + off + __popc(bal & ((1u << lane) - 1u))] = ent;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                int tot = 0;
-                for (int k = 0; k < nw; ++k) tot += warp_tot[k];
-                ibase += tot;
-            }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) base += n;
-        __syncthreads();
+__device__ void concat_lists(const DevLevelT<R>* __restrict__ lvs, int jmin, int jmax, const GridLists& g) {
+    const int j = jmin + int(blockIdx.x);
+    if (j > jmax) return;
+    int base[LIST_COUNTS] = {0, 0, 0};
+    for (int i = jmin; i < j; ++i)
+        for (int q = 0; q < LIST_COUNTS; ++q) base[q] += lvs[i].npatches[q];
+    const DevLevelT<R>& L = lvs[j];
+    const int32_t* src[LIST_COUNTS] = {L.patches, L.clist, L.ilist};
+    int32_t* dst[LIST_COUNTS] = {g.all, g.core, g.irr};
+    for (int q = 0; q < LIST_COUNTS; ++q) {
+        const int n = L.npatches[q];
+        for (int i = threadIdx.x; i < n; i += blockDim.x) dst[q][base[q] + i] = src[q][i];
+        if (j == jmax && threadIdx.x == 0) g.count[q] = base[q] + n;
     }
-    if (threadIdx.x == 0) *count = base, *irr_count = ibase;
-    // the point work lists are rebuilt from these lists next (wl_build)
-    for (int j = jmin + int(threadIdx.x); j <= jmax && threadIdx.x < 32; j += 32)
-        if (lvs[j].wl_n)
-            for (int k = 0; k < WL_WORDS; ++k) lvs[j].wl_n[k] = 0;
+    if (threadIdx.x < WL_WORDS && L.wl_n) L.wl_n[threadIdx.x] = 0;
 }
 
 // offset of work list k of a level in wl

@@ -19,6 +19,17 @@ constexpr int MLP_PARAMS = NF * NH + NH + NH + 1;   // W1[NF][NH], b1[NH], w2[NH
 // level's live-node count, taken in the same pass (wl_n[WL_LIVE]).
 constexpr int WL_GN = 0, WL_GE = 1, WL_CN = 2, WL_RE = 3, WL_DN = 4, WL_KINDS = 5, WL_LIVE = 5, WL_WORDS = 6;
 
+// The core of the active grid.  A live node's or edge's update reads fluxes, potential
+// vorticities, divergences and Bernoulli functions owned by nodes within two hops of
+// a live node of its level, the restriction to the coarser level reads fluxes and
+// divergences owned by nodes within two hops of one (tests/core_reach_check.cpp), and a
+// divergence reads fluxes a hop further; the ghost band reaches five hops, so that
+// ghost values can be predicted from the coarser level.  A patch without a node within
+// CORE_HOPS hops of a live node therefore holds nothing that the trend of a live point
+// reads, and the passes over live points and their trend skip it.
+constexpr int CORE_HOPS = 3;
+constexpr int LIST_COUNTS = 3;   // counts kept per level (DevLevelT::npatches)
+
 // Work-list entry: (level << LVL_SHIFT) | patch; patch == npatch stands for the two poles.
 constexpr int LVL_SHIFT = 27;
 constexpr int32_t PATCH_MASK = (1 << LVL_SHIFT) - 1;
@@ -91,7 +102,12 @@ struct DevLevelT {
     uint8_t *prop, *prop_prev;     // [npatch+1] proposal for the next / used by the last mask
     uint8_t* pexact;               // [npatch+1] patch holds a point of the exact rules' set
     int32_t* patches;              // [npatch + 1] active patch list (+ pole entry), level-tagged
-    int32_t* npatches;             // [1]
+    int32_t* npatches;             // [LIST_COUNTS] entries of patches, clist, ilist
+    // of the active patches those whose points the trend of a live point can reach (the
+    // core: a node within CORE_HOPS hops of a live node of the level), and of these the
+    // ones whose tile is not regular; same order and entries as `patches`
+    uint8_t* kflag;                // [npatch+1] patch is in the core
+    int32_t *clist, *ilist;        // [npatch + 1]
     // work lists of the stage's point-wise phases, rebuilt with the active lists
     // (after every adaptation): ghost nodes [N], ghost edges [E], covered nodes [N],
     // edges with a covered end [E], available nodes with a covered node among them and

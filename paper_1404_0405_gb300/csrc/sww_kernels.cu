@@ -481,6 +481,7 @@ __global__ void k_patch_flags(const DevLevelT<R>* __restrict__ lvs, Span sp, con
                 if (L.prop[pid]) atomicAdd(&lstat[2], 1ull);
             }
             L.pflag[pid] = uint8_t(any);
+            L.kflag[pid] = uint8_t(any);   // every active patch counts as core (a superset is allowed)
         }
     }
 }
@@ -491,13 +492,12 @@ template <class R>
 __global__ void k_patch_scan(const DevLevelT<R>* __restrict__ lvs, int ja, const int32_t* sig_any, int tail_j) {
     int j = ja + int(blockIdx.x);
     if (j == tail_j && !sig_any[j - 1]) return;
-    patch_scan_level(lvs[j]);
+    patch_scan_level(lvs[j], j == ja);
 }
 
 template <class R>
-__global__ void k_concat(const DevLevelT<R>* __restrict__ lvs, int jmin, int jmax, int32_t* all, int32_t* count,
-                         int32_t* irr, int32_t* irr_count) {
-    concat_lists(lvs, jmin, jmax, all, count, irr, irr_count);
+__global__ void k_concat(const DevLevelT<R>* __restrict__ lvs, int jmin, int jmax, GridLists lists) {
+    concat_lists(lvs, jmin, jmax, lists);
 }
 
 // the point work lists of every level from the all-level list
@@ -640,11 +640,11 @@ void launch_patches_all(const DevLevelT<R>* lvs, const Span& patches, cudaStream
 }
 
 template <class R>
-void launch_concat(const DevLevelT<R>* lvs, int jmin, int jmax, int32_t* all, int32_t* count, int32_t* irr,
-                   int32_t* irr_count, int P, unsigned grid, cudaStream_t s) {
+void launch_concat(const DevLevelT<R>* lvs, int jmin, int jmax, const GridLists& lists, int P, unsigned grid,
+                   cudaStream_t s) {
     g_launches += 2;
-    k_concat<R><<<1, 1024, 0, s>>>(lvs, jmin, jmax, all, count, irr, irr_count);
-    k_wl_build<R><<<grid, TPB, 0, s>>>(lvs, all, count, P);
+    k_concat<R><<<unsigned(jmax - jmin + 1), 1024, 0, s>>>(lvs, jmin, jmax, lists);
+    k_wl_build<R><<<grid, TPB, 0, s>>>(lvs, lists.all, lists.count, P);
 }
 
 template <class R>
@@ -696,8 +696,7 @@ void launch_convert(const A* x, B* y, int64_t n, cudaStream_t s) {
                                     cudaStream_t);                                                           \
     template void launch_mark_support<R>(const WorkT<R>&, cudaStream_t);                                     \
     template void launch_patches_all<R>(const DevLevelT<R>*, const Span&, cudaStream_t);                     \
-    template void launch_concat<R>(const DevLevelT<R>*, int, int, int32_t*, int32_t*, int32_t*, int32_t*, int,     \
-                                   unsigned, cudaStream_t);         \
+    template void launch_concat<R>(const DevLevelT<R>*, int, int, const GridLists&, int, unsigned, cudaStream_t);    \
     template int sums_blocks<R>(const DevLevelT<R>&);                                                        \
     template void launch_sums<R>(const DevLevelT<R>&, double, double, double*, double*, cudaStream_t);       \
     template void launch_count<R>(const DevLevelT<R>&, unsigned long long*, cudaStream_t);

@@ -27,6 +27,14 @@ struct WorkT {
     unsigned grid;
 };
 
+// The all-level lists of a handle (level order, ascending patches): every active patch,
+// the core (CORE_HOPS), and of the core the entries whose tile is not regular, with their
+// lengths in count[0..2].
+struct GridLists {
+    int32_t *all, *core, *irr;
+    int32_t* count;
+};
+
 // Levels ja..jb of a multi-level dense launch; off[j - ja] is the first thread of
 // level j and off[jb + 1 - ja] the total.  Level tail_j (-1: none; only ever jb) is a
 // tail level of tail_n items covered by a fixed number of striding threads.
@@ -88,12 +96,11 @@ template <class R> void launch_mask(const MaskArgsT<R>& a, cudaStream_t s);
 template <class R> void launch_live_all(const DevLevelT<R>* lvs, const Span& nodes, const Span& edges, cudaStream_t s);
 template <class R> void launch_covered_all(const DevLevelT<R>* lvs, const Span& nodes_c, cudaStream_t s);
 template <class R> void launch_patches_all(const DevLevelT<R>* lvs, const Span& patches, cudaStream_t s);
-// the all-level active list from the levels' lists, its entries whose tile is not
-// regular (irregular list, same order), and the levels' point work lists (patch
+// the all-level lists from the levels' lists, and the levels' point work lists (patch
 // area P; grid: blocks of the list launch)
 template <class R>
-void launch_concat(const DevLevelT<R>* lvs, int jmin, int jmax, int32_t* all, int32_t* count, int32_t* irr,
-                   int32_t* irr_count, int P, unsigned grid, cudaStream_t s);
+void launch_concat(const DevLevelT<R>* lvs, int jmin, int jmax, const GridLists& lists, int P, unsigned grid,
+                   cudaStream_t s);
 template <class R> int sums_blocks(const DevLevelT<R>& L);
 template <class R>
 void launch_sums(const DevLevelT<R>& L, double H, double g, double* part, double* out, cudaStream_t s);

@@ -62,11 +62,6 @@ __device__ __forceinline__ const DevLevelT<R>* stage_levels(DevLevelT<R>* sl, co
     __shared__ DevLevelT<R> sl_[MAXL]; \
     const DevLevelT<R>* lvs = stage_levels(sl_, M.lvs, B.ja, M.jmax)
 
-template <class Lv>
-__device__ __forceinline__ int64_t patch_of(const Lv& L, int64_t x) {
-    return x < L.nelem ? x / (L.p * L.p) : L.npatch;
-}
-
 __device__ __forceinline__ bool span_find(const Span& sp, int64_t t, int& j, int64_t& i) {
     for (j = sp.ja; j <= sp.jb; ++j)
         if (t < sp.off[j + 1 - sp.ja]) {
@@ -115,10 +110,10 @@ __global__ void k_prop_any(const __grid_constant__ MaskBatch<R, CAP> B) {
 // Own features of a patch: log2(1 + max|h~|/eps_h) over its live odd nodes,
 // log2(1 + max|u~|/eps_u) over its live interior edges and the pair coefficients of
 // the coarse edges under its even nodes, and the fraction of its nodes that are
-// live.  An inactive patch has no live point: all three are 0 (k_feat_clear, one
-// thread per patch; the pole entry is cleared too and recomputed when listed).
-// The active patches of levels Jmin+1..jb come from the active list, one warp per
-// entry (one lane per node of the patch).
+// live.  A patch that is not active or not in the core has no live point: all three are
+// 0 (k_feat_clear, one thread per patch; the pole entry is cleared too and recomputed
+// when listed).  The core patches of levels Jmin+1..jb come from the core list, one
+// warp per entry (one lane per node of the patch).
 template <class R, int CAP>
 __global__ void k_feat_clear(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
@@ -128,7 +123,7 @@ __global__ void k_feat_clear(const __grid_constant__ MaskBatch<R, CAP> B) {
         return;
     const DevLevelT<R>& L = M.lvs[j];
     const int64_t np1 = L.npatch + 1;
-    if (P == L.npatch || !L.pflag[P]) L.pfeat[0 * np1 + P] = 0.f, L.pfeat[1 * np1 + P] = 0.f, L.pfeat[6 * np1 + P] = 0.f;
+    if (P == L.npatch || !L.pflag[P] || !L.kflag[P]) L.pfeat[0 * np1 + P] = 0.f, L.pfeat[1 * np1 + P] = 0.f, L.pfeat[6 * np1 + P] = 0.f;
 }
 
 template <class R, int CAP>
@@ -140,8 +135,8 @@ __global__ void k_feat_own(const __grid_constant__ MaskBatch<R, CAP> B) {
     const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
     // the thresholds once per thread, in FP32
     const float eh = float(M.thr[0] > 0 ? M.thr[0] : 1.0), eu = float(M.thr[1] > 0 ? M.thr[1] : 1.0);
-    for (int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; w < *M.active_count; w += nw) {
-        const int32_t ent = M.active[w];
+    for (int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; w < M.lists.count[1]; w += nw) {
+        const int32_t ent = M.lists.core[w];
         const int j = ent >> LVL_SHIFT;
         if (j <= B.ja || j > M.jb) continue;
         const int64_t P = ent & PATCH_MASK;
@@ -255,6 +250,7 @@ __global__ void k_clear_flags(const __grid_constant__ MaskBatch<R, CAP> B) {
     if (!span_find(B.patches, int64_t(blockIdx.x) * blockDim.x + threadIdx.x, j, P) || j > M.jb) return;
     const DevLevelT<R>& L = M.lvs[j];
     L.zflag[P] = 0, L.sflag[P] = 0, L.cflag[P] = 0, L.lflag[P] = 0, L.gflag[P] = 0;
+    L.kflag[P] = 0;
 }
 
 // the significance bytes of the previous mask, over its candidates (they stay
@@ -267,8 +263,8 @@ __global__ void k_clear_sig_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     ITEMS(K_NODE, lvs, none, M.cand, M.cand_count, B.P) { L.sig[id] = 0; });
 }
 
-// significance over the items of the active patches above Jmin; the patch of each
-// significant coefficient is recorded
+// significance over the items of the core patches above Jmin (only live points carry
+// coefficients); the patch of each significant coefficient is recorded
 template <class R, int CAP>
 __global__ void k_sig_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
@@ -276,7 +272,7 @@ __global__ void k_sig_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     DevLevelT<R> none{};
     const R eh = sig_thr<R>(M.thr[0]), eu = sig_thr<R>(M.thr[1]);
     int32_t* sig_any = M.sig_any;
-    ITEMS(K_NODE | K_EDGE | K_CEDGE, lvs, none, M.active, M.active_count, B.P) {
+    ITEMS(K_NODE | K_EDGE | K_CEDGE, lvs, none, M.lists.core, M.lists.count + 1, B.P) {
         if (L.J == B.ja) return;
         const DevLevelT<R>& C = lvs[L.J - 1];
         bool any;
@@ -291,7 +287,7 @@ __global__ void k_sig_list(const __grid_constant__ MaskBatch<R, CAP> B) {
         }
         if (any) {
             sig_any[L.J] = 1;
-            L.sflag[el < 0 ? L.npatch : el / (L.p * L.p)] = 1;
+            L.sflag[el < 0 ? L.npatch : patch_of(L, el)] = 1;
         }
     });
 }
@@ -302,8 +298,8 @@ template <class R, int CAP>
 __global__ void k_seed(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < *M.active_count; t += stride) {
-        const int32_t ent = M.active[t];
+    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < M.lists.count[0]; t += stride) {
+        const int32_t ent = M.lists.all[t];
         const int j = ent >> LVL_SHIFT;
         const int64_t P = ent & PATCH_MASK;
         const DevLevelT<R>& L = M.lvs[j];
@@ -454,14 +450,15 @@ __global__ void k_live_edges_list(const __grid_constant__ MaskBatch<R, CAP> B) {
 }
 
 template <class R, int CAP>
-__global__ void k_dilate_list(const __grid_constant__ MaskBatch<R, CAP> B, int forward) {
+__global__ void k_dilate_list(const __grid_constant__ MaskBatch<R, CAP> B, int forward, int core) {
     MEMBER;
     if (M.jb == B.ja) return;
     STAGE_LEVELS;
     DevLevelT<R> none{};
     ITEMS(K_NODE, lvs, none, M.gcand, M.gcand_count, B.P) {
         if (L.J == B.ja) return;
-        dilate_node(L, id, forward != 0);
+        // after CORE_HOPS hops: the patches of the core
+        if (dilate_node(L, id, forward != 0) && core) L.kflag[patch_of(L, id)] = 1;
     });
 }
 
@@ -551,14 +548,14 @@ __global__ void k_patch_scan_b(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
     const int j = B.ja + int(blockIdx.x);
     if (j > M.jb) return;
-    patch_scan_level(M.lvs[j]);
+    patch_scan_level(M.lvs[j], j == B.ja);
 }
 
-// the member's all-level and irregular lists (one block per member)
+// the member's all-level lists (one block per level)
 template <class R, int CAP>
 __global__ void k_concat_b(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
-    concat_lists(M.lvs, B.ja, M.jmax, M.all, M.all_count, M.irr, M.irr_count);
+    concat_lists(M.lvs, B.ja, M.jmax, M.lists);
 }
 
 // the point work lists of the member's levels from its all-level list
@@ -567,7 +564,7 @@ __global__ void k_wl_build_b(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
     STAGE_LEVELS;
     DevLevelT<R> none{};
-    ITEMS(K_NODE | K_EDGE, lvs, none, M.all, M.all_count, B.P) { wl_item(L, kind, id); });
+    ITEMS(K_NODE | K_EDGE, lvs, none, M.lists.all, M.lists.count, B.P) { wl_item(L, kind, id); });
 }
 
 }  // namespace
@@ -639,7 +636,8 @@ void launch_mask_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s
     go(k_flag_scan<R, CAP>, unsigned(jb - ja + 1), unsigned(b.nm), 1024, s, b, 2);
     go(k_cat<R, CAP>, 1u, unsigned(b.nm), 1024, s, b, 2);
     if (jb > ja) {
-        for (int h = 0; h < b.hops; ++h) go(k_dilate_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b, h % 2 == 0 ? 1 : 0);
+        for (int h = 0; h < b.hops; ++h)
+            go(k_dilate_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b, h % 2 == 0 ? 1 : 0, h + 1 == CORE_HOPS ? 1 : 0);
         go(k_ghost_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b, b.hops % 2 == 1 ? 1 : 0);
         go(k_covered_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     }
@@ -654,7 +652,7 @@ void launch_mask_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s
 template <class R, int CAP>
 void launch_concat_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s) {
     if (b.nm < 1 || b.nm > CAP) throw std::runtime_error("mask batch size");
-    go(k_concat_b<R, CAP>, 1u, unsigned(b.nm), 1024, s, b);
+    go(k_concat_b<R, CAP>, unsigned(b.jmax_max - b.ja + 1), unsigned(b.nm), 1024, s, b);
     go(k_wl_build_b<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
 }
 

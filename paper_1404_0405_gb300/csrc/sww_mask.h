@@ -11,17 +11,14 @@
 
 namespace sww {
 
-// One member's mask: its levels, the all-level active list of the grid before the
+// One member's mask: its levels, the all-level lists of the grid before the
 // mask, the candidate lists (built into the levels' cand/gcand arrays and
-// concatenated into cand/gcand), the rebuilt all-level and irregular lists, its
-// thresholds and counters.  Levels Jmin..jb take part (jb = min(top + 1, jmax)).
+// concatenated into cand/gcand), its thresholds and counters.  Levels Jmin..jb take part (jb = min(top + 1, jmax)).
 template <class R>
 struct MaskMember {
     const DevLevelT<R>* lvs;             // device array of levels 0..jmax
-    const int32_t* active;               // all-level active list before the mask
-    const int32_t* active_count;
+    GridLists lists;                     // all-level lists: the grid before the mask, then rebuilt
     int32_t *cand, *cand_count, *gcand, *gcand_count;
-    int32_t *all, *all_count, *irr, *irr_count;
     const double* thr;                   // eps_h, eps_u
     int32_t* sig_any;                    // [jmax + 2] per level: a significant point or a proposed patch
     unsigned long long* lstat;           // learned-proposal counters (misses, over, proposed) or null
@@ -53,8 +50,8 @@ void launch_mask_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s
 // proposal roll before a mask (post 0) or after it (post 1)
 template <class R, int CAP>
 void launch_proposal_batch(const MaskBatch<R, CAP>& b, unsigned grid, int post, cudaStream_t s);
-// the all-level and irregular lists of every member from its level lists, and the
-// levels' point work lists (grid: blocks per member of the list launch)
+// the all-level lists of every member from its level lists, and the levels' point
+// work lists (grid: blocks per member of the list launch)
 template <class R, int CAP>
 void launch_concat_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s);
 

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ DevLevelT<R> sl[MAXL];
     __shared__ int cnt[MAXL][WL_KINDS];
-    __shared__ int n_all, n_irr, start_ok;
+    __shared__ int n_core, n_irr, start_ok;
     __shared__ unsigned start_base;
     {
         const int words = int((a.jmax + 1) * sizeof(DevLevelT<R>) / sizeof(int));
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
             // a launch that follows a failed one leaves at once (its barrier count is stale)
             start_ok = *reinterpret_cast<volatile int*>(a.err) == 0;
             start_base = a.bar[GridBarrier::BASE];
-            n_all = *a.all_count, n_irr = *a.irr_count;
+            n_core = a.lists.count[1], n_irr = a.lists.count[2];
         }
         __syncthreads();
         if (!start_ok) return;
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
     }
     // the trend: the irregular patches' F and q one thread an item, then a regular patch
     // a team at a time (patches dealt out over the SMs first)
-    entry_items(a.irr_list, n_irr, 5, a.P, [&](int32_t ent, uint32_t local) {
+    entry_items(a.lists.irr, n_irr, 5, a.P, [&](int32_t ent, uint32_t local) {
         irregular_fq(lv[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), local, a.P, H);
     });
     {
@@ -213,13 +213,13 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
         const int team = int(threadIdx.x) / TM::NT;
         bool ok = true;
         if (team < TM::N)
-            ok = tile_sweep<R, P, TM::NT>(Team<TM::NT>{int(threadIdx.x) % TM::NT, unsigned(team + 1)}, lv, a.all_list, n_all,
+            ok = tile_sweep<R, P, TM::NT>(Team<TM::NT>{int(threadIdx.x) % TM::NT, unsigned(team + 1)}, lv, a.lists.core, n_core,
                                           int(team * gridDim.x + blockIdx.x), int(TM::N * gridDim.x), H, g,
                                           smem + team * Tile<R, P>::BYTES, a.err, limit);
         if (!__syncthreads_and(ok)) return;
     }
     if (!gb.sync()) return;
-    entry_items(a.irr_list, n_irr, 4, a.P, [&](int32_t ent, uint32_t local) {
+    entry_items(a.lists.irr, n_irr, 4, a.P, [&](int32_t ent, uint32_t local) {
         auto body = [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
             if (kind == K_NODE)
                 node_at(L, id, g);
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
     if (blockIdx.x == 0 && threadIdx.x == 0) a.bar[GridBarrier::BASE] = gb.target;
     const R dt = R(a.dt ? *a.dt : 0.0);
     const RKStageR<R> sr(a.st);
-    entry_items(a.all_list, n_all, 4, a.P, [&](int32_t ent, uint32_t local) {
+    entry_items(a.lists.core, n_core, 4, a.P, [&](int32_t ent, uint32_t local) {
         auto body = [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
             if (kind == K_NODE)
                 update_node(L, id, sr, dt);

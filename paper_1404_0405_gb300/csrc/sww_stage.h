@@ -10,7 +10,7 @@
 namespace sww {
 
 // Arguments of one persistent stage: levels (device array of jmax + 1 records),
-// the all-level work list, patch area P, the levels, the constants, the stage
+// the all-level lists, patch area P, the levels, the constants, the stage
 // coefficients and the time step, and the barrier state: STAGE_BAR_WORDS words, zero
 // before the first launch (the arrival count and its value when a launch begins, each
 // in its own 128-byte line), err set on a timed-out wait.
@@ -19,10 +19,7 @@ constexpr int STAGE_BAR_WORDS = 32 * 2;
 template <class R>
 struct StageArgs {
     const DevLevelT<R>* lvs;
-    const int32_t* all_list;
-    const int32_t* all_count;
-    const int32_t* irr_list;    // entries of all_list whose tile is not regular
-    const int32_t* irr_count;
+    GridLists lists;
     int P;
     int jmin, jtop, jmax;
     double H, g;
@@ -38,12 +35,11 @@ struct StageArgs {
 };
 
 // One member of an ensemble stage: its level records (contiguous, levels 0..jmax),
-// its all-level active list, its time step and its top level.
+// its all-level lists, its time step and its top level.
 template <class R>
 struct MemberRef {
     const DevLevelT<R>* lvs;
-    const int32_t* all_list;
-    const int32_t* all_count;
+    GridLists lists;
     double* dt;
     int jtop;
     unsigned long long* red;   // [RED_WORDS] reduction words (CFL step, live maxima; see RED_WORDS)
@@ -55,8 +51,6 @@ struct MemberRef {
     int j1;                    // top level of the inverse transform (min(jtop + 1, jmax))
     int jmax;
     int* err;                  // error flag of the member's bounded waits (barriers, bulk copies)
-    const int32_t* irr_list;   // entries of all_list whose tile is not regular
-    const int32_t* irr_count;
 };
 
 // One RK stage of nm members (m: device array of nm refs, nm <= 128) with a common

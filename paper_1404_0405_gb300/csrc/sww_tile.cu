@@ -3,7 +3,7 @@
 // regular:
 //
 //   k_tile_trend  one block per active patch at a time (blocks grouped per
-//                 member, striding over the member's all-level list): a regular
+//                 member, striding over the member's core list): a regular
 //                 patch runs tile_trend (F, q, div F, K, B, q F^perp from its tile in
 //                 shared memory, its geometry block brought in by a bulk copy one
 //                 patch ahead); the irregular ones (a pentagon or a pole within
@@ -65,13 +65,13 @@ __global__ void __launch_bounds__(TILE_TPB, tile_min_blocks<P>()) k_tile_trend(B
     const R H = R(a.H);
     // the irregular patches' items first, over the member's blocks
     const int lp = __ffs(a.P) - 1;
-    const uint32_t n = uint32_t(*mr->irr_count) * (5u << lp);
+    const uint32_t n = uint32_t(mr->lists.count[2]) * (5u << lp);
     for (uint32_t it = uint32_t(b) * blockDim.x + threadIdx.x; it < n; it += uint32_t(bpm) * blockDim.x) {
         const uint32_t e = (it >> lp) / 5;
-        const int32_t ent = mr->irr_list[e];
+        const int32_t ent = mr->lists.irr[e];
         irregular_fq(sl[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), it - ((e * 5) << lp), a.P, H);
     }
-    tile_sweep<R, P, TILE_TPB>(Team<TILE_TPB>{int(threadIdx.x), 0u}, sl, mr->all_list, *mr->all_count, b, bpm, H, R(a.g),
+    tile_sweep<R, P, TILE_TPB>(Team<TILE_TPB>{int(threadIdx.x), 0u}, sl, mr->lists.core, mr->lists.count[1], b, bpm, H, R(a.g),
                                smem, mr->err, COPY_WAIT_CYCLES);
 }
 
@@ -92,10 +92,10 @@ __global__ void __launch_bounds__(TILE_TPB) k_tile_irr(BatchArgs<R> a, int bpm) 
     stage_records(sl, mr, a.jmin);
     const R g = R(a.g);
     const int lp = __ffs(a.P) - 1;
-    const uint32_t n = uint32_t(*mr->irr_count) * (4u << lp);
+    const uint32_t n = uint32_t(mr->lists.count[2]) * (4u << lp);
     for (uint32_t it = uint32_t(b) * blockDim.x + threadIdx.x; it < n; it += uint32_t(bpm) * blockDim.x) {
         const uint32_t e = (it >> lp) / 4;
-        const int32_t ent = mr->irr_list[e];
+        const int32_t ent = mr->lists.irr[e];
         const DevLevelT<R>& L = sl[ent >> LVL_SHIFT];
         auto body = [&](const DevLevelT<R>& LL, int kind, int64_t id, int64_t) {
             if (kind == K_NODE)
