@@ -50,15 +50,6 @@ void ck(cudaError_t e, const char* what) {
     if (e != cudaSuccess) throw CudaError(std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-__global__ void k_set(double* p, double v) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *p = v;
-}
-
-// reduction words of the time step (see RED_WORDS): the maxima start at zero
-__global__ void k_reset_red(unsigned long long* red) {
-    if (blockIdx.x == 0 && threadIdx.x < RED_WORDS) red[threadIdx.x] = 0ull;
-}
-
 // per level: the active patch list's size at out[j], the live nodes at
 // out[jmax + 1 + j]
 template <class R>
@@ -144,7 +135,7 @@ struct Geometry {
             F.J = D.J, F.n = D.n, F.p = D.p, F.np = D.np, F.nelem = D.nelem, F.N = D.N, F.E = D.E, F.T = D.T;
             F.npatch = D.npatch, F.dx = D.dx, F.kx2 = D.kx2;
             F.en = D.en, F.et = D.et, F.tn = D.tn, F.te = D.te, F.deg = D.deg, F.ring_e = D.ring_e, F.ring_n = D.ring_n, F.f2c = D.f2c;
-            F.cor_i = D.cor_i, F.par = D.par, F.fe_kind = D.fe_kind, F.fe_ce = D.fe_ce, F.vst = D.vst;
+            F.cor_i = D.cor_i, F.par = D.par, F.fe_kind = D.fe_kind, F.fe_ce = D.fe_ce, F.fe_ot = D.fe_ot, F.vst = D.vst;
             F.c2f = D.c2f, F.mid = D.mid, F.half = D.half, F.mk_i = D.mk_i, F.rf_fi = D.rf_fi, F.rf_ci = D.rf_ci;
             F.ppar = D.ppar, F.pnbr = D.pnbr, F.pchild = D.pchild;
             F.thalo = D.thalo, F.tirr = D.tirr;
@@ -230,11 +221,7 @@ struct sww_handle {
     struct {
         uint8_t* refs = nullptr;    // device MemberRef array
         uint8_t* h_refs = nullptr;  // pinned staging of the refs
-        unsigned* bar = nullptr;
-        int* err = nullptr;
-        int* h_err = nullptr;
         cudaEvent_t ev = nullptr;
-        unsigned grid = 0;
         uint8_t* out = nullptr;     // device read-back records (BatchOut per member)
         uint8_t* h_out = nullptr;   // pinned copy
     } ens;
@@ -247,7 +234,8 @@ struct sww_handle {
     int32_t *d_counts = nullptr, *sig_any = nullptr;
     GridLists lists{};              // all-level lists
     int64_t irr_bound = 0;          // a bound on the entries whose tile is not regular
-    uint8_t* self_ref = nullptr;    // device MemberRef of this handle (its own trend launches)
+    BatchOut* out = nullptr;        // read-back record of a step (device and pinned copy)
+    BatchOut* h_out = nullptr;
     // candidate lists of the list-based mask (all levels)
     int32_t *cand = nullptr, *cand_count = nullptr, *gcand = nullptr, *gcand_count = nullptr;
     int64_t total_entries = 0;
@@ -259,7 +247,8 @@ struct sww_handle {
     double t = 0, last_dt = 0;
     int64_t steps = 0;
     bool has_state = false;
-    // captured steps: (part, top level, adapt, dt, stage blocks) -> graph and its kernel count
+    // captured steps: (part and size class, top level, adapt, dt, stage blocks) -> graph
+    // and its kernel count
     std::map<std::tuple<int, int, int, double, unsigned>, std::pair<cudaGraphExec_t, int64_t>> graphs;
     // tracing: per-class event pairs
     uint32_t prof_mask = 0;
@@ -299,10 +288,10 @@ struct sww_handle {
         if (h_counts) cudaFreeHost(h_counts);
         if (h_err) cudaFreeHost(h_err);
         if (ens.h_refs) cudaFreeHost(ens.h_refs);
-        if (ens.h_err) cudaFreeHost(ens.h_err);
         if (ens.h_out) cudaFreeHost(ens.h_out);
         if (ens.ev) cudaEventDestroy(ens.ev);
         if (h_dt) cudaFreeHost(h_dt);
+        if (h_out) cudaFreeHost(h_out);
         for (void* p : allocs) cudaFree(p);
         if (stream) cudaStreamDestroy(stream);
     }
@@ -368,6 +357,17 @@ void upload_geometry(Geometry& G, HostLevel& L, bool fine_side, bool coarse_side
         D.ptw = G.up_slots(L.ptw, 4);
         D.fe_kind = G.up(L.fe_kind);
         D.fe_ce = G.up(L.fe_ce);
+        // the other half of each half's coarse edge
+        std::vector<int32_t> first(L.E / 4 + 1, -1), ot(L.E, -1);
+        for (int64_t e = 0; e < L.E; ++e) {
+            if (L.fe_kind[e] == 2) continue;
+            int32_t& f = first[L.fe_ce[e]];
+            if (f < 0)
+                f = int32_t(e);
+            else
+                ot[e] = f, ot[f] = int32_t(e);
+        }
+        D.fe_ot = G.up(ot);
         D.vst = G.up_slots(L.vst, VST);
         D.vw = G.up_slots(L.vw, VST);
     }
@@ -608,67 +608,56 @@ template <class R>
 WorkT<R> work_all(const sww_handle* h) {
     return WorkT<R>{dlv<R>(h), h->lists.all, h->lists.count, h->S, h->grid_all};
 }
-// the patches that hold or border live points (CORE_HOPS), for passes over live points
-template <class R>
-WorkT<R> work_core(const sww_handle* h) {
-    return WorkT<R>{dlv<R>(h), h->lists.core, h->lists.count + 1, h->S, h->grid_all};
-}
-template <class R>
-WorkT<R> work_level(const sww_handle* h, int j) {
-    const DevLevelT<R>& L = lvl<R>(h)[j];
-    return WorkT<R>{nullptr, L.patches, L.npatches, h->S, h->grid_lv[j]};
-}
-template <class R>
-WorkT<R> work_level_core(const sww_handle* h, int j) {
-    const DevLevelT<R>& L = lvl<R>(h)[j];
-    return WorkT<R>{nullptr, L.clist, L.npatches + 1, h->S, h->grid_lv[j]};
-}
-
 // ------------------------------------------------------------------ sequences
 
-template <class R>
-void fill_ghosts(sww_handle* h) {
-    auto& lv = lvl<R>(h);
-    for (int j = h->cfg.jmin + 1; j <= h->jtop; ++j) {
-        Trace t(h, SWW_K_FILL);
-        launch_fill(lv[j], lv[j - 1], work_level<R>(h, j), h->stream);
-    }
-}
+// classes of the parts of launch_stage_batch_part
+constexpr int STAGE_PART_CLASS[5] = {SWW_K_FILL, SWW_K_TREND, SWW_K_IRREG, SWW_K_RESTRICT, SWW_K_UPDATE};
 
-// one trend evaluation (Sec. 3.1): ghosts, q/K/B/F/qF^perp on every level, then the
-// restriction of B, F and q F^perp from the top level down to Jmin
-template <class R>
-void trend(sww_handle* h) {
-    const int j0 = h->cfg.jmin;
-    cudaStream_t s = h->stream;
-    auto& lv = lvl<R>(h);
-    fill_ghosts<R>(h);
-    {
-        // the structured trend of every active patch, then the irregular patches'
-        // node and Coriolis terms (one member: this handle)
-        BatchArgs<R> a{reinterpret_cast<const MemberRef<R>*>(h->self_ref), 1, h->S, j0, h->jtop, h->cfg.H, h->cfg.g,
-                       RKStage{}, nullptr, nullptr, 0.0, nullptr};
-        { Trace t(h, SWW_K_TREND); ck(launch_tile_trend(a, h->total_entries, h->irr_bound, h->nsm, 1, s), "trend"); }
-        { Trace t(h, SWW_K_IRREG); ck(launch_tile_trend(a, h->total_entries, h->irr_bound, h->nsm, 2, s), "trend"); }
-    }
-    for (int j = h->jtop - 1; j >= j0; --j) {
-        { Trace t(h, SWW_K_RESTRICT); launch_restrict(lv[j], lv[j + 1], work_level<R>(h, j), s); }
-        { Trace t(h, SWW_K_NODE); launch_div(lv[j], work_level<R>(h, j), s); }
-    }
+// log2 of the active patches as of the last read-back: launches of a captured step get
+// their grids from it, so a step is captured again when the grid has doubled
+int size_class(const sww_handle* h) {
+    int64_t n = 1;
+    for (int j = h->cfg.jmin; j <= h->cfg.jmax; ++j) n += h->h_counts[j];
+    int c = 0;
+    while (n >>= 1) ++c;
+    return c;
 }
 
 template <class R>
-void update(sww_handle* h, const RKStage& st) {
-    Trace t(h, SWW_K_UPDATE);
-    launch_update(work_core<R>(h), st, h->dt, h->stream);
+MemberRef<R> member_ref(const sww_handle* h);
+
+// The handle's own phases as a batch of one: its record passed with each launch, and
+// bounds of its list entries per level for the grid sizes (the lists' lengths are read
+// on the device).
+template <class R>
+struct Self {
+    BatchArgs<R> a;
+    int64_t entries[16] = {};
+    explicit Self(const sww_handle* h) {
+        a = BatchArgs<R>{nullptr, 1, h->S, h->cfg.jmin, h->jtop, h->cfg.H, h->cfg.g, RKStage{}, 0.0, h->out, -1.0, -1.0,
+                         member_ref<R>(h)};
+        const int64_t cap = int64_t(1) << (size_class(h) + 1);
+        for (int j = h->cfg.jmin; j <= h->cfg.jmax; ++j) entries[j] = std::min<int64_t>(meta(h, j).npatch + 1, cap);
+    }
+};
+
+// one RK stage, a launch per phase (Sec. 3.1): ghosts, q/K/B/F/qF^perp on every level, the
+// restriction of B, F and q F^perp from the top level down to Jmin, the update
+template <class R>
+void stage_phases(sww_handle* h, const RKStage& st) {
+    Self<R> w(h);
+    w.a.st = st;
+    for (int part = 0; part < 5; ++part) {
+        Trace t(h, STAGE_PART_CLASS[part]);
+        ck(launch_stage_batch_part(w.a, w.entries, h->irr_bound, h->nsm, part, h->stream), "stage");
+    }
 }
 
 // trend and RK stage: one persistent cooperative launch, or one launch per phase
 template <class R>
 void stage(sww_handle* h, const RKStage& st) {
     if (!h->stage_blocks) {
-        trend<R>(h);
-        update<R>(h, st);
+        stage_phases<R>(h, st);
         return;
     }
     Trace t(h, SWW_K_STAGE);
@@ -687,15 +676,6 @@ int barrier_status(sww_handle* h) {
     return fail(SWW_E_TIMEOUT, "a bounded wait of the RK stage (grid barrier or bulk copy) timed out");
 }
 
-template <class R>
-void compute_dt(sww_handle* h) {
-    Trace t(h, SWW_K_DT);
-    count_launch(1);
-    k_reset_red<<<1, 32, 0, h->stream>>>(h->red);
-    launch_dt(work_core<R>(h), h->cfg.H, h->cfg.g, h->red, h->stream);
-    launch_dt_final<R>(dlv<R>(h), h->red, h->cfg.cfl, h->dt, h->stream);
-}
-
 // list sizes of every level into pinned host memory (read after the next sync)
 template <class R>
 void read_counts(sww_handle* h) {
@@ -704,6 +684,16 @@ void read_counts(sww_handle* h) {
     ck(cudaMemcpyAsync(h->h_counts, h->d_counts, sizeof(int32_t) * 2 * (h->cfg.jmax + 1), cudaMemcpyDeviceToHost,
                        h->stream),
        "counts");
+}
+
+// a step's read-back record into the handle's host copies
+void take_record(sww_handle* h, const BatchOut& o) {
+    *h->h_dt = o.dt;
+    *h->h_err = o.err;
+    for (int j = 0; j <= h->cfg.jmax && j < 16; ++j) {
+        h->h_counts[j] = o.counts[j];
+        h->h_counts[h->cfg.jmax + 1 + j] = o.live[j];
+    }
 }
 
 // top level with any live or ghost point (after the stream has synchronised)
@@ -824,15 +814,11 @@ void mask_only(sww_handle* h) {
 
 template <class R>
 void mask_and_inverse(sww_handle* h) {
-    const int j0 = h->cfg.jmin, j1 = std::min(h->jtop + 1, h->cfg.jmax);
-    cudaStream_t s = h->stream;
-    auto& lv = lvl<R>(h);
     mask_only<R>(h);
     // inverse transform of the retained coefficients, coarse to fine, ghosts per level
-    for (int j = j0 + 1; j <= j1; ++j) {
-        { Trace t(h, SWW_K_INVERSE); launch_inverse(lv[j], lv[j - 1], work_level_core<R>(h, j), s); }
-        { Trace t(h, SWW_K_FILL); launch_fill(lv[j], lv[j - 1], work_level<R>(h, j), s); }
-    }
+    Trace t(h, SWW_K_INVERSE);
+    Self<R> w(h);
+    ck(launch_batch_adapt_post(w.a, w.entries, w.a.one.j1, h->nsm, h->stream), "inverse");
 }
 
 // relative coefficient tolerance: eps, or eps^{3/2} when eps is read as the trend
@@ -841,13 +827,11 @@ double eps_coeff(const sww_config& c) { return c.regime == 1 ? c.eps * std::sqrt
 
 template <class R>
 void adapt(sww_handle* h, double eh, double eu) {
-    cudaStream_t s = h->stream;
-    { Trace t(h, SWW_K_COEFF); launch_details(work_core<R>(h), h->cfg.jmin, s); }
     {
-        Trace t(h, SWW_K_MASK);
-        ck(cudaMemsetAsync(h->red + 2, 0, 2 * sizeof(unsigned long long), s), "memset red");
-        launch_maxabs(work_core<R>(h), h->red, s);
-        launch_thresholds(h->red, eps_coeff(h->cfg), eh, eu, h->cfg.advect, h->thr, s);
+        Trace t(h, SWW_K_COEFF);
+        Self<R> w(h);
+        w.a.eps_h = eh, w.a.eps_u = eu;
+        ck(launch_batch_adapt_pre(w.a, w.entries, h->nsm, h->stream), "adapt");
     }
     mask_and_inverse<R>(h);
 }
@@ -872,46 +856,30 @@ const RKStage* stages(int rk, int& n) {
 }
 
 // One RK step with its partial transform and (optionally) adaptation; ends with the
-// device-to-host copies of the time step and the list sizes.  part 1 is what comes
-// before the RK stages (time step, RK base), part 2 what follows them; part 0 is the
-// whole step.
-// part 0: the whole step; 1: time step and RK base only; 2: after the stages
-// (partial transform, ghosts, adaptation, read-backs); 3: adaptation and
-// read-backs only (the rest ran batched over an ensemble); 4: the mask only
+// device-to-host copy of its read-back record.  part 0: the whole step; 4: the mask
+// only.
 template <class R>
 void one_step(sww_handle* h, double dt, bool do_adapt, int part = 0) {
-    const int j0 = h->cfg.jmin;
-    auto& lv = lvl<R>(h);
-    if (part == 4) {   // the mask alone (coefficients, thresholds and inverse batched)
+    if (part == 4) {   // the mask alone (the rest ran batched over an ensemble)
         mask_only<R>(h);
         return;
     }
-    if (part == 0 || part == 1) {
-        if (dt > 0) {
-            count_launch(1);
-            k_set<<<1, 32, 0, h->stream>>>(h->dt, dt);
-        } else {
-            compute_dt<R>(h);
-        }
-        { Trace t(h, SWW_K_UPDATE); launch_save_base(work_core<R>(h), h->stream); }
+    {
+        Trace t(h, SWW_K_DT);
+        Self<R> w(h);
+        ck(launch_batch_pre(w.a, w.entries, h->nsm, dt, h->stream), "time step");
     }
-    if (part == 0) {
-        int ns;
-        const RKStage* st = stages(h->cfg.rk, ns);
-        for (int k = 0; k < ns; ++k) stage<R>(h, st[k]);
-    }
-    if (part == 1) return;
-    if (part != 3) {
-        for (int j = h->jtop - 1; j >= j0; --j) {
-            Trace t(h, SWW_K_PARTIAL);
-            launch_partial(lv[j], lv[j + 1], work_level<R>(h, j), h->stream);
-        }
-        fill_ghosts<R>(h);
+    int ns;
+    const RKStage* st = stages(h->cfg.rk, ns);
+    for (int k = 0; k < ns; ++k) stage<R>(h, st[k]);
+    Self<R> w(h);
+    {
+        Trace t(h, SWW_K_PARTIAL);
+        ck(launch_batch_post(w.a, w.entries, h->nsm, h->stream), "partial transform");
     }
     if (do_adapt) adapt<R>(h, -1.0, -1.0);
-    read_counts<R>(h);
-    ck(cudaMemcpyAsync(h->h_dt, h->dt, sizeof(double), cudaMemcpyDeviceToHost, h->stream), "dt");
-    ck(cudaMemcpyAsync(h->h_err, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "err");
+    ck(launch_batch_out(w.a, h->stream), "read-back");
+    ck(cudaMemcpyAsync(h->h_out, h->out, sizeof(BatchOut), cudaMemcpyDeviceToHost, h->stream), "read-back");
 }
 
 // Run one step (or part of one) through a captured graph (eager when tracing).
@@ -922,7 +890,7 @@ void run_step_t(sww_handle* h, double dt, bool do_adapt, int part = 0) {
         return;
     }
     const unsigned mode = h->stage_blocks;
-    auto key = std::make_tuple(part, h->jtop, int(do_adapt), dt > 0 ? dt : -1.0, mode);
+    auto key = std::make_tuple(part * 64 + size_class(h), h->jtop, int(do_adapt), dt > 0 ? dt : -1.0, mode);
     auto it = h->graphs.find(key);
     if (it == h->graphs.end()) {
         if (h->graphs.size() >= 24) h->drop_graphs();
@@ -971,15 +939,9 @@ void ensure_ensemble(sww_handle* lead) {
     auto& E = lead->ens;
     if (E.refs) return;
     E.refs = lead->alloc<uint8_t>(sizeof(MemberRef<double>) * 128);
-    E.bar = lead->alloc<unsigned>(STAGE_BAR_WORDS);
-    E.err = lead->alloc<int>(1);
     E.out = lead->alloc<uint8_t>(sizeof(BatchOut) * 128);
-    ck(cudaMemset(E.bar, 0, STAGE_BAR_WORDS * sizeof(unsigned)), "memset");
-    ck(cudaMemset(E.err, 0, sizeof(int)), "memset");
     ck(cudaMallocHost(&E.h_refs, sizeof(MemberRef<double>) * 128), "cudaMallocHost");
-    ck(cudaMallocHost(&E.h_err, sizeof(int)), "cudaMallocHost");
     ck(cudaMallocHost(&E.h_out, sizeof(BatchOut) * 128), "cudaMallocHost");
-    *E.h_err = 0;
     ck(cudaEventCreateWithFlags(&E.ev, cudaEventDisableTiming), "cudaEventCreate");
 }
 
@@ -1016,8 +978,8 @@ BatchArgs<R> ensemble_refs(sww_handle* const* hs, int n, std::vector<int64_t>& e
             entries[j] += meta(hs[i], j).npatch + 1;
     int ns;
     const RKStage* st = stages(lead->cfg.rk, ns);
-    return BatchArgs<R>{reinterpret_cast<const MemberRef<R>*>(E.refs), n, lead->S, lead->cfg.jmin, jtop,
-                        lead->cfg.H, lead->cfg.g, st[0], E.bar, E.err, 0.0, E.out};
+    return BatchArgs<R>{reinterpret_cast<const MemberRef<R>*>(E.refs), n, lead->S, lead->cfg.jmin, jtop, lead->cfg.H,
+                        lead->cfg.g, st[0], 0.0, E.out, -1.0, -1.0, MemberRef<R>{}};
 }
 
 // One step of every member with the work batched over members (persistent = 3), on
@@ -1042,12 +1004,11 @@ void ensemble_phased(sww_handle* const* hs, int n, double dt, bool do_adapt) {
         Trace t(lead, SWW_K_DT);
         ck(launch_batch_pre(a, entries.data(), lead->nsm, dt, s), "batched ensemble step");
     }
-    static const int part_cls[5] = {SWW_K_FILL, SWW_K_TREND, SWW_K_IRREG, SWW_K_RESTRICT, SWW_K_UPDATE};
     for (int k = 0; k < ns; ++k) {
         Trace t(lead, SWW_K_STAGE);
         a.st = st[k];
         for (int part = 0; part < 5; ++part) {
-            Trace tp(lead, part_cls[part]);
+            Trace tp(lead, STAGE_PART_CLASS[part]);
             ck(launch_stage_batch_part(a, entries.data(), irr_entries, lead->nsm, part, s), "batched ensemble stage");
         }
     }
@@ -1231,15 +1192,8 @@ int create_handle(const sww_config* cfg, void* stream, std::shared_ptr<Geometry>
         ck(cudaMemset(h->thr, 0, 2 * sizeof(double)), "memset");
         ck(cudaMemset(h->dt, 0, sizeof(double)), "memset");
         h->jtop = cfg->jmax;
-        // the handle's own member record (the fields its trend launches read are fixed)
-        h->self_ref = h->alloc<uint8_t>(sizeof(MemberRef<double>));
-        if (fp32) {
-            MemberRef<float> r = member_ref<float>(h);
-            ck(cudaMemcpy(h->self_ref, &r, sizeof(r), cudaMemcpyHostToDevice), "member record");
-        } else {
-            MemberRef<double> r = member_ref<double>(h);
-            ck(cudaMemcpy(h->self_ref, &r, sizeof(r), cudaMemcpyHostToDevice), "member record");
-        }
+        h->out = h->alloc<BatchOut>(1);
+        ck(cudaMallocHost(&h->h_out, sizeof(BatchOut)), "cudaMallocHost");
         ck(cudaDeviceSynchronize(), "create");
         return SWW_OK;
     });
@@ -1404,6 +1358,7 @@ int sww_adapt(sww_handle* h, double eps_h, double eps_u) {
         by_prec(h, [&](auto r) {
             using R = decltype(r);
             Join jn(h);
+            ck(cudaMemsetAsync(h->red + 2, 0, 2 * sizeof(unsigned long long), h->stream), "memset red");
             adapt<R>(h, eps_h, eps_u);
             read_counts<R>(h);
             check_launch();
@@ -1478,6 +1433,7 @@ int sww_step(sww_handle* h, double dt, int nsteps, int do_adapt) {
                 check_launch();
             }
             ck(cudaStreamSynchronize(h->stream), "step");
+            take_record(h, *h->h_out);
             if (int rc = barrier_status(h)) return rc;
             double d = *h->h_dt;
             if (!std::isfinite(d) || !(d > 0)) return fail(SWW_E_NUMERIC, "non-finite or non-positive time step");
@@ -1515,8 +1471,9 @@ int sww_step_ensemble(sww_handle* const* hs, int n, double dt, int nsteps, int d
             ck(cudaEventRecord(h->ev_in, h->user), "join in");
             ck(cudaStreamWaitEvent(h->stream, h->ev_in, 0), "join in");
         }
-        auto finish = [&](sww_handle* h) -> int {
+        auto finish = [&](sww_handle* h, const BatchOut* o) -> int {
             ck(cudaStreamSynchronize(h->stream), "step");
+            take_record(h, *o);
             if (int rc = barrier_status(h)) return rc;
             double d = *h->h_dt;
             if (!std::isfinite(d) || !(d > 0)) return fail(SWW_E_NUMERIC, "non-finite or non-positive time step");
@@ -1543,16 +1500,7 @@ int sww_step_ensemble(sww_handle* const* hs, int n, double dt, int nsteps, int d
                 check_launch();
                 ck(cudaStreamSynchronize(hs[0]->stream), "step");
                 const BatchOut* o = reinterpret_cast<const BatchOut*>(hs[0]->ens.h_out);
-                for (int i = 0; i < n && rc == SWW_OK; ++i) {
-                    sww_handle* h = hs[i];
-                    *h->h_dt = o[i].dt;
-                    *h->h_err = o[i].err;
-                    for (int j = 0; j <= h->cfg.jmax && j < 16; ++j) {
-                        h->h_counts[j] = o[i].counts[j];
-                        h->h_counts[h->cfg.jmax + 1 + j] = o[i].live[j];
-                    }
-                    rc = finish(h);
-                }
+                for (int i = 0; i < n && rc == SWW_OK; ++i) rc = finish(hs[i], o + i);
             }
             join_out();
             return rc;
@@ -1580,11 +1528,11 @@ int sww_step_ensemble(sww_handle* const* hs, int n, double dt, int nsteps, int d
         for (int i = 0; i < n; ++i) launch(hs[i]);
         for (int s = 1; s < nsteps && rc == SWW_OK; ++s)
             for (int i = 0; i < n && rc == SWW_OK; ++i) {
-                rc = finish(hs[i]);
+                rc = finish(hs[i], hs[i]->h_out);
                 if (rc == SWW_OK) launch(hs[i]);
             }
         for (int i = 0; i < n; ++i) {
-            int r = finish(hs[i]);
+            int r = finish(hs[i], hs[i]->h_out);
             if (rc == SWW_OK) rc = r;
         }
         join_out();
@@ -1666,8 +1614,8 @@ int sww_forward(sww_handle* h) {
             using R = decltype(r);
             Join jn(h);
             Trace t(h, SWW_K_COEFF);
-            launch_details(work_core<R>(h), h->cfg.jmin, h->stream);
-            check_launch();
+            Self<R> w(h);
+            ck(launch_batch_details(w.a, w.entries, h->nsm, h->stream), "coefficients");
             return 0;
         });
         ck(cudaStreamSynchronize(h->stream), "forward");
@@ -1682,13 +1630,11 @@ int sww_inverse(sww_handle* h) {
         by_prec(h, [&](auto r) {
             using R = decltype(r);
             Join jn(h);
-            auto& lv = lvl<R>(h);
-            cudaStream_t s = h->stream;
-            launch_mark_support(work_all<R>(h), s);
-            for (int j = h->cfg.jmin + 1; j <= h->jtop; ++j) {
-                { Trace t(h, SWW_K_INVERSE); launch_inverse(lv[j], lv[j - 1], work_level_core<R>(h, j), s); }
-                { Trace t(h, SWW_K_FILL); launch_fill(lv[j], lv[j - 1], work_level<R>(h, j), s); }
-            }
+            launch_mark_support(work_all<R>(h), h->stream);
+            Trace t(h, SWW_K_INVERSE);
+            Self<R> w(h);
+            w.a.one.j1 = h->jtop;
+            ck(launch_batch_adapt_post(w.a, w.entries, h->jtop, h->nsm, h->stream), "inverse");
             check_launch();
             return 0;
         });

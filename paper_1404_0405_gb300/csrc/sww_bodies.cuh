@@ -184,18 +184,32 @@ __device__ __forceinline__ void for_items(const Lv* __restrict__ lvs, const Lv& 
 
 // ---------------------------------------------------------------------------- trend bodies (Sec. 3.1)
 
+// The bodies below load what they need in groups issued together and test the flags
+// afterwards: a short-circuit test per neighbour makes each load wait for the one before
+// (a divergence's six ring edges took 4 us of a stage's phase that way, 2 us now).
+
 // potential vorticity q = (curl u + f)/h at a triangle (dual cell)
 template <class R>
 __device__ __forceinline__ void pv_at(const DevLevelT<R>& L, int64_t t, R H) {
     if (L.advect) return;   // no velocity trend, no q
-    int32_t n0 = L.tn[t], n1 = L.tn[L.T + t], n2 = L.tn[2 * L.T + t];
-    int32_t c0 = L.te[t], c1 = L.te[L.T + t], c2 = L.te[2 * L.T + t];
-    if (!(L.nflag[n0] & AVAIL) || !(L.nflag[n1] & AVAIL) || !(L.nflag[n2] & AVAIL)) return;
-    if (!(L.eflag[c0 >> 1] & AVAIL) || !(L.eflag[c1 >> 1] & AVAIL) || !(L.eflag[c2 >> 1] & AVAIL)) return;
-    R circ = esign<R>(c0) * L.u[c0 >> 1] * geo<R>(L.d_e, c0 >> 1) + esign<R>(c1) * L.u[c1 >> 1] * geo<R>(L.d_e, c1 >> 1) +
-             esign<R>(c2) * L.u[c2 >> 1] * geo<R>(L.d_e, c2 >> 1);
-    R hv = geo<R>(L.kite, t) * (H + L.dh[n0]) + geo<R>(L.kite, L.T + t) * (H + L.dh[n1]) +
-           geo<R>(L.kite, 2 * L.T + t) * (H + L.dh[n2]);
+    int32_t n[3], c[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) n[k] = L.tn[k * L.T + t], c[k] = L.te[k * L.T + t];
+    uint8_t nf[3], ef[3];
+    R dh[3], u[3];
+    double de[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        nf[k] = L.nflag[n[k]], ef[k] = L.eflag[c[k] >> 1];
+        dh[k] = L.dh[n[k]], u[k] = L.u[c[k] >> 1], de[k] = L.d_e[c[k] >> 1];
+    }
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ok = ok & ((nf[k] & AVAIL) != 0) & ((ef[k] & AVAIL) != 0);
+    if (!ok) return;
+    R circ = esign<R>(c[0]) * u[0] * to_r<R>(de[0]) + esign<R>(c[1]) * u[1] * to_r<R>(de[1]) +
+             esign<R>(c[2]) * u[2] * to_r<R>(de[2]);
+    R hv = geo<R>(L.kite, t) * (H + dh[0]) + geo<R>(L.kite, L.T + t) * (H + dh[1]) + geo<R>(L.kite, 2 * L.T + t) * (H + dh[2]);
     R Av = geo<R>(L.A_v, t);
     if (viscous(L)) L.zeta[t] = circ / Av;
     L.q[t] = (circ / Av + geo<R>(L.f_v, t)) / (hv / Av);
@@ -204,32 +218,59 @@ __device__ __forceinline__ void pv_at(const DevLevelT<R>& L, int64_t t, R H) {
 // thickness flux F = h_e u at an edge
 template <class R>
 __device__ __forceinline__ void flux_at(const DevLevelT<R>& L, int64_t e, R H) {
-    if (!(L.eflag[e] & AVAIL)) return;
-    int32_t a = L.en[e], b = L.en[L.E + e];
-    if (!(L.nflag[a] & AVAIL) || !(L.nflag[b] & AVAIL)) return;
-    L.F[e] = R(0.5) * ((H + L.dh[a]) + (H + L.dh[b])) * L.u[e];
+    const uint8_t fe = L.eflag[e];
+    const int32_t a = L.en[e], b = L.en[L.E + e];
+    const R u = L.u[e];
+    const uint8_t fa = L.nflag[a], fb = L.nflag[b];
+    const R ha = L.dh[a], hb = L.dh[b];
+    if (!(((fe & AVAIL) != 0) & ((fa & AVAIL) != 0) & ((fb & AVAIL) != 0))) return;
+    L.F[e] = R(0.5) * ((H + ha) + (H + hb)) * u;
     // viscous form: diffusive height flux -nu grad(dh) (joins F in the divergence)
-    if (viscous(L)) L.Fd[e] = -R(L.nu) * (L.dh[b] - L.dh[a]) / geo<R>(L.d_e, e);
+    if (viscous(L)) L.Fd[e] = -R(L.nu) * (hb - ha) / geo<R>(L.d_e, e);
 }
+
+// the ring of node v: its edges' codes, and their flags, total height flux and lengths
+template <class R>
+struct Ring {
+    int32_t code[6];
+    uint8_t ef[6];
+    R F[6];
+    double le[6];
+    __device__ __forceinline__ Ring(const DevLevelT<R>& L, int64_t v) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) code[k] = L.ring_e[k * L.N + v];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const int64_t e = edge(k);
+            ef[k] = L.eflag[e], F[k] = L.F[e], le[k] = L.l_e[e];
+        }
+        if (viscous(L)) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) F[k] = F[k] + L.Fd[edge(k)];
+        }
+    }
+    // ring slot 5 of a pentagon is padded with -1: edge 0 is read and not used
+    __device__ __forceinline__ int64_t edge(int k) const { return code[k] < 0 ? 0 : code[k] >> 1; }
+};
 
 // divergence of the height flux (with the diffusive flux of the viscous form) at a node
 template <class R>
 __device__ __forceinline__ void div_at(const DevLevelT<R>& L, int64_t v) {
-    if (!(L.nflag[v] & AVAIL)) return;
+    const uint8_t fv = L.nflag[v];
     const int dg = L.deg[v];
+    const double Av = L.A_i[v];
+    if (!(fv & AVAIL)) return;
+    const Ring<R> g(L, v);
     R div = R(0);
     bool ok = true;   // every ring edge available (else nothing is written)
-    const bool visc = viscous(L);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        if (k >= dg) break;
-        const int32_t code = L.ring_e[k * L.N + v];
-        const int64_t e = code >> 1;
-        ok = ok && (L.eflag[e] & AVAIL);
-        div += esign<R>(code) * (visc ? L.F[e] + L.Fd[e] : L.F[e]) * geo<R>(L.l_e, e);
-    }
+    for (int k = 0; k < 6; ++k)
+        if (k < dg) {
+            ok = ok & ((g.ef[k] & AVAIL) != 0);
+            div += esign<R>(g.code[k]) * g.F[k] * to_r<R>(g.le[k]);
+        }
     if (!ok) return;
-    L.c[v] = div / geo<R>(L.A_i, v);
+    L.c[v] = div / to_r<R>(Av);
 }
 
 // a node whose divergence the restricted fluxes change: available, with a covered
@@ -253,23 +294,26 @@ __device__ __forceinline__ bool restricted_div_node(const DevLevelT<R>& L, int64
 template <class R>
 __device__ __forceinline__ void node_at(const DevLevelT<R>& L, int64_t v, R g) {
     if (L.advect) return div_at(L, v);   // prescribed velocity: no Bernoulli function
-    if (!(L.nflag[v] & AVAIL)) return;
+    const uint8_t fv = L.nflag[v];
     const int dg = L.deg[v];
+    if (!(fv & AVAIL)) return;
+    const Ring<R> r(L, v);
+    R u[6];
+    double de[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) u[k] = L.u[r.edge(k)], de[k] = L.d_e[r.edge(k)];
     R div = R(0), ke = R(0), du = R(0);
     bool ok = true;   // every ring edge available (else nothing is written)
     const bool visc = viscous(L);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        if (k >= dg) break;
-        const int32_t code = L.ring_e[k * L.N + v];
-        const int64_t e = code >> 1;
-        ok = ok && (L.eflag[e] & AVAIL);
-        R ue = L.u[e];
-        const R le = geo<R>(L.l_e, e);
-        div += esign<R>(code) * (visc ? L.F[e] + L.Fd[e] : L.F[e]) * le;
-        if (visc) du += esign<R>(code) * ue * le;
-        ke += R(0.25) * le * geo<R>(L.d_e, e) * ue * ue;
-    }
+    for (int k = 0; k < 6; ++k)
+        if (k < dg) {
+            ok = ok & ((r.ef[k] & AVAIL) != 0);
+            const R le = to_r<R>(r.le[k]);
+            div += esign<R>(r.code[k]) * r.F[k] * le;
+            if (visc) du += esign<R>(r.code[k]) * u[k] * le;
+            ke += R(0.25) * le * to_r<R>(de[k]) * u[k] * u[k];
+        }
     if (!ok) return;
     R A = geo<R>(L.A_i, v);
     // viscous form: -nu div u joins B (so that -grad B gains +nu grad div u)
@@ -352,42 +396,62 @@ __device__ __forceinline__ void update_edge(const DevLevelT<R>& L, int64_t e, co
 
 // ---------------------------------------------------------------------------- prolongation (Eqs. 1-2)
 
-// ghost node of level F from level C (inverse transform with zero coefficients)
+// ghost node i of level F (of its list WL_GN) from level C: inverse transform with zero
+// coefficients
 template <class R>
 __device__ __forceinline__ void fill_node(const DevLevelT<R>& F, const DevLevelT<R>& C, int64_t i) {
-    if (!(F.nflag[i] & GHOST)) return;
-    int32_t k = F.f2c[i];
+    const int32_t k = F.f2c[i];
     if (k >= 0) {
         F.dh[i] = C.dh[k];
         return;
     }
+    int32_t p[4], c[4];
+    R w[4], a[4], b[4];
+    uint8_t f[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) p[q] = F.par[q * F.N + i], w[q] = F.ptw[q * F.N + i];
+    // the parents of an odd node are even: each has a coarse node
+#pragma unroll
+    for (int q = 0; q < 4; ++q) f[q] = F.nflag[p[q]], a[q] = F.dh[p[q]], c[q] = F.f2c[p[q]];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = C.dh[c[q]];
     R s = R(0);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        int32_t p = F.par[q * F.N + i];
-        R v = (F.nflag[p] & LIVE) ? F.dh[p] : C.dh[F.f2c[p]];
-        s += F.ptw[q * F.N + i] * v;
+        const R v = (f[q] & LIVE) ? a[q] : b[q];
+        s += w[q] * v;
     }
     F.dh[i] = s;
 }
 
+// the half of a coarse edge with coarse velocity uc, from its own prediction and the
+// other half's, when neither is live
+template <class R>
+__device__ __forceinline__ R half_value(R P, R Po, R uc) { return P + R(0.5) * (R(2) * uc - P - Po); }
+
+// ghost edge i of level F (of its list WL_GE) from level C.  Both halves of a coarse edge
+// need both predictions, so the item of the first half writes the second too when that
+// is a ghost as well (then the list does not hold the second, see wl_item): 24
+// stencil entries a pair instead of 48.
 template <class R>
 __device__ __forceinline__ void fill_edge(const DevLevelT<R>& F, const DevLevelT<R>& C, int64_t i) {
-    if (F.advect || !(F.eflag[i] & GHOST)) return;   // prescribed velocity is kept everywhere
-    int kind = F.fe_kind[i];
-    R P = predict(F, C.u, i);
-    if (kind == 2) {
+    if (F.advect) return;   // prescribed velocity is kept everywhere
+    const int32_t o = F.fe_ot[i];
+    const int32_t E = F.fe_ce[i];
+    const R P = predict(F, C.u, i);
+    if (o < 0) {
         F.u[i] = P;
         return;
     }
-    int64_t E = F.fe_ce[i];
-    int32_t other = C.half[(kind == 0 ? C.E : 0) + E];
-    R uc = C.u[E];
-    if (F.eflag[other] & LIVE) {
-        F.u[i] = R(2) * uc - F.u[other];
+    const uint8_t fo = F.eflag[o];
+    const R uo = F.u[o], uc = C.u[E];
+    if (fo & LIVE) {
+        F.u[i] = R(2) * uc - uo;
     } else {
-        R Po = predict(F, C.u, other);
-        F.u[i] = P + R(0.5) * (R(2) * uc - P - Po);
+        const R Po = predict(F, C.u, o);
+        F.u[i] = half_value(P, Po, uc);
+        // only the first half reaches here when both are ghosts
+        if (fo & GHOST) F.u[o] = half_value(Po, P, uc);
     }
 }
 
@@ -401,15 +465,19 @@ template <class R>
 __device__ __forceinline__ void details_item(const DevLevelT<R>& L, const DevLevelT<R>& C, int kind, int64_t id,
                                              int64_t el) {
     if (kind == K_NODE) {
-        if (L.f2c[id] < 0 && (L.nflag[id] & LIVE)) L.hdet[id] = height_detail(L, id);
+        const int32_t k = L.f2c[id];
+        const uint8_t f = L.nflag[id];
+        if ((k < 0) & ((f & LIVE) != 0)) L.hdet[id] = height_detail(L, id);
     } else if (kind == K_EDGE) {
-        if (L.fe_kind[id] == 2 && (L.eflag[id] & LIVE)) L.ui[id] = L.u[id] - predict(L, C.u, id);
+        const int fk = L.fe_kind[id];
+        const uint8_t f = L.eflag[id];
+        if ((fk == 2) & ((f & LIVE) != 0)) L.ui[id] = L.u[id] - predict(L, C.u, id);
     } else {
         int32_t ce = L.f2c[el];
         if (ce < 0) return;
         int64_t E = id * C.nelem + ce;
         int32_t h0 = C.half[E], h1 = C.half[C.E + E];
-        if ((L.eflag[h0] & LIVE) || (L.eflag[h1] & LIVE)) {
+        if ((L.eflag[h0] | L.eflag[h1]) & LIVE) {
             R a = L.u[h0] - predict(L, C.u, h0);
             R b = L.u[h1] - predict(L, C.u, h1);
             L.ue[E] = R(0.5) * (a - b);
@@ -423,39 +491,64 @@ __device__ __forceinline__ void details_item(const DevLevelT<R>& L, const DevLev
 template <class R>
 __device__ __forceinline__ void inverse_a_item(const DevLevelT<R>& L, const DevLevelT<R>& C, int kind, int64_t id) {
     if (kind == K_NODE) {
-        if (!(L.nflag[id] & LIVE) || L.f2c[id] < 0) return;
-        int32_t k = L.f2c[id];
+        const uint8_t f = L.nflag[id];
+        const int32_t k = L.f2c[id];
+        if (!(f & LIVE) | (k < 0)) return;
         R s = C.dh[k];
 #pragma unroll
-        for (int q = 0; q < 12; ++q) {
-            int32_t m = C.mk_i[q * C.N + k];
-            if (m >= 0 && (L.nflag[m] & LIVE) && (L.nflag[m] & WASLIVE)) s -= C.mk_w[q * C.N + k] * L.hdet[m];
+        for (int g = 0; g < 12; g += 6) {
+            int32_t m[6];
+            R w[6], d[6];
+            uint8_t mf[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) m[q] = C.mk_i[(g + q) * C.N + k], w[q] = C.mk_w[(g + q) * C.N + k];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const int64_t x = m[q] < 0 ? 0 : m[q];   // padded with -1 at the pentagons
+                mf[q] = L.nflag[x], d[q] = L.hdet[x];
+            }
+#pragma unroll
+            for (int q = 0; q < 6; ++q)
+                if ((m[q] >= 0) & ((mf[q] & (LIVE | WASLIVE)) == (LIVE | WASLIVE))) s -= w[q] * d[q];
         }
         L.dh[id] = s;
         return;
     }
-    int64_t i = id;
-    if (L.advect || !(L.eflag[i] & LIVE)) return;   // a prescribed velocity is kept as set
-    int fk = L.fe_kind[i];
-    R Pr = predict(L, C.u, i);
-    if (fk == 2) {
-        L.u[i] = Pr + ((L.eflag[i] & WASLIVE) ? L.ui[i] : R(0));
-    } else {
-        int64_t E = L.fe_ce[i];
-        int32_t h0 = C.half[E], h1 = C.half[C.E + E];
-        int32_t other = fk == 0 ? h1 : h0;
-        R Po = predict(L, C.u, other);
-        R delta = R(0.5) * (R(2) * C.u[E] - Pr - Po);
-        R d = ((L.eflag[h0] | L.eflag[h1]) & WASLIVE) ? L.ue[E] : R(0);
+    const int64_t i = id;
+    if (L.advect) return;   // a prescribed velocity is kept as set
+    const uint8_t fi = L.eflag[i];
+    const int32_t o = L.fe_ot[i], E = L.fe_ce[i];
+    const int fk = L.fe_kind[i];
+    if (!(fi & LIVE)) return;
+    if (o < 0) {
+        const R Pr = predict(L, C.u, i), d = L.ui[i];
+        L.u[i] = Pr + ((fi & WASLIVE) ? d : R(0));
+        return;
+    }
+    // the halves of a coarse edge share their predictions: the first half's item writes
+    // both when both are live
+    const uint8_t fo = L.eflag[o];
+    if ((fk == 1) & ((fo & LIVE) != 0)) return;
+    const R Pr = predict(L, C.u, i), Po = predict(L, C.u, o);
+    const R uc = C.u[E], de = L.ue[E];
+    const R d = ((fi | fo) & WASLIVE) ? de : R(0);
+    {
+        const R delta = R(0.5) * (R(2) * uc - Pr - Po);
         L.u[i] = Pr + delta + (fk == 0 ? d : -d);
+    }
+    if (fo & LIVE) {
+        const R delta = R(0.5) * (R(2) * uc - Po - Pr);
+        L.u[o] = Po + delta - d;
     }
 }
 
 // (b) odd nodes from the even ones
 template <class R>
 __device__ __forceinline__ void inverse_b_item(const DevLevelT<R>& L, int64_t id) {
-    if (!(L.nflag[id] & LIVE) || L.f2c[id] >= 0) return;
-    R s = (L.nflag[id] & WASLIVE) ? L.hdet[id] : R(0);
+    const uint8_t f = L.nflag[id];
+    const int32_t k = L.f2c[id];
+    if (!(f & LIVE) | (k >= 0)) return;
+    R s = (f & WASLIVE) ? L.hdet[id] : R(0);
 #pragma unroll
     for (int q = 0; q < 4; ++q) s += L.ptw[q * L.N + id] * L.dh[L.par[q * L.N + id]];
     L.dh[id] = s;
@@ -464,33 +557,58 @@ __device__ __forceinline__ void inverse_b_item(const DevLevelT<R>& L, int64_t id
 #define ITEMS(KINDS, lvs, one, list, count, P) \
     for_items<KINDS>(lvs, one, list, count, P, [&](const auto& L, int kind, int64_t id, int64_t el)
 
-// restriction from F = level j+1 to C = level j at one item of C (Sec. 3.1): B by
-// injection at covered nodes, flux by R_F on faces of covered nodes, Coriolis
-// tendency by R_u where both ends are covered
+// restriction from F = level j+1 to C = level j (Sec. 3.1), at a covered node (list
+// WL_CN): B by injection
 template <class R>
-__device__ __forceinline__ void restrict_item(const DevLevelT<R>& L, const DevLevelT<R>& F, int kind, int64_t id) {
-    if (kind == K_NODE) {
-        if (!L.advect && (L.nflag[id] & COVERED)) L.B[id] = F.B[L.c2f[id]];
-        return;
-    }
-    int64_t i = id;
-    bool ca = L.nflag[L.en[i]] & COVERED, cb = L.nflag[L.en[L.E + i]] & COVERED;
-    if (ca || cb) {
-        // the restricted total height flux (mass flux plus the viscous form's
-        // diffusive flux) goes to F; the coarse diffusive flux is then zero
-        const bool visc = viscous(L);
-        R s = R(0);
+__device__ __forceinline__ void restrict_node(const DevLevelT<R>& L, const DevLevelT<R>& F, int64_t id) {
+    if (!L.advect) L.B[id] = F.B[L.c2f[id]];
+}
+
+// at an edge with a covered end (list WL_RE): flux by R_F, Coriolis tendency by R_u where
+// both ends are covered
+template <class R>
+__device__ __forceinline__ void restrict_edge(const DevLevelT<R>& L, const DevLevelT<R>& F, int64_t i) {
+    const uint8_t both = L.nflag[L.en[i]] & L.nflag[L.en[L.E + i]];
+    // the restricted total height flux (mass flux plus the viscous form's diffusive
+    // flux) goes to F; the coarse diffusive flux is then zero
+    const bool visc = viscous(L);
+    R s = R(0);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            const int32_t f = L.rf_fi[k * L.E + i];
-            s += L.rf_fw[k * L.E + i] * (visc ? F.F[f] + F.Fd[f] : F.F[f]);
+    for (int k = 0; k < 12; ++k) {
+        const int32_t f = L.rf_fi[k * L.E + i];
+        s += L.rf_fw[k * L.E + i] * (visc ? F.F[f] + F.Fd[f] : F.F[f]);
+    }
+#pragma unroll
+    for (int k = 0; k < 11; ++k) s += L.rf_cw[k * L.E + i] * F.c[L.rf_ci[k * L.E + i]];
+    L.F[i] = s / geo<R>(L.l_e, i);
+    if (visc) L.Fd[i] = R(0);
+    if ((both & COVERED) && !L.advect) L.Q[i] = R(0.5) * (F.Q[L.half[i]] + F.Q[L.half[L.E + i]]);
+}
+
+// partial height transform (Eq. Rh) at a covered node of C (list WL_CN) from F = the level
+// above: the details of M_k, all live, four at a time (the twelve one after another
+// are a chain of 36 loads)
+template <class R>
+__device__ __forceinline__ void partial_node(const DevLevelT<R>& C, const DevLevelT<R>& F, int64_t id) {
+    R s = F.dh[C.c2f[id]];
+#pragma unroll
+    for (int g = 0; g < 12; g += 4) {
+        int32_t m[4];
+        R w[4], d[4];
+        uint8_t mf[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) m[q] = C.mk_i[(g + q) * C.N + id], w[q] = C.mk_w[(g + q) * C.N + id];
+        // a pentagon's padded -1 reads M_k's first node instead, unused
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t x = m[q] < 0 ? C.mk_i[id] : m[q];
+            mf[q] = F.nflag[x], d[q] = height_detail(F, x);
         }
 #pragma unroll
-        for (int k = 0; k < 11; ++k) s += L.rf_cw[k * L.E + i] * F.c[L.rf_ci[k * L.E + i]];
-        L.F[i] = s / geo<R>(L.l_e, i);
-        if (visc) L.Fd[i] = R(0);
+        for (int q = 0; q < 4; ++q)
+            if ((m[q] >= 0) & ((mf[q] & LIVE) != 0)) s += w[q] * d[q];
     }
-    if (ca && cb && !L.advect) L.Q[i] = R(0.5) * (F.Q[L.half[i]] + F.Q[L.half[L.E + i]]);
+    C.dh[id] = s;
 }
 
 // ---------------------------------------------------------------------------- mask items (Sec. 2.3)
@@ -510,7 +628,10 @@ __device__ __forceinline__ float sig_thr<float>(double e) { return __double2floa
 
 template <class R>
 __device__ __forceinline__ bool sig_node(const DevLevelT<R>& F, int64_t i, R eh) {
-    if (F.f2c[i] < 0 && (F.nflag[i] & LIVE) && fabs(F.hdet[i]) >= eh) {
+    const int32_t k = F.f2c[i];
+    const uint8_t f = F.nflag[i];
+    const R d = F.hdet[i];
+    if ((k < 0) & ((f & LIVE) != 0) & (fabs(d) >= eh)) {
         F.sig[i] = 1;
         return true;
     }
@@ -519,7 +640,10 @@ __device__ __forceinline__ bool sig_node(const DevLevelT<R>& F, int64_t i, R eh)
 
 template <class R>
 __device__ __forceinline__ bool sig_edge(const DevLevelT<R>& F, int64_t i, R eu) {
-    if (F.fe_kind[i] == 2 && (F.eflag[i] & LIVE) && fabs(F.ui[i]) >= eu) {
+    const int k = F.fe_kind[i];
+    const uint8_t f = F.eflag[i];
+    const R d = F.ui[i];
+    if ((k == 2) & ((f & LIVE) != 0) & (fabs(d) >= eu)) {
         F.sig[F.en[i]] = 1;
         F.sig[F.en[F.E + i]] = 1;
         return true;
@@ -530,7 +654,8 @@ __device__ __forceinline__ bool sig_edge(const DevLevelT<R>& F, int64_t i, R eu)
 template <class R>
 __device__ __forceinline__ bool sig_cedge(const DevLevelT<R>& F, const DevLevelT<R>& C, int64_t i, R eu) {
     const int32_t h0 = C.half[i], h1 = C.half[C.E + i];
-    if (((F.eflag[h0] & LIVE) || (F.eflag[h1] & LIVE)) && fabs(F.ue[i]) >= eu) {
+    const R d = F.ue[i];
+    if ((((F.eflag[h0] | F.eflag[h1]) & LIVE) != 0) & (fabs(d) >= eu)) {
         F.sig[C.c2f[C.en[i]]] = 1;
         F.sig[C.c2f[C.en[C.E + i]]] = 1;
         F.sig[C.mid[i]] = 1;
@@ -841,7 +966,10 @@ __device__ __forceinline__ void wl_item(const DevLevelT<R>& L, int kind, int64_t
         wl_push(L, WL_DN, restricted_div_node(L, id), int32_t(id));
     } else {
         const uint8_t f = L.eflag[id];
-        wl_push(L, WL_GE, (f & GHOST) != 0, int32_t(id));
+        // the first half of a coarse edge fills a ghost second half too (fill_edge)
+        bool ge = (f & GHOST) != 0;
+        if (ge && L.fe_kind[id] == 1 && (L.eflag[L.fe_ot[id]] & GHOST)) ge = false;
+        wl_push(L, WL_GE, ge, int32_t(id));
         const bool r = ((L.nflag[L.en[id]] | L.nflag[L.en[L.E + id]]) & COVERED) != 0;
         wl_push(L, WL_RE, r, int32_t(id));
     }

@@ -14,7 +14,8 @@ constexpr uint8_t AVAIL = LIVE | GHOST;
 constexpr int NF = 8, NH = 32, NB = 24;
 constexpr int MLP_PARAMS = NF * NH + NH + NH + 1;   // W1[NF][NH], b1[NH], w2[NH], b2
 
-// Work lists of a level (DevLevelT::wl): ghost nodes, ghost edges, covered nodes,
+// Work lists of a level (DevLevelT::wl): ghost nodes, ghost edges (of two ghost halves of
+// a coarse edge only the first, which fills both), covered nodes,
 // edges with a covered end, nodes whose divergence the restriction changes; and the
 // level's live-node count, taken in the same pass (wl_n[WL_LIVE]).
 constexpr int WL_GN = 0, WL_GE = 1, WL_CN = 2, WL_RE = 3, WL_DN = 4, WL_KINDS = 5, WL_LIVE = 5, WL_WORDS = 6;
@@ -73,6 +74,7 @@ struct DevLevelT {
     const R* ptw;                  // [4*N] s~_km
     const int8_t* fe_kind;         // [E] 0/1 half of a coarse edge, 2 interior
     const int32_t* fe_ce;          // [E] coarse edge of a half
+    const int32_t* fe_ot;          // [E] the other half of that coarse edge (-1: interior edge)
     const int32_t* vst;            // [12*E] coarse stencil
     const R* vw;                   // [12*E]
     // coarse side of the pair (J, J+1)

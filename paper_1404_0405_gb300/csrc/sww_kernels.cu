@@ -29,98 +29,6 @@ constexpr int TPB = 256;
 
 #include "sww_bodies.cuh"
 
-// ---------------------------------------------------------------------------- list kernels
-
-template <class R>
-__global__ void k_update(const DevLevelT<R>* __restrict__ lvs, const int32_t* list, const int32_t* count, int P,
-                         RKStage st, const double* __restrict__ dtp) {
-    DevLevelT<R> none{};
-    R dt = R(dtp ? *dtp : 0.0);
-    const RKStageR<R> sr(st);
-    ITEMS(K_NODE | K_EDGE, lvs, none, list, count, P) {
-        if (kind == K_NODE)
-            update_node(L, id, sr, dt);
-        else
-            update_edge(L, id, sr, dt);
-    });
-}
-
-template <class R>
-__global__ void k_save_base(const DevLevelT<R>* __restrict__ lvs, const int32_t* list, const int32_t* count, int P) {
-    DevLevelT<R> none{};
-    ITEMS(K_NODE | K_EDGE, lvs, none, list, count, P) {
-        if (kind == K_NODE) {
-            if (L.nflag[id] & LIVE) L.dh0[id] = L.dh[id];
-        } else if (L.eflag[id] & LIVE) {
-            L.u0[id] = L.u[id];
-        }
-    });
-}
-
-// ghosts of level F from level C over F's work list
-template <class R>
-__global__ void k_fill(DevLevelT<R> F, DevLevelT<R> C, const int32_t* list, const int32_t* count, int P) {
-    ITEMS(K_NODE | K_EDGE, (const DevLevelT<R>*)nullptr, F, list, count, P) {
-        if (kind == K_NODE)
-            fill_node(L, C, id);
-        else
-            fill_edge(L, C, id);
-    });
-}
-
-// restriction from F = level j+1 to C = level j (Sec. 3.1)
-template <class R>
-__global__ void k_restrict(DevLevelT<R> C, DevLevelT<R> F, const int32_t* list, const int32_t* count, int P) {
-    ITEMS(K_NODE | K_EDGE, (const DevLevelT<R>*)nullptr, C, list, count, P) { restrict_item(L, F, kind, id); });
-}
-
-template <class R>
-__global__ void k_div(DevLevelT<R> C, const int32_t* list, const int32_t* count, int P) {
-    ITEMS(K_NODE, (const DevLevelT<R>*)nullptr, C, list, count, P) {
-        if (restricted_div_node(L, id)) div_at(L, id);
-    });
-}
-
-// R_h at covered nodes of C from level F (Eq. Rh; coefficients of non-live points are zero)
-template <class R>
-__global__ void k_partial(DevLevelT<R> C, DevLevelT<R> F, const int32_t* list, const int32_t* count, int P) {
-    ITEMS(K_NODE, (const DevLevelT<R>*)nullptr, C, list, count, P) {
-        if (!(L.nflag[id] & COVERED)) return;
-        R s = F.dh[L.c2f[id]];
-#pragma unroll
-        for (int q = 0; q < 12; ++q) {
-            int32_t m = L.mk_i[q * L.N + id];
-            if (m < 0 || !(F.nflag[m] & LIVE)) continue;
-            s += L.mk_w[q * L.N + id] * height_detail(F, m);
-        }
-        L.dh[id] = s;
-    });
-}
-
-// wavelet coefficients at live points (body details_item)
-template <class R>
-__global__ void k_details(const DevLevelT<R>* __restrict__ lvs, const int32_t* list, const int32_t* count, int P,
-                          int jmin) {
-    DevLevelT<R> none{};
-    ITEMS(K_NODE | K_EDGE | K_CEDGE, lvs, none, list, count, P) {
-        if (L.J == jmin) return;
-        details_item(L, lvs[L.J - 1], kind, id, el);
-    });
-}
-
-// inverse transform of the retained coefficients onto the live points of F:
-// (a) even nodes and all edges from level C, (b) odd nodes from the even ones
-// (bodies inverse_a_item, inverse_b_item)
-template <class R>
-__global__ void k_inverse_a(DevLevelT<R> F, DevLevelT<R> C, const int32_t* list, const int32_t* count, int P) {
-    ITEMS(K_NODE | K_EDGE, (const DevLevelT<R>*)nullptr, F, list, count, P) { inverse_a_item(L, C, kind, id); });
-}
-
-template <class R>
-__global__ void k_inverse_b(DevLevelT<R> F, const int32_t* list, const int32_t* count, int P) {
-    ITEMS(K_NODE, (const DevLevelT<R>*)nullptr, F, list, count, P) { inverse_b_item(L, id); });
-}
-
 // ---------------------------------------------------------------------------- reductions
 
 // block-wide reduction; `idle` is the operation's identity (fills lanes without a warp)
@@ -139,80 +47,9 @@ __device__ T block_reduce(T v, Op op, T* sh, T idle) {
     return v;
 }
 
-struct MaxOp {
-    __device__ unsigned long long operator()(unsigned long long a, unsigned long long b) const { return a > b ? a : b; }
-};
-struct MinOp {
-    __device__ unsigned long long operator()(unsigned long long a, unsigned long long b) const { return a < b ? a : b; }
-};
 struct AddOp {
     __device__ unsigned long long operator()(unsigned long long a, unsigned long long b) const { return a + b; }
 };
-
-// max |dh| over live nodes, max |u| over live edges: compared as keys of the field
-// type, widened to FP64 once per block (bit patterns of non-negative doubles)
-template <class R>
-__global__ void k_maxabs(const DevLevelT<R>* __restrict__ lvs, const int32_t* list, const int32_t* count, int S,
-                         unsigned long long* red) {
-    __shared__ unsigned long long sh[32];
-    DevLevelT<R> none{};
-    unsigned long long a = 0, b = 0;
-    ITEMS(K_NODE | K_EDGE, lvs, none, list, count, S) {
-        if (kind == K_NODE) {
-            if (L.nflag[id] & LIVE) a = max(a, abs_key(L.dh[id]));
-        } else if (L.eflag[id] & LIVE) {
-            b = max(b, abs_key(L.u[id]));
-        }
-    });
-    a = block_reduce(a, MaxOp(), sh, 0ull);
-    if (threadIdx.x == 0 && a) atomicMax(&red[2], dbits(key_value<R>(a)));
-    b = block_reduce(b, MaxOp(), sh, 0ull);
-    if (threadIdx.x == 0 && b) atomicMax(&red[3], dbits(key_value<R>(b)));
-}
-
-// largest omega^2 = f^2 + g h (pi/dx)^2 over live nodes (none with a prescribed
-// velocity, which carries no waves) and, per level, the largest |u| over live
-// edges with u != 0 (NaN left out, as dx/|u| with u NaN takes no part); the step
-// itself in k_dt_final
-template <class R>
-__global__ void k_dt(const DevLevelT<R>* __restrict__ lvs, const int32_t* list, const int32_t* count, int S, double H,
-                     double g, unsigned long long* red) {
-    __shared__ unsigned long long sh[32];
-    __shared__ unsigned long long slev[RED_WORDS - RED_LEVEL];
-    if (threadIdx.x < RED_WORDS - RED_LEVEL) slev[threadIdx.x] = 0ull;
-    __syncthreads();
-    DevLevelT<R> none{};
-    unsigned long long a = 0;
-    LevelMax um;
-    ITEMS(K_NODE | K_EDGE, lvs, none, list, count, S) {
-        if (kind == K_NODE) {
-            if (L.advect || !(L.nflag[id] & LIVE)) return;
-            a = max(a, dbits(omega2_at(L, id, H, g)));
-        } else if (L.eflag[id] & LIVE) {
-            const unsigned long long k = abs_key(L.u[id]);
-            if (k && k <= inf_key<R>()) um.add(L.J, k, slev);
-        }
-    });
-    um.flush(slev);
-    a = block_reduce(a, MaxOp(), sh, 0ull);   // synchronises the block: slev is complete
-    if (threadIdx.x == 0 && a) atomicMax(&red[0], a);
-    if (threadIdx.x < RED_WORDS - RED_LEVEL && slev[threadIdx.x]) atomicMax(&red[RED_LEVEL + threadIdx.x], slev[threadIdx.x]);
-}
-
-template <class R>
-__global__ void k_dt_final(const DevLevelT<R>* lvs, const unsigned long long* red, double cfl, double* dt) {
-    if (threadIdx.x || blockIdx.x) return;
-    *dt = cfl_step<R>(lvs, red, cfl);
-}
-
-// a prescribed velocity takes no part in the significance test (eps_u infinite
-// unless given)
-__global__ void k_thresholds(const unsigned long long* red, double eps, double eps_h, double eps_u, int advect,
-                             double* thr) {
-    if (threadIdx.x || blockIdx.x) return;
-    thr[0] = eps_h > 0 ? eps_h : eps * __longlong_as_double(static_cast<long long>(red[2]));
-    thr[1] = eps_u > 0 ? eps_u : advect ? INFINITY : eps * __longlong_as_double(static_cast<long long>(red[3]));
-}
 
 // Neumaier-compensated partial sums of mass and energy over level Jmin (dense)
 __device__ __forceinline__ void neumaier(double& s, double& c, double x) {
@@ -519,58 +356,6 @@ template <class R>
 static int64_t span(const DevLevelT<R>& L) { return L.E > L.N ? L.E : L.N; }
 
 template <class R>
-void launch_update(const WorkT<R>& W, const RKStage& st, const double* dt, cudaStream_t s) {
-    LIST(k_update<R>, W.lvs, W.list, W.count, W.S, st, dt);
-}
-template <class R>
-void launch_save_base(const WorkT<R>& W, cudaStream_t s) {
-    LIST(k_save_base<R>, W.lvs, W.list, W.count, W.S);
-}
-template <class R>
-void launch_fill(const DevLevelT<R>& F, const DevLevelT<R>& C, const WorkT<R>& W, cudaStream_t s) {
-    LIST(k_fill<R>, F, C, W.list, W.count, W.S);
-}
-template <class R>
-void launch_restrict(const DevLevelT<R>& C, const DevLevelT<R>& F, const WorkT<R>& W, cudaStream_t s) {
-    LIST(k_restrict<R>, C, F, W.list, W.count, W.S);
-}
-template <class R>
-void launch_div(const DevLevelT<R>& C, const WorkT<R>& W, cudaStream_t s) {
-    LIST(k_div<R>, C, W.list, W.count, W.S);
-}
-template <class R>
-void launch_partial(const DevLevelT<R>& C, const DevLevelT<R>& F, const WorkT<R>& W, cudaStream_t s) {
-    LIST(k_partial<R>, C, F, W.list, W.count, W.S);
-}
-template <class R>
-void launch_details(const WorkT<R>& W, int jmin, cudaStream_t s) {
-    LIST(k_details<R>, W.lvs, W.list, W.count, W.S, jmin);
-}
-template <class R>
-void launch_inverse(const DevLevelT<R>& F, const DevLevelT<R>& C, const WorkT<R>& W, cudaStream_t s) {
-    LIST(k_inverse_a<R>, F, C, W.list, W.count, W.S);
-    LIST(k_inverse_b<R>, F, W.list, W.count, W.S);
-}
-template <class R>
-void launch_maxabs(const WorkT<R>& W, unsigned long long* red, cudaStream_t s) {
-    LIST(k_maxabs<R>, W.lvs, W.list, W.count, W.S, red);
-}
-template <class R>
-void launch_dt(const WorkT<R>& W, double H, double g, unsigned long long* red, cudaStream_t s) {
-    LIST(k_dt<R>, W.lvs, W.list, W.count, W.S, H, g, red);
-}
-template <class R>
-void launch_dt_final(const DevLevelT<R>* lvs, const unsigned long long* red, double cfl, double* dt, cudaStream_t s) {
-    g_launches++;
-    k_dt_final<R><<<1, 32, 0, s>>>(lvs, red, cfl, dt);
-}
-void launch_thresholds(const unsigned long long* red, double eps, double eh, double eu, int advect, double* thr,
-                       cudaStream_t s) {
-    g_launches++;
-    k_thresholds<<<1, 32, 0, s>>>(red, eps, eh, eu, advect, thr);
-}
-
-template <class R>
 void launch_restrict_full(const DevLevelT<R>& C, const DevLevelT<R>& F, cudaStream_t s) {
     DENSE(k_restrict_full<R>, span(C), C, F);
 }
@@ -677,17 +462,6 @@ void launch_convert(const A* x, B* y, int64_t n, cudaStream_t s) {
 }
 
 #define SWW_INSTANTIATE(R)                                                                                   \
-    template void launch_update<R>(const WorkT<R>&, const RKStage&, const double*, cudaStream_t);            \
-    template void launch_save_base<R>(const WorkT<R>&, cudaStream_t);                                        \
-    template void launch_fill<R>(const DevLevelT<R>&, const DevLevelT<R>&, const WorkT<R>&, cudaStream_t);   \
-    template void launch_restrict<R>(const DevLevelT<R>&, const DevLevelT<R>&, const WorkT<R>&, cudaStream_t); \
-    template void launch_div<R>(const DevLevelT<R>&, const WorkT<R>&, cudaStream_t);                          \
-    template void launch_partial<R>(const DevLevelT<R>&, const DevLevelT<R>&, const WorkT<R>&, cudaStream_t); \
-    template void launch_details<R>(const WorkT<R>&, int, cudaStream_t);                                     \
-    template void launch_inverse<R>(const DevLevelT<R>&, const DevLevelT<R>&, const WorkT<R>&, cudaStream_t); \
-    template void launch_maxabs<R>(const WorkT<R>&, unsigned long long*, cudaStream_t);                      \
-    template void launch_dt<R>(const WorkT<R>&, double, double, unsigned long long*, cudaStream_t);          \
-    template void launch_dt_final<R>(const DevLevelT<R>*, const unsigned long long*, double, double*, cudaStream_t); \
     template void launch_restrict_full<R>(const DevLevelT<R>&, const DevLevelT<R>&, cudaStream_t);           \
     template void launch_mask<R>(const MaskArgsT<R>&, cudaStream_t);                                         \
     template void launch_live_all<R>(const DevLevelT<R>*, const Span&, const Span&, cudaStream_t);           \

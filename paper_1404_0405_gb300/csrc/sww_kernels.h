@@ -63,24 +63,6 @@ struct MaskArgsT {
 };
 
 // Launchers; R = double (FP64 form) or float (FP32 form), instantiated for both.
-// list kernels (active patches)
-template <class R> void launch_update(const WorkT<R>& W, const RKStage& st, const double* dt, cudaStream_t s);
-template <class R> void launch_save_base(const WorkT<R>& W, cudaStream_t s);
-template <class R> void launch_fill(const DevLevelT<R>& F, const DevLevelT<R>& C, const WorkT<R>& W, cudaStream_t s);
-// restriction of B, F, q F^perp from level j+1 (F) to level j (C); then the
-// divergence of the restricted fluxes at C's nodes
-template <class R> void launch_restrict(const DevLevelT<R>& C, const DevLevelT<R>& F, const WorkT<R>& W, cudaStream_t s);
-template <class R> void launch_div(const DevLevelT<R>& C, const WorkT<R>& W, cudaStream_t s);
-template <class R> void launch_partial(const DevLevelT<R>& C, const DevLevelT<R>& F, const WorkT<R>& W, cudaStream_t s);
-template <class R> void launch_details(const WorkT<R>& W, int jmin, cudaStream_t s);
-template <class R> void launch_inverse(const DevLevelT<R>& F, const DevLevelT<R>& C, const WorkT<R>& W, cudaStream_t s);
-template <class R> void launch_maxabs(const WorkT<R>& W, unsigned long long* red, cudaStream_t s);
-template <class R> void launch_dt(const WorkT<R>& W, double H, double g, unsigned long long* red, cudaStream_t s);
-template <class R>
-void launch_dt_final(const DevLevelT<R>* lvs, const unsigned long long* red, double cfl, double* dt, cudaStream_t s);
-void launch_thresholds(const unsigned long long* red, double eps, double eh, double eu, int advect, double* thr,
-                       cudaStream_t s);
-
 // dense level kernels (masks, initialisation, diagnostics)
 template <class R> void launch_restrict_full(const DevLevelT<R>& C, const DevLevelT<R>& F, cudaStream_t s);
 // full level F from the full level below (zero coefficients away from live points)

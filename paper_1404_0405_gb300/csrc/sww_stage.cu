@@ -234,7 +234,12 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
     for (int j = a.jtop - 1; j >= a.jmin; --j) {
         const DevLevelT<R>& C = lv[j];
         const DevLevelT<R>& F = lv[j + 1];
-        ph.run([&](int k, int64_t id) { restrict_item(C, F, k == 0 ? K_NODE : K_EDGE, id); });
+        ph.run([&](int k, int64_t id) {
+            if (k == 0)
+                restrict_node(C, F, id);
+            else
+                restrict_edge(C, F, id);
+        });
         ph.first(C, cnt, j, WL_DN, -1);
         if (!gb.sync()) return;
         ph.run([&](int, int64_t id) { div_at(C, id); });

@@ -53,18 +53,18 @@ struct MemberRef {
     int* err;                  // error flag of the member's bounded waits (barriers, bulk copies)
 };
 
-// One RK stage of nm members (m: device array of nm refs, nm <= 128) with a common
-// patch area P, Jmin, mean depth H and gravity g.
+// The phases of a step over nm members (m: device array of nm refs, nm <= 128; null: the
+// one member `one`) with a common patch area P, Jmin, mean depth H and gravity g.
 template <class R>
 struct BatchArgs {
     const MemberRef<R>* m;
     int nm, P, jmin, jtop_max;
     double H, g;
     RKStage st;
-    unsigned* bar;
-    int* err;
-    double dt_given;   // phases before the stages: > 0 sets every member's time step
-    void* out;         // read-back records, one per member (BatchOut, below)
+    double dt_given;       // phases before the stages: > 0 sets every member's time step
+    void* out;             // read-back records, one per member (BatchOut, below)
+    double eps_h, eps_u;   // > 0: every member's thresholds, instead of relative ones
+    MemberRef<R> one;
 };
 
 // Read-back record of one member after a batched step: dt, the error flag, and the
@@ -99,13 +99,10 @@ template <class R>
 cudaError_t launch_tile_trend(const BatchArgs<R>& a, int64_t entries, int64_t irr_entries, int nsm, int parts,
                               cudaStream_t s);
 // One RK stage as one regular launch per phase over all members (level-serial
-// phases once per level); level_entries[j] bounds the members' level-j list
-// entries in total, irr_entries their irregular entries (for the grid sizes).
-template <class R>
-cudaError_t launch_stage_batch_phases(const BatchArgs<R>& a, const int64_t* level_entries, int64_t irr_entries, int nsm,
-                                      cudaStream_t s);
-// The same stage in parts: 0 the ghosts, 1 the structured trend, 2 the irregular
-// patches, 3 the restrictions and divergences level by level, 4 the update.
+// phases once per level), in parts: 0 the ghosts, 1 the structured trend, 2 the
+// irregular patches, 3 the restrictions and divergences level by level, 4 the update.
+// level_entries[j] bounds the members' level-j list entries in total, irr_entries
+// their irregular entries (for the grid sizes).
 template <class R>
 cudaError_t launch_stage_batch_part(const BatchArgs<R>& a, const int64_t* level_entries, int64_t irr_entries, int nsm,
                                     int part, cudaStream_t s);
@@ -117,6 +114,12 @@ cudaError_t launch_batch_pre(const BatchArgs<R>& a, const int64_t* level_entries
 // ghosts (Jmin+1 up to the top) of every member.
 template <class R>
 cudaError_t launch_batch_post(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);
+// Every member's ghosts, Jmin+1 up to the top.
+template <class R>
+cudaError_t launch_batch_fill(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);
+// The wavelet coefficients of every live point and the live maxima.
+template <class R>
+cudaError_t launch_batch_details(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);
 // Before the members' masks: wavelet coefficients, live maxima and thresholds.
 template <class R>
 cudaError_t launch_batch_adapt_pre(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);

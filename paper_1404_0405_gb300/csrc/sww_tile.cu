@@ -56,11 +56,11 @@ template <int P>
 constexpr int tile_min_blocks() { return P >= 16 ? 4 : 5; }
 
 template <class R, int P>
-__global__ void __launch_bounds__(TILE_TPB, tile_min_blocks<P>()) k_tile_trend(BatchArgs<R> a, int bpm) {
+__global__ void __launch_bounds__(TILE_TPB, tile_min_blocks<P>()) k_tile_trend(const __grid_constant__ BatchArgs<R> a, int bpm) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ DevLevelT<R> sl[MAXL];
     const int m = blockIdx.x / bpm, b = blockIdx.x % bpm;
-    const MemberRef<R>* mr = a.m + m;
+    const MemberRef<R>* mr = a.m ? a.m + m : &a.one;
     stage_records(sl, mr, a.jmin);
     const R H = R(a.H);
     // the irregular patches' items first, over the member's blocks
@@ -85,10 +85,10 @@ __global__ void __launch_bounds__(TILE_TPB) k_tile_geo(DevLevelT<R> L, R* out) {
 }
 
 template <class R>
-__global__ void __launch_bounds__(TILE_TPB) k_tile_irr(BatchArgs<R> a, int bpm) {
+__global__ void __launch_bounds__(TILE_TPB, 5) k_tile_irr(const __grid_constant__ BatchArgs<R> a, int bpm) {
     __shared__ DevLevelT<R> sl[MAXL];
     const int m = blockIdx.x / bpm, b = blockIdx.x % bpm;
-    const MemberRef<R>* mr = a.m + m;
+    const MemberRef<R>* mr = a.m ? a.m + m : &a.one;
     stage_records(sl, mr, a.jmin);
     const R g = R(a.g);
     const int lp = __ffs(a.P) - 1;
@@ -151,7 +151,7 @@ cudaError_t launch_trend_p(const BatchArgs<R>& a, int64_t entries, int64_t irr_e
 template <class R>
 cudaError_t launch_tile_trend(const BatchArgs<R>& a, int64_t entries, int64_t irr_entries, int nsm, int parts,
                               cudaStream_t s) {
-    if (a.nm < 1 || a.nm > MAXM) return cudaErrorInvalidValue;
+    if (a.nm < 1 || a.nm > MAXM || (!a.m && a.nm != 1)) return cudaErrorInvalidValue;
     switch (a.P) {
         case 16: return launch_trend_p<R, 4>(a, entries, irr_entries, nsm, parts, s);
         case 64: return launch_trend_p<R, 8>(a, entries, irr_entries, nsm, parts, s);
