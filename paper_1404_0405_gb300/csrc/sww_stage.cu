@@ -20,10 +20,14 @@
 // blocks, one patch per 512-thread block and a barrier of 304 blocks; 148 and 93 us
 // now.  The barrier itself costs 1.4 us.
 //
-// Loads of this translation unit bypass L1 (compiled with -dlcm=cg): values written
-// by other blocks in one phase are read in the next.  Every barrier wait is bounded:
-// after about two seconds a block sets the error flag and the kernel returns; so does
-// the wait for a patch's geometry block (a bulk copy).
+// Values written by other blocks in one phase are read in the next: the barrier's
+// release and acquire at GPU scope, between two block barriers, order them (the acquire
+// also drops the SM's stale L1 lines), so loads may use L1, where the gathers of
+// neighbouring items meet: with L1 bypassed a stage of the 23 400-cell jet took 79 us
+// instead of 75 (FP32) and 136 instead of 131 (FP64).
+//
+// Every barrier wait is bounded: after about two seconds a block sets the error flag and
+// the kernel returns; so does the wait for a patch's geometry block (a bulk copy).
 #include <cuda_runtime.h>
 
 #include <algorithm>
