@@ -90,7 +90,8 @@ typedef struct {
                           The ABI's double arrays are converted at the boundary.     */
     int persistent;    /* RK stages.  0: one cooperative launch per stage (all phases of
                           the trend and the update, grid barriers between them) for a
-                          handle stepping alone, one launch per phase inside
+                          handle stepping alone on up to 16383 active patches, one launch
+                          per phase on larger grids and inside
                           sww_step_ensemble (the members' steps then overlap); 3:
                           inside sww_step_ensemble, one regular launch per phase of
                           the step over all members, each member's mask on its own

@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "grid.h"
+#include "pdl.cuh"
 #include "sww.h"
 #include "sww_core.cuh"
 #include "sww_internal.h"
@@ -622,6 +623,20 @@ int size_class(const sww_handle* h) {
     while (n >>= 1) ++c;
     return c;
 }
+// From 2^14 active patches a stage is one launch per phase instead of one cooperative
+// launch: the phases fill the GPU then, and their kernels keep more warps resident (FP32
+// turbulence, us per step persistent / phases: 3 400 patches 768 / 813, 13 640 1857 /
+// 1848, 52 632 6531 / 6076).
+constexpr int PHASES_CLASS = 14;
+// short kernels are chained: by the size class for a handle alone (its launches are
+// captured per class), by the members' active patches for a batch
+bool chained(const sww_handle* h) { return (int64_t(2) << size_class(h)) <= CHAIN_PATCHES; }
+bool chained(sww_handle* const* hs, int n) {
+    int64_t p = 0;
+    for (int i = 0; i < n; ++i)
+        for (int j = hs[i]->cfg.jmin; j <= hs[i]->cfg.jmax; ++j) p += hs[i]->h_counts[j];
+    return p <= CHAIN_PATCHES;
+}
 
 template <class R>
 MemberRef<R> member_ref(const sww_handle* h);
@@ -634,8 +649,8 @@ struct Self {
     BatchArgs<R> a;
     int64_t entries[16] = {};
     explicit Self(const sww_handle* h) {
-        a = BatchArgs<R>{nullptr, 1, h->S, h->cfg.jmin, h->jtop, h->cfg.H, h->cfg.g, RKStage{}, 0.0, h->out, -1.0, -1.0,
-                         member_ref<R>(h)};
+        a = BatchArgs<R>{nullptr, 1, h->S, h->cfg.jmin, h->jtop, h->cfg.H, h->cfg.g, RKStage{}, 0.0, h->out, chained(h), -1.0,
+                         -1.0, member_ref<R>(h)};
         const int64_t cap = int64_t(1) << (size_class(h) + 1);
         for (int j = h->cfg.jmin; j <= h->cfg.jmax; ++j) entries[j] = std::min<int64_t>(meta(h, j).npatch + 1, cap);
     }
@@ -656,7 +671,7 @@ void stage_phases(sww_handle* h, const RKStage& st) {
 // trend and RK stage: one persistent cooperative launch, or one launch per phase
 template <class R>
 void stage(sww_handle* h, const RKStage& st) {
-    if (!h->stage_blocks) {
+    if (!h->stage_blocks || size_class(h) >= PHASES_CLASS) {
         stage_phases<R>(h, st);
         return;
     }
@@ -802,6 +817,7 @@ void mask_only(sww_handle* h) {
     Trace tm(h, SWW_K_MASK);
     MaskBatch<R, 1> b{};
     mask_batch_head(b, h, 1, j1, h->cfg.jmax);
+    b.chain = chained(h);
     b.m[0] = mask_member<R>(h);
     launch_proposal_batch(b, h->grid_all, 0, s);
     if (list_mask(h))
@@ -979,7 +995,7 @@ BatchArgs<R> ensemble_refs(sww_handle* const* hs, int n, std::vector<int64_t>& e
     int ns;
     const RKStage* st = stages(lead->cfg.rk, ns);
     return BatchArgs<R>{reinterpret_cast<const MemberRef<R>*>(E.refs), n, lead->S, lead->cfg.jmin, jtop, lead->cfg.H,
-                        lead->cfg.g, st[0], 0.0, E.out, -1.0, -1.0, MemberRef<R>{}};
+                        lead->cfg.g, st[0], 0.0, E.out, chained(hs, n), -1.0, -1.0, MemberRef<R>{}};
 }
 
 // One step of every member with the work batched over members (persistent = 3), on
@@ -1034,6 +1050,7 @@ void ensemble_phased(sww_handle* const* hs, int n, double dt, bool do_adapt) {
                 jmax_max = std::max(jmax_max, hs[i]->cfg.jmax);
             }
             mask_batch_head(*b, lead, n, jb_max, jmax_max);
+            b->chain = a.chain;
             // blocks per member of the list passes: two waves of 8 blocks of 256 per SM
             // over all members (measured 8 % faster than one wave on the 64-member jet)
             const unsigned grid = unsigned(std::max(1, std::min<int>(int(lead->grid_all), 16 * lead->nsm / n)));

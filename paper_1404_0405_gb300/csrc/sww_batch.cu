@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "pdl.cuh"
 #include "sww_core.cuh"
 #include "sww_kernels.h"
 #include "sww_stage.h"
@@ -101,6 +102,7 @@ constexpr int phase_blocks() {
 
 template <class R, int PH>
 __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const __grid_constant__ BatchArgs<R> a, int j, int bpm) {
+    chain_wait();
     const int m = blockIdx.x / bpm, b = blockIdx.x % bpm;
     const MemberRef<R>* mr = a.m ? a.m + m : &a.one;
     // one block per member
@@ -272,8 +274,7 @@ int batch_bpm(const BatchArgs<R>& a, int64_t entries, int slots, int nsm) {
 template <int PH, class R>
 cudaError_t batch_go(const BatchArgs<R>& a, int j, int bpm, cudaStream_t s) {
     count_launch(1);
-    k_phase<R, PH><<<unsigned(a.nm * bpm), BATCH_TPB, 0, s>>>(a, j, bpm);
-    return cudaGetLastError();
+    return launch_chain(a.chain, k_phase<R, PH>, dim3(unsigned(a.nm * bpm)), dim3(BATCH_TPB), 0, s, a, j, bpm);
 }
 
 template <class R>

@@ -30,6 +30,7 @@
 
 #include "sww_core.cuh"
 #include "sww_kernels.h"
+#include "pdl.cuh"
 #include "sww_mask.h"
 
 namespace sww {
@@ -40,7 +41,10 @@ namespace {
 
 constexpr int TPB = 256;
 
-#define MEMBER const MaskMember<R>& M = B.m[blockIdx.y]
+// the member of this block; waits for the launch before (pdl.cuh)
+#define MEMBER    \
+    chain_wait(); \
+    const MaskMember<R>& M = B.m[blockIdx.y]
 
 constexpr int MAXL = 12;
 
@@ -571,10 +575,11 @@ __global__ void k_wl_build_b(const __grid_constant__ MaskBatch<R, CAP> B) {
 
 namespace {
 // one launch of `kernel` over gx blocks per member (threads: TPB unless given)
-template <class K, class... A>
-void go(K kernel, unsigned gx, unsigned nm, unsigned threads, cudaStream_t s, const A&... args) {
+template <class R, int CAP, class K, class... A>
+void go(K kernel, unsigned gx, unsigned nm, unsigned threads, cudaStream_t s, const MaskBatch<R, CAP>& b, const A&... args) {
     count_launch(1);
-    kernel<<<dim3(std::max(gx, 1u), nm), threads, 0, s>>>(args...);
+    if (launch_chain(b.chain, kernel, dim3(std::max(gx, 1u), nm), dim3(threads), 0, s, b, args...) != cudaSuccess)
+        throw std::runtime_error("mask launch");
 }
 }  // namespace
 

@@ -35,6 +35,7 @@ struct MaskMember {
 template <class R, int CAP>
 struct MaskBatch {
     int nm, P, ja, jb_max, jmax_max, hops, rings;
+    bool chain;   // chained launches (pdl.cuh)
     Span patches, patches_f, props;
     MaskMember<R> m[CAP];
 };

@@ -63,6 +63,7 @@ struct BatchArgs {
     RKStage st;
     double dt_given;       // phases before the stages: > 0 sets every member's time step
     void* out;             // read-back records, one per member (BatchOut, below)
+    bool chain;            // chained launches (pdl.cuh)
     double eps_h, eps_u;   // > 0: every member's thresholds, instead of relative ones
     MemberRef<R> one;
 };

@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "pdl.cuh"
 #include "sww_core.cuh"
 #include "sww_kernels.h"
 #include "sww_stage.h"
@@ -59,6 +60,7 @@ template <class R, int P>
 __global__ void __launch_bounds__(TILE_TPB, tile_min_blocks<P>()) k_tile_trend(const __grid_constant__ BatchArgs<R> a, int bpm) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ DevLevelT<R> sl[MAXL];
+    chain_wait();
     const int m = blockIdx.x / bpm, b = blockIdx.x % bpm;
     const MemberRef<R>* mr = a.m ? a.m + m : &a.one;
     stage_records(sl, mr, a.jmin);
@@ -87,6 +89,7 @@ __global__ void __launch_bounds__(TILE_TPB) k_tile_geo(DevLevelT<R> L, R* out) {
 template <class R>
 __global__ void __launch_bounds__(TILE_TPB, 5) k_tile_irr(const __grid_constant__ BatchArgs<R> a, int bpm) {
     __shared__ DevLevelT<R> sl[MAXL];
+    chain_wait();
     const int m = blockIdx.x / bpm, b = blockIdx.x % bpm;
     const MemberRef<R>* mr = a.m ? a.m + m : &a.one;
     stage_records(sl, mr, a.jmin);
@@ -131,8 +134,7 @@ cudaError_t launch_trend_p(const BatchArgs<R>& a, int64_t entries, int64_t irr_e
     const int cap = std::max(1, per_sm * nsm / a.nm);
     const int bpm = int(std::max<int64_t>(1, std::min<int64_t>((entries + a.nm - 1) / a.nm, cap)));
     count_launch(1);
-    k_tile_trend<R, P><<<unsigned(a.nm * bpm), TILE_TPB, smem, s>>>(a, bpm);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chain(a.chain, k_tile_trend<R, P>, dim3(unsigned(a.nm * bpm)), dim3(TILE_TPB), smem, s, a, bpm);
     if (e != cudaSuccess) return e;
     }
     if (!(parts & 2)) return cudaSuccess;
@@ -142,8 +144,7 @@ cudaError_t launch_trend_p(const BatchArgs<R>& a, int64_t entries, int64_t irr_e
     const int bpm2 = int(std::max<int64_t>(1, std::min<int64_t>((items + TILE_TPB - 1) / TILE_TPB,
                                                                    std::max(1, 16 * nsm / a.nm))));
     count_launch(1);
-    k_tile_irr<R><<<unsigned(a.nm * bpm2), TILE_TPB, 0, s>>>(a, bpm2);
-    return cudaGetLastError();
+    return launch_chain(a.chain, k_tile_irr<R>, dim3(unsigned(a.nm * bpm2)), dim3(TILE_TPB), 0, s, a, bpm2);
 }
 
 }  // namespace
