@@ -148,14 +148,25 @@ def _ptr(a):
     raise TypeError(type(a))
 
 
+def _addr(a):
+    """Address of a numpy array or a torch tensor."""
+    return a.data_ptr() if hasattr(a, "data_ptr") else _ptr(a)[0]
+
+
+_current_stream = None   # torch.cuda.current_stream once torch is known to have CUDA
+
+
 def _default_stream():
-    try:
-        import torch
-        if torch.cuda.is_available():
-            return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    except ImportError:
-        pass
-    return ctypes.c_void_p(None)
+    global _current_stream
+    if _current_stream is None:
+        try:
+            import torch
+            if not torch.cuda.is_available():
+                return None
+            _current_stream = torch.cuda.current_stream
+        except ImportError:
+            return None
+    return _current_stream().cuda_stream
 
 
 def step_ensemble(models, dt=-1.0, nsteps=1, adapt=True):
@@ -169,18 +180,18 @@ def mlp_loss_grad(X, y, params, pos_weight, work, out, stream=None):
     """Device tensors: X[n, 8], y[n], params[MLP_PARAMS], work[MLP_WORK], out[MLP_PARAMS + 1]
     (gradient, then the mean loss) -- sww_mlp_loss_grad."""
     st = stream if stream is not None else _default_stream()
-    _check(load().sww_mlp_loss_grad(_ptr(X)[0], _ptr(y)[0], X.shape[0], _ptr(params)[0], float(pos_weight),
-                                    _ptr(work)[0], _ptr(out)[0], st))
+    _check(load().sww_mlp_loss_grad(_addr(X), _addr(y), X.shape[0], _addr(params), float(pos_weight), _addr(work), _addr(out),
+                                    st))
 
 
 def mlp_adam(params, grad, m, v, t, lr, stream=None):
     st = stream if stream is not None else _default_stream()
-    _check(load().sww_mlp_adam(_ptr(params)[0], _ptr(grad)[0], _ptr(m)[0], _ptr(v)[0], int(t), float(lr), st))
+    _check(load().sww_mlp_adam(_addr(params), _addr(grad), _addr(m), _addr(v), int(t), float(lr), st))
 
 
 def mlp_predict(X, params, out, stream=None):
     st = stream if stream is not None else _default_stream()
-    _check(load().sww_mlp_predict(_ptr(X)[0], X.shape[0], _ptr(params)[0], _ptr(out)[0], st))
+    _check(load().sww_mlp_predict(_addr(X), X.shape[0], _addr(params), _addr(out), st))
 
 
 class Model:
