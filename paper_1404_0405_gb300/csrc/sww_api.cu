@@ -642,6 +642,16 @@ int size_class(const sww_handle* h) {
     while (n >>= 1) ++c;
     return c;
 }
+// Blocks of 256 of the mask's list launches: blocks_per_sm per SM on small grids, and on
+// grids whose nodes (at the size class's upper bound) outnumber those threads as many
+// as they need, up to 16 per SM.  With two or four blocks per SM the first adaptation of
+// a full level 9 grid ran each thread through 18 to 35 dependent items in turn.
+unsigned list_grid(const sww_handle* h, int64_t patches) {
+    const int64_t need = blocks_for(patches * h->S, 256), most = 16 * int64_t(h->nsm);
+    return unsigned(std::max<int64_t>(h->grid_all, std::min(need, most)));
+}
+unsigned list_grid(const sww_handle* h) { return list_grid(h, std::min(h->total_entries, int64_t(2) << size_class(h))); }
+
 // From 2^14 active patches a stage is one launch per phase instead of one cooperative
 // launch: the phases fill the GPU then, and their kernels keep more warps resident (FP32
 // turbulence, us per step persistent / phases: 3 400 patches 768 / 813, 13 640 1857 /
@@ -668,8 +678,8 @@ struct Self {
     BatchArgs<R> a;
     int64_t entries[16] = {};
     explicit Self(const sww_handle* h) {
-        a = BatchArgs<R>{nullptr, 1, h->S, h->cfg.jmin, h->jtop, h->cfg.H, h->cfg.g, RKStage{}, 0.0, h->out, chained(h), -1.0,
-                         -1.0, member_ref<R>(h)};
+        a = BatchArgs<R>{nullptr, 1, h->S, h->cfg.jmin, h->jtop, h->cfg.H, h->cfg.g, R(h->cfg.H), R(h->cfg.g),
+                         StageCoef<R>{}, 0.0, h->out, chained(h), -1.0, -1.0, member_ref<R>(h)};
         const int64_t cap = int64_t(1) << (size_class(h) + 1);
         for (int j = h->cfg.jmin; j <= h->cfg.jmax; ++j) entries[j] = std::min<int64_t>(meta(h, j).npatch + 1, cap);
     }
@@ -695,7 +705,7 @@ void stage(sww_handle* h, const RKStage& st) {
         return;
     }
     Trace t(h, SWW_K_STAGE);
-    StageArgs<R> a{dlv<R>(h), h->lists, h->S, h->cfg.jmin, h->jtop, h->cfg.jmax, h->cfg.H, h->cfg.g, st, h->dt, h->bar,
+    StageArgs<R> a{dlv<R>(h), h->lists, h->S, h->cfg.jmin, h->jtop, h->cfg.jmax, R(h->cfg.H), R(h->cfg.g), st, h->dt, h->bar,
                    h->err, h->spin_cycles, h->skip_block};
     ck(launch_stage(a, h->stage_blocks, h->stream), "persistent stage launch");
 }
@@ -838,13 +848,14 @@ void mask_only(sww_handle* h) {
     mask_batch_head(b, h, 1, j1, h->cfg.jmax);
     b.chain = chained(h);
     b.m[0] = mask_member<R>(h);
-    launch_proposal_batch(b, h->grid_all, 0, s);
+    const unsigned grid = list_grid(h);
+    launch_proposal_batch(b, grid, 0, s);
     if (list_mask(h))
-        launch_mask_batch(b, h->grid_all, s);
+        launch_mask_batch(b, grid, s);
     else
         launch_mask(mask_args<R>(h, j0, j1), s);
-    launch_proposal_batch(b, h->grid_all, 1, s);
-    launch_concat_batch(b, h->grid_all, s);
+    launch_proposal_batch(b, grid, 1, s);
+    launch_concat_batch(b, grid, s);
 }
 
 template <class R>
@@ -875,16 +886,16 @@ const RKStage* stages(int rk, int& n) {
     // classical RK4 (acc holds k1 + 2 k2 + 2 k3) and the 4-stage, third-order SSP
     // scheme of Spiteri & Ruuth (Sec. 3.1)
     static const RKStage rk4[4] = {
-        {1, 1.0, 0.0, 0.5, 0.0, 0.0, 1.0},
-        {1, 1.0, 0.0, 0.5, 0.0, 1.0, 2.0},
-        {1, 1.0, 0.0, 1.0, 0.0, 1.0, 2.0},
-        {1, 1.0, 0.0, 1.0 / 6.0, 1.0 / 6.0, 1.0, 0.0},
+        {1, 1.0, 0.0, 0.5, 0.0, 0.0, 1.0, 1, 0},
+        {1, 1.0, 0.0, 0.5, 0.0, 1.0, 2.0, 0, 0},
+        {1, 1.0, 0.0, 1.0, 0.0, 1.0, 2.0, 0, 0},
+        {1, 1.0, 0.0, 1.0 / 6.0, 1.0 / 6.0, 0.0, 0.0, 0, 1},
     };
     static const RKStage ssp[4] = {
-        {1, 0.0, 1.0, 0.5, 0.0, 0.0, 0.0},
-        {1, 0.0, 1.0, 0.5, 0.0, 0.0, 0.0},
-        {1, 2.0 / 3.0, 1.0 / 3.0, 1.0 / 6.0, 0.0, 0.0, 0.0},
-        {1, 0.0, 1.0, 0.5, 0.0, 0.0, 0.0},
+        {1, 0.0, 1.0, 0.5, 0.0, 0.0, 0.0, 1, 0},
+        {1, 0.0, 1.0, 0.5, 0.0, 0.0, 0.0, 0, 0},
+        {1, 2.0 / 3.0, 1.0 / 3.0, 1.0 / 6.0, 0.0, 0.0, 0.0, 0, 0},
+        {1, 0.0, 1.0, 0.5, 0.0, 0.0, 0.0, 0, 1},
     };
     n = 4;
     return rk == SWW_SSP43 ? ssp : rk4;
@@ -1014,7 +1025,8 @@ BatchArgs<R> ensemble_refs(sww_handle* const* hs, int n, std::vector<int64_t>& e
     int ns;
     const RKStage* st = stages(lead->cfg.rk, ns);
     return BatchArgs<R>{reinterpret_cast<const MemberRef<R>*>(E.refs), n, lead->S, lead->cfg.jmin, jtop, lead->cfg.H,
-                        lead->cfg.g, st[0], 0.0, E.out, chained(hs, n), -1.0, -1.0, MemberRef<R>{}};
+                        lead->cfg.g, R(lead->cfg.H), R(lead->cfg.g), StageCoef<R>(st[0]), 0.0, E.out, chained(hs, n),
+                        -1.0, -1.0, MemberRef<R>{}};
 }
 
 // One step of every member with the work batched over members (persistent = 3), on
@@ -1343,7 +1355,7 @@ static int set_state_at(sww_handle* h, const double* dh, const double* u, int J,
             }
             for (int j = J; j > j0; --j) launch_restrict_full(lv[j - 1], lv[j], s);
             MaskArgsT<R> a = mask_args<R>(h, j0, J, false);
-            launch_live_all(dlv<R>(h), a.nodes, a.edges, s);
+            launch_live_all(dlv<R>(h), a.edges, s);
             for (int j = J + 1; j <= j1; ++j) {
                 const DevLevelT<R>& L = lv[j];
                 ck(cudaMemsetAsync(L.nflag, 0, L.N, s), "memset flags");
@@ -1359,7 +1371,7 @@ static int set_state_at(sww_handle* h, const double* dh, const double* u, int J,
             if (J > j0) launch_covered_all(dlv<R>(h), a.nodes_c, s);
             MaskArgsT<R> b = mask_args<R>(h, j0, j1, false);
             launch_patches_all(dlv<R>(h), b.patches, s);
-            launch_concat(dlv<R>(h), j0, j1, h->lists, h->S, h->grid_all, s);
+            launch_concat(dlv<R>(h), j0, j1, h->lists, h->S, list_grid(h, h->total_entries), s);
             read_counts<R>(h);
             check_launch();
             return 0;
@@ -1446,7 +1458,7 @@ int sww_rhs(sww_handle* h) {
         by_prec(h, [&](auto r) {
             using R = decltype(r);
             Join jn(h);
-            RKStage none{0, 0, 0, 0, 0, 0, 0};
+            RKStage none{0, 0, 0, 0, 0, 0, 0, 0, 1};
             stage<R>(h, none);
             ck(cudaMemcpyAsync(h->h_err, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "err");
             check_launch();
@@ -1866,7 +1878,7 @@ int sww_load(sww_handle* h, const char* path) {
                 ck(cudaMemcpyAsync(h->thr, thr, sizeof(thr), cudaMemcpyHostToDevice, s), "load thr");
                 MaskArgsT<R> a = mask_args<R>(h, j0, j1, false);
                 launch_patches_all(dlv<R>(h), a.patches, s);
-                launch_concat(dlv<R>(h), j0, j1, h->lists, h->S, h->grid_all, s);
+                launch_concat(dlv<R>(h), j0, j1, h->lists, h->S, list_grid(h, h->total_entries), s);
                 read_counts<R>(h);
                 check_launch();
                 ck(cudaStreamSynchronize(s), "load");   // host buffers live on this frame

@@ -1,5 +1,5 @@
 // The phases of a step as one regular launch each, for every member of an ensemble or
-// for one handle: time step and RK base; each stage's trend and update (Sec. 3.1, in
+// for one handle: time step; each stage's trend and update (Sec. 3.1, in
 // the order of the persistent stage): ghosts level by level, the structured trend and
 // the irregular patches (sww_tile.cu), the restrictions level by level, the update; the
 // partial transform and ghosts; coefficients, maxima and thresholds; the inverse
@@ -37,7 +37,7 @@ constexpr int BATCH_TPB = 256;
 constexpr int MAXL = 12;
 constexpr int MAXM = 128;
 enum {
-    PH_FILL = 0, PH_RESTRICT, PH_DIV, PH_UPDATE, PH_SAVE, PH_DT, PH_DT_FINAL, PH_PARTIAL,
+    PH_FILL = 0, PH_RESTRICT, PH_DIV, PH_UPDATE, PH_SET_DT, PH_DT, PH_DT_FINAL, PH_PARTIAL,
     PH_DETAILS, PH_THRESH, PH_INV_A, PH_INV_B, PH_INV_FILL, PH_OUT
 };
 
@@ -106,8 +106,15 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
     const int m = blockIdx.x / bpm, b = blockIdx.x % bpm;
     const MemberRef<R>* mr = a.m ? a.m + m : &a.one;
     // one block per member
-    if constexpr (PH == PH_DT_FINAL) {
-        if (threadIdx.x == 0) *mr->dt = cfl_step<R>(mr->lvs, mr->red, mr->cfl);
+    if constexpr (PH == PH_DT_FINAL || PH == PH_SET_DT) {
+        // the step, CFL or given; the reduction words are left at zero for the step's maxima
+        // and the next step
+        if (threadIdx.x < 32) {
+            const double dt = PH == PH_SET_DT ? a.dt_given : cfl_step<R>(mr->lvs, mr->red, mr->cfl);
+            __syncwarp();
+            if (threadIdx.x == 0) *mr->dt = dt;
+            if (threadIdx.x < RED_WORDS) mr->red[threadIdx.x] = 0ull;
+        }
         return;
     }
     if constexpr (PH == PH_THRESH) {   // given, or relative to the live maxima (a prescribed velocity has no threshold)
@@ -173,25 +180,6 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
     } else if constexpr (PH == PH_PARTIAL) {
         // R_h at covered nodes of level j from level j + 1 (Eq. Rh)
         member_wl(sl[j], WL_CN, -1, b, bpm, [&](int, int64_t id) { partial_node(sl[j], sl[j + 1], id); });
-    } else if constexpr (PH == PH_SAVE) {
-        // the RK base, and the time step: given (a.dt > 0) or its reduction words reset
-        if (b == 0 && threadIdx.x == 0) {
-            if (a.dt_given > 0) {
-                *mr->dt = a.dt_given;
-                mr->red[2] = 0ull;
-                mr->red[3] = 0ull;
-            } else {
-                for (int w = 0; w < RED_WORDS; ++w) mr->red[w] = 0ull;
-            }
-        }
-        member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
-                                      [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
-                                          if (kind == K_NODE) {
-                                              if (L.nflag[id] & LIVE) L.dh0[id] = L.dh[id];
-                                          } else if (L.eflag[id] & LIVE) {
-                                              L.u0[id] = L.u[id];
-                                          }
-                                      });
     } else if constexpr (PH == PH_DT) {
         // largest omega^2 over live nodes (none with a prescribed velocity) and, per level,
         // largest |u| over live edges with u != 0 (NaN left out, as dx/|u| with u NaN takes
@@ -224,15 +212,15 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         // doubles); the details only read dh and u
         __shared__ unsigned long long shm[BATCH_TPB / 32];
         unsigned long long hmax = 0, umax = 0;
-        member_items<K_NODE | K_EDGE | K_CEDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
-                                                [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t el) {
-                                                    if (kind == K_NODE) {
-                                                        if (L.nflag[id] & LIVE) hmax = max(hmax, abs_key(L.dh[id]));
-                                                    } else if (kind == K_EDGE) {
-                                                        if (L.eflag[id] & LIVE) umax = max(umax, abs_key(L.u[id]));
-                                                    }
-                                                    if (L.J > a.jmin) details_item(L, (&L)[-1], kind, id, el);
-                                                });
+        member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
+                                      [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
+                                          if (kind == K_NODE) {
+                                              if (L.nflag[id] & LIVE) hmax = max(hmax, abs_key(L.dh[id]));
+                                          } else {
+                                              if (L.eflag[id] & LIVE) umax = max(umax, abs_key(L.u[id]));
+                                          }
+                                          if (L.J > a.jmin) details_item(L, (&L)[-1], kind, id);
+                                      });
         hmax = block_reduce_u64(hmax, MaxU64(), shm);
         umax = block_reduce_u64(umax, MaxU64(), shm);
         if (threadIdx.x == 0) {
@@ -248,15 +236,14 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         member_items<K_NODE>(sl, sl[j].clist, sl[j].npatches[1], a.P, b, bpm,
                              [&](const DevLevelT<R>& L, int, int64_t id, int64_t) { inverse_b_item(L, id); });
     } else {
-        static_assert(PH == PH_UPDATE || PH == PH_DT_FINAL || PH == PH_THRESH || PH == PH_OUT, "phase");
-        const R dt = R(mr->dt ? *mr->dt : 0.0);
-        const RKStageR<R> sr(a.st);
+        static_assert(PH == PH_UPDATE || PH == PH_SET_DT || PH == PH_DT_FINAL || PH == PH_THRESH || PH == PH_OUT, "phase");
+        const R dt = to_r<R>(mr->dt ? *mr->dt : 0.0);
         member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
                                       [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
                                           if (kind == K_NODE)
-                                              update_node(L, id, sr, dt);
+                                              update_node(L, id, a.st, dt);
                                           else
-                                              update_edge(L, id, sr, dt);
+                                              update_edge(L, id, a.st, dt);
                                       });
     }
 }
@@ -323,12 +310,9 @@ cudaError_t launch_batch_pre(const BatchArgs<R>& a, const int64_t* level_entries
     const int64_t all = entries_to(a, level_entries);
     BatchArgs<R> b = a;
     b.dt_given = dt;
-    cudaError_t e = batch_go<PH_SAVE>(b, 0, batch_bpm(b, all, 4, nsm), s);
-    if (e == cudaSuccess && !(dt > 0)) {
-        e = batch_go<PH_DT>(b, 0, batch_bpm(b, all, 4, nsm), s);
-        if (e == cudaSuccess) e = batch_go<PH_DT_FINAL>(b, 0, 1, s);
-    }
-    return e;
+    if (dt > 0) return batch_go<PH_SET_DT>(b, 0, 1, s);
+    cudaError_t e = batch_go<PH_DT>(b, 0, batch_bpm(b, all, 4, nsm), s);
+    return e == cudaSuccess ? batch_go<PH_DT_FINAL>(b, 0, 1, s) : e;
 }
 
 template <class R>
@@ -348,7 +332,7 @@ cudaError_t launch_batch_post(const BatchArgs<R>& a, const int64_t* level_entrie
 template <class R>
 cudaError_t launch_batch_details(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s) {
     if (!batch_ok(a, a.jtop_max)) return cudaErrorInvalidValue;
-    return batch_go<PH_DETAILS>(a, 0, batch_bpm(a, entries_to(a, level_entries), 7, nsm), s);
+    return batch_go<PH_DETAILS>(a, 0, batch_bpm(a, entries_to(a, level_entries), 4, nsm), s);
 }
 
 template <class R>

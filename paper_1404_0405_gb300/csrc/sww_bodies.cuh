@@ -94,15 +94,15 @@ struct LevelMax {
 
 // Advective bound min over live edges of dx_j / |u| (Sec. 3.1's CFL condition):
 // for one level, a correctly rounded dx_j / a falls as a grows, so the minimum is
-// dx_j over the level's largest |u|; then the step cfl * min(1/omega, that bound).
+// dx_j over the level's largest |u|; then the step cfl * min(1/omega, that bound).  By
+// one warp, a level a lane; the value is lane 0's.
 template <class R>
 __device__ __forceinline__ double cfl_step(const DevLevelT<R>* lvs, const unsigned long long* red, double cfl) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long k = lane < RED_WORDS - RED_LEVEL ? red[RED_LEVEL + lane] : 0ull;
+    double r = k ? lvs[lane].dx / key_value<R>(k) : INFINITY;
+    for (int o = 16; o > 0; o >>= 1) r = fmin(r, __shfl_xor_sync(0xffffffffu, r, o));
     const double w = sqrt(__longlong_as_double(static_cast<long long>(red[0])));
-    double r = INFINITY;
-    for (int j = 0; j < RED_WORDS - RED_LEVEL; ++j) {
-        const unsigned long long k = red[RED_LEVEL + j];
-        if (k) r = fmin(r, lvs[j].dx / key_value<R>(k));
-    }
     return cfl * fmin(1.0 / w, r);
 }
 
@@ -113,18 +113,17 @@ __device__ __forceinline__ int64_t patch_of(const Lv& L, int64_t x) {
 }
 
 // Item kinds of a work-list entry, in slot order.
-constexpr int K_NODE = 1, K_EDGE = 2, K_TRI = 4, K_CEDGE = 8;
+constexpr int K_NODE = 1, K_EDGE = 2, K_TRI = 4;
 
 template <int KINDS>
 __host__ __device__ constexpr int slots_of() {
-    return ((KINDS & K_NODE) ? 1 : 0) + ((KINDS & K_EDGE) ? 3 : 0) + ((KINDS & K_TRI) ? 2 : 0) + ((KINDS & K_CEDGE) ? 3 : 0);
+    return ((KINDS & K_NODE) ? 1 : 0) + ((KINDS & K_EDGE) ? 3 : 0) + ((KINDS & K_TRI) ? 2 : 0);
 }
 
 // Visit the items of the entries of a work list, one thread per item:
 // body(L, kind, id, elem).  An entry covers slots x P threads (P = configured patch
-// area): one slot of nodes, three of edges (orientation 0, 1, 2), two of triangles
-// and three of the edges of the coarse element under an even element (id = the
-// orientation), as KINDS selects.  A pole entry yields the two pole nodes with
+// area): one slot of nodes, three of edges (orientation 0, 1, 2) and two of triangles,
+// as KINDS selects.  A pole entry yields the two pole nodes with
 // elem = -1.  Entries name their level in `lvs` (multi-level lists) or all belong
 // to `one` when lvs is null.
 // Item `local` (0 <= local < slots x P) of work-list entry patch `pat` of level L:
@@ -160,9 +159,7 @@ __device__ __forceinline__ void visit_item(const Lv& L, int64_t pat, uint32_t lo
             body(L, K_TRI, slot * L.nelem + el, el);
             return;
         }
-        slot -= 2;
     }
-    if (KINDS & K_CEDGE) body(L, K_CEDGE, int64_t(slot), el);
 }
 
 template <int KINDS, class Lv, class Body>
@@ -353,21 +350,17 @@ __device__ __forceinline__ void coriolis_at(const DevLevelT<R>& L, int64_t e) {
 // trend and one Runge-Kutta stage at a live point (terms with a zero coefficient
 // are skipped, so stale storage never enters):
 //   y <- a*y0 + b*y + (cdt*dt)*k + (ddt*dt)*acc,   acc <- al*acc + be*k
-// An RK stage in the working precision: the coefficients converted and their zero
-// tests taken once per thread, not at every point (the FP64 pipe is narrow)
 template <class R>
-struct RKStageR {
-    R a, b, cdt, ddt, al, be;
-    bool apply, ha, hb, hddt, hacc, hal;
-    __device__ explicit RKStageR(const RKStage& st)
-        : a(R(st.a)), b(R(st.b)), cdt(R(st.cdt)), ddt(R(st.ddt)), al(R(st.al)), be(R(st.be)), apply(st.apply != 0),
-          ha(st.a != 0.0), hb(st.b != 0.0), hddt(st.ddt != 0.0), hacc(st.al != 0.0 || st.be != 0.0), hal(st.al != 0.0) {}
-};
-
-template <class R>
-__device__ __forceinline__ void rk_apply(const RKStageR<R>& st, R dt, R k, R* y, const R* y0, R* acc) {
+__device__ __forceinline__ void rk_apply(const StageCoef<R>& st, R dt, R k, R* y, R* y0, R* acc) {
     R v = st.cdt * dt * k;
-    if (st.ha) v += st.a * *y0;
+    R b = R(0);
+    if (st.base) {
+        b = *y;
+        *y0 = b;
+    } else if (st.ha) {
+        b = *y0;
+    }
+    if (st.ha) v += st.a * b;
     if (st.hb) v += st.b * *y;
     if (st.hddt) v += st.ddt * dt * *acc;
     if (st.hacc) *acc = (st.hal ? st.al * *acc : R(0)) + st.be * k;
@@ -375,22 +368,22 @@ __device__ __forceinline__ void rk_apply(const RKStageR<R>& st, R dt, R k, R* y,
 }
 
 template <class R>
-__device__ __forceinline__ void update_node(const DevLevelT<R>& L, int64_t v, const RKStageR<R>& st, R dt) {
+__device__ __forceinline__ void update_node(const DevLevelT<R>& L, int64_t v, const StageCoef<R>& st, R dt) {
     if (!(L.nflag[v] & LIVE)) return;
     R k = -L.c[v];
-    L.dht[v] = k;
+    if (st.trend) L.dht[v] = k;
     if (st.apply) rk_apply(st, dt, k, &L.dh[v], &L.dh0[v], &L.dha[v]);
 }
 
 template <class R>
-__device__ __forceinline__ void update_edge(const DevLevelT<R>& L, int64_t e, const RKStageR<R>& st, R dt) {
+__device__ __forceinline__ void update_edge(const DevLevelT<R>& L, int64_t e, const StageCoef<R>& st, R dt) {
     if (!(L.eflag[e] & LIVE)) return;
     if (L.advect) {   // prescribed velocity: zero trend, u untouched
-        L.ut[e] = R(0);
+        if (st.trend) L.ut[e] = R(0);
         return;
     }
     R k = L.Q[e] - (L.B[L.en[L.E + e]] - L.B[L.en[e]]) / geo<R>(L.d_e, e);
-    L.ut[e] = k;
+    if (st.trend) L.ut[e] = k;
     if (st.apply) rk_apply(st, dt, k, &L.u[e], &L.u0[e], &L.ua[e]);
 }
 
@@ -460,28 +453,27 @@ __device__ __forceinline__ void fill_edge(const DevLevelT<R>& F, const DevLevelT
 
 // wavelet coefficients at a live point of F > Jmin from C = the level below
 // (Eqs. 1-2; velocity transform of Sec. 4.1): h~ at odd nodes, u~ at interior fine
-// edges, u~_E at the edges of the coarse element under each even fine element
+// edges, and u~_E of a coarse edge at its first half (visited by elements and their
+// edges alone: a pass over the coarse edges under even elements keeps a quarter of its
+// threads busy)
 template <class R>
-__device__ __forceinline__ void details_item(const DevLevelT<R>& L, const DevLevelT<R>& C, int kind, int64_t id,
-                                             int64_t el) {
+__device__ __forceinline__ void details_item(const DevLevelT<R>& L, const DevLevelT<R>& C, int kind, int64_t id) {
     if (kind == K_NODE) {
         const int32_t k = L.f2c[id];
         const uint8_t f = L.nflag[id];
         if ((k < 0) & ((f & LIVE) != 0)) L.hdet[id] = height_detail(L, id);
-    } else if (kind == K_EDGE) {
-        const int fk = L.fe_kind[id];
-        const uint8_t f = L.eflag[id];
-        if ((fk == 2) & ((f & LIVE) != 0)) L.ui[id] = L.u[id] - predict(L, C.u, id);
-    } else {
-        int32_t ce = L.f2c[el];
-        if (ce < 0) return;
-        int64_t E = id * C.nelem + ce;
-        int32_t h0 = C.half[E], h1 = C.half[C.E + E];
-        if ((L.eflag[h0] | L.eflag[h1]) & LIVE) {
-            R a = L.u[h0] - predict(L, C.u, h0);
-            R b = L.u[h1] - predict(L, C.u, h1);
-            L.ue[E] = R(0.5) * (a - b);
-        }
+        return;
+    }
+    const int fk = L.fe_kind[id];
+    const uint8_t f = L.eflag[id];
+    const int32_t o = L.fe_ot[id];
+    if (fk == 1) return;
+    if (fk == 2) {
+        if (f & LIVE) L.ui[id] = L.u[id] - predict(L, C.u, id);
+    } else if ((f | L.eflag[o]) & LIVE) {
+        R a = L.u[id] - predict(L, C.u, id);
+        R b = L.u[o] - predict(L, C.u, o);
+        L.ue[L.fe_ce[id]] = R(0.5) * (a - b);
     }
 }
 
@@ -638,30 +630,26 @@ __device__ __forceinline__ bool sig_node(const DevLevelT<R>& F, int64_t i, R eh)
     return false;
 }
 
+// a fine edge of kind 2, or the coarse edge of a first half (kind 0)
 template <class R>
-__device__ __forceinline__ bool sig_edge(const DevLevelT<R>& F, int64_t i, R eu) {
+__device__ __forceinline__ bool sig_edge(const DevLevelT<R>& F, const DevLevelT<R>& C, int64_t i, R eu) {
     const int k = F.fe_kind[i];
     const uint8_t f = F.eflag[i];
-    const R d = F.ui[i];
-    if ((k == 2) & ((f & LIVE) != 0) & (fabs(d) >= eu)) {
+    if (k == 1) return false;
+    if (k == 2) {
+        const R d = F.ui[i];
+        if (!((f & LIVE) != 0 & fabs(d) >= eu)) return false;
         F.sig[F.en[i]] = 1;
         F.sig[F.en[F.E + i]] = 1;
         return true;
     }
-    return false;
-}
-
-template <class R>
-__device__ __forceinline__ bool sig_cedge(const DevLevelT<R>& F, const DevLevelT<R>& C, int64_t i, R eu) {
-    const int32_t h0 = C.half[i], h1 = C.half[C.E + i];
-    const R d = F.ue[i];
-    if ((((F.eflag[h0] | F.eflag[h1]) & LIVE) != 0) & (fabs(d) >= eu)) {
-        F.sig[C.c2f[C.en[i]]] = 1;
-        F.sig[C.c2f[C.en[C.E + i]]] = 1;
-        F.sig[C.mid[i]] = 1;
-        return true;
-    }
-    return false;
+    const int32_t E = F.fe_ce[i];
+    const R d = F.ue[E];
+    if (!(((f | F.eflag[F.fe_ot[i]]) & LIVE) != 0 & fabs(d) >= eu)) return false;
+    F.sig[C.c2f[C.en[E]]] = 1;
+    F.sig[C.c2f[C.en[C.E + E]]] = 1;
+    F.sig[C.mid[E]] = 1;
+    return true;
 }
 
 // T = S + same-level neighbours of S + children of the coarser significance set; a
@@ -719,11 +707,15 @@ __device__ __forceinline__ uint8_t live_node(const DevLevelT<R>& L, int64_t i, b
     return lv;
 }
 
-// an edge is live when an end node is
+// An edge is live when an end node is: from the closure marks (every node when `all`), not
+// from the node flags, so that nodes and edges take their flags in one pass.  A mark is
+// 0 at a node outside the mask's candidates (a marked node was live and its patch
+// active, a seed of the next mask).
 template <class R>
-__device__ __forceinline__ void live_edge(const DevLevelT<R>& L, int64_t e) {
+__device__ __forceinline__ void live_edge(const DevLevelT<R>& L, int64_t e, bool all) {
     const uint8_t was = (L.eflag[e] & LIVE) ? WASLIVE : 0;
-    L.eflag[e] = uint8_t((((L.nflag[L.en[e]] | L.nflag[L.en[L.E + e]]) & LIVE) ? LIVE : 0) | was);
+    const bool lv = all || (L.tmask[L.en[e]] | L.tmask[L.en[L.E + e]]);
+    L.eflag[e] = uint8_t((lv ? LIVE : 0) | was);
 }
 
 // one neighbour hop of the ghost band: band1 <- dilate(band0) when `forward`,
@@ -931,47 +923,75 @@ __device__ __forceinline__ int64_t wl_off(const DevLevelT<R>& L, int k) {
     return k == WL_GN ? 0 : k == WL_GE ? L.N : k == WL_CN ? L.N + L.E : k == WL_RE ? 2 * L.N + L.E : 2 * L.N + 2 * L.E;
 }
 
-// warp-aggregated append of v to work list k of L when pred (the lanes of the warp
-// that reach the call take part).  All lanes of a warp belong to one level: the
-// work-list build visits 4 x P items per list entry (node and edge slots), with
-// P >= 16 (patch sides 4, 8, 16) a multiple of 32.
-template <class R>
-__device__ __forceinline__ void wl_push(const DevLevelT<R>& L, int k, bool pred, int32_t v) {
-    const unsigned act = __activemask();
-    const unsigned m = __ballot_sync(act, pred);
-    if (!pred) return;
-    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(&L.wl_n[k], __popc(m));
-    base = __shfl_sync(m, base, leader);
-    L.wl[wl_off(L, k) + base + __popc(m & ((1u << lane) - 1u))] = v;
-}
-
-// The point work lists of one item of an active patch (node or edge, see
-// visit_item): ghost points, covered nodes, edges with a covered end, and
+// The point work lists and the live-node counts of the entries of `list`, a warp an entry
+// (warp w of nw warps): ghost points, covered nodes, edges with a covered end, and
 // available nodes with a covered node among themselves and their neighbours (their
-// divergence changes with the restricted fluxes); and the count of live nodes.
-// The order of the lists is not fixed; every item's work is independent of it.
+// divergence changes with the restricted fluxes).  The warp goes through the entry's
+// node and edge slots 256 items at a time, keeps in which lists each belongs, and then
+// reserves its room with one addition per list, by a lane each.  (With one addition per
+// 32 items they queued on the lists' counters: 260 us for the 52 632 patches of
+// turbulence at Jmax 9, 142 us now.)  The order of the lists is not fixed; every item's
+// work is independent of it.
 template <class R>
-__device__ __forceinline__ void wl_item(const DevLevelT<R>& L, int kind, int64_t id) {
+__device__ __forceinline__ unsigned wl_member(const DevLevelT<R>& L, int kind, int64_t id) {
     if (kind == K_NODE) {
         const uint8_t f = L.nflag[id];
-        {   // the level's live nodes (warp-aggregated)
-            const unsigned act = __activemask();
-            const unsigned m = __ballot_sync(act, (f & LIVE) != 0);
-            if ((threadIdx.x & 31) == __ffs(act) - 1 && m) atomicAdd(&L.wl_n[WL_LIVE], __popc(m));
-        }
-        wl_push(L, WL_GN, (f & GHOST) != 0, int32_t(id));
-        wl_push(L, WL_CN, (f & COVERED) != 0, int32_t(id));
-        wl_push(L, WL_DN, restricted_div_node(L, id), int32_t(id));
-    } else {
-        const uint8_t f = L.eflag[id];
-        // the first half of a coarse edge fills a ghost second half too (fill_edge)
-        bool ge = (f & GHOST) != 0;
-        if (ge && L.fe_kind[id] == 1 && (L.eflag[L.fe_ot[id]] & GHOST)) ge = false;
-        wl_push(L, WL_GE, ge, int32_t(id));
-        const bool r = ((L.nflag[L.en[id]] | L.nflag[L.en[L.E + id]]) & COVERED) != 0;
-        wl_push(L, WL_RE, r, int32_t(id));
+        return ((f & LIVE) ? 1u << WL_LIVE : 0u) | ((f & GHOST) ? 1u << WL_GN : 0u) | ((f & COVERED) ? 1u << WL_CN : 0u) |
+               (restricted_div_node(L, id) ? 1u << WL_DN : 0u);
     }
+    const uint8_t f = L.eflag[id];
+    const int32_t na = L.en[id], nb = L.en[L.E + id];
+    // the first half of a coarse edge fills a ghost second half too (fill_edge)
+    bool ge = (f & GHOST) != 0;
+    if (ge && L.fe_kind[id] == 1 && (L.eflag[L.fe_ot[id]] & GHOST)) ge = false;
+    return (ge ? 1u << WL_GE : 0u) | (((L.nflag[na] | L.nflag[nb]) & COVERED) ? 1u << WL_RE : 0u);
 }
 
+template <class R>
+__device__ void wl_build(const DevLevelT<R>* __restrict__ lvs, const int32_t* __restrict__ list, int count, int P, int w,
+                         int nw) {
+    constexpr int G = 8;   // groups of 32 items a round
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const int groups = 4 * P / 32;   // P >= 16
+    for (int t = w; t < count; t += nw) {
+        const int32_t ent = list[t];
+        const DevLevelT<R>& L = lvs[ent >> LVL_SHIFT];
+        for (int g0 = 0; g0 < groups; g0 += G) {
+            int32_t id[G];
+            unsigned in[G];
+            int n = 0;   // lane k < WL_WORDS: entries of list k
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                in[g] = 0u, id[g] = 0;
+                auto body = [&](const DevLevelT<R>& LL, int kind, int64_t i, int64_t) {
+                    id[g] = int32_t(i);
+                    in[g] = wl_member(LL, kind, i);
+                };
+                if (g0 + g < groups)
+                    visit_item<K_NODE | K_EDGE>(L, int64_t(ent & PATCH_MASK), uint32_t((g0 + g) * 32 + lane), P, body);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+#pragma unroll
+                for (int k = 0; k < WL_WORDS; ++k) {
+                    const int c = __popc(__ballot_sync(0xffffffffu, in[g] >> k & 1u));
+                    if (lane == k) n += c;
+                }
+            int at = 0;
+            if (lane < WL_WORDS && n) at = atomicAdd(&L.wl_n[lane], n);
+#pragma unroll
+            for (int k = 0; k < WL_KINDS; ++k) {
+                int pos = __shfl_sync(0xffffffffu, at, k);
+                int32_t* __restrict__ out = L.wl + wl_off(L, k);
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const unsigned m = __ballot_sync(0xffffffffu, in[g] >> k & 1u);
+                    if (in[g] >> k & 1u) out[pos + __popc(m & below)] = id[g];
+                    pos += __popc(m);
+                }
+            }
+        }
+    }
+}

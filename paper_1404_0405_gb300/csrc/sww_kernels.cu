@@ -234,8 +234,7 @@ __global__ void k_sig(const DevLevelT<R>* __restrict__ lvs, Span sp, const doubl
         bool any = false;
         const R eh = sig_thr<R>(thr[0]), eu = sig_thr<R>(thr[1]);
         if (i < F.N) any |= sig_node(F, i, eh);
-        if (i < F.E) any |= sig_edge(F, i, eu);
-        if (i < C.E) any |= sig_cedge(F, C, i, eu);
+        if (i < F.E) any |= sig_edge(F, C, i, eu);
         if (any) sig_any[j] = 1;
     });
 }
@@ -253,14 +252,16 @@ __global__ void k_close(DevLevelT<R> F, DevLevelT<R> Fp, int has_finer, const in
     for (int64_t x = gid(); x < F.N; x += stride) close_node(F, Fp, has_finer != 0, x);
 }
 
+// live flags of the nodes and edges (sp: the edges of the levels; every point of level
+// all_level, of every level when it is -2)
 template <class R>
 __global__ void k_live(const DevLevelT<R>* __restrict__ lvs, Span sp, int all_level, const int32_t* sig_any) {
-    DENSE_EACH(sp, gid(), sig_any) { live_node(lvs[j], i, all_level == -2 || j == all_level); });
-}
-
-template <class R>
-__global__ void k_live_edges(const DevLevelT<R>* __restrict__ lvs, Span sp, const int32_t* sig_any) {
-    DENSE_EACH(sp, gid(), sig_any) { live_edge(lvs[j], i); });
+    DENSE_EACH(sp, gid(), sig_any) {
+        const DevLevelT<R>& L = lvs[j];
+        const bool all = all_level == -2 || j == all_level;
+        if (i < L.N) live_node(L, i, all);
+        live_edge(L, i, all);
+    });
 }
 
 template <class R>
@@ -341,8 +342,7 @@ __global__ void k_concat(const DevLevelT<R>* __restrict__ lvs, int jmin, int jma
 template <class R>
 __global__ void k_wl_build(const DevLevelT<R>* __restrict__ lvs, const int32_t* __restrict__ list,
                            const int32_t* __restrict__ count, int P) {
-    DevLevelT<R> none{};
-    ITEMS(K_NODE | K_EDGE, lvs, none, list, count, P) { wl_item(L, kind, id); });
+    wl_build(lvs, list, *count, P, int(gid() >> 5), int(gridDim.x * blockDim.x >> 5));
 }
 
 }  // namespace
@@ -395,8 +395,7 @@ void launch_mask(const MaskArgsT<R>& a, cudaStream_t s) {
         k_close<R><<<grid, TPB, 0, s>>>(F, finer ? a.host[j + 1] : F, finer, any, tail);
     }
     // live flags, ghost band, covered nodes, patch lists (levels ja..jb)
-    MULTI(k_live<R>, a.nodes, a.lvs, a.nodes, a.ja, any);
-    MULTI(k_live_edges<R>, a.edges, a.lvs, a.edges, any);
+    MULTI(k_live<R>, a.edges, a.lvs, a.edges, a.ja, any);
     for (int h = 0; h < a.hops; ++h) MULTI(k_dilate<R>, a.nodes_f, a.lvs, a.nodes_f, h % 2 == 0, any);
     MULTI(k_ghost<R>, a.edges_f, a.lvs, a.edges_f, a.hops % 2 == 1, any);
     if (a.jb > a.ja) MULTI(k_covered<R>, a.nodes_c, a.lvs, a.nodes_c);
@@ -406,9 +405,8 @@ void launch_mask(const MaskArgsT<R>& a, cudaStream_t s) {
 }
 
 template <class R>
-void launch_live_all(const DevLevelT<R>* lvs, const Span& nodes, const Span& edges, cudaStream_t s) {
-    MULTI(k_live<R>, nodes, lvs, nodes, -2, nullptr);
-    MULTI(k_live_edges<R>, edges, lvs, edges, nullptr);
+void launch_live_all(const DevLevelT<R>* lvs, const Span& edges, cudaStream_t s) {
+    MULTI(k_live<R>, edges, lvs, edges, -2, nullptr);
 }
 
 template <class R>
@@ -464,7 +462,7 @@ void launch_convert(const A* x, B* y, int64_t n, cudaStream_t s) {
 #define SWW_INSTANTIATE(R)                                                                                   \
     template void launch_restrict_full<R>(const DevLevelT<R>&, const DevLevelT<R>&, cudaStream_t);           \
     template void launch_mask<R>(const MaskArgsT<R>&, cudaStream_t);                                         \
-    template void launch_live_all<R>(const DevLevelT<R>*, const Span&, const Span&, cudaStream_t);           \
+    template void launch_live_all<R>(const DevLevelT<R>*, const Span&, cudaStream_t);                        \
     template void launch_covered_all<R>(const DevLevelT<R>*, const Span&, cudaStream_t);                     \
     template void launch_uniform<R>(const DevLevelT<R>&, const DevLevelT<R>&, const R*, const R*, R*, R*,       \
                                     cudaStream_t);                                                           \

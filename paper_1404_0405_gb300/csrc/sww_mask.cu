@@ -137,8 +137,11 @@ __global__ void k_feat_own(const __grid_constant__ MaskBatch<R, CAP> B) {
     STAGE_LEVELS;
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t(gridDim.x) * blockDim.x) >> 5;
-    // the thresholds once per thread, in FP32
-    const float eh = float(M.thr[0] > 0 ? M.thr[0] : 1.0), eu = float(M.thr[1] > 0 ? M.thr[1] : 1.0);
+    // the thresholds in FP32, by one thread
+    __shared__ float thr[2];
+    if (threadIdx.x < 2) thr[threadIdx.x] = float(M.thr[threadIdx.x] > 0 ? M.thr[threadIdx.x] : 1.0);
+    __syncthreads();
+    const float eh = thr[0], eu = thr[1];
     for (int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; w < M.lists.count[1]; w += nw) {
         const int32_t ent = M.lists.core[w];
         const int j = ent >> LVL_SHIFT;
@@ -274,21 +277,15 @@ __global__ void k_sig_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
     STAGE_LEVELS;
     DevLevelT<R> none{};
-    const R eh = sig_thr<R>(M.thr[0]), eu = sig_thr<R>(M.thr[1]);
+    // in the field type, by one thread: FP64 conversions queue on their pipe
+    __shared__ R thr[2];
+    if (threadIdx.x < 2) thr[threadIdx.x] = sig_thr<R>(M.thr[threadIdx.x]);
+    __syncthreads();
+    const R eh = thr[0], eu = thr[1];
     int32_t* sig_any = M.sig_any;
-    ITEMS(K_NODE | K_EDGE | K_CEDGE, lvs, none, M.lists.core, M.lists.count + 1, B.P) {
+    ITEMS(K_NODE | K_EDGE, lvs, none, M.lists.core, M.lists.count + 1, B.P) {
         if (L.J == B.ja) return;
-        const DevLevelT<R>& C = lvs[L.J - 1];
-        bool any;
-        if (kind == K_NODE) {
-            any = sig_node(L, id, eh);
-        } else if (kind == K_EDGE) {
-            any = sig_edge(L, id, eu);
-        } else {
-            const int32_t ce = L.f2c[el];
-            if (ce < 0) return;
-            any = sig_cedge(L, C, id * C.nelem + ce, eu);
-        }
+        const bool any = kind == K_NODE ? sig_node(L, id, eh) : sig_edge(L, lvs[L.J - 1], id, eu);
         if (any) {
             sig_any[L.J] = 1;
             L.sflag[el < 0 ? L.npatch : patch_of(L, el)] = 1;
@@ -440,17 +437,12 @@ __global__ void k_live_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
     STAGE_LEVELS;
     DevLevelT<R> none{};
-    ITEMS(K_NODE, lvs, none, M.cand, M.cand_count, B.P) {
-        if (live_node(L, id, L.J == B.ja)) L.lflag[patch_of(L, id)] = 1;
+    ITEMS(K_NODE | K_EDGE, lvs, none, M.cand, M.cand_count, B.P) {
+        if (kind == K_EDGE)
+            live_edge(L, id, L.J == B.ja);
+        else if (live_node(L, id, L.J == B.ja))
+            L.lflag[patch_of(L, id)] = 1;
     });
-}
-
-template <class R, int CAP>
-__global__ void k_live_edges_list(const __grid_constant__ MaskBatch<R, CAP> B) {
-    MEMBER;
-    STAGE_LEVELS;
-    DevLevelT<R> none{};
-    ITEMS(K_EDGE, lvs, none, M.cand, M.cand_count, B.P) { live_edge(L, id); });
 }
 
 template <class R, int CAP>
@@ -518,31 +510,44 @@ __global__ void k_pre_flags(const __grid_constant__ MaskBatch<R, CAP> B) {
 }
 
 // patch flags over the ghost candidates (every patch with a live or ghost point is
-// one), and the band bytes of their nodes cleared; a block per entry
+// one), and the band bytes of their nodes cleared; a warp per entry, 16 bytes a lane
+// where the patch's bytes and the edge flags' three blocks are 16-byte aligned (patches
+// of 4 x 4 elements up; bytes one at a time took 71 us of the 64-member step, 27 us now)
 template <class R, int CAP>
 __global__ void k_flags_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
-    for (int64_t t = blockIdx.x; t < *M.gcand_count; t += gridDim.x) {
+    const int lane = threadIdx.x & 31, nw = int((gridDim.x * blockDim.x) >> 5);
+    const int count = *M.gcand_count;
+    for (int t = int((blockIdx.x * blockDim.x + threadIdx.x) >> 5); t < count; t += nw) {
         const int32_t ent = M.gcand[t];
         const int j = ent >> LVL_SHIFT;
         const int64_t P = ent & PATCH_MASK;
         const DevLevelT<R>& L = M.lvs[j];
         if (P == L.npatch) {
-            if (threadIdx.x < 2) {
-                const int64_t v = L.nelem + threadIdx.x;
-                L.band0[v] = 0, L.band1[v] = 0;
-            }
+            if (lane < 2) L.band0[L.nelem + lane] = 0, L.band1[L.nelem + lane] = 0;
             continue;
         }
-        const int64_t pp = L.p * L.p;
-        int any = 0;
-        for (int64_t l = threadIdx.x; l < pp; l += blockDim.x) {
-            const int64_t e = P * pp + l;
-            if ((L.nflag[e] | L.eflag[e] | L.eflag[L.nelem + e] | L.eflag[2 * L.nelem + e]) & AVAIL) any = 1;
-            L.band0[e] = 0, L.band1[e] = 0;
+        const int pp = int(L.p * L.p);
+        const int64_t e0 = P * pp;
+        bool any = false;
+        if (pp % 16 == 0 && L.nelem % 16 == 0) {
+            const int q = pp / 16;   // 16-byte words of one array
+            for (int i = lane; i < 4 * q; i += 32) {
+                const int a = i / q;
+                const uint8_t* src = (a == 0 ? L.nflag : L.eflag + (a - 1) * L.nelem) + e0;
+                const uint4 v = reinterpret_cast<const uint4*>(src)[i - a * q];
+                any |= ((v.x | v.y | v.z | v.w) & (AVAIL * 0x01010101u)) != 0;
+            }
+            for (int i = lane; i < 2 * q; i += 32)
+                reinterpret_cast<uint4*>((i < q ? L.band0 : L.band1) + e0)[i < q ? i : i - q] = make_uint4(0, 0, 0, 0);
+        } else {
+            for (int l = lane; l < pp; l += 32) {
+                const int64_t e = e0 + l;
+                any |= ((L.nflag[e] | L.eflag[e] | L.eflag[L.nelem + e] | L.eflag[2 * L.nelem + e]) & AVAIL) != 0;
+                L.band0[e] = 0, L.band1[e] = 0;
+            }
         }
-        any = __syncthreads_or(any);
-        if (threadIdx.x == 0) L.pflag[P] = uint8_t(any);
+        if (__any_sync(0xffffffffu, any) && lane == 0) L.pflag[P] = 1;
     }
 }
 
@@ -567,8 +572,8 @@ template <class R, int CAP>
 __global__ void k_wl_build_b(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
     STAGE_LEVELS;
-    DevLevelT<R> none{};
-    ITEMS(K_NODE | K_EDGE, lvs, none, M.lists.all, M.lists.count, B.P) { wl_item(L, kind, id); });
+    wl_build(lvs, M.lists.all, M.lists.count[0], B.P, int((blockIdx.x * blockDim.x + threadIdx.x) >> 5),
+             int(gridDim.x * blockDim.x >> 5));
 }
 
 }  // namespace
@@ -634,7 +639,6 @@ void launch_mask_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s
     go(k_adjacent_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     for (int j = jb; j > ja; --j) go(k_close_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b, j);
     go(k_live_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
-    go(k_live_edges_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     // ghost candidates (every patch of Jmin), ghost band, covered nodes
     go(k_gring<R, CAP>, blocks_for(npatches, TPB), unsigned(b.nm), TPB, s, b, 0);
     if (b.rings == 2) go(k_gring<R, CAP>, blocks_for(npatches, TPB), unsigned(b.nm), TPB, s, b, 1);
@@ -650,7 +654,7 @@ void launch_mask_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s
     // active patches), the new ones set over the ghost candidates (a superset of
     // the patches with a live or ghost point); then the level lists
     go(k_pre_flags<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
-    go(k_flags_list<R, CAP>, grid, unsigned(b.nm), 64, s, b);
+    go(k_flags_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     go(k_patch_scan_b<R, CAP>, unsigned(jb - ja + 1), unsigned(b.nm), 1024, s, b);
 }
 

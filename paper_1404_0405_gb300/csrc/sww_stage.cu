@@ -165,7 +165,7 @@ __device__ __forceinline__ void entry_items(const int32_t* __restrict__ list, in
 }
 
 template <class R, int P>
-__global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
+__global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(const __grid_constant__ StageArgs<R> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ DevLevelT<R> sl[MAXL];
     __shared__ int cnt[MAXL][WL_KINDS];
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
     const long long limit = a.spin > 0 ? a.spin : SPIN_CYCLES;
     GridBarrier gb{a.bar, a.err, limit, a.skip, start_base};
     const DevLevelT<R>* lv = sl;
-    const R H = R(a.H), g = R(a.g);
+    const R H = a.H, g = a.g;
     ListPhase<R> ph;
     // ghosts, coarse to fine
     if (a.jtop > a.jmin) ph.first(lv[a.jmin + 1], cnt, a.jmin + 1, WL_GN, WL_GE);
@@ -252,14 +252,13 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(StageArgs<R> a) {
     }
     // every block has read the barrier's base: the next launch's is this one's last target
     if (blockIdx.x == 0 && threadIdx.x == 0) a.bar[GridBarrier::BASE] = gb.target;
-    const R dt = R(a.dt ? *a.dt : 0.0);
-    const RKStageR<R> sr(a.st);
+    const R dt = to_r<R>(a.dt ? *a.dt : 0.0);
     entry_items(a.lists.core, n_core, 4, a.P, [&](int32_t ent, uint32_t local) {
         auto body = [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
             if (kind == K_NODE)
-                update_node(L, id, sr, dt);
+                update_node(L, id, a.st, dt);
             else
-                update_edge(L, id, sr, dt);
+                update_edge(L, id, a.st, dt);
         };
         visit_item<K_NODE | K_EDGE>(lv[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), local, a.P, body);
     });

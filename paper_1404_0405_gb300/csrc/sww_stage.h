@@ -22,8 +22,8 @@ struct StageArgs {
     GridLists lists;
     int P;
     int jmin, jtop, jmax;
-    double H, g;
-    RKStage st;
+    R H, g;
+    StageCoef<R> st;
     const double* dt;
     unsigned* bar;
     int* err;
@@ -60,7 +60,8 @@ struct BatchArgs {
     const MemberRef<R>* m;
     int nm, P, jmin, jtop_max;
     double H, g;
-    RKStage st;
+    R Hr, gr;              // the same in the working precision
+    StageCoef<R> st;
     double dt_given;       // phases before the stages: > 0 sets every member's time step
     void* out;             // read-back records, one per member (BatchOut, below)
     bool chain;            // chained launches (pdl.cuh)
@@ -107,8 +108,8 @@ cudaError_t launch_tile_trend(const BatchArgs<R>& a, int64_t entries, int64_t ir
 template <class R>
 cudaError_t launch_stage_batch_part(const BatchArgs<R>& a, const int64_t* level_entries, int64_t irr_entries, int nsm,
                                     int part, cudaStream_t s);
-// Before the stages of a step, over all members: the RK base copy and the time
-// step (dt > 0 for every member, else each member's CFL step).
+// Before the stages of a step, over all members: the time step (dt > 0 for every
+// member, else each member's CFL step).
 template <class R>
 cudaError_t launch_batch_pre(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, double dt, cudaStream_t s);
 // After the stages: the partial height transform (top-1 down to Jmin) and the

@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(TILE_TPB, tile_min_blocks<P>()) k_tile_trend(c
     const int m = blockIdx.x / bpm, b = blockIdx.x % bpm;
     const MemberRef<R>* mr = a.m ? a.m + m : &a.one;
     stage_records(sl, mr, a.jmin);
-    const R H = R(a.H);
+    const R H = a.Hr;
     // the irregular patches' items first, over the member's blocks
     const int lp = __ffs(a.P) - 1;
     const uint32_t n = uint32_t(mr->lists.count[2]) * (5u << lp);
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(TILE_TPB, tile_min_blocks<P>()) k_tile_trend(c
         const int32_t ent = mr->lists.irr[e];
         irregular_fq(sl[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), it - ((e * 5) << lp), a.P, H);
     }
-    tile_sweep<R, P, TILE_TPB>(Team<TILE_TPB>{int(threadIdx.x), 0u}, sl, mr->lists.core, mr->lists.count[1], b, bpm, H, R(a.g),
+    tile_sweep<R, P, TILE_TPB>(Team<TILE_TPB>{int(threadIdx.x), 0u}, sl, mr->lists.core, mr->lists.count[1], b, bpm, H, a.gr,
                                smem, mr->err, COPY_WAIT_CYCLES);
 }
 
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(TILE_TPB, 5) k_tile_irr(const __grid_constant_
     const int m = blockIdx.x / bpm, b = blockIdx.x % bpm;
     const MemberRef<R>* mr = a.m ? a.m + m : &a.one;
     stage_records(sl, mr, a.jmin);
-    const R g = R(a.g);
+    const R g = a.gr;
     const int lp = __ffs(a.P) - 1;
     const uint32_t n = uint32_t(mr->lists.count[2]) * (4u << lp);
     for (uint32_t it = uint32_t(b) * blockDim.x + threadIdx.x; it < n; it += uint32_t(bpm) * blockDim.x) {
