@@ -1360,6 +1360,9 @@ static int set_state_at(sww_handle* h, const double* dh, const double* u, int J,
                 const DevLevelT<R>& L = lv[j];
                 ck(cudaMemsetAsync(L.nflag, 0, L.N, s), "memset flags");
                 ck(cudaMemsetAsync(L.eflag, 0, L.E, s), "memset flags");
+                // marks of an earlier state's last mask
+                ck(cudaMemsetAsync(L.tmask, 0, L.N, s), "memset marks");
+                ck(cudaMemsetAsync(L.sig, 0, L.N, s), "memset marks");
                 ck(cudaMemsetAsync(L.dh, 0, L.N * sizeof(R), s), "memset state");
                 ck(cudaMemsetAsync(L.u, 0, L.E * sizeof(R), s), "memset state");
             }
