@@ -209,7 +209,11 @@ __device__ __forceinline__ void pv_at(const DevLevelT<R>& L, int64_t t, R H) {
     R hv = geo<R>(L.kite, t) * (H + dh[0]) + geo<R>(L.kite, L.T + t) * (H + dh[1]) + geo<R>(L.kite, 2 * L.T + t) * (H + dh[2]);
     R Av = geo<R>(L.A_v, t);
     if (viscous(L)) L.zeta[t] = circ / Av;
-    L.q[t] = (circ / Av + geo<R>(L.f_v, t)) / (hv / Av);
+    // one division in the FP64 form (the FP64 pipe is narrow)
+    if constexpr (sizeof(R) == 8)
+        L.q[t] = (circ + geo<R>(L.f_v, t) * Av) / hv;
+    else
+        L.q[t] = (circ / Av + geo<R>(L.f_v, t)) / (hv / Av);
 }
 
 // thickness flux F = h_e u at an edge
@@ -323,15 +327,17 @@ __device__ __forceinline__ void node_at(const DevLevelT<R>& L, int64_t v, R g) {
 template <class R>
 __device__ __forceinline__ void coriolis_at(const DevLevelT<R>& L, int64_t e) {
     if (L.advect || !(L.eflag[e] & LIVE)) return;
-    R qe = R(0.5) * (L.q[L.et[e]] + L.q[L.et[L.E + e]]);
+    // the factors 1/2 of the q averages out of the sum (exact: powers of two)
+    R qe = L.q[L.et[e]] + L.q[L.et[L.E + e]];
     R s = R(0);
 #pragma unroll
     for (int k = 0; k < 10; ++k) {
         int32_t e2 = L.cor_i[k * L.E + e];
         R w = geo<R>(L.cor_w, k * L.E + e);
-        R q2 = R(0.5) * (L.q[L.et[e2]] + L.q[L.et[L.E + e2]]);
-        s += w * L.F[e2] * R(0.5) * (qe + q2);
+        R q2 = L.q[L.et[e2]] + L.q[L.et[L.E + e2]];
+        s += w * L.F[e2] * (qe + q2);
     }
+    s *= R(0.25);
     // viscous form: -nu grad^perp curl u, grad^perp zeta = (1/l_e) sum_{v at e} t_{e,v} zeta_v
     if (viscous(L)) {
         R gp = R(0);

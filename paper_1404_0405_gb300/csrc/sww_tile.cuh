@@ -163,16 +163,25 @@ __device__ __forceinline__ constexpr int kite_off(int k) {
     return ring_tri_off<W, NN>(k) - (k & 1) * NN + (3 * (k & 1) + (k >> 1)) * NN;
 }
 
+// The FP64 form is bound by the FP64 pipe (one warp instruction per 16 clocks and SM), so
+// its tiles take the products they share once: l_e F_e per edge instead of per edge and
+// neighbour, 1/A_i per node, one division for q.  The FP32 form keeps the order of
+// operations of the tabulated bodies.
+template <class R>
+constexpr bool fp64_form = sizeof(R) == 8;
+
 // q F^perp at the live edge of orientation O from node slot x: the two cells'
 // contributions n_{e,i} sum_{m=1..5} n_{e',i} (1/2 - sum of the fractions passed) l_{e'}
 // F_{e'} (q_e + q_{e'})/2, over d_e (edge e sits at ring position O of its origin and
-// O + 3 of its end); a node's kite fractions are its kites times is (1 / their sum)
+// O + 3 of its end); a node's kite fractions are its kites times is (1 / their sum).  The
+// factors 1/2 of the q averages are taken out of the sum (exact: powers of two).  F holds
+// l_e F_e in the FP64 form.
 template <class R, int W, int NN, int O>
 __device__ __forceinline__ R tile_coriolis(int x, const R* q, const R* F, const R* le, const R* de, const R* kt,
                                            const R* is) {
     constexpr int xe = O == 0 ? W : O == 1 ? W + 1 : 1;   // end node slot - origin node slot
     const int y = O * NN + x;
-    const R qe = R(0.5) * (q[x + ring_tri_off<W, NN>(O)] + q[x + ring_tri_off<W, NN>((O + 5) % 6)]);
+    const R qe = q[x + ring_tri_off<W, NN>(O)] + q[x + ring_tri_off<W, NN>((O + 5) % 6)];
     const R inv_d = R(1) / de[y];
     R s = R(0);
 #pragma unroll
@@ -188,12 +197,16 @@ __device__ __forceinline__ R tile_coriolis(int x, const R* q, const R* F, const 
             csum += kt[kite_off<W, NN>(kp) + xv] * inv_s;
             const int y2 = xv + ring_edge_off<W, NN>(kk);
             const R n2 = kk < 3 ? R(1) : R(-1);
-            const R q2 = R(0.5) * (q[xv + ring_tri_off<W, NN>(kk)] + q[xv + ring_tri_off<W, NN>((kk + 5) % 6)]);
-            const R w = ne * n2 * (R(0.5) - csum) * le[y2] * inv_d;
-            s += w * F[y2] * R(0.5) * (qe + q2);
+            const R q2 = q[xv + ring_tri_off<W, NN>(kk)] + q[xv + ring_tri_off<W, NN>((kk + 5) % 6)];
+            if constexpr (fp64_form<R>) {
+                s += ne * n2 * (R(0.5) - csum) * F[y2] * (qe + q2);
+            } else {
+                const R w = ne * n2 * (R(0.5) - csum) * le[y2] * inv_d;
+                s += w * F[y2] * (qe + q2);
+            }
         }
     }
-    return s;
+    return fp64_form<R> ? R(0.25) * s * inv_d : R(0.25) * s;
 }
 
 // The halo ids a thread's slots need for one tile (own slots: unused), loaded one
@@ -402,6 +415,7 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
                 if (plan.e[i] < 0) L.F[o * nelem + base + (-plan.e[i] - 1 - o * PP)] = f;
             }
         }
+        if constexpr (fp64_form<R>) f *= le[y];
         F[y] = f;
     }
 #pragma unroll
@@ -421,7 +435,10 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
             const R hv = kt[(3 * t) * NN + x] * (H + dh[x]) + kt[(3 * t + 1) * NN + x] * (H + dh[n1]) +
                          kt[(3 * t + 2) * NN + x] * (H + dh[n2]);
             const R A = av[z];
-            qq = (circ / A + fv[z]) / (hv / A);
+            if constexpr (fp64_form<R>)
+                qq = (circ + fv[z] * A) / hv;
+            else
+                qq = (circ / A + fv[z]) / (hv / A);
             if (c < 0) L.q[t * nelem + base + (-c - 1 - t * PP)] = qq;
         }
         q[z] = qq;
@@ -441,14 +458,25 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
                 const int y = x + ring_edge_off<W, NN>(k);
                 okr = okr && (ef[y] & AVAIL);
                 const R n = k < 3 ? R(1) : R(-1);
-                div += n * F[y] * le[y];
-                ke += R(0.25) * le[y] * de[y] * u[y] * u[y];
+                if constexpr (fp64_form<R>) {
+                    div += n * F[y];
+                    ke += le[y] * de[y] * (u[y] * u[y]);
+                } else {
+                    div += n * F[y] * le[y];
+                    ke += R(0.25) * le[y] * de[y] * u[y] * u[y];
+                }
             }
             if (!okr) continue;
             const int32_t v = base + i;
             const R A = ai[i];
-            L.c[v] = div / A;
-            L.B[v] = g * dh[x] + ke / A;
+            if constexpr (fp64_form<R>) {
+                const R inv_a = R(1) / A;
+                L.c[v] = div * inv_a;
+                L.B[v] = g * dh[x] + R(0.25) * ke * inv_a;
+            } else {
+                L.c[v] = div / A;
+                L.B[v] = g * dh[x] + ke / A;
+            }
         } else {
             const int o = (w - PP) / PP, i = (w - PP) - o * PP, x = T::at(i / P, i % P);
             if (!(ef[o * NN + x] & LIVE)) continue;
