@@ -58,7 +58,7 @@ __global__ void k_gather_counts(const DevLevelT<R>* lvs, int jmin, int jmax, int
     int j = jmin + int(threadIdx.x);
     if (j <= jmax) {
         out[j] = *lvs[j].npatches;
-        out[jmax + 1 + j] = lvs[j].wl_n[WL_LIVE];
+        out[jmax + 1 + j] = lvs[j].wl_n[WL_LN];
     }
 }
 
@@ -515,9 +515,9 @@ void alloc_state(sww_handle* h, int j) {
     D.clist = h->alloc<int32_t>(D.npatch + 1);
     D.ilist = h->alloc<int32_t>(D.npatch + 1);
     D.npatches = h->alloc<int32_t>(LIST_COUNTS);
-    D.wl = h->alloc<int32_t>(3 * N + 2 * E);
-    D.wl_n = h->alloc<int32_t>(WL_WORDS);
-    ck(cudaMemset(D.wl_n, 0, WL_WORDS * sizeof(int32_t)), "memset");
+    D.wl = h->alloc<int32_t>(4 * N + 3 * E);
+    D.wl_n = h->alloc<int32_t>(WL_KINDS);
+    ck(cudaMemset(D.wl_n, 0, WL_KINDS * sizeof(int32_t)), "memset");
     uint8_t** cf[] = {&D.zflag, &D.sflag, &D.cflag, &D.lflag, &D.gflag};
     for (auto p : cf) {
         *p = h->alloc<uint8_t>(D.npatch + 1);
@@ -809,7 +809,7 @@ MaskMember<R> mask_member(const sww_handle* h) {
     m.thr = h->thr, m.sig_any = h->sig_any, m.lstat = h->lstat, m.net = h->d_net;
     m.logit_tau = std::log(h->tau / (1.f - h->tau));
     m.learn = h->learn_mode;
-    m.jb = std::min(h->jtop + 1, h->cfg.jmax), m.jmax = h->cfg.jmax;
+    m.jtop = h->jtop, m.jb = std::min(h->jtop + 1, h->cfg.jmax), m.jmax = h->cfg.jmax;
     return m;
 }
 

@@ -61,23 +61,6 @@ __device__ unsigned long long block_reduce_u64(unsigned long long v, Op op, unsi
     return sh[0];
 }
 
-// items of `n_entries` entries of `list` (levels from the staged records `sl`),
-// block b of bpm blocks of the member
-template <int KINDS, class R, class Body>
-__device__ __forceinline__ void member_items(const DevLevelT<R>* sl, const int32_t* __restrict__ list,
-                                             int64_t n_entries, int P, int b, int bpm, Body body) {
-    constexpr uint32_t NS = slots_of<KINDS>();
-    const int lp = __ffs(P) - 1;
-    const uint32_t n = uint32_t(n_entries) * (NS << lp);
-    const uint32_t stride = uint32_t(bpm) * blockDim.x;
-    for (uint32_t it = uint32_t(b) * blockDim.x + threadIdx.x; it < n; it += stride) {
-        const uint32_t e = (it >> lp) / NS;
-        const int32_t ent = list[e];
-        const DevLevelT<R>& L = sl[ent >> LVL_SHIFT];
-        visit_item<KINDS>(L, int64_t(ent & PATCH_MASK), it - ((e * NS) << lp), P, body);
-    }
-}
-
 // items of work lists k0 and k1 (k1 < 0: none) of level L, block b of the
 // member's bpm blocks: body(0, id) for list k0, body(1, id) for list k1
 template <class R, class Body>
@@ -132,7 +115,7 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         if (t < 16) {
             const bool in = t >= a.jmin && t <= mr->jmax;
             o->counts[t] = in ? *mr->lvs[t].npatches : 0;
-            o->live[t] = in ? mr->lvs[t].wl_n[WL_LIVE] : 0;
+            o->live[t] = in ? mr->lvs[t].wl_n[WL_LN] : 0;
         }
         if (t == 0) {
             o->dt = *mr->dt;
@@ -159,6 +142,14 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         for (int k = threadIdx.x; k < words; k += blockDim.x) dst[k] = src[k];
     }
     __syncthreads();
+    // the live points of every level
+    constexpr bool all_live = PH == PH_UPDATE || PH == PH_DT || PH == PH_DETAILS;
+    __shared__ LiveItems live;
+    const int first = b * int(blockDim.x) + int(threadIdx.x), stride = bpm * int(blockDim.x);
+    if constexpr (all_live) {
+        live.init(sl, a.jmin, jtop);
+        __syncthreads();
+    }
     if constexpr (PH == PH_FILL || PH == PH_INV_FILL) {
         // ghost nodes and edges of level j from level j - 1
         member_wl(sl[j], WL_GN, WL_GE, b, bpm, [&](int k, int64_t id) {
@@ -190,16 +181,14 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         __syncthreads();
         unsigned long long wmax = 0;
         LevelMax um;
-        member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
-                                      [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
-                                          if (kind == K_NODE) {
-                                              if (L.advect || !(L.nflag[id] & LIVE)) return;
-                                              wmax = max(wmax, dbits(omega2_at(L, id, a.H, a.g)));
-                                          } else if (L.eflag[id] & LIVE) {
-                                              const unsigned long long k = abs_key(L.u[id]);
-                                              if (k && k <= inf_key<R>()) um.add(L.J, k, slev);
-                                          }
-                                      });
+        live.run(sl, a.jmin, jtop, first, stride, [&](const DevLevelT<R>& L, int kind, int64_t id) {
+            if (kind == K_NODE) {
+                if (!L.advect) wmax = max(wmax, dbits(omega2_at(L, id, a.H, a.g)));
+            } else {
+                const unsigned long long k = abs_key(L.u[id]);
+                if (k && k <= inf_key<R>()) um.add(L.J, k, slev);
+            }
+        });
         um.flush(slev);
         wmax = block_reduce_u64(wmax, MaxU64(), sh);   // synchronises the block: slev is complete
         if (threadIdx.x == 0 && wmax) atomicMax(&mr->red[0], wmax);
@@ -212,15 +201,13 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         // doubles); the details only read dh and u
         __shared__ unsigned long long shm[BATCH_TPB / 32];
         unsigned long long hmax = 0, umax = 0;
-        member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
-                                      [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
-                                          if (kind == K_NODE) {
-                                              if (L.nflag[id] & LIVE) hmax = max(hmax, abs_key(L.dh[id]));
-                                          } else {
-                                              if (L.eflag[id] & LIVE) umax = max(umax, abs_key(L.u[id]));
-                                          }
-                                          if (L.J > a.jmin) details_item(L, (&L)[-1], kind, id);
-                                      });
+        live.run(sl, a.jmin, jtop, first, stride, [&](const DevLevelT<R>& L, int kind, int64_t id) {
+            if (kind == K_NODE)
+                hmax = max(hmax, abs_key(L.dh[id]));
+            else
+                umax = max(umax, abs_key(L.u[id]));
+            if (L.J > a.jmin) details_item(L, (&L)[-1], kind, id);
+        });
         hmax = block_reduce_u64(hmax, MaxU64(), shm);
         umax = block_reduce_u64(umax, MaxU64(), shm);
         if (threadIdx.x == 0) {
@@ -228,23 +215,19 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
             if (umax) atomicMax(&mr->red[3], dbits(key_value<R>(umax)));
         }
     } else if constexpr (PH == PH_INV_A) {
-        member_items<K_NODE | K_EDGE>(sl, sl[j].clist, sl[j].npatches[1], a.P, b, bpm,
-                                      [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
-                                          inverse_a_item(L, (&L)[-1], kind, id);
-                                      });
+        member_wl(sl[j], WL_LN, WL_LE, b, bpm,
+                  [&](int k, int64_t id) { inverse_a_item(sl[j], sl[j - 1], k == 0 ? K_NODE : K_EDGE, id); });
     } else if constexpr (PH == PH_INV_B) {
-        member_items<K_NODE>(sl, sl[j].clist, sl[j].npatches[1], a.P, b, bpm,
-                             [&](const DevLevelT<R>& L, int, int64_t id, int64_t) { inverse_b_item(L, id); });
+        member_wl(sl[j], WL_LN, -1, b, bpm, [&](int, int64_t id) { inverse_b_item(sl[j], id); });
     } else {
         static_assert(PH == PH_UPDATE || PH == PH_SET_DT || PH == PH_DT_FINAL || PH == PH_THRESH || PH == PH_OUT, "phase");
         const R dt = to_r<R>(mr->dt ? *mr->dt : 0.0);
-        member_items<K_NODE | K_EDGE>(sl, mr->lists.core, mr->lists.count[1], a.P, b, bpm,
-                                      [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
-                                          if (kind == K_NODE)
-                                              update_node(L, id, a.st, dt);
-                                          else
-                                              update_edge(L, id, a.st, dt);
-                                      });
+        live.run(sl, a.jmin, jtop, first, stride, [&](const DevLevelT<R>& L, int kind, int64_t id) {
+            if (kind == K_NODE)
+                update_node(L, id, a.st, dt);
+            else
+                update_edge(L, id, a.st, dt);
+        });
     }
 }
 

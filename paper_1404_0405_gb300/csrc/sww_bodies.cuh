@@ -375,7 +375,6 @@ __device__ __forceinline__ void rk_apply(const StageCoef<R>& st, R dt, R k, R* y
 
 template <class R>
 __device__ __forceinline__ void update_node(const DevLevelT<R>& L, int64_t v, const StageCoef<R>& st, R dt) {
-    if (!(L.nflag[v] & LIVE)) return;
     R k = -L.c[v];
     if (st.trend) L.dht[v] = k;
     if (st.apply) rk_apply(st, dt, k, &L.dh[v], &L.dh0[v], &L.dha[v]);
@@ -383,7 +382,6 @@ __device__ __forceinline__ void update_node(const DevLevelT<R>& L, int64_t v, co
 
 template <class R>
 __device__ __forceinline__ void update_edge(const DevLevelT<R>& L, int64_t e, const StageCoef<R>& st, R dt) {
-    if (!(L.eflag[e] & LIVE)) return;
     if (L.advect) {   // prescribed velocity: zero trend, u untouched
         if (st.trend) L.ut[e] = R(0);
         return;
@@ -457,29 +455,29 @@ __device__ __forceinline__ void fill_edge(const DevLevelT<R>& F, const DevLevelT
 
 // ---------------------------------------------------------------------------- transforms (Eqs. 1-2)
 
+// A coarse edge has a coefficient when one of its halves is live; it is taken at the first
+// half (kind 0) when that is live, else at the second.  Live half i of the other half o,
+// kind k: whether i is the one.
+__device__ __forceinline__ bool pair_at(int k, uint8_t other_flag) { return k == 0 || !(other_flag & LIVE); }
+
 // wavelet coefficients at a live point of F > Jmin from C = the level below
 // (Eqs. 1-2; velocity transform of Sec. 4.1): h~ at odd nodes, u~ at interior fine
-// edges, and u~_E of a coarse edge at its first half (visited by elements and their
-// edges alone: a pass over the coarse edges under even elements keeps a quarter of its
-// threads busy)
+// edges, u~_E of a coarse edge at one of its live halves
 template <class R>
 __device__ __forceinline__ void details_item(const DevLevelT<R>& L, const DevLevelT<R>& C, int kind, int64_t id) {
     if (kind == K_NODE) {
-        const int32_t k = L.f2c[id];
-        const uint8_t f = L.nflag[id];
-        if ((k < 0) & ((f & LIVE) != 0)) L.hdet[id] = height_detail(L, id);
+        if (L.f2c[id] < 0) L.hdet[id] = height_detail(L, id);
         return;
     }
-    const int fk = L.fe_kind[id];
-    const uint8_t f = L.eflag[id];
     const int32_t o = L.fe_ot[id];
-    if (fk == 1) return;
-    if (fk == 2) {
-        if (f & LIVE) L.ui[id] = L.u[id] - predict(L, C.u, id);
-    } else if ((f | L.eflag[o]) & LIVE) {
-        R a = L.u[id] - predict(L, C.u, id);
-        R b = L.u[o] - predict(L, C.u, o);
-        L.ue[L.fe_ce[id]] = R(0.5) * (a - b);
+    const int fk = L.fe_kind[id];
+    if (o >= 0 && !pair_at(fk, L.eflag[o])) return;
+    const R di = L.u[id] - predict(L, C.u, id);
+    if (o < 0) {
+        L.ui[id] = di;
+    } else {
+        const R d_o = L.u[o] - predict(L, C.u, o);
+        L.ue[L.fe_ce[id]] = fk == 0 ? R(0.5) * (di - d_o) : R(0.5) * (d_o - di);
     }
 }
 
@@ -489,9 +487,8 @@ __device__ __forceinline__ void details_item(const DevLevelT<R>& L, const DevLev
 template <class R>
 __device__ __forceinline__ void inverse_a_item(const DevLevelT<R>& L, const DevLevelT<R>& C, int kind, int64_t id) {
     if (kind == K_NODE) {
-        const uint8_t f = L.nflag[id];
         const int32_t k = L.f2c[id];
-        if (!(f & LIVE) | (k < 0)) return;
+        if (k < 0) return;
         R s = C.dh[k];
 #pragma unroll
         for (int g = 0; g < 12; g += 6) {
@@ -517,7 +514,6 @@ __device__ __forceinline__ void inverse_a_item(const DevLevelT<R>& L, const DevL
     const uint8_t fi = L.eflag[i];
     const int32_t o = L.fe_ot[i], E = L.fe_ce[i];
     const int fk = L.fe_kind[i];
-    if (!(fi & LIVE)) return;
     if (o < 0) {
         const R Pr = predict(L, C.u, i), d = L.ui[i];
         L.u[i] = Pr + ((fi & WASLIVE) ? d : R(0));
@@ -545,7 +541,7 @@ template <class R>
 __device__ __forceinline__ void inverse_b_item(const DevLevelT<R>& L, int64_t id) {
     const uint8_t f = L.nflag[id];
     const int32_t k = L.f2c[id];
-    if (!(f & LIVE) | (k >= 0)) return;
+    if (k >= 0) return;
     R s = (f & WASLIVE) ? L.hdet[id] : R(0);
 #pragma unroll
     for (int q = 0; q < 4; ++q) s += L.ptw[q * L.N + id] * L.dh[L.par[q * L.N + id]];
@@ -624,34 +620,32 @@ __device__ __forceinline__ double sig_thr<double>(double e) { return e; }
 template <>
 __device__ __forceinline__ float sig_thr<float>(double e) { return __double2float_ru(e); }
 
+// at a live node
 template <class R>
 __device__ __forceinline__ bool sig_node(const DevLevelT<R>& F, int64_t i, R eh) {
     const int32_t k = F.f2c[i];
-    const uint8_t f = F.nflag[i];
     const R d = F.hdet[i];
-    if ((k < 0) & ((f & LIVE) != 0) & (fabs(d) >= eh)) {
+    if ((k < 0) & (fabs(d) >= eh)) {
         F.sig[i] = 1;
         return true;
     }
     return false;
 }
 
-// a fine edge of kind 2, or the coarse edge of a first half (kind 0)
+// at a live edge: its own coefficient, or its coarse edge's (pair_at)
 template <class R>
 __device__ __forceinline__ bool sig_edge(const DevLevelT<R>& F, const DevLevelT<R>& C, int64_t i, R eu) {
+    const int32_t o = F.fe_ot[i], E = F.fe_ce[i];
     const int k = F.fe_kind[i];
-    const uint8_t f = F.eflag[i];
-    if (k == 1) return false;
-    if (k == 2) {
-        const R d = F.ui[i];
-        if (!((f & LIVE) != 0 & fabs(d) >= eu)) return false;
+    if (o < 0) {
+        if (!(fabs(F.ui[i]) >= eu)) return false;
         F.sig[F.en[i]] = 1;
         F.sig[F.en[F.E + i]] = 1;
         return true;
     }
-    const int32_t E = F.fe_ce[i];
+    const uint8_t fo = F.eflag[o];
     const R d = F.ue[E];
-    if (!(((f | F.eflag[F.fe_ot[i]]) & LIVE) != 0 & fabs(d) >= eu)) return false;
+    if (!(pair_at(k, fo) & (fabs(d) >= eu))) return false;
     F.sig[C.c2f[C.en[E]]] = 1;
     F.sig[C.c2f[C.en[C.E + E]]] = 1;
     F.sig[C.mid[E]] = 1;
@@ -920,29 +914,71 @@ __device__ void concat_lists(const DevLevelT<R>* __restrict__ lvs, int jmin, int
         for (int i = threadIdx.x; i < n; i += blockDim.x) dst[q][base[q] + i] = src[q][i];
         if (j == jmax && threadIdx.x == 0) g.count[q] = base[q] + n;
     }
-    if (threadIdx.x < WL_WORDS && L.wl_n) L.wl_n[threadIdx.x] = 0;
+    if (threadIdx.x < WL_KINDS && L.wl_n) L.wl_n[threadIdx.x] = 0;
 }
 
 // offset of work list k of a level in wl
 template <class R>
 __device__ __forceinline__ int64_t wl_off(const DevLevelT<R>& L, int k) {
-    return k == WL_GN ? 0 : k == WL_GE ? L.N : k == WL_CN ? L.N + L.E : k == WL_RE ? 2 * L.N + L.E : 2 * L.N + 2 * L.E;
+    const int edges = k <= WL_GE ? 0 : k <= WL_RE ? 1 : 2;   // lists of edges before list k
+    return (k - edges) * L.N + edges * L.E;
 }
 
-// The point work lists and the live-node counts of the entries of `list`, a warp an entry
-// (warp w of nw warps): ghost points, covered nodes, edges with a covered end, and
+// The live points of levels ja..jb of one block's shared copy of the level records, item i
+// of n(): off[j - ja] the items before level j.  A thread's items rise, so it steps its
+// level up as it goes.  Passes over live points that visited every item of the core
+// patches kept under half of their threads busy (41 % of the core's nodes are live on
+// the jet at eps 1e-2, 31 % on a 64-member ensemble).
+struct LiveItems {
+    int off[14], nodes[14];
+
+    // by the whole block, then a block barrier by the caller
+    template <class R>
+    __device__ void init(const DevLevelT<R>* lv, int ja, int jb) {
+        if (threadIdx.x < 32) {
+            const int lane = threadIdx.x, j = ja + lane;
+            const int nn = j <= jb ? lv[j].wl_n[WL_LN] : 0, n = j <= jb ? nn + lv[j].wl_n[WL_LE] : 0;
+            int incl = n;
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (lane < 14) off[lane] = incl - n, nodes[lane] = nn;
+        }
+    }
+    // items first, first + stride, ...: body(L, kind, id)
+    template <class R, class Body>
+    __device__ __forceinline__ void run(const DevLevelT<R>* lv, int ja, int jb, int first, int stride, Body body) const {
+        int j = ja;
+        const int n = off[jb + 1 - ja];
+        for (int i = first; i < n; i += stride) {
+            while (i >= off[j + 1 - ja]) ++j;
+            const DevLevelT<R>& L = lv[j];
+            const int nn = nodes[j - ja], k = i - off[j - ja];
+            if (k < nn)
+                body(L, K_NODE, int64_t(L.wl[wl_off(L, WL_LN) + k]));
+            else
+                body(L, K_EDGE, int64_t(L.wl[wl_off(L, WL_LE) + (k - nn)]));
+        }
+    }
+};
+
+// The point work lists of the entries of `list`, a warp an entry (warp w of nw warps):
+// live points, ghost points, covered nodes, edges with a covered end, and
 // available nodes with a covered node among themselves and their neighbours (their
 // divergence changes with the restricted fluxes).  The warp goes through the entry's
 // node and edge slots 256 items at a time, keeps in which lists each belongs, and then
 // reserves its room with one addition per list, by a lane each.  (With one addition per
 // 32 items they queued on the lists' counters: 260 us for the 52 632 patches of
-// turbulence at Jmax 9, 142 us now.)  The order of the lists is not fixed; every item's
+// turbulence at Jmax 9, 136 us now, with
+// the lists of live points.)  The order of the lists is not fixed; every item's
 // work is independent of it.
 template <class R>
 __device__ __forceinline__ unsigned wl_member(const DevLevelT<R>& L, int kind, int64_t id) {
     if (kind == K_NODE) {
         const uint8_t f = L.nflag[id];
-        return ((f & LIVE) ? 1u << WL_LIVE : 0u) | ((f & GHOST) ? 1u << WL_GN : 0u) | ((f & COVERED) ? 1u << WL_CN : 0u) |
+        return ((f & LIVE) ? 1u << WL_LN : 0u) | ((f & GHOST) ? 1u << WL_GN : 0u) | ((f & COVERED) ? 1u << WL_CN : 0u) |
                (restricted_div_node(L, id) ? 1u << WL_DN : 0u);
     }
     const uint8_t f = L.eflag[id];
@@ -950,54 +986,73 @@ __device__ __forceinline__ unsigned wl_member(const DevLevelT<R>& L, int kind, i
     // the first half of a coarse edge fills a ghost second half too (fill_edge)
     bool ge = (f & GHOST) != 0;
     if (ge && L.fe_kind[id] == 1 && (L.eflag[L.fe_ot[id]] & GHOST)) ge = false;
-    return (ge ? 1u << WL_GE : 0u) | (((L.nflag[na] | L.nflag[nb]) & COVERED) ? 1u << WL_RE : 0u);
+    return ((f & LIVE) ? 1u << WL_LE : 0u) | (ge ? 1u << WL_GE : 0u) | (((L.nflag[na] | L.nflag[nb]) & COVERED) ? 1u << WL_RE : 0u);
 }
 
-template <class R>
-__device__ void wl_build(const DevLevelT<R>* __restrict__ lvs, const int32_t* __restrict__ list, int count, int P, int w,
-                         int nw) {
-    constexpr int G = 8;   // groups of 32 items a round
-    const int lane = threadIdx.x & 31;
+// one entry of patch area P: its G groups of 32 items from g0 on
+template <int P, int G, class R>
+__device__ __forceinline__ void wl_groups(const DevLevelT<R>& L, int64_t pat, int g0, int lane) {
     const unsigned below = (1u << lane) - 1u;
-    const int groups = 4 * P / 32;   // P >= 16
+    // a group holds nodes (its items below P), edges, or for P = 16 both
+    auto holds = [](int g, int k) {
+        const bool node = k == WL_GN || k == WL_CN || k == WL_DN || k == WL_LN;
+        return node ? g * 32 < P : (g + 1) * 32 > P;
+    };
+    int32_t id[G];
+    unsigned in[G], m[G][WL_KINDS];
+    int n = 0;   // lane k: entries of list k
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        in[g] = 0u, id[g] = 0;
+        auto body = [&](const DevLevelT<R>& LL, int kind, int64_t i, int64_t) {
+            id[g] = int32_t(i);
+            in[g] = wl_member(LL, kind, i);
+        };
+        visit_item<K_NODE | K_EDGE>(L, pat, uint32_t((g0 + g) * 32 + lane), P, body);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int k = 0; k < WL_KINDS; ++k)
+            if (holds(g0 + g, k)) {
+                m[g][k] = __ballot_sync(0xffffffffu, in[g] >> k & 1u);
+                if (lane == k) n += __popc(m[g][k]);
+            }
+    int at = 0;
+    if (lane < WL_KINDS && n) at = atomicAdd(&L.wl_n[lane], n);
+#pragma unroll
+    for (int k = 0; k < WL_KINDS; ++k) {
+        int pos = __shfl_sync(0xffffffffu, at, k);
+        int32_t* __restrict__ out = L.wl + wl_off(L, k);
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            if (holds(g0 + g, k)) {
+                if (in[g] >> k & 1u) out[pos + __popc(m[g][k] & below)] = id[g];
+                pos += __popc(m[g][k]);
+            }
+    }
+}
+
+template <int P, class R>
+__device__ __forceinline__ void wl_entries(const DevLevelT<R>* __restrict__ lvs, const int32_t* __restrict__ list,
+                                           int count, int w, int nw) {
+    constexpr int NG = 4 * P / 32, G = NG < 8 ? NG : 8;
     for (int t = w; t < count; t += nw) {
         const int32_t ent = list[t];
         const DevLevelT<R>& L = lvs[ent >> LVL_SHIFT];
-        for (int g0 = 0; g0 < groups; g0 += G) {
-            int32_t id[G];
-            unsigned in[G];
-            int n = 0;   // lane k < WL_WORDS: entries of list k
 #pragma unroll
-            for (int g = 0; g < G; ++g) {
-                in[g] = 0u, id[g] = 0;
-                auto body = [&](const DevLevelT<R>& LL, int kind, int64_t i, int64_t) {
-                    id[g] = int32_t(i);
-                    in[g] = wl_member(LL, kind, i);
-                };
-                if (g0 + g < groups)
-                    visit_item<K_NODE | K_EDGE>(L, int64_t(ent & PATCH_MASK), uint32_t((g0 + g) * 32 + lane), P, body);
-            }
-            __syncwarp();
-#pragma unroll
-            for (int g = 0; g < G; ++g)
-#pragma unroll
-                for (int k = 0; k < WL_WORDS; ++k) {
-                    const int c = __popc(__ballot_sync(0xffffffffu, in[g] >> k & 1u));
-                    if (lane == k) n += c;
-                }
-            int at = 0;
-            if (lane < WL_WORDS && n) at = atomicAdd(&L.wl_n[lane], n);
-#pragma unroll
-            for (int k = 0; k < WL_KINDS; ++k) {
-                int pos = __shfl_sync(0xffffffffu, at, k);
-                int32_t* __restrict__ out = L.wl + wl_off(L, k);
-#pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    const unsigned m = __ballot_sync(0xffffffffu, in[g] >> k & 1u);
-                    if (in[g] >> k & 1u) out[pos + __popc(m & below)] = id[g];
-                    pos += __popc(m);
-                }
-            }
-        }
+        for (int g0 = 0; g0 < NG; g0 += G) wl_groups<P, G>(L, int64_t(ent & PATCH_MASK), g0, int(threadIdx.x & 31));
     }
+}
+
+template <class R>
+__device__ __forceinline__ void wl_build(const DevLevelT<R>* __restrict__ lvs, const int32_t* __restrict__ list, int count,
+                                         int P, int w, int nw) {
+    if (P == 64)
+        wl_entries<64>(lvs, list, count, w, nw);
+    else if (P == 16)
+        wl_entries<16>(lvs, list, count, w, nw);
+    else
+        wl_entries<256>(lvs, list, count, w, nw);
 }

@@ -15,10 +15,9 @@ constexpr int NF = 8, NH = 32, NB = 24;
 constexpr int MLP_PARAMS = NF * NH + NH + NH + 1;   // W1[NF][NH], b1[NH], w2[NH], b2
 
 // Work lists of a level (DevLevelT::wl): ghost nodes, ghost edges (of two ghost halves of
-// a coarse edge only the first, which fills both), covered nodes,
-// edges with a covered end, nodes whose divergence the restriction changes; and the
-// level's live-node count, taken in the same pass (wl_n[WL_LIVE]).
-constexpr int WL_GN = 0, WL_GE = 1, WL_CN = 2, WL_RE = 3, WL_DN = 4, WL_KINDS = 5, WL_LIVE = 5, WL_WORDS = 6;
+// a coarse edge only the first, which fills both), covered nodes, edges with a covered
+// end, nodes whose divergence the restriction changes, live nodes, live edges.
+constexpr int WL_GN = 0, WL_GE = 1, WL_CN = 2, WL_RE = 3, WL_DN = 4, WL_LN = 5, WL_LE = 6, WL_KINDS = 7;
 
 // The core of the active grid.  A live node's or edge's update reads fluxes, potential
 // vorticities, divergences and Bernoulli functions owned by nodes within two hops of
@@ -110,11 +109,9 @@ struct DevLevelT {
     // ones whose tile is not regular; same order and entries as `patches`
     uint8_t* kflag;                // [npatch+1] patch is in the core
     int32_t *clist, *ilist;        // [npatch + 1]
-    // work lists of the stage's point-wise phases, rebuilt with the active lists
-    // (after every adaptation): ghost nodes [N], ghost edges [E], covered nodes [N],
-    // edges with a covered end [E], available nodes with a covered node among them and
-    // their neighbours [N], at offsets 0, N, N+E, 2N+E, 2N+2E of wl; their counts in
-    // wl_n[0..4]; wl_n[WL_LIVE] the level's live nodes
+    // work lists of the point-wise phases, rebuilt with the active lists (after every
+    // adaptation): list k (WL_GN ...) at wl_off(k) of wl, its length in wl_n[k]; lists of
+    // nodes hold at most N ids, of edges E: 4 N + 3 E in all
     int32_t* wl;
     int32_t* wl_n;
     // candidate patches of the list-based mask (index npatch: the two poles)

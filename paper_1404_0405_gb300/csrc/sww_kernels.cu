@@ -233,8 +233,8 @@ __global__ void k_sig(const DevLevelT<R>* __restrict__ lvs, Span sp, const doubl
         const DevLevelT<R>& C = lvs[j - 1];
         bool any = false;
         const R eh = sig_thr<R>(thr[0]), eu = sig_thr<R>(thr[1]);
-        if (i < F.N) any |= sig_node(F, i, eh);
-        if (i < F.E) any |= sig_edge(F, C, i, eu);
+        if (i < F.N && (F.nflag[i] & LIVE)) any |= sig_node(F, i, eh);
+        if (i < F.E && (F.eflag[i] & LIVE)) any |= sig_edge(F, C, i, eu);
         if (any) sig_any[j] = 1;
     });
 }
@@ -340,7 +340,7 @@ __global__ void k_concat(const DevLevelT<R>* __restrict__ lvs, int jmin, int jma
 
 // the point work lists of every level from the all-level list
 template <class R>
-__global__ void k_wl_build(const DevLevelT<R>* __restrict__ lvs, const int32_t* __restrict__ list,
+__global__ void __launch_bounds__(TPB, 4) k_wl_build(const DevLevelT<R>* __restrict__ lvs, const int32_t* __restrict__ list,
                            const int32_t* __restrict__ count, int P) {
     wl_build(lvs, list, *count, P, int(gid() >> 5), int(gridDim.x * blockDim.x >> 5));
 }

@@ -270,27 +270,30 @@ __global__ void k_clear_sig_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     ITEMS(K_NODE, lvs, none, M.cand, M.cand_count, B.P) { L.sig[id] = 0; });
 }
 
-// significance over the items of the core patches above Jmin (only live points carry
-// coefficients); the patch of each significant coefficient is recorded
+// significance over the live points above Jmin (only they carry coefficients); the
+// patch of each significant coefficient is recorded
 template <class R, int CAP>
 __global__ void k_sig_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
+    if (M.jtop == B.ja) return;
     STAGE_LEVELS;
-    DevLevelT<R> none{};
     // in the field type, by one thread: FP64 conversions queue on their pipe
     __shared__ R thr[2];
+    __shared__ LiveItems live;
     if (threadIdx.x < 2) thr[threadIdx.x] = sig_thr<R>(M.thr[threadIdx.x]);
+    live.init(lvs, B.ja + 1, M.jtop);
     __syncthreads();
     const R eh = thr[0], eu = thr[1];
     int32_t* sig_any = M.sig_any;
-    ITEMS(K_NODE | K_EDGE, lvs, none, M.lists.core, M.lists.count + 1, B.P) {
-        if (L.J == B.ja) return;
-        const bool any = kind == K_NODE ? sig_node(L, id, eh) : sig_edge(L, lvs[L.J - 1], id, eu);
-        if (any) {
-            sig_any[L.J] = 1;
-            L.sflag[el < 0 ? L.npatch : patch_of(L, el)] = 1;
-        }
-    });
+    live.run(lvs, B.ja + 1, M.jtop, int(blockIdx.x * blockDim.x + threadIdx.x), int(gridDim.x * blockDim.x),
+             [&](const DevLevelT<R>& L, int kind, int64_t id) {
+                 const bool any = kind == K_NODE ? sig_node(L, id, eh) : sig_edge(L, lvs[L.J - 1], id, eu);
+                 if (any) {
+                     sig_any[L.J] = 1;
+                     // an edge's patch: that of the node of its element
+                     L.sflag[patch_of(L, kind == K_NODE ? id : int64_t(uint32_t(id) % uint32_t(L.nelem)))] = 1;
+                 }
+             });
 }
 
 // seeds: every active patch, and the patches over an active patch holding a
@@ -569,7 +572,7 @@ __global__ void k_concat_b(const __grid_constant__ MaskBatch<R, CAP> B) {
 
 // the point work lists of the member's levels from its all-level list
 template <class R, int CAP>
-__global__ void k_wl_build_b(const __grid_constant__ MaskBatch<R, CAP> B) {
+__global__ void __launch_bounds__(TPB, 4) k_wl_build_b(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
     STAGE_LEVELS;
     wl_build(lvs, M.lists.all, M.lists.count[0], B.P, int((blockIdx.x * blockDim.x + threadIdx.x) >> 5),

@@ -25,7 +25,7 @@ struct MaskMember {
     const MlpWeights* net;               // device weights of the proposal (learn == 2)
     float logit_tau;                     // proposal threshold on the logit
     int learn;                           // 0 off, 1 features only, 2 features and proposal
-    int jb, jmax;
+    int jtop, jb, jmax;                  // top live level, jb = min(jtop + 1, jmax)
 };
 
 // The members of one mask launch sequence (by value in every launch: CAP members

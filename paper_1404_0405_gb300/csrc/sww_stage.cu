@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(const __grid_constant__ 
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ DevLevelT<R> sl[MAXL];
     __shared__ int cnt[MAXL][WL_KINDS];
+    __shared__ LiveItems live;
     __shared__ int n_core, n_irr, start_ok;
     __shared__ unsigned start_base;
     {
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(const __grid_constant__ 
         }
         __syncthreads();
         if (!start_ok) return;
+        live.init(sl, a.jmin, a.jtop);
         for (int k = threadIdx.x; k < (a.jtop + 1) * WL_KINDS; k += blockDim.x)
             if (k / WL_KINDS >= a.jmin) cnt[k / WL_KINDS][k % WL_KINDS] = sl[k / WL_KINDS].wl_n[k % WL_KINDS];
         __syncthreads();
@@ -253,14 +255,11 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(const __grid_constant__ 
     // every block has read the barrier's base: the next launch's is this one's last target
     if (blockIdx.x == 0 && threadIdx.x == 0) a.bar[GridBarrier::BASE] = gb.target;
     const R dt = to_r<R>(a.dt ? *a.dt : 0.0);
-    entry_items(a.lists.core, n_core, 4, a.P, [&](int32_t ent, uint32_t local) {
-        auto body = [&](const DevLevelT<R>& L, int kind, int64_t id, int64_t) {
-            if (kind == K_NODE)
-                update_node(L, id, a.st, dt);
-            else
-                update_edge(L, id, a.st, dt);
-        };
-        visit_item<K_NODE | K_EDGE>(lv[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), local, a.P, body);
+    live.run(lv, a.jmin, a.jtop, first_item(), int(gridDim.x * blockDim.x), [&](const DevLevelT<R>& L, int kind, int64_t id) {
+        if (kind == K_NODE)
+            update_node(L, id, a.st, dt);
+        else
+            update_edge(L, id, a.st, dt);
     });
 }
 
