@@ -494,12 +494,13 @@ void alloc_state(sww_handle* h, int j) {
     D.nu = h->cfg.nu;
     D.advect = h->cfg.advect;
     D.ue = h->alloc<R>(coarse_E);
-    // byte arrays padded to a multiple of 16 bytes (zeroed): the structured trend
-    // copies the aligned 32-bit word holding a flag
+    // byte arrays padded to a multiple of 16 bytes (zeroed): the patch flags read them by
+    // 16-byte words
     const int64_t N16 = (N + 15) / 16 * 16, E16 = (E + 15) / 16 * 16;
     uint8_t** bN[] = {&D.nflag, &D.sig, &D.tmask, &D.band0, &D.band1};
     for (auto p : bN) *p = h->alloc<uint8_t>(N16);
     D.eflag = h->alloc<uint8_t>(E16);
+    D.tvalid = h->alloc<uint32_t>(D.thalo ? size_t(D.npatch) * tile_valid_words(h->cfg.patch) : 1);
     D.pflag = h->alloc<uint8_t>(D.npatch);
     D.kflag = h->alloc<uint8_t>(D.npatch + 1);
     ck(cudaMemset(D.pflag, 0, D.npatch), "memset");

@@ -971,9 +971,8 @@ struct LiveItems {
 // node and edge slots 256 items at a time, keeps in which lists each belongs, and then
 // reserves its room with one addition per list, by a lane each.  (With one addition per
 // 32 items they queued on the lists' counters: 260 us for the 52 632 patches of
-// turbulence at Jmax 9, 136 us now, with
-// the lists of live points.)  The order of the lists is not fixed; every item's
-// work is independent of it.
+// turbulence at Jmax 9, 136 us now, the lists of live points included.)  The order of
+// the lists is not fixed; every item's work is independent of it.
 template <class R>
 __device__ __forceinline__ unsigned wl_member(const DevLevelT<R>& L, int kind, int64_t id) {
     if (kind == K_NODE) {

@@ -91,6 +91,7 @@ struct DevLevelT {
     const int32_t* thalo;          // [npatch * halo]
     const uint8_t* tirr;           // [npatch + 1]
     const R* tgeo;                 // [npatch * geometry block words]: geometry blocks of the regular patches
+    uint32_t* tvalid;              // [npatch * TileValid words]: which tile slots hold values (sww_valid.cuh)
     // state and work arrays
     R *dh, *u, *dh0, *u0, *dha, *ua, *dht, *ut;
     R *F, *q, *B, *c, *Q;

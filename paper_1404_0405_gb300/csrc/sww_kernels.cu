@@ -16,6 +16,7 @@
 
 #include "sww_core.cuh"
 #include "sww_kernels.h"
+#include "tile.h"
 
 namespace sww {
 
@@ -28,6 +29,7 @@ namespace {
 constexpr int TPB = 256;
 
 #include "sww_bodies.cuh"
+#include "sww_valid.cuh"
 
 // ---------------------------------------------------------------------------- reductions
 
@@ -340,9 +342,15 @@ __global__ void k_concat(const DevLevelT<R>* __restrict__ lvs, int jmin, int jma
 
 // the point work lists of every level from the all-level list
 template <class R>
-__global__ void __launch_bounds__(TPB, 4) k_wl_build(const DevLevelT<R>* __restrict__ lvs, const int32_t* __restrict__ list,
-                           const int32_t* __restrict__ count, int P) {
-    wl_build(lvs, list, *count, P, int(gid() >> 5), int(gridDim.x * blockDim.x >> 5));
+__global__ void __launch_bounds__(TPB, 4) k_wl_build(const DevLevelT<R>* __restrict__ lvs, GridLists lists, int P) {
+    wl_build(lvs, lists.all, lists.count[0], P, int(gid() >> 5), int(gridDim.x * blockDim.x >> 5));
+}
+
+// the validity words of the regular core patches, of side P
+template <class R, int P>
+__global__ void __launch_bounds__(TPB, valid_blocks<P>()) k_valid(const DevLevelT<R>* __restrict__ lvs, GridLists lists) {
+    __shared__ uint32_t sh[TPB / 32 * TileValid<P>::SCRATCH];
+    tile_valid_entries<R, P>(lvs, lists.core, lists.count[1], int(gid() >> 5), int(gridDim.x * blockDim.x >> 5), sh);
 }
 
 }  // namespace
@@ -425,9 +433,11 @@ void launch_patches_all(const DevLevelT<R>* lvs, const Span& patches, cudaStream
 template <class R>
 void launch_concat(const DevLevelT<R>* lvs, int jmin, int jmax, const GridLists& lists, int P, unsigned grid,
                    cudaStream_t s) {
-    g_launches += 2;
+    g_launches += 3;
     k_concat<R><<<unsigned(jmax - jmin + 1), 1024, 0, s>>>(lvs, jmin, jmax, lists);
-    k_wl_build<R><<<grid, TPB, 0, s>>>(lvs, lists.all, lists.count, P);
+    k_wl_build<R><<<grid, TPB, 0, s>>>(lvs, lists, P);
+    auto valid = P == 64 ? k_valid<R, 8> : P == 16 ? k_valid<R, 4> : k_valid<R, 16>;
+    valid<<<grid, TPB, 0, s>>>(lvs, lists);
 }
 
 template <class R>

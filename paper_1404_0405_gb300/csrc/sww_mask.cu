@@ -32,12 +32,14 @@
 #include "sww_kernels.h"
 #include "pdl.cuh"
 #include "sww_mask.h"
+#include "tile.h"
 
 namespace sww {
 
 namespace {
 
 #include "sww_bodies.cuh"
+#include "sww_valid.cuh"
 
 constexpr int TPB = 256;
 
@@ -579,6 +581,16 @@ __global__ void __launch_bounds__(TPB, 4) k_wl_build_b(const __grid_constant__ M
              int(gridDim.x * blockDim.x >> 5));
 }
 
+// the validity words of its regular core patches of side P
+template <class R, int CAP, int P>
+__global__ void __launch_bounds__(TPB, valid_blocks<P>()) k_valid_b(const __grid_constant__ MaskBatch<R, CAP> B) {
+    MEMBER;
+    STAGE_LEVELS;
+    __shared__ uint32_t sh[TPB / 32 * TileValid<P>::SCRATCH];
+    tile_valid_entries<R, P>(lvs, M.lists.core, M.lists.count[1], int((blockIdx.x * blockDim.x + threadIdx.x) >> 5),
+                             int(gridDim.x * blockDim.x >> 5), sh);
+}
+
 }  // namespace
 
 namespace {
@@ -666,6 +678,8 @@ void launch_concat_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t
     if (b.nm < 1 || b.nm > CAP) throw std::runtime_error("mask batch size");
     go(k_concat_b<R, CAP>, unsigned(b.jmax_max - b.ja + 1), unsigned(b.nm), 1024, s, b);
     go(k_wl_build_b<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
+    auto valid = b.P == 64 ? k_valid_b<R, CAP, 8> : b.P == 16 ? k_valid_b<R, CAP, 4> : k_valid_b<R, CAP, 16>;
+    go(valid, grid, unsigned(b.nm), TPB, s, b);
 }
 
 #define MASK_INST(R, CAP)                                                                                   \

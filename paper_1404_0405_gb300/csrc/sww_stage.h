@@ -89,6 +89,8 @@ cudaError_t launch_stage(const StageArgs<R>& a, unsigned grid, cudaStream_t s);
 // words of the geometry block of one tile of side `side` (4, 8 or 16; 0 otherwise)
 template <class R>
 size_t tile_geo_words(int side);
+// words of the validity block of one tile of side `side` (sww_valid.cuh)
+size_t tile_valid_words(int side);
 // the geometry blocks of L's regular patches into out ([npatch * words], zeroed by
 // the caller), for tiles of side `side` (sww_tile.cu)
 template <class R>

@@ -183,6 +183,10 @@ size_t tile_geo_words(int side) {
     }
 }
 
+size_t tile_valid_words(int side) {
+    return size_t(side == 4 ? TileValid<4>::WORDS : side == 8 ? TileValid<8>::WORDS : TileValid<16>::WORDS);
+}
+
 template <class R>
 cudaError_t build_tile_geo(const DevLevelT<R>& L, int side, R* out, cudaStream_t s) {
     switch (side) {

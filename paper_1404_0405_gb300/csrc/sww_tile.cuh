@@ -6,9 +6,9 @@
 // threads of a team (the block, or NT of its threads) call tile_trend and
 // tile_sweep together (they synchronise the team).
 //
-// Per tile: depth and velocity with their flags over the tile range (velocity
-// signs turned to the local directions), copied asynchronously through the
-// patch's halo table while the previous patch is worked on; and the patch's
+// Per tile: depth and velocity over the tile range (velocity signs turned to the
+// local directions), copied asynchronously through the patch's halo table while the
+// previous patch is worked on; which slots hold values (TileValid); and the patch's
 // geometry block (TileGeo: edge lengths d_e and l_e, for
 // each triangle its three kite areas, its area and its Coriolis parameter, the
 // inverse kite sums of the nodes and the cell areas), the FP64 tables rounded
@@ -26,6 +26,7 @@
 // available nodes, Q at live edges, for the patch's own points.
 #pragma once
 // (tile.h is included at file scope by the translation unit)
+#include "sww_valid.cuh"
 
 // NT threads that work on one patch: the whole block (barrier 0), or one of several
 // teams of a block, each with a hardware barrier of its own, so that a large block
@@ -72,16 +73,17 @@ struct Tile {
     static constexpr int HALO = S.halo();
     using G = TileGeo<R, P>;
     static constexpr size_t up16(size_t x) { return (x + 15) / 16 * 16; }
+    using V = TileValid<P>;
     // shared-memory layout (bytes): two geometry buffers and two buffers of staged
     // fields (patch i of a block's sweep uses buffers i mod 2), F and q, the
-    // geometry buffers' mbarriers
+    // buffers' mbarriers
     static constexpr size_t OFF_GEO = 0;   // R[2][G::WORDS]
-    // staged fields: dh[NN], u[3 NN] (local direction), the flag words as copied
-    // nfw[NN], efw[3 NN] (uint32), the flags nf[NN], ef[3 NN]
-    static constexpr size_t STAGED = up16(sizeof(R) * 4 * NN + 4 * 4 * NN + 4 * NN);
+    // staged: dh[NN], u[3 NN] (local direction), and the validity words: of edge and
+    // triangle slots at ST_NFW, of own nodes and edges at ST_EFW
+    static constexpr size_t ST_DH = 0, ST_U = sizeof(R) * NN, ST_EF = ST_U, ST_NFW = up16(sizeof(R) * 4 * NN),
+                            ST_EFW = ST_NFW + 4 * V::N;
+    static constexpr size_t STAGED = ST_NFW + V::BYTES;
     static constexpr size_t OFF_STG = OFF_GEO + 2 * size_t(G::BYTES);   // [2][STAGED]
-    static constexpr size_t ST_DH = 0, ST_U = sizeof(R) * NN, ST_NFW = sizeof(R) * 4 * NN, ST_EFW = ST_NFW + 4 * NN,
-                            ST_NF = ST_EFW + 4 * 3 * NN, ST_EF = ST_NF + NN;
     static constexpr size_t OFF_F = OFF_STG + 2 * STAGED;                 // R[3 NN]
     static constexpr size_t OFF_Q = OFF_F + sizeof(R) * 3 * NN;           // R[2 NN]
     static constexpr size_t OFF_BAR = up16(OFF_Q + sizeof(R) * 2 * NN);   // uint64[2]
@@ -128,13 +130,6 @@ struct TilePlan {
         }
     }
 };
-
-// the structured path applies: a regular tile of a level with tiles, inviscid and
-// with the velocity free (the viscous and advection forms take the tabulated path)
-template <class R>
-__device__ __forceinline__ bool tile_regular(const DevLevelT<R>& L, int64_t pat) {
-    return pat < L.npatch && L.thalo != nullptr && L.tirr[pat] == 0 && !viscous(L) && !L.advect;
-}
 
 // position (a, b) of tile slot x = (a + 1) W + (b + 1)
 template <int W>
@@ -306,55 +301,48 @@ __device__ void tile_geo_build(const DevLevelT<R>& L, int64_t pat, R* __restrict
 }
 
 // Starts this thread's element copies of the fields of tile (L, pat) into staged
-// buffer `stg`: dh and u at its slots, and for the flags the aligned 32-bit word
-// holding each flag byte (the flag arrays are padded to a multiple of 16 bytes),
-// with the byte's position in the word and the velocity's direction flip left in
-// nf and ef for tile_trend to apply.
+// buffer `stg`: dh and u at its slots.  Bit i of the result: the velocity of edge slot i of
+// this thread has to be turned to the local direction.
 template <class R, int P, int NT>
-__device__ __forceinline__ void tile_fetch(const DevLevelT<R>& L, int64_t pat, int tid, const TilePlan<P, NT>& plan,
-                                           const TileCodes<P, NT>& codes, unsigned char* stg) {
+__device__ __forceinline__ unsigned tile_fetch(const DevLevelT<R>& L, int64_t pat, int tid, const TilePlan<P, NT>& plan,
+                                               const TileCodes<P, NT>& codes, unsigned char* stg) {
     using T = Tile<R, P>;
     using PL = TilePlan<P, NT>;
     constexpr int PP = P * P;
     R* dh = reinterpret_cast<R*>(stg + T::ST_DH);
     R* u = reinterpret_cast<R*>(stg + T::ST_U);
-    uint32_t* nfw = reinterpret_cast<uint32_t*>(stg + T::ST_NFW);
-    uint32_t* efw = reinterpret_cast<uint32_t*>(stg + T::ST_EFW);
-    uint8_t* nf = stg + T::ST_NF;
-    uint8_t* ef = stg + T::ST_EF;
     const int32_t nelem = int32_t(L.nelem), base = int32_t(pat) * PP;
+    unsigned turn = 0u;
 #pragma unroll
     for (int i = 0; i < PL::SN; ++i) {
         const int c = plan.n[i];
         if (c == PL::NONE) continue;
-        const int x = tid + i * NT;
-        const int32_t v = c < 0 ? base + (-c - 1) : codes.n[i];
-        async_copy<sizeof(R)>(dh + x, L.dh + v);
-        async_copy<4>(nfw + x, L.nflag + (v & ~3));
-        nf[x] = uint8_t(v & 3);
+        async_copy<sizeof(R)>(dh + tid + i * NT, L.dh + (c < 0 ? base + (-c - 1) : codes.n[i]));
     }
 #pragma unroll
     for (int i = 0; i < PL::SE; ++i) {
-        const int c = plan.e[i], y = tid + i * NT;
+        const int c = plan.e[i];
         if (c == PL::NONE) continue;
         bool rev;
         const int32_t e = slot_edge<P>(c, codes.e[i], nelem, base, rev);
-        async_copy<sizeof(R)>(u + y, L.u + e);
-        async_copy<4>(efw + y, L.eflag + (e & ~3));
-        ef[y] = uint8_t((e & 3) | (rev ? 4 : 0));
+        async_copy<sizeof(R)>(u + tid + i * NT, L.u + e);
+        if (rev) turn |= 1u << i;
     }
     async_commit();
+    return turn;
 }
 
 // The trend of one regular tile (all threads of the team): its fields fetched
-// into staged-field buffer `k` (tile_fetch), its geometry block in `geo` (shared
-// memory) once wait_geo() has returned true.  After the staging barrier the
+// into staged-field buffer `k` (tile_fetch, `turn` its result), its geometry block in
+// `geo` (shared memory) and its validity words in the staged buffer once wait_geo() has
+// returned true.  After the staging barrier the
 // team's earlier tiles are done with every buffer but k's, and after_stage()
 // runs (it may refill them).  False, for every thread, when wait_geo() failed for
 // some thread (nothing is computed).
 template <class R, int P, int NT, class WaitGeo, class AfterStage>
 __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t pat, R H, R g, const TilePlan<P, NT>& plan,
-                           unsigned char* smem, int k, const R* geo, WaitGeo wait_geo, AfterStage after_stage) {
+                           unsigned char* smem, int k, unsigned turn, const R* geo, WaitGeo wait_geo,
+                           AfterStage after_stage) {
     using T = Tile<R, P>;
     using G = TileGeo<R, P>;
     using PL = TilePlan<P, NT>;
@@ -362,10 +350,10 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
     unsigned char* stg = smem + T::OFF_STG + k * T::STAGED;
     R* __restrict__ dh = reinterpret_cast<R*>(stg + T::ST_DH);
     R* __restrict__ u = reinterpret_cast<R*>(stg + T::ST_U);
-    const uint32_t* __restrict__ nfw = reinterpret_cast<const uint32_t*>(stg + T::ST_NFW);
-    const uint32_t* __restrict__ efw = reinterpret_cast<const uint32_t*>(stg + T::ST_EFW);
-    uint8_t* __restrict__ nf = stg + T::ST_NF;
-    uint8_t* __restrict__ ef = stg + T::ST_EF;
+    using V = TileValid<P>;
+    const uint32_t* __restrict__ valid = reinterpret_cast<const uint32_t*>(stg + T::ST_NFW);
+    // bit of slot i (a word a warp)
+    auto has = [&](int first, int i) { return (valid[first + (i >> 5)] >> (i & 31) & 1u) != 0; };
     R* __restrict__ F = reinterpret_cast<R*>(smem + T::OFF_F);
     R* __restrict__ q = reinterpret_cast<R*>(smem + T::OFF_Q);
     const R* __restrict__ de = geo + G::DE;
@@ -378,27 +366,12 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
     const int32_t nelem = int32_t(L.nelem);
     const int32_t base = int32_t(pat) * PP;
     const int tid = team.tid;
-    // --- the fields tile_fetch copied for this thread's slots: the flag bytes out of
-    // their words (the byte's position was left in nf/ef), the velocity turned to the
-    // local direction
+    // --- the velocities tile_fetch copied for this thread's slots turned to the local
+    // direction
     async_wait_all();
 #pragma unroll
-    for (int i = 0; i < PL::SN; ++i) {
-        const int x = tid + i * NT;
-        if (plan.n[i] == PL::NONE) continue;
-        nf[x] = uint8_t(nfw[x] >> (8 * nf[x]));
-    }
-#pragma unroll
-    for (int i = 0; i < PL::SE; ++i) {
-        const int y = tid + i * NT;
-        if (plan.e[i] == PL::NONE) {
-            if (y < 3 * NN) ef[y] = 0;
-            continue;
-        }
-        const uint8_t m = ef[y];
-        ef[y] = uint8_t(efw[y] >> (8 * (m & 3)));
-        if (m & 4) u[y] = -u[y];
-    }
+    for (int i = 0; i < PL::SE; ++i)
+        if (turn >> i & 1u) u[tid + i * NT] = -u[tid + i * NT];
     if (!team.sync_and(wait_geo())) return false;
     after_stage();
     // --- F at edges, q at triangles
@@ -408,12 +381,10 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
         if (plan.e[i] == PL::NONE) continue;
         const int o = y / NN, x = y - o * NN;
         R f = R(0);
-        if (ef[y] & AVAIL) {
+        if (has(V::F, y)) {
             const int x2 = x + (o == 0 ? W : o == 1 ? W + 1 : 1);
-            if ((nf[x] & AVAIL) && (nf[x2] & AVAIL)) {
-                f = R(0.5) * ((H + dh[x]) + (H + dh[x2])) * u[y];
-                if (plan.e[i] < 0) L.F[o * nelem + base + (-plan.e[i] - 1 - o * PP)] = f;
-            }
+            f = R(0.5) * ((H + dh[x]) + (H + dh[x2])) * u[y];
+            if (plan.e[i] < 0) L.F[o * nelem + base + (-plan.e[i] - 1 - o * PP)] = f;
         }
         if constexpr (fp64_form<R>) f *= le[y];
         F[y] = f;
@@ -429,8 +400,7 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
         const int n1 = t == 0 ? x + W : x + W + 1, n2 = t == 0 ? x + W + 1 : x + 1;
         const int s0 = t == 0 ? x : NN + x, s1 = t == 0 ? 2 * NN + x + W : x + 1, s2 = t == 0 ? NN + x : 2 * NN + x;
         R qq = R(0);
-        if ((nf[x] & AVAIL) && (nf[n1] & AVAIL) && (nf[n2] & AVAIL) && (ef[s0] & AVAIL) && (ef[s1] & AVAIL) &&
-            (ef[s2] & AVAIL)) {
+        if (has(V::Q, z)) {
             const R circ = u[s0] * de[s0] + (t == 0 ? R(1) : R(-1)) * u[s1] * de[s1] + R(-1) * u[s2] * de[s2];
             const R hv = kt[(3 * t) * NN + x] * (H + dh[x]) + kt[(3 * t + 1) * NN + x] * (H + dh[n1]) +
                          kt[(3 * t + 2) * NN + x] * (H + dh[n2]);
@@ -450,13 +420,11 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
     for (int w = tid; w < 4 * PP; w += NT) {
         if (w < PP) {
             const int i = w, x = T::at(i / P, i % P);
-            if (!(nf[x] & AVAIL)) continue;
-            bool okr = true;
+            if (!has(V::N, i)) continue;
             R div = R(0), ke = R(0);
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 const int y = x + ring_edge_off<W, NN>(k);
-                okr = okr && (ef[y] & AVAIL);
                 const R n = k < 3 ? R(1) : R(-1);
                 if constexpr (fp64_form<R>) {
                     div += n * F[y];
@@ -466,7 +434,6 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
                     ke += R(0.25) * le[y] * de[y] * u[y] * u[y];
                 }
             }
-            if (!okr) continue;
             const int32_t v = base + i;
             const R A = ai[i];
             if constexpr (fp64_form<R>) {
@@ -479,7 +446,7 @@ __device__ bool tile_trend(const Team<NT>& team, const DevLevelT<R>& L, int64_t 
             }
         } else {
             const int o = (w - PP) / PP, i = (w - PP) - o * PP, x = T::at(i / P, i % P);
-            if (!(ef[o * NN + x] & LIVE)) continue;
+            if (!has(V::E, w - PP)) continue;
             const R Q = o == 0 ? tile_coriolis<R, W, NN, 0>(x, q, F, le, de, kt, is)
                                : o == 1 ? tile_coriolis<R, W, NN, 1>(x, q, F, le, de, kt, is)
                                         : tile_coriolis<R, W, NN, 2>(x, q, F, le, de, kt, is);
@@ -504,6 +471,7 @@ __device__ bool tile_sweep(const Team<NT>& team, const DevLevelT<R>* lv, const i
                            R H, R g, unsigned char* smem, int* err, long long limit) {
     using T = Tile<R, P>;
     using G = TileGeo<R, P>;
+    using V = TileValid<P>;
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + T::OFF_BAR);
     R* gbuf = reinterpret_cast<R*>(smem + T::OFF_GEO);
     if (team.tid == 0) {
@@ -524,24 +492,29 @@ __device__ bool tile_sweep(const Team<NT>& team, const DevLevelT<R>* lv, const i
         c.load(lv[ent >> LVL_SHIFT], ent & PATCH_MASK, plan);
     };
     // list entry e (regular, halo ids c) into buffers k: its fields and, from
-    // thread 0, its geometry block
-    auto start = [&](int e, const TileCodes<P, NT>& c, int k) {
+    // thread 0, its geometry block and validity words
+    auto start = [&](int e, const TileCodes<P, NT>& c, int k) -> unsigned {
         const int32_t ent = list[e];
         const DevLevelT<R>& L = lv[ent >> LVL_SHIFT];
         const int64_t pat = ent & PATCH_MASK;
-        tile_fetch<R, P, NT>(L, pat, team.tid, plan, c, smem + T::OFF_STG + k * T::STAGED);
+        unsigned char* stg = smem + T::OFF_STG + k * T::STAGED;
+        const unsigned turn = tile_fetch<R, P, NT>(L, pat, team.tid, plan, c, stg);
         if (team.tid == 0) {
-            fence_async_shared();   // the buffer's last readers are behind a team barrier
-            bulk_load(gbuf + k * G::WORDS, L.tgeo + pat * G::WORDS, G::BYTES, bar + k);
+            fence_async_shared();   // the buffers' last readers are behind a team barrier
+            bulk_expect(G::BYTES + V::BYTES, bar + k);
+            bulk_copy(gbuf + k * G::WORDS, L.tgeo + pat * G::WORDS, G::BYTES, bar + k);
+            bulk_copy(stg + T::ST_NFW, L.tvalid + pat * V::WORDS, V::BYTES, bar + k);
         }
+        return turn;
     };
     TileCodes<P, NT> c1, c2;   // halo ids of the next patch and of the one after
+    unsigned turn = 0u, turn1 = 0u;   // of the current patch and of the next
     bool reg = regular(first);
     bool reg1 = regular(first + stride);
     if (reg) {
         TileCodes<P, NT> c0;
         codes_of(first, c0);
-        start(first, c0, 0);
+        turn = start(first, c0, 0);
     }
     if (reg1) codes_of(first + stride, c1);
     unsigned ph = 0;   // bit k: parity of buffer k's next phase
@@ -555,10 +528,10 @@ __device__ bool tile_sweep(const Team<NT>& team, const DevLevelT<R>* lv, const i
             const uint32_t parity = (ph >> k) & 1u;
             ph ^= 1u << k;
             const bool done = tile_trend<R, P, NT>(
-                team, L, ent & PATCH_MASK, H, g, plan, smem, k, gbuf + k * G::WORDS,
+                team, L, ent & PATCH_MASK, H, g, plan, smem, k, turn, gbuf + k * G::WORDS,
                 [&]() { return mbar_wait(bar + k, parity, limit); },
                 [&]() {
-                    if (reg1) start(e + stride, c1, k ^ 1);
+                    if (reg1) turn1 = start(e + stride, c1, k ^ 1);
                 });
             if (!done) {
                 // this patch's bulk copy did not land in time: report it, give it one
@@ -570,8 +543,9 @@ __device__ bool tile_sweep(const Team<NT>& team, const DevLevelT<R>* lv, const i
         } else if (reg1) {
             // the next patch's buffers may still be read by a thread behind in the patch before
             team.sync();
-            start(e + stride, c1, k ^ 1);
+            turn1 = start(e + stride, c1, k ^ 1);
         }
+        turn = turn1;
         c1 = c2;
         reg = reg1;
         reg1 = reg2;
