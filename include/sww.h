@@ -90,8 +90,9 @@ typedef struct {
                           The ABI's double arrays are converted at the boundary.     */
     int persistent;    /* RK stages.  0: one cooperative launch per stage (all phases of
                           the trend and the update, grid barriers between them) for a
-                          handle stepping alone on up to 16383 active patches, one launch
-                          per phase on larger grids and inside
+                          handle stepping alone on grids of fewer than 2^17 live nodes
+                          (FP32; 2^20 in FP64), one launch per phase on larger grids and
+                          inside
                           sww_step_ensemble (the members' steps then overlap); 3:
                           inside sww_step_ensemble, one regular launch per phase of
                           the step over all members, each member's mask on its own

@@ -653,11 +653,16 @@ unsigned list_grid(const sww_handle* h, int64_t patches) {
 }
 unsigned list_grid(const sww_handle* h) { return list_grid(h, std::min(h->total_entries, int64_t(2) << size_class(h))); }
 
-// From 2^14 active patches a stage is one launch per phase instead of one cooperative
-// launch: the phases fill the GPU then, and their kernels keep more warps resident (FP32
-// turbulence, us per step persistent / phases: 3 400 patches 768 / 813, 13 640 1857 /
-// 1848, 52 632 6531 / 6076).
-constexpr int PHASES_CLASS = 14;
+// Live nodes from which a stage is one launch per phase instead of one cooperative launch:
+// the phases fill the GPU then, and their kernels keep more warps resident; in FP64 the
+// FP64 pipe bounds both, so the line lies higher.  Us per step, cooperative / phases: FP32
+// 71 000 live nodes 830 / 862, 218 000 777 / 711, 817 000 2020 / 1640; FP64 218 000
+// 1430 / 1543, 870 000 4479 / 4567.
+bool stage_by_phases(const sww_handle* h) {
+    int64_t live = 0;
+    for (int j = h->cfg.jmin; j <= h->cfg.jmax; ++j) live += h->h_counts[h->cfg.jmax + 1 + j];
+    return !h->stage_blocks || live >= (h->cfg.precision == SWW_FP32 ? int64_t(1) << 17 : int64_t(1) << 20);
+}
 // short kernels are chained: by the size class for a handle alone (its launches are
 // captured per class), by the members' active patches for a batch
 bool chained(const sww_handle* h) { return (int64_t(2) << size_class(h)) <= CHAIN_PATCHES; }
@@ -701,7 +706,7 @@ void stage_phases(sww_handle* h, const RKStage& st) {
 // trend and RK stage: one persistent cooperative launch, or one launch per phase
 template <class R>
 void stage(sww_handle* h, const RKStage& st) {
-    if (!h->stage_blocks || size_class(h) >= PHASES_CLASS) {
+    if (stage_by_phases(h)) {
         stage_phases<R>(h, st);
         return;
     }
@@ -936,7 +941,7 @@ void run_step_t(sww_handle* h, double dt, bool do_adapt, int part = 0) {
         one_step<R>(h, dt, do_adapt, part);
         return;
     }
-    const unsigned mode = h->stage_blocks;
+    const unsigned mode = stage_by_phases(h) ? 0 : h->stage_blocks;
     auto key = std::make_tuple(part * 64 + size_class(h), h->jtop, int(do_adapt), dt > 0 ? dt : -1.0, mode);
     auto it = h->graphs.find(key);
     if (it == h->graphs.end()) {

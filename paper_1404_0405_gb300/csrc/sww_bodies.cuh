@@ -28,6 +28,15 @@ __device__ __forceinline__ R predict(const DevLevelT<R>& F, const R* __restrict_
     return s;
 }
 
+// the same through stencil ids already read
+template <class R>
+__device__ __forceinline__ R predict_from(const DevLevelT<R>& F, const R* __restrict__ uc, int64_t fe, const int32_t* st) {
+    R s = R(0);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) s += F.vw[k * F.E + fe] * uc[st[k]];
+    return s;
+}
+
 template <class R>
 __device__ __forceinline__ R height_detail(const DevLevelT<R>& F, int64_t x) {
     R s = F.dh[x];

@@ -9,22 +9,23 @@
 //   -> restriction of B, F, q F^perp and div, top-1 down to Jmin (two phases a level)
 //   -> RK stage update of the live points (all levels)
 //
-// One block of 1024 threads per SM.  The phases of a small grid are bound by
-// latency: a barrier, then a chain of dependent gathers.  So the level-serial phases
-// run over the point work lists (their lengths staged once per block) with each
-// warp's first id loaded before the barrier; consecutive warps of a list go to
+// One block of 512 threads per SM, up to 128 registers a thread (with 1024 threads of 64
+// the ids read ahead spill: 75 us a stage instead of 69 on the jet below in FP32, 118
+// instead of 101 in FP64).  The phases of a small grid are bound by latency: a barrier,
+// then a chain of dependent gathers.  So the level-serial phases run over the point work
+// lists (their lengths staged once per block) with the ids of each thread's first item
+// read ahead while its block waits (ListPhase); consecutive warps of a list go to
 // different SMs, which also spreads the FP64 work (the FP64 pipe starts one warp
-// instruction per 16 clocks and SM); and the block's teams (Team) each work on a
-// patch of their own in the trend.  On the jet of 23 400 live cells on five levels a
-// stage took 206 us (FP64) and 134 us (FP32) with the patches' items dealt out in whole
-// blocks, one patch per 512-thread block and a barrier of 304 blocks; 148 and 93 us
-// now.  The barrier itself costs 1.4 us.
+// instruction per 16 clocks and SM); and the block's teams (Team) each work on a patch
+// of their own in the trend.  On the jet of 23 400 live cells on five levels a stage took
+// 206 us (FP64) and 134 us (FP32) with the patches' items dealt out in whole blocks, one
+// patch per block at a time and a barrier of 304 blocks; 101 and 69 us now.  The barrier
+// itself costs 1.4 us.
 //
 // Values written by other blocks in one phase are read in the next: the barrier's
 // release and acquire at GPU scope, between two block barriers, order them (the acquire
 // also drops the SM's stale L1 lines), so loads may use L1, where the gathers of
-// neighbouring items meet: with L1 bypassed a stage of the 23 400-cell jet took 79 us
-// instead of 75 (FP32) and 136 instead of 131 (FP64).
+// neighbouring items meet (with L1 bypassed a stage of that jet took 3 to 5 % longer).
 //
 // Every barrier wait is bounded: after about two seconds a block sets the error flag and
 // the kernel returns; so does the wait for a patch's geometry block (a bulk copy).
@@ -46,7 +47,7 @@ namespace {
 #include "sww_bodies.cuh"
 #include "sww_tile.cuh"
 
-constexpr int STAGE_TPB = 1024;
+constexpr int STAGE_TPB = 512;
 constexpr int MAXL = 12;
 constexpr long long SPIN_CYCLES = 4000000000ll;   // ~2 s at 2 GHz
 
@@ -83,21 +84,33 @@ struct GridBarrier {
     int skip;
     unsigned target;
 
-    // arrives and waits: false, for every thread of the block, when the wait timed
-    // out (after `limit` cycles; the error flag is set), another block has reported
-    // an error, or the block is the one told to leave without arriving (fault
-    // injection).  A block that leaves arrives nowhere again, so no block passes a
-    // later barrier.
-    __device__ bool sync() {
-        bool ok = true;
+    bool left = false;   // thread 0 of a block that did not arrive
+
+    // The block arrives (its writes of the phase before are released).  Between arriving and
+    // waiting a thread may read what does not change during a stage.
+    __device__ void arrive() {
         __syncthreads();
         if (threadIdx.x == 0) {
             if (int(blockIdx.x) == skip) {
-                ok = false;
+                left = true;
             } else {
                 __threadfence();
                 red_release(bar);
                 target += gridDim.x;
+            }
+        }
+    }
+
+    // waits for all blocks: false, for every thread of the block, when the wait timed out
+    // (after `limit` cycles; the error flag is set), another block has reported an error,
+    // or the block is the one told to leave without arriving (fault injection).  A block
+    // that leaves arrives nowhere again, so no block passes a later barrier.
+    __device__ bool wait() {
+        bool ok = true;
+        if (threadIdx.x == 0) {
+            if (left) {
+                ok = false;
+            } else {
                 const long long t0 = clock64();
                 unsigned polls = 0;
                 while (int(ld_acquire(bar) - target) < 0) {
@@ -116,6 +129,10 @@ struct GridBarrier {
         }
         return __syncthreads_and(ok);
     }
+    __device__ bool sync() {
+        arrive();
+        return wait();
+    }
 };
 
 // This thread's first item of a phase: consecutive warps of items go to consecutive
@@ -125,31 +142,170 @@ __device__ __forceinline__ int first_item() {
     return int(((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31));
 }
 
-// One level-serial phase over work lists k0 and (k1 >= 0) k1 of level L: item i < n0 of
-// the first, then the second.  first() loads this thread's first id (before the
-// barrier that precedes the phase: lists do not change during a stage), run() visits
-// the items.
+// One level-serial phase over work lists k0 and (k1 >= 0) k1 of level L, item i < n0 of
+// the first, then the second; a thread's first item is read ahead of the phase: its id and
+// the ids it gathers through (lists, tables and flags do not change during a stage), between
+// the block's arrival at the barrier before the phase and its wait.  Then the phase is one
+// round of gathers instead of three or four rounds of dependent loads.  Items further on
+// (grids beyond one item a thread) take the general bodies, whose arithmetic is the same.
 template <class R>
 struct ListPhase {
     const DevLevelT<R>* L = nullptr;
     int n0 = 0, n1 = 0, k0 = 0, k1 = -1;
-    int32_t id = 0;
+    // read ahead (by the phase's own functions below)
+    int32_t id = -1, a = 0, b = 0, s[24];
+    uint32_t f = 0;
+
     __device__ __forceinline__ int32_t load(int i) const {
         return i < n0 ? L->wl[wl_off(*L, k0) + i] : L->wl[wl_off(*L, k1) + (i - n0)];
     }
-    __device__ __forceinline__ void first(const DevLevelT<R>& lev, const int (&cnt)[MAXL][WL_KINDS], int j, int a, int b) {
-        L = &lev, k0 = a, k1 = b;
-        n0 = cnt[j][a], n1 = b >= 0 ? cnt[j][b] : 0;
+    __device__ __forceinline__ bool first(const DevLevelT<R>& lev, const int (&cnt)[MAXL][WL_KINDS], int j, int ka, int kb) {
+        L = &lev, k0 = ka, k1 = kb;
+        n0 = cnt[j][ka], n1 = kb >= 0 ? cnt[j][kb] : 0;
         const int i = first_item();
-        if (i < n0 + n1) id = load(i);
+        id = i < n0 + n1 ? load(i) : -1;
+        return i < n0;
     }
+    // the items after the thread's first
     template <class Body>
-    __device__ __forceinline__ void run(Body body) {
-        for (int i = first_item(); i < n0 + n1; i += int(gridDim.x * blockDim.x)) {
-            body(i < n0 ? 0 : 1, int64_t(id));
-            const int ni = i + int(gridDim.x * blockDim.x);
-            if (ni < n0 + n1) id = load(ni);
+    __device__ __forceinline__ void rest(Body body) const {
+        const int stride = int(gridDim.x * blockDim.x);
+        for (int i = first_item() + stride; i < n0 + n1; i += stride) body(i < n0 ? 0 : 1, int64_t(load(i)));
+    }
+
+    // ---- ghosts of L (WL_GN, WL_GE) from C, as fill_node and fill_edge
+    __device__ __forceinline__ void ahead_fill(const DevLevelT<R>& F, const int (&cnt)[MAXL][WL_KINDS], int j) {
+        const bool node = first(F, cnt, j, WL_GN, WL_GE);
+        if (id < 0) return;
+        f = 0u;
+        if (node) {
+            a = F.f2c[id];
+            if (a >= 0) return;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q] = F.par[q * F.N + id];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                s[4 + q] = F.f2c[s[q]];
+                if (F.nflag[s[q]] & LIVE) f |= 1u << q;
+            }
+        } else {
+            a = F.fe_ot[id], b = F.fe_ce[id];
+#pragma unroll
+            for (int k = 0; k < 12; ++k) s[k] = F.vst[k * F.E + id];
+            if (a >= 0) {
+                f = F.eflag[a];
+#pragma unroll
+                for (int k = 0; k < 12; ++k) s[12 + k] = F.vst[k * F.E + a];
+            }
         }
+    }
+    __device__ __forceinline__ void run_fill(const DevLevelT<R>& F, const DevLevelT<R>& C) {
+        if (id >= 0 && first_item() < n0) {
+            if (a >= 0) {
+                F.dh[id] = C.dh[a];
+            } else {
+                R w[4], v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) w[q] = F.ptw[q * F.N + id], v[q] = (f >> q & 1u) ? F.dh[s[q]] : C.dh[s[4 + q]];
+                R sum = R(0);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) sum += w[q] * v[q];
+                F.dh[id] = sum;
+            }
+        } else if (id >= 0 && !F.advect) {
+            const R P = predict_from(F, C.u, id, s);
+            if (a < 0) {
+                F.u[id] = P;
+            } else {
+                const R uc = C.u[b];
+                if (f & LIVE) {
+                    F.u[id] = R(2) * uc - F.u[a];
+                } else {
+                    const R Po = predict_from(F, C.u, a, s + 12);
+                    F.u[id] = half_value(P, Po, uc);
+                    if (f & GHOST) F.u[a] = half_value(Po, P, uc);
+                }
+            }
+        }
+        rest([&](int k, int64_t x) {
+            if (k == 0)
+                fill_node(F, C, x);
+            else
+                fill_edge(F, C, x);
+        });
+    }
+
+    // ---- restriction to L (WL_CN, WL_RE) from F, as restrict_node and restrict_edge
+    __device__ __forceinline__ void ahead_restrict(const DevLevelT<R>& C, const int (&cnt)[MAXL][WL_KINDS], int j) {
+        const bool node = first(C, cnt, j, WL_CN, WL_RE);
+        if (id < 0) return;
+        if (node) {
+            a = C.c2f[id];
+        } else {
+            const int32_t na = C.en[id], nb = C.en[C.E + id];
+#pragma unroll
+            for (int k = 0; k < 12; ++k) s[k] = C.rf_fi[k * C.E + id];
+#pragma unroll
+            for (int k = 0; k < 11; ++k) s[12 + k] = C.rf_ci[k * C.E + id];
+            a = C.half[id], b = C.half[C.E + id];
+            f = C.nflag[na] & C.nflag[nb];
+        }
+    }
+    __device__ __forceinline__ void run_restrict(const DevLevelT<R>& C, const DevLevelT<R>& F) {
+        if (id >= 0 && first_item() < n0) {
+            if (!C.advect) C.B[id] = F.B[a];
+        } else if (id >= 0) {
+            const bool visc = viscous(C);
+            R sum = R(0);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) sum += C.rf_fw[k * C.E + id] * (visc ? F.F[s[k]] + F.Fd[s[k]] : F.F[s[k]]);
+#pragma unroll
+            for (int k = 0; k < 11; ++k) sum += C.rf_cw[k * C.E + id] * F.c[s[12 + k]];
+            C.F[id] = sum / geo<R>(C.l_e, id);
+            if (visc) C.Fd[id] = R(0);
+            if ((f & COVERED) && !C.advect) C.Q[id] = R(0.5) * (F.Q[a] + F.Q[b]);
+        }
+        rest([&](int k, int64_t x) {
+            if (k == 0)
+                restrict_node(C, F, x);
+            else
+                restrict_edge(C, F, x);
+        });
+    }
+
+    // ---- divergence of the restricted fluxes of L (WL_DN), as div_at
+    __device__ __forceinline__ void ahead_div(const DevLevelT<R>& C, const int (&cnt)[MAXL][WL_KINDS], int j) {
+        first(C, cnt, j, WL_DN, -1);
+        if (id < 0) return;
+        const uint8_t fv = C.nflag[id];
+        a = C.deg[id];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) s[k] = C.ring_e[k * C.N + id];
+        uint8_t ok = 0xff;
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if (k < a) ok = (C.eflag[s[k] >> 1] & AVAIL) ? ok : 0;
+        f = (fv & AVAIL) ? ok : 0;
+    }
+    __device__ __forceinline__ void run_div(const DevLevelT<R>& C) {
+        if (id >= 0 && f) {
+            const bool visc = viscous(C);
+            R F[6];
+            double le[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const int64_t e = s[k] < 0 ? 0 : s[k] >> 1;   // slot 5 of a pentagon: -1, not used
+                F[k] = C.F[e], le[k] = C.l_e[e];
+                if (visc) F[k] = F[k] + C.Fd[e];
+            }
+            const double A = C.A_i[id];
+            R div = R(0);
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                if (k < a) div += esign<R>(s[k]) * F[k] * to_r<R>(le[k]);
+            C.c[id] = div / to_r<R>(A);
+        }
+        rest([&](int, int64_t x) { div_at(C, x); });
     }
 };
 
@@ -196,18 +352,12 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(const __grid_constant__ 
     const R H = a.H, g = a.g;
     ListPhase<R> ph;
     // ghosts, coarse to fine
-    if (a.jtop > a.jmin) ph.first(lv[a.jmin + 1], cnt, a.jmin + 1, WL_GN, WL_GE);
+    if (a.jtop > a.jmin) ph.ahead_fill(lv[a.jmin + 1], cnt, a.jmin + 1);
     for (int j = a.jmin + 1; j <= a.jtop; ++j) {
-        const DevLevelT<R>& F = lv[j];
-        const DevLevelT<R>& C = lv[j - 1];
-        ph.run([&](int k, int64_t id) {
-            if (k == 0)
-                fill_node(F, C, id);
-            else
-                fill_edge(F, C, id);
-        });
-        if (j < a.jtop) ph.first(lv[j + 1], cnt, j + 1, WL_GN, WL_GE);
-        if (!gb.sync()) return;
+        ph.run_fill(lv[j], lv[j - 1]);
+        gb.arrive();
+        if (j < a.jtop) ph.ahead_fill(lv[j + 1], cnt, j + 1);
+        if (!gb.wait()) return;
     }
     // the trend: the irregular patches' F and q one thread an item, then a regular patch
     // a team at a time (patches dealt out over the SMs first)
@@ -234,23 +384,19 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(const __grid_constant__ 
         };
         visit_item<K_NODE | K_EDGE>(lv[ent >> LVL_SHIFT], int64_t(ent & PATCH_MASK), local, a.P, body);
     });
-    // restriction, fine to coarse
-    if (a.jtop > a.jmin) ph.first(lv[a.jtop - 1], cnt, a.jtop - 1, WL_CN, WL_RE);
-    if (!gb.sync()) return;
+    // restriction, fine to coarse; then the update
+    gb.arrive();
+    if (a.jtop > a.jmin) ph.ahead_restrict(lv[a.jtop - 1], cnt, a.jtop - 1);
+    if (!gb.wait()) return;
     for (int j = a.jtop - 1; j >= a.jmin; --j) {
-        const DevLevelT<R>& C = lv[j];
-        const DevLevelT<R>& F = lv[j + 1];
-        ph.run([&](int k, int64_t id) {
-            if (k == 0)
-                restrict_node(C, F, id);
-            else
-                restrict_edge(C, F, id);
-        });
-        ph.first(C, cnt, j, WL_DN, -1);
-        if (!gb.sync()) return;
-        ph.run([&](int, int64_t id) { div_at(C, id); });
-        if (j > a.jmin) ph.first(lv[j - 1], cnt, j - 1, WL_CN, WL_RE);
-        if (!gb.sync()) return;
+        ph.run_restrict(lv[j], lv[j + 1]);
+        gb.arrive();
+        ph.ahead_div(lv[j], cnt, j);
+        if (!gb.wait()) return;
+        ph.run_div(lv[j]);
+        gb.arrive();
+        if (j > a.jmin) ph.ahead_restrict(lv[j - 1], cnt, j - 1);
+        if (!gb.wait()) return;
     }
     // every block has read the barrier's base: the next launch's is this one's last target
     if (blockIdx.x == 0 && threadIdx.x == 0) a.bar[GridBarrier::BASE] = gb.target;
