@@ -88,11 +88,11 @@ typedef struct {
                           tables rounded once; thresholds, time step and the
                           compensated mass/energy sums in FP64 on the FP32 values.
                           The ABI's double arrays are converted at the boundary.     */
-    int persistent;    /* RK stages.  0: one cooperative launch per stage (all phases of
-                          the trend and the update, grid barriers between them) for a
-                          handle stepping alone on grids of fewer than 2^17 live nodes
-                          (FP32; 2^20 in FP64), one launch per phase on larger grids and
-                          inside
+    int persistent;    /* Steps.  0: one cooperative launch from the time step to the
+                          coefficients (grid barriers between the phases) and one for the
+                          inverse transform, for a handle stepping alone on grids of
+                          fewer than 2^17 live nodes (FP32; 2^20 in FP64); one launch
+                          per phase on larger grids and inside
                           sww_step_ensemble (the members' steps then overlap); 3:
                           inside sww_step_ensemble, one regular launch per phase of
                           the step over all members, each member's mask on its own
@@ -294,7 +294,7 @@ enum {
     SWW_K_MASK = 9,      /* thresholds, significance, closure, ghosts, patches       */
     SWW_K_INVERSE = 10,  /* inverse transform onto the new mask                      */
     SWW_K_DT = 11,       /* CFL time step reduction                                  */
-    SWW_K_STAGE = 12,    /* persistent RK stage (trend and update in one launch)     */
+    SWW_K_STAGE = 12,    /* persistent RK stage (a launch each while being profiled) */
     SWW_K_NCLASS = 13
 };
 

@@ -653,11 +653,11 @@ unsigned list_grid(const sww_handle* h, int64_t patches) {
 }
 unsigned list_grid(const sww_handle* h) { return list_grid(h, std::min(h->total_entries, int64_t(2) << size_class(h))); }
 
-// Live nodes from which a stage is one launch per phase instead of one cooperative launch:
+// Live nodes from which a stage is one launch per phase instead of part of a cooperative launch:
 // the phases fill the GPU then, and their kernels keep more warps resident; in FP64 the
 // FP64 pipe bounds both, so the line lies higher.  Us per step, cooperative / phases: FP32
-// 71 000 live nodes 830 / 862, 218 000 777 / 711, 817 000 2020 / 1640; FP64 218 000
-// 1430 / 1543, 870 000 4479 / 4567.
+// 71 000 live nodes 763 / 848, 218 000 779 / 712, 817 000 2140 / 1649; FP64 218 000
+// 1431 / 1548, 870 000 4589 / 4580.
 bool stage_by_phases(const sww_handle* h) {
     int64_t live = 0;
     for (int j = h->cfg.jmin; j <= h->cfg.jmax; ++j) live += h->h_counts[h->cfg.jmax + 1 + j];
@@ -703,6 +703,12 @@ void stage_phases(sww_handle* h, const RKStage& st) {
     }
 }
 
+template <class R>
+StageArgs<R> stage_args(const sww_handle* h) {
+    return StageArgs<R>{dlv<R>(h), h->lists, h->S, h->cfg.jmin, h->jtop, h->cfg.jmax, R(h->cfg.H), R(h->cfg.g), h->dt, h->bar,
+                        h->err, h->spin_cycles, h->skip_block};
+}
+
 // trend and RK stage: one persistent cooperative launch, or one launch per phase
 template <class R>
 void stage(sww_handle* h, const RKStage& st) {
@@ -711,8 +717,8 @@ void stage(sww_handle* h, const RKStage& st) {
         return;
     }
     Trace t(h, SWW_K_STAGE);
-    StageArgs<R> a{dlv<R>(h), h->lists, h->S, h->cfg.jmin, h->jtop, h->cfg.jmax, R(h->cfg.H), R(h->cfg.g), st, h->dt, h->bar,
-                   h->err, h->spin_cycles, h->skip_block};
+    StageArgs<R> a = stage_args<R>(h);
+    a.st[0] = st;
     ck(launch_stage(a, h->stage_blocks, h->stream), "persistent stage launch");
 }
 
@@ -723,6 +729,7 @@ int barrier_status(sww_handle* h) {
     *h->h_err = 0;
     ck(cudaMemset(h->err, 0, sizeof(int)), "reset err");
     ck(cudaMemset(h->bar, 0, STAGE_BAR_WORDS * sizeof(unsigned)), "reset barrier");
+    ck(cudaMemset(h->red, 0, RED_WORDS * sizeof(unsigned long long)), "reset maxima");
     return fail(SWW_E_TIMEOUT, "a bounded wait of the RK stage (grid barrier or bulk copy) timed out");
 }
 
@@ -864,12 +871,20 @@ void mask_only(sww_handle* h) {
     launch_concat_batch(b, grid, s);
 }
 
+// The mask, then the inverse transform of the retained coefficients, coarse to fine, ghosts
+// per level: one cooperative launch within a persistent step (whose caller reads the flag
+// of its bounded waits), else a launch per phase
 template <class R>
-void mask_and_inverse(sww_handle* h) {
+void mask_and_inverse(sww_handle* h, bool persistent = false) {
     mask_only<R>(h);
-    // inverse transform of the retained coefficients, coarse to fine, ghosts per level
     Trace t(h, SWW_K_INVERSE);
     Self<R> w(h);
+    if (persistent) {
+        StageArgs<R> a = stage_args<R>(h);
+        a.jtop = w.a.one.j1;
+        ck(launch_inverse(a, h->stage_blocks, h->stream), "persistent inverse launch");
+        return;
+    }
     ck(launch_batch_adapt_post(w.a, w.entries, w.a.one.j1, h->nsm, h->stream), "inverse");
 }
 
@@ -916,20 +931,31 @@ void one_step(sww_handle* h, double dt, bool do_adapt, int part = 0) {
         mask_only<R>(h);
         return;
     }
-    {
-        Trace t(h, SWW_K_DT);
-        Self<R> w(h);
-        ck(launch_batch_pre(w.a, w.entries, h->nsm, dt, h->stream), "time step");
-    }
     int ns;
     const RKStage* st = stages(h->cfg.rk, ns);
-    for (int k = 0; k < ns; ++k) stage<R>(h, st[k]);
     Self<R> w(h);
-    {
-        Trace t(h, SWW_K_PARTIAL);
-        ck(launch_batch_post(w.a, w.entries, h->nsm, h->stream), "partial transform");
+    if (!stage_by_phases(h) && !h->prof_mask) {
+        // time step, stages, partial transform and coefficients in one cooperative launch
+        StageArgs<R> a = stage_args<R>(h);
+        a.ns = ns;
+        for (int k = 0; k < ns; ++k) a.st[k] = st[k];
+        a.pre = dt > 0 ? 2 : 1, a.dt_given = dt, a.post = true, a.details = do_adapt;
+        a.Hd = h->cfg.H, a.gd = h->cfg.g, a.cfl = h->cfg.cfl, a.red = h->red;
+        a.thr = h->thr, a.eps_c = w.a.one.eps_c, a.advect = h->cfg.advect != 0;
+        ck(launch_stage(a, h->stage_blocks, h->stream), "persistent step launch");
+        if (do_adapt) mask_and_inverse<R>(h, true);
+    } else {
+        {
+            Trace t(h, SWW_K_DT);
+            ck(launch_batch_pre(w.a, w.entries, h->nsm, dt, h->stream), "time step");
+        }
+        for (int k = 0; k < ns; ++k) stage<R>(h, st[k]);
+        {
+            Trace t(h, SWW_K_PARTIAL);
+            ck(launch_batch_post(w.a, w.entries, h->nsm, h->stream), "partial transform");
+        }
+        if (do_adapt) adapt<R>(h, -1.0, -1.0);
     }
-    if (do_adapt) adapt<R>(h, -1.0, -1.0);
     ck(launch_batch_out(w.a, h->stream), "read-back");
     ck(cudaMemcpyAsync(h->h_out, h->out, sizeof(BatchOut), cudaMemcpyDeviceToHost, h->stream), "read-back");
 }

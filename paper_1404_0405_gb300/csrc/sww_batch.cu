@@ -38,49 +38,32 @@ constexpr int MAXL = 12;
 constexpr int MAXM = 128;
 enum {
     PH_FILL = 0, PH_RESTRICT, PH_DIV, PH_UPDATE, PH_SET_DT, PH_DT, PH_DT_FINAL, PH_PARTIAL,
-    PH_DETAILS, PH_THRESH, PH_INV_A, PH_INV_B, PH_INV_FILL, PH_OUT
+    PH_DETAILS, PH_THRESH, PH_INV_A, PH_INV_B, PH_OUT
 };
 
-struct MaxU64 {
-    __device__ unsigned long long operator()(unsigned long long x, unsigned long long y) const { return x > y ? x : y; }
-};
-
-// block reduction of one word per thread (every thread returns the block's value)
-template <class Op>
-__device__ unsigned long long block_reduce_u64(unsigned long long v, Op op, unsigned long long* sh) {
-    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_down_sync(0xffffffffu, v, o));
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-    __syncthreads();
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < nw; ++k) v = op(v, sh[k]);
-        sh[0] = v;
-    }
-    __syncthreads();
-    return sh[0];
-}
-
-// items of work lists k0 and k1 (k1 < 0: none) of level L, block b of the
-// member's bpm blocks: body(0, id) for list k0, body(1, id) for list k1
+// items of work lists k0, k1 and k2 (< 0: none) of level L, block b of the member's bpm
+// blocks: body(0, id) for list k0, body(1, id) for list k1, body(2, id) for list k2
 template <class R, class Body>
-__device__ __forceinline__ void member_wl(const DevLevelT<R>& L, int k0, int k1, int b, int bpm, Body body) {
-    const int n0 = L.wl_n[k0], n1 = k1 >= 0 ? L.wl_n[k1] : 0;
+__device__ __forceinline__ void member_wl(const DevLevelT<R>& L, int k0, int k1, int k2, int b, int bpm, Body body) {
+    const int n0 = L.wl_n[k0], n1 = n0 + (k1 >= 0 ? L.wl_n[k1] : 0), n2 = n1 + (k2 >= 0 ? L.wl_n[k2] : 0);
     const int32_t* __restrict__ l0 = L.wl + wl_off(L, k0);
     const int32_t* __restrict__ l1 = k1 >= 0 ? L.wl + wl_off(L, k1) : l0;
-    for (int i = b * int(blockDim.x) + int(threadIdx.x); i < n0 + n1; i += bpm * int(blockDim.x)) {
+    const int32_t* __restrict__ l2 = k2 >= 0 ? L.wl + wl_off(L, k2) : l0;
+    for (int i = b * int(blockDim.x) + int(threadIdx.x); i < n2; i += bpm * int(blockDim.x)) {
         if (i < n0)
             body(0, int64_t(l0[i]));
-        else
+        else if (i < n1)
             body(1, int64_t(l1[i - n0]));
+        else
+            body(2, int64_t(l2[i - n1]));
     }
 }
 
 template <int PH>
 constexpr int phase_blocks() {
-    return PH == PH_FILL || PH == PH_INV_FILL || PH == PH_RESTRICT || PH == PH_PARTIAL || PH == PH_DETAILS || PH == PH_INV_A || PH == PH_DIV
+    return PH == PH_FILL || PH == PH_INV_B || PH == PH_RESTRICT || PH == PH_PARTIAL || PH == PH_DETAILS || PH == PH_INV_A || PH == PH_DIV
                ? 4
-               : PH == PH_INV_B ? 6 : 8;
+               : 8;
 }
 
 template <class R, int PH>
@@ -101,12 +84,7 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         return;
     }
     if constexpr (PH == PH_THRESH) {   // given, or relative to the live maxima (a prescribed velocity has no threshold)
-        if (threadIdx.x == 0) {
-            const double h = __longlong_as_double(static_cast<long long>(mr->red[2]));
-            const double u = __longlong_as_double(static_cast<long long>(mr->red[3]));
-            mr->thr[0] = a.eps_h > 0 ? a.eps_h : mr->eps_c * h;
-            mr->thr[1] = a.eps_u > 0 ? a.eps_u : mr->advect ? INFINITY : mr->eps_c * u;
-        }
+        if (threadIdx.x == 0) thresholds(mr->thr, mr->red, a.eps_h, a.eps_u, mr->eps_c, mr->advect != 0);
         return;
     }
     if constexpr (PH == PH_OUT) {
@@ -125,7 +103,7 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
     }
     const int jtop = mr->jtop;
     // level-serial phases skip the members that do not reach the level
-    constexpr bool inv = PH == PH_INV_A || PH == PH_INV_B || PH == PH_INV_FILL;
+    constexpr bool inv = PH == PH_INV_A || PH == PH_INV_B;
     constexpr bool down = PH == PH_RESTRICT || PH == PH_DIV || PH == PH_PARTIAL;
     if (PH == PH_FILL && j > jtop) return;
     if (down && j > jtop - 1) return;
@@ -134,7 +112,7 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
     // reaches one level above the top)
     __shared__ DevLevelT<R> sl[MAXL];
     {
-        const int lo = (PH == PH_FILL || PH == PH_INV_A || PH == PH_INV_FILL) ? j - 1 : (down || inv) ? j : a.jmin;
+        const int lo = (PH == PH_FILL || inv) ? j - 1 : down ? j : a.jmin;
         const int hi = (PH == PH_RESTRICT || PH == PH_PARTIAL) ? j + 1 : (PH == PH_FILL || PH == PH_DIV || inv) ? j : jtop;
         const int words = int((hi - lo + 1) * sizeof(DevLevelT<R>) / sizeof(int));
         const int* src = reinterpret_cast<const int*>(mr->lvs + lo);
@@ -150,75 +128,39 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         live.init(sl, a.jmin, jtop);
         __syncthreads();
     }
-    if constexpr (PH == PH_FILL || PH == PH_INV_FILL) {
-        // ghost nodes and edges of level j from level j - 1
-        member_wl(sl[j], WL_GN, WL_GE, b, bpm, [&](int k, int64_t id) {
+    if constexpr (PH == PH_FILL || PH == PH_INV_B) {
+        // ghost nodes and edges of level j from level j - 1; with the inverse transform's odd
+        // nodes (both read even nodes and the level below only)
+        member_wl(sl[j], WL_GN, WL_GE, PH == PH_INV_B ? WL_LN : -1, b, bpm, [&](int k, int64_t id) {
             if (k == 0)
                 fill_node(sl[j], sl[j - 1], id);
-            else
+            else if (k == 1)
                 fill_edge(sl[j], sl[j - 1], id);
+            else
+                inverse_b_item(sl[j], id);
         });
     } else if constexpr (PH == PH_RESTRICT) {
         // covered nodes and the edges with a covered end of level j
-        member_wl(sl[j], WL_CN, WL_RE, b, bpm, [&](int k, int64_t id) {
+        member_wl(sl[j], WL_CN, WL_RE, -1, b, bpm, [&](int k, int64_t id) {
             if (k == 0)
                 restrict_node(sl[j], sl[j + 1], id);
             else
                 restrict_edge(sl[j], sl[j + 1], id);
         });
     } else if constexpr (PH == PH_DIV) {
-        member_wl(sl[j], WL_DN, -1, b, bpm, [&](int, int64_t id) { div_at(sl[j], id); });
+        member_wl(sl[j], WL_DN, -1, -1, b, bpm, [&](int, int64_t id) { div_at(sl[j], id); });
     } else if constexpr (PH == PH_PARTIAL) {
         // R_h at covered nodes of level j from level j + 1 (Eq. Rh)
-        member_wl(sl[j], WL_CN, -1, b, bpm, [&](int, int64_t id) { partial_node(sl[j], sl[j + 1], id); });
+        member_wl(sl[j], WL_CN, -1, -1, b, bpm, [&](int, int64_t id) { partial_node(sl[j], sl[j + 1], id); });
     } else if constexpr (PH == PH_DT) {
-        // largest omega^2 over live nodes (none with a prescribed velocity) and, per level,
-        // largest |u| over live edges with u != 0 (NaN left out, as dx/|u| with u NaN takes
-        // no part); the step in PH_DT_FINAL
-        __shared__ unsigned long long sh[BATCH_TPB / 32];
-        __shared__ unsigned long long slev[RED_WORDS - RED_LEVEL];
-        if (threadIdx.x < RED_WORDS - RED_LEVEL) slev[threadIdx.x] = 0ull;
-        __syncthreads();
-        unsigned long long wmax = 0;
-        LevelMax um;
-        live.run(sl, a.jmin, jtop, first, stride, [&](const DevLevelT<R>& L, int kind, int64_t id) {
-            if (kind == K_NODE) {
-                if (!L.advect) wmax = max(wmax, dbits(omega2_at(L, id, a.H, a.g)));
-            } else {
-                const unsigned long long k = abs_key(L.u[id]);
-                if (k && k <= inf_key<R>()) um.add(L.J, k, slev);
-            }
-        });
-        um.flush(slev);
-        wmax = block_reduce_u64(wmax, MaxU64(), sh);   // synchronises the block: slev is complete
-        if (threadIdx.x == 0 && wmax) atomicMax(&mr->red[0], wmax);
-        if (threadIdx.x < RED_WORDS - RED_LEVEL && slev[threadIdx.x])
-            atomicMax(&mr->red[RED_LEVEL + threadIdx.x], slev[threadIdx.x]);
+        __shared__ unsigned long long sh[BATCH_TPB / 32], slev[RED_WORDS - RED_LEVEL];
+        cfl_maxima(live, sl, a.jmin, jtop, first, stride, a.H, a.g, mr->red, sh, slev);   // the step in PH_DT_FINAL
     } else if constexpr (PH == PH_DETAILS) {
-        // the wavelet coefficients (levels above Jmin) and, in the same pass, max |dh|
-        // over live nodes and max |u| over live edges of every level: compared as keys of
-        // the field type, widened to FP64 once per block (bit patterns of non-negative
-        // doubles); the details only read dh and u
         __shared__ unsigned long long shm[BATCH_TPB / 32];
-        unsigned long long hmax = 0, umax = 0;
-        live.run(sl, a.jmin, jtop, first, stride, [&](const DevLevelT<R>& L, int kind, int64_t id) {
-            if (kind == K_NODE)
-                hmax = max(hmax, abs_key(L.dh[id]));
-            else
-                umax = max(umax, abs_key(L.u[id]));
-            if (L.J > a.jmin) details_item(L, (&L)[-1], kind, id);
-        });
-        hmax = block_reduce_u64(hmax, MaxU64(), shm);
-        umax = block_reduce_u64(umax, MaxU64(), shm);
-        if (threadIdx.x == 0) {
-            if (hmax) atomicMax(&mr->red[2], dbits(key_value<R>(hmax)));
-            if (umax) atomicMax(&mr->red[3], dbits(key_value<R>(umax)));
-        }
+        details_and_maxima(live, sl, a.jmin, jtop, first, stride, mr->red, shm);
     } else if constexpr (PH == PH_INV_A) {
-        member_wl(sl[j], WL_LN, WL_LE, b, bpm,
+        member_wl(sl[j], WL_LN, WL_LE, -1, b, bpm,
                   [&](int k, int64_t id) { inverse_a_item(sl[j], sl[j - 1], k == 0 ? K_NODE : K_EDGE, id); });
-    } else if constexpr (PH == PH_INV_B) {
-        member_wl(sl[j], WL_LN, -1, b, bpm, [&](int, int64_t id) { inverse_b_item(sl[j], id); });
     } else {
         static_assert(PH == PH_UPDATE || PH == PH_SET_DT || PH == PH_DT_FINAL || PH == PH_THRESH || PH == PH_OUT, "phase");
         const R dt = to_r<R>(mr->dt ? *mr->dt : 0.0);
@@ -332,8 +274,7 @@ cudaError_t launch_batch_adapt_post(const BatchArgs<R>& a, const int64_t* level_
     for (int j = a.jmin + 1; j <= j1_max && e == cudaSuccess; ++j) {
         const int k = batch_bpm(a, level_entries[j], 4, nsm);
         e = batch_go<PH_INV_A>(a, j, k, s);
-        if (e == cudaSuccess) e = batch_go<PH_INV_B>(a, j, batch_bpm(a, level_entries[j], 1, nsm), s);
-        if (e == cudaSuccess) e = batch_go<PH_INV_FILL>(a, j, k, s);
+        if (e == cudaSuccess) e = batch_go<PH_INV_B>(a, j, k, s);
     }
     return e;
 }

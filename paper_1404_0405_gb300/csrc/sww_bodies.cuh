@@ -973,6 +973,84 @@ struct LiveItems {
     }
 };
 
+struct MaxU64 {
+    __device__ unsigned long long operator()(unsigned long long x, unsigned long long y) const { return x > y ? x : y; }
+};
+
+// block reduction of one word per thread (every thread returns the block's value); sh: a
+// word per warp
+template <class Op>
+__device__ unsigned long long block_reduce_u64(unsigned long long v, Op op, unsigned long long* sh) {
+    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_down_sync(0xffffffffu, v, o));
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+    __syncthreads();
+    if (l == 0) sh[w] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < nw; ++k) v = op(v, sh[k]);
+        sh[0] = v;
+    }
+    __syncthreads();
+    return sh[0];
+}
+
+// Into red: the largest omega^2 over live nodes (none with a prescribed velocity) and, per
+// level, the largest |u| over live edges with u != 0 (NaN left out, as dx/|u| with u NaN
+// takes no part).  By whole blocks; sh as above, slev: a word per level.
+template <class R>
+__device__ __forceinline__ void cfl_maxima(const LiveItems& live, const DevLevelT<R>* lv, int jmin, int jtop, int first, int stride,
+                                           double H, double g, unsigned long long* red, unsigned long long* sh,
+                                           unsigned long long* slev) {
+    if (threadIdx.x < RED_WORDS - RED_LEVEL) slev[threadIdx.x] = 0ull;
+    __syncthreads();
+    unsigned long long wmax = 0;
+    LevelMax um;
+    live.run(lv, jmin, jtop, first, stride, [&](const DevLevelT<R>& L, int kind, int64_t id) {
+        if (kind == K_NODE) {
+            if (!L.advect) wmax = max(wmax, dbits(omega2_at(L, id, H, g)));
+        } else {
+            const unsigned long long k = abs_key(L.u[id]);
+            if (k && k <= inf_key<R>()) um.add(L.J, k, slev);
+        }
+    });
+    um.flush(slev);
+    wmax = block_reduce_u64(wmax, MaxU64(), sh);   // synchronises the block: slev is complete
+    if (threadIdx.x == 0 && wmax) atomicMax(&red[0], wmax);
+    if (threadIdx.x < RED_WORDS - RED_LEVEL && slev[threadIdx.x]) atomicMax(&red[RED_LEVEL + threadIdx.x], slev[threadIdx.x]);
+}
+
+// The wavelet coefficients (levels above Jmin) and, in the same pass, max |dh| over live
+// nodes and max |u| over live edges of every level into red[2..3]: compared as keys of the
+// field type, widened to FP64 once per block (bit patterns of non-negative doubles); the
+// details only read dh and u
+template <class R>
+__device__ __forceinline__ void details_and_maxima(const LiveItems& live, const DevLevelT<R>* lv, int jmin, int jtop, int first,
+                                                   int stride, unsigned long long* red, unsigned long long* sh) {
+    unsigned long long hmax = 0, umax = 0;
+    live.run(lv, jmin, jtop, first, stride, [&](const DevLevelT<R>& L, int kind, int64_t id) {
+        if (kind == K_NODE)
+            hmax = max(hmax, abs_key(L.dh[id]));
+        else
+            umax = max(umax, abs_key(L.u[id]));
+        if (L.J > jmin) details_item(L, (&L)[-1], kind, id);
+    });
+    hmax = block_reduce_u64(hmax, MaxU64(), sh);
+    umax = block_reduce_u64(umax, MaxU64(), sh);
+    if (threadIdx.x == 0) {
+        if (hmax) atomicMax(&red[2], dbits(key_value<R>(hmax)));
+        if (umax) atomicMax(&red[3], dbits(key_value<R>(umax)));
+    }
+}
+
+// the thresholds: given (> 0), or relative to the maxima (a prescribed velocity has none)
+__device__ __forceinline__ void thresholds(double* thr, const unsigned long long* red, double eps_h, double eps_u, double eps_c,
+                                           bool advect) {
+    const double h = __longlong_as_double(static_cast<long long>(red[2]));
+    const double u = __longlong_as_double(static_cast<long long>(red[3]));
+    thr[0] = eps_h > 0 ? eps_h : eps_c * h;
+    thr[1] = eps_u > 0 ? eps_u : advect ? INFINITY : eps_c * u;
+}
+
 // The point work lists of the entries of `list`, a warp an entry (warp w of nw warps):
 // live points, ghost points, covered nodes, edges with a covered end, and
 // available nodes with a covered node among themselves and their neighbours (their

@@ -9,12 +9,14 @@
 
 namespace sww {
 
-// Arguments of one persistent stage: levels (device array of jmax + 1 records),
-// the all-level lists, patch area P, the levels, the constants, the stage
-// coefficients and the time step, and the barrier state: STAGE_BAR_WORDS words, zero
-// before the first launch (the arrival count and its value when a launch begins, each
-// in its own 128-byte line), err set on a timed-out wait.
+// Arguments of a persistent launch: one stage (ns 1), or the ns <= 4 stages of a step with
+// its time step before them and its partial transform and coefficients after.  Levels
+// (device array of jmax + 1 records), the all-level lists, patch area P, the levels, the
+// constants, the stages' coefficients and the time step, and the barrier state:
+// STAGE_BAR_WORDS words, zero before the first launch (the arrival count and its value
+// when a launch begins, each in its own 128-byte line), err set on a timed-out wait.
 constexpr int STAGE_BAR_WORDS = 32 * 2;
+constexpr int STEP_STAGES = 4;
 
 template <class R>
 struct StageArgs {
@@ -23,8 +25,7 @@ struct StageArgs {
     int P;
     int jmin, jtop, jmax;
     R H, g;
-    StageCoef<R> st;
-    const double* dt;
+    double* dt;
     unsigned* bar;
     int* err;
     // bounded barrier waits: a wait gives up after `spin` clock cycles (<= 0: the
@@ -32,6 +33,16 @@ struct StageArgs {
     // at the first barrier without arriving, so the others' waits run out
     long long spin = 0;
     int skip = -1;
+    int ns = 1;
+    StageCoef<R> st[STEP_STAGES];
+    // before the stages: 0 *dt as it is, 1 the CFL step, 2 dt_given; after them: the partial
+    // transform with the ghosts (post), then the coefficients, maxima and thresholds
+    // (details).  The members below are read only then.
+    int pre = 0;
+    bool post = false, details = false, advect = false;
+    double dt_given = 0, Hd = 0, gd = 0, cfl = 0, eps_c = 0;
+    unsigned long long* red = nullptr;
+    double* thr = nullptr;
 };
 
 // One member of an ensemble stage: its level records (contiguous, levels 0..jmax),
@@ -86,6 +97,9 @@ template <class R>
 unsigned stage_grid(int P, int nsm);
 template <class R>
 cudaError_t launch_stage(const StageArgs<R>& a, unsigned grid, cudaStream_t s);
+// the inverse transform and ghosts up to level a.jtop in one cooperative launch
+template <class R>
+cudaError_t launch_inverse(const StageArgs<R>& a, unsigned grid, cudaStream_t s);
 // words of the geometry block of one tile of side `side` (4, 8 or 16; 0 otherwise)
 template <class R>
 size_t tile_geo_words(int side);

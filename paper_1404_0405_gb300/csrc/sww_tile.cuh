@@ -550,6 +550,8 @@ __device__ bool tile_sweep(const Team<NT>& team, const DevLevelT<R>* lv, const i
         reg = reg1;
         reg1 = reg2;
     }
+    team.sync();
+    if (team.tid == 0) mbar_inval(bar), mbar_inval(bar + 1);   // a later sweep makes its own
     return true;
 }
 

@@ -1,9 +1,10 @@
 """The persistent stage with its teams of threads per patch against one launch per
-phase, for every patch side (4: teams of 128 threads, 8: of 256, 16: of 512)
-and both precisions, from grids with fewer patches than teams up, and for the viscous form, whose patches all take the tabulated path.  The bodies and their
-order are the same, so the inviscid results agree bit for bit; the compiler may
-contract the viscous terms differently in the two kernels, so those are compared to
-rounding (1e-12 of the field's maximum in FP64, 2e-6 in FP32)."""
+phase, for every patch side (4: teams of 128 threads, 8: of 256, 16: of 512) and both
+precisions, from grids with fewer patches than teams up, and for the viscous form, whose
+patches all take the tabulated path.  The bodies and their order are the same, so the
+inviscid results agree bit for bit; the compiler may contract the viscous terms
+differently in the two kernels, so those are compared to rounding (1e-12 of the field's
+maximum in FP64, 2e-6 in FP32)."""
 import numpy as np
 import pytest
 
