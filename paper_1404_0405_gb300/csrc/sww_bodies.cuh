@@ -790,9 +790,10 @@ __device__ __forceinline__ unsigned flag_bits(const uint8_t* __restrict__ flag, 
 // The indices of the nonzero bytes of flag[0..n) into out (tag | index), in
 // ascending order, by one block: each thread takes 32 consecutive flags per pass
 // (two 16-byte loads), the block forms an exclusive prefix of the counts, and each
-// thread writes its entries.  flag must be 16-byte aligned.  Returns the count (in
-// every thread).
-__device__ int compact_flags(const uint8_t* __restrict__ flag, int64_t n, int32_t tag, int32_t* __restrict__ out) {
+// thread writes its entries, to out and to out2.  flag must be 16-byte aligned.  Returns
+// the count (in every thread).
+__device__ int compact_flags(const uint8_t* __restrict__ flag, int64_t n, int32_t tag, int32_t* __restrict__ out,
+                             int32_t* __restrict__ out2) {
     __shared__ int wsum[32];
     __shared__ int total;
     if (threadIdx.x == 0) total = 0;
@@ -823,7 +824,8 @@ __device__ int compact_flags(const uint8_t* __restrict__ flag, int64_t n, int32_
         int pos = total + wsum[w] + incl - cnt;
         while (bits) {
             const int k = __ffs(bits) - 1;
-            out[pos++] = tag | int32_t(i0 + k);
+            out[pos] = out2[pos] = tag | int32_t(i0 + k);
+            ++pos;
             bits &= bits - 1u;
         }
         __syncthreads();
@@ -851,9 +853,11 @@ __device__ void patch_scan_level(const DevLevelT<R>& L, bool whole) {
     __syncthreads();
     for (int64_t start = 0; start < L.npatch; start += 32 * int64_t(blockDim.x)) {
         const int64_t i0 = start + 32 * int64_t(threadIdx.x);
+        // the three arrays' loads issued together
         const unsigned a = flag_bits(L.pflag, i0, L.npatch);
-        const unsigned c = a & (whole || !a ? ~0u : flag_bits(L.kflag, i0, L.npatch));
-        const unsigned r = c & (all_irr || !c ? ~0u : flag_bits(L.tirr, i0, L.npatch));
+        const unsigned core = whole ? ~0u : flag_bits(L.kflag, i0, L.npatch);
+        const unsigned irr = all_irr ? ~0u : flag_bits(L.tirr, i0, L.npatch);
+        const unsigned c = a & core, r = c & irr;
         const U64 cnt = U64(__popc(a)) | U64(__popc(c)) << 32;
         const unsigned cnt_i = __popc(r);
         U64 incl = cnt;

@@ -250,24 +250,20 @@ __global__ void k_propose(const __grid_constant__ MaskBatch<R, CAP> B) {
 
 // ------------------------------------------------------------------ mask passes
 
-// all candidate flags of the member's levels ja..jb to zero
+// all candidate flags of the member's levels ja..jb to zero (a thread a patch), and the
+// significance bytes of the previous mask, over its candidates (they stay readable
+// until the next mask)
 template <class R, int CAP>
-__global__ void k_clear_flags(const __grid_constant__ MaskBatch<R, CAP> B) {
-    MEMBER;
-    int j;
-    int64_t P;
-    if (!span_find(B.patches, int64_t(blockIdx.x) * blockDim.x + threadIdx.x, j, P) || j > M.jb) return;
-    const DevLevelT<R>& L = M.lvs[j];
-    L.zflag[P] = 0, L.sflag[P] = 0, L.cflag[P] = 0, L.lflag[P] = 0, L.gflag[P] = 0;
-    L.kflag[P] = 0;
-}
-
-// the significance bytes of the previous mask, over its candidates (they stay
-// readable until the next mask)
-template <class R, int CAP>
-__global__ void k_clear_sig_list(const __grid_constant__ MaskBatch<R, CAP> B) {
+__global__ void k_clear(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
     STAGE_LEVELS;
+    int j;
+    int64_t P;
+    if (span_find(B.patches, int64_t(blockIdx.x) * blockDim.x + threadIdx.x, j, P) && j <= M.jb) {
+        const DevLevelT<R>& L = lvs[j];
+        L.zflag[P] = 0, L.sflag[P] = 0, L.cflag[P] = 0, L.lflag[P] = 0, L.gflag[P] = 0;
+        L.kflag[P] = 0;
+    }
     DevLevelT<R> none{};
     ITEMS(K_NODE, lvs, none, M.cand, M.cand_count, B.P) { L.sig[id] = 0; });
 }
@@ -378,40 +374,38 @@ __global__ void k_gring(const __grid_constant__ MaskBatch<R, CAP> B, int pass) {
     (pass == 0 && B.rings == 2 ? L.cflag : L.gflag)[P] = c;
 }
 
-// compact flags of every level (one block per level) into level-tagged lists:
-// which 1 candidates (cflag -> cand), 2 ghost candidates (gflag -> gcand)
+// the flags of every level (one block per level) compacted into level-tagged lists, the
+// level's own and the all-level one: which 1 candidates (cflag -> cand), 2 ghost candidates
+// (gflag -> gcand).  A block counts the flags of the levels below its own (32 a thread, two
+// loads) for its place in the all-level list, instead of a launch that copies the lists
+// one after the other (10 us with the scan's; 5 us so, jet of 23 400 live cells).
 template <class R, int CAP>
 __global__ void k_flag_scan(const __grid_constant__ MaskBatch<R, CAP> B, int which) {
     MEMBER;
     const int j = B.ja + int(blockIdx.x);
     if (j > M.jb) return;
+    __shared__ int below;
+    if (threadIdx.x == 0) below = 0;
+    __syncthreads();
+    int mine = 0;
+    for (int i = B.ja; i < j; ++i) {
+        const DevLevelT<R>& L = M.lvs[i];
+        const uint8_t* flag = which == 1 ? L.cflag : L.gflag;
+        const int64_t n = L.npatch + 1;
+        for (int64_t i0 = 32 * int64_t(threadIdx.x); i0 < n; i0 += 32 * int64_t(blockDim.x)) mine += __popc(flag_bits(flag, i0, n));
+    }
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, o);
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&below, mine);
+    __syncthreads();
+    const int base = below;
     const DevLevelT<R>& L = M.lvs[j];
     const uint8_t* flag = which == 1 ? L.cflag : L.gflag;
-    int32_t* out = which == 1 ? L.cand : L.gcand;
-    int32_t* nout = which == 1 ? L.ncand : L.ngcand;
-    const int n = compact_flags(flag, L.npatch + 1, int32_t(L.J) << LVL_SHIFT, out);
-    if (threadIdx.x == 0) *nout = n;
-}
-
-// concatenation of the candidate lists of the member's levels ja..jb (one block)
-template <class R, int CAP>
-__global__ void k_cat(const __grid_constant__ MaskBatch<R, CAP> B, int which) {
-    MEMBER;
-    int32_t* all = which == 1 ? M.cand : M.gcand;
-    int32_t* count = which == 1 ? M.cand_count : M.gcand_count;
-    __shared__ int base;
-    if (threadIdx.x == 0) base = 0;
-    __syncthreads();
-    for (int j = B.ja; j <= M.jb; ++j) {
-        const DevLevelT<R>& L = M.lvs[j];
-        const int32_t* src = which == 1 ? L.cand : L.gcand;
-        const int n = which == 1 ? *L.ncand : *L.ngcand;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) all[base + i] = src[i];
-        __syncthreads();
-        if (threadIdx.x == 0) base += n;
-        __syncthreads();
+    const int n = compact_flags(flag, L.npatch + 1, int32_t(L.J) << LVL_SHIFT, which == 1 ? L.cand : L.gcand,
+                                (which == 1 ? M.cand : M.gcand) + base);
+    if (threadIdx.x == 0) {
+        *(which == 1 ? L.ncand : L.ngcand) = n;
+        if (j == M.jb) *(which == 1 ? M.cand_count : M.gcand_count) = base + n;
     }
-    if (threadIdx.x == 0) *count = base;
 }
 
 template <class R, int CAP>
@@ -479,31 +473,19 @@ __global__ void k_ghost_list(const __grid_constant__ MaskBatch<R, CAP> B, int in
     });
 }
 
+// covered nodes; and before the new patch flags, the learned proposal's counts (misses,
+// over-refined, proposed; levels above Jmin) and the old flags cleared, over the
+// candidates (a superset of the old active patches and of the exact set)
 template <class R, int CAP>
 __global__ void k_covered_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     MEMBER;
-    if (M.jb == B.ja) return;
     STAGE_LEVELS;
-    DevLevelT<R> none{};
-    const int jtop = M.jb;
-    ITEMS(K_NODE, lvs, none, M.cand, M.cand_count, B.P) {
-        if (L.J >= jtop) return;
-        covered_node(L, lvs[L.J + 1], id);
-    });
-}
-
-// before the new patch flags: the learned proposal's counts (misses, over-refined,
-// proposed; levels above Jmin) and the old flags cleared, over the candidates (a
-// superset of the old active patches and of the exact set)
-template <class R, int CAP>
-__global__ void k_pre_flags(const __grid_constant__ MaskBatch<R, CAP> B) {
-    MEMBER;
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < *M.cand_count; t += stride) {
         const int32_t ent = M.cand[t];
         const int j = ent >> LVL_SHIFT;
         const int64_t P = ent & PATCH_MASK;
-        const DevLevelT<R>& L = M.lvs[j];
+        const DevLevelT<R>& L = lvs[j];
         if (P >= L.npatch) continue;
         if (M.lstat && j > B.ja) {
             if (L.pexact[P] && !L.pflag[P]) atomicAdd(&M.lstat[0], 1ull);
@@ -512,6 +494,13 @@ __global__ void k_pre_flags(const __grid_constant__ MaskBatch<R, CAP> B) {
         }
         L.pflag[P] = 0;
     }
+    if (M.jb == B.ja) return;
+    DevLevelT<R> none{};
+    const int jtop = M.jb;
+    ITEMS(K_NODE, lvs, none, M.cand, M.cand_count, B.P) {
+        if (L.J >= jtop) return;
+        covered_node(L, lvs[L.J + 1], id);
+    });
 }
 
 // patch flags over the ghost candidates (every patch with a live or ghost point is
@@ -631,8 +620,7 @@ void launch_mask_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s
     const int ja = b.ja, jb = b.jb_max;
     const int64_t npatches = b.patches.off[jb + 1 - ja];
     // seeds
-    go(k_clear_flags<R, CAP>, blocks_for(npatches, TPB), unsigned(b.nm), TPB, s, b);
-    go(k_clear_sig_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
+    go(k_clear<R, CAP>, std::max<unsigned>(grid, blocks_for(npatches, TPB)), unsigned(b.nm), TPB, s, b);
     go(k_sig_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     go(k_seed<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     // candidates, from the top level down (Jmin and whole-lozenge levels: every patch)
@@ -649,7 +637,6 @@ void launch_mask_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s
         }
     }
     go(k_flag_scan<R, CAP>, unsigned(jb - ja + 1), unsigned(b.nm), 1024, s, b, 1);
-    go(k_cat<R, CAP>, 1u, unsigned(b.nm), 1024, s, b, 1);
     // the set T, its closure from the top level down, live flags
     go(k_adjacent_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     for (int j = jb; j > ja; --j) go(k_close_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b, j);
@@ -658,17 +645,15 @@ void launch_mask_batch(const MaskBatch<R, CAP>& b, unsigned grid, cudaStream_t s
     go(k_gring<R, CAP>, blocks_for(npatches, TPB), unsigned(b.nm), TPB, s, b, 0);
     if (b.rings == 2) go(k_gring<R, CAP>, blocks_for(npatches, TPB), unsigned(b.nm), TPB, s, b, 1);
     go(k_flag_scan<R, CAP>, unsigned(jb - ja + 1), unsigned(b.nm), 1024, s, b, 2);
-    go(k_cat<R, CAP>, 1u, unsigned(b.nm), 1024, s, b, 2);
     if (jb > ja) {
         for (int h = 0; h < b.hops; ++h)
             go(k_dilate_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b, h % 2 == 0 ? 1 : 0, h + 1 == CORE_HOPS ? 1 : 0);
         go(k_ghost_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b, b.hops % 2 == 1 ? 1 : 0);
-        go(k_covered_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     }
-    // patch flags: the old ones cleared over the candidates (a superset of the old
-    // active patches), the new ones set over the ghost candidates (a superset of
+    // covered nodes; patch flags: the old ones cleared over the candidates (a superset of
+    // the old active patches), the new ones set over the ghost candidates (a superset of
     // the patches with a live or ghost point); then the level lists
-    go(k_pre_flags<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
+    go(k_covered_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     go(k_flags_list<R, CAP>, grid, unsigned(b.nm), TPB, s, b);
     go(k_patch_scan_b<R, CAP>, unsigned(jb - ja + 1), unsigned(b.nm), 1024, s, b);
 }
