@@ -336,17 +336,20 @@ __device__ __forceinline__ void node_at(const DevLevelT<R>& L, int64_t v, R g) {
 template <class R>
 __device__ __forceinline__ void coriolis_at(const DevLevelT<R>& L, int64_t e) {
     if (L.advect || !(L.eflag[e] & LIVE)) return;
-    // the factors 1/2 of the q averages out of the sum (exact: powers of two)
-    R qe = L.q[L.et[e]] + L.q[L.et[L.E + e]];
+    // FP64: the factors 1/2 of the q averages out of the sum (powers of two).  Not in FP32,
+    // where the products of a field that dies away reach the subnormals and would round
+    // elsewhere
+    constexpr R hq = sizeof(R) == 8 ? R(1) : R(0.5);
+    R qe = hq * (L.q[L.et[e]] + L.q[L.et[L.E + e]]);
     R s = R(0);
 #pragma unroll
     for (int k = 0; k < 10; ++k) {
         int32_t e2 = L.cor_i[k * L.E + e];
         R w = geo<R>(L.cor_w, k * L.E + e);
-        R q2 = L.q[L.et[e2]] + L.q[L.et[L.E + e2]];
-        s += w * L.F[e2] * (qe + q2);
+        R q2 = hq * (L.q[L.et[e2]] + L.q[L.et[L.E + e2]]);
+        s += w * L.F[e2] * hq * (qe + q2);
     }
-    s *= R(0.25);
+    if constexpr (sizeof(R) == 8) s *= R(0.25);
     // viscous form: -nu grad^perp curl u, grad^perp zeta = (1/l_e) sum_{v at e} t_{e,v} zeta_v
     if (viscous(L)) {
         R gp = R(0);

@@ -168,15 +168,17 @@ constexpr bool fp64_form = sizeof(R) == 8;
 // q F^perp at the live edge of orientation O from node slot x: the two cells'
 // contributions n_{e,i} sum_{m=1..5} n_{e',i} (1/2 - sum of the fractions passed) l_{e'}
 // F_{e'} (q_e + q_{e'})/2, over d_e (edge e sits at ring position O of its origin and
-// O + 3 of its end); a node's kite fractions are its kites times is (1 / their sum).  The
-// factors 1/2 of the q averages are taken out of the sum (exact: powers of two).  F holds
-// l_e F_e in the FP64 form.
+// O + 3 of its end); a node's kite fractions are its kites times is (1 / their sum).  In the
+// FP64 form F holds l_e F_e, and the factors 1/2 of the q averages are taken out of the sum
+// (powers of two; in FP32 the products of a field that dies away reach the subnormals and
+// would round elsewhere).
 template <class R, int W, int NN, int O>
 __device__ __forceinline__ R tile_coriolis(int x, const R* q, const R* F, const R* le, const R* de, const R* kt,
                                            const R* is) {
     constexpr int xe = O == 0 ? W : O == 1 ? W + 1 : 1;   // end node slot - origin node slot
     const int y = O * NN + x;
-    const R qe = q[x + ring_tri_off<W, NN>(O)] + q[x + ring_tri_off<W, NN>((O + 5) % 6)];
+    constexpr R hq = fp64_form<R> ? R(1) : R(0.5);
+    const R qe = hq * (q[x + ring_tri_off<W, NN>(O)] + q[x + ring_tri_off<W, NN>((O + 5) % 6)]);
     const R inv_d = R(1) / de[y];
     R s = R(0);
 #pragma unroll
@@ -192,16 +194,16 @@ __device__ __forceinline__ R tile_coriolis(int x, const R* q, const R* F, const 
             csum += kt[kite_off<W, NN>(kp) + xv] * inv_s;
             const int y2 = xv + ring_edge_off<W, NN>(kk);
             const R n2 = kk < 3 ? R(1) : R(-1);
-            const R q2 = q[xv + ring_tri_off<W, NN>(kk)] + q[xv + ring_tri_off<W, NN>((kk + 5) % 6)];
+            const R q2 = hq * (q[xv + ring_tri_off<W, NN>(kk)] + q[xv + ring_tri_off<W, NN>((kk + 5) % 6)]);
             if constexpr (fp64_form<R>) {
                 s += ne * n2 * (R(0.5) - csum) * F[y2] * (qe + q2);
             } else {
                 const R w = ne * n2 * (R(0.5) - csum) * le[y2] * inv_d;
-                s += w * F[y2] * (qe + q2);
+                s += w * F[y2] * hq * (qe + q2);
             }
         }
     }
-    return fp64_form<R> ? R(0.25) * s * inv_d : R(0.25) * s;
+    return fp64_form<R> ? R(0.25) * s * inv_d : s;
 }
 
 // The halo ids a thread's slots need for one tile (own slots: unused), loaded one
