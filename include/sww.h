@@ -28,8 +28,8 @@
  *     of its own, joined to the caller's stream with events).  Calls that
  *     return host data, and sww_step, wait for their own work to finish.
  *   - sww_step replays one CUDA graph per step (captured on first use for each
- *     top level and time-step mode); it reads the new time step and the work-list
- *     sizes back to the host once per step.
+ *     top level, size class of the active grid and time-step mode); it reads the
+ *     new time step and the work-list sizes back to the host once per step.
  */
 #ifndef SWW_H
 #define SWW_H
@@ -79,7 +79,8 @@ typedef struct {
     int rk;            /* SWW_RK4 or SWW_SSP43                                         */
     double cfl;        /* dt = cfl * min(1/omega_max, min dx/|u|) when dt <= 0         */
     double eps;        /* relative threshold: eps_h = eps*max|dh|, eps_u = eps*max|u| (see regime); 0 keeps every point */
-    int blocks_per_sm; /* work-list launches: blocks of 256 threads per SM (0: 4)           */
+    int blocks_per_sm; /* list passes of small grids: blocks of 256 threads per SM (0: 4);
+                          larger grids take up to 16                                 */
     int precision;     /* SWW_FP64: fields and arithmetic in FP64.  SWW_FP32: fields,
                           stencils and transforms in FP32; the spherical geometry
                           (areas, lengths, kite areas, Coriolis parameter, TRiSK

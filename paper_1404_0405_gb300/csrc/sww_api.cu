@@ -3,7 +3,7 @@
 //
 // The library issues its work on a stream of its own, joined to the caller's
 // stream with events at the start and end of every call.  A step is captured once
-// as a CUDA graph per (top level, time-step mode) and replayed; the only host
+// as a CUDA graph per (size class, top level, time-step mode) and replayed; the only host
 // round trip per step reads the new time step and the per-level work-list sizes.
 #include <cuda_runtime.h>
 
@@ -236,7 +236,7 @@ struct sww_handle {
     GridLists lists{};              // all-level lists
     int64_t irr_bound = 0;          // a bound on the entries whose tile is not regular
     BatchOut* out = nullptr;        // read-back record of a step (device and pinned copy)
-    BatchOut* h_out = nullptr;
+    BatchOut* h_out = nullptr;   // in h_counts' allocation
     // candidate lists of the list-based mask (all levels)
     int32_t *cand = nullptr, *cand_count = nullptr, *gcand = nullptr, *gcand_count = nullptr;
     int64_t total_entries = 0;
@@ -292,7 +292,6 @@ struct sww_handle {
         if (ens.h_out) cudaFreeHost(ens.h_out);
         if (ens.ev) cudaEventDestroy(ens.ev);
         if (h_dt) cudaFreeHost(h_dt);
-        if (h_out) cudaFreeHost(h_out);
         for (void* p : allocs) cudaFree(p);
         if (stream) cudaStreamDestroy(stream);
     }
@@ -482,60 +481,37 @@ void alloc_state(sww_handle* h, int j) {
         D = h->geo->lv[j];
     // a level with tiles has its geometry blocks (the structured trend copies them)
     if (D.thalo && !D.tgeo) throw std::runtime_error("tile geometry blocks missing");
-    const int64_t N = D.N, E = D.E, T = D.T;
+    const int64_t N = D.N, E = D.E, T = D.T, NP = D.npatch + 1;
     const int64_t coarse_E = j > h->cfg.jmin ? h->geo->lv[j - 1].E : 1;
-    R** dN[] = {&D.dh, &D.dh0, &D.dha, &D.dht, &D.B, &D.c, &D.hdet};
-    for (auto p : dN) *p = h->alloc<R>(N);
-    R** dE[] = {&D.u, &D.u0, &D.ua, &D.ut, &D.F, &D.Q, &D.ui, &D.Fd};
-    for (auto p : dE) *p = h->alloc<R>(E);
-    D.q = h->alloc<R>(T);
-    D.zeta = h->alloc<R>(T);
-    ck(cudaMemset(D.zeta, 0, T * sizeof(R)), "memset");
+    const int64_t valid = D.thalo ? D.npatch * int64_t(tile_valid_words(h->cfg.patch)) : 1;
+    // the level's arrays in one allocation, each on a 256-byte boundary: called without a
+    // base for the size, then with it
+    auto lay = [&](unsigned char* base) -> size_t {
+        size_t off = 0;
+        auto take = [&](auto*& p, int64_t n) {
+            using T_ = std::remove_reference_t<decltype(*p)>;
+            p = base ? reinterpret_cast<T_*>(base + off) : nullptr;
+            off += (size_t(n) * sizeof(T_) + 255) / 256 * 256;
+        };
+        for (R** p : {&D.dh, &D.dh0, &D.dha, &D.dht, &D.B, &D.c, &D.hdet}) take(*p, N);
+        for (R** p : {&D.u, &D.u0, &D.ua, &D.ut, &D.F, &D.Q, &D.ui, &D.Fd}) take(*p, E);
+        take(D.q, T), take(D.zeta, T), take(D.ue, coarse_E);
+        // padded to a multiple of 16 bytes: the patch flags read them by 16-byte words
+        for (uint8_t** p : {&D.nflag, &D.sig, &D.tmask, &D.band0, &D.band1}) take(*p, N);
+        take(D.eflag, E);
+        for (uint8_t** p : {&D.pflag, &D.kflag, &D.prop, &D.prop_prev, &D.pexact, &D.zflag, &D.sflag, &D.cflag, &D.lflag, &D.gflag})
+            take(*p, NP);
+        for (int32_t** p : {&D.patches, &D.clist, &D.ilist, &D.cand, &D.ncand, &D.gcand, &D.ngcand}) take(*p, NP);
+        take(D.pfeat, NF * NP), take(D.npatches, LIST_COUNTS), take(D.wl_n, WL_KINDS);
+        take(D.tvalid, valid), take(D.wl, 4 * N + 3 * E);
+        return off;
+    };
+    const size_t bytes = lay(nullptr);
+    unsigned char* base = h->alloc<unsigned char>(bytes);
+    ck(cudaMemset(base, 0, bytes), "memset");
+    lay(base);
     D.nu = h->cfg.nu;
     D.advect = h->cfg.advect;
-    D.ue = h->alloc<R>(coarse_E);
-    // byte arrays padded to a multiple of 16 bytes (zeroed): the patch flags read them by
-    // 16-byte words
-    const int64_t N16 = (N + 15) / 16 * 16, E16 = (E + 15) / 16 * 16;
-    uint8_t** bN[] = {&D.nflag, &D.sig, &D.tmask, &D.band0, &D.band1};
-    for (auto p : bN) *p = h->alloc<uint8_t>(N16);
-    D.eflag = h->alloc<uint8_t>(E16);
-    D.tvalid = h->alloc<uint32_t>(D.thalo ? size_t(D.npatch) * tile_valid_words(h->cfg.patch) : 1);
-    D.pflag = h->alloc<uint8_t>(D.npatch);
-    D.kflag = h->alloc<uint8_t>(D.npatch + 1);
-    ck(cudaMemset(D.pflag, 0, D.npatch), "memset");
-    ck(cudaMemset(D.kflag, 0, D.npatch + 1), "memset");
-    D.pfeat = h->alloc<float>(NF * (D.npatch + 1));
-    D.prop = h->alloc<uint8_t>(D.npatch + 1);
-    D.prop_prev = h->alloc<uint8_t>(D.npatch + 1);
-    D.pexact = h->alloc<uint8_t>(D.npatch + 1);
-    uint8_t* pz[] = {D.prop, D.prop_prev, D.pexact};
-    for (uint8_t* p : pz) ck(cudaMemset(p, 0, D.npatch + 1), "memset");
-    ck(cudaMemset(D.pfeat, 0, NF * (D.npatch + 1) * sizeof(float)), "memset");
-    D.patches = h->alloc<int32_t>(D.npatch + 1);
-    D.clist = h->alloc<int32_t>(D.npatch + 1);
-    D.ilist = h->alloc<int32_t>(D.npatch + 1);
-    D.npatches = h->alloc<int32_t>(LIST_COUNTS);
-    D.wl = h->alloc<int32_t>(4 * N + 3 * E);
-    D.wl_n = h->alloc<int32_t>(WL_KINDS);
-    ck(cudaMemset(D.wl_n, 0, WL_KINDS * sizeof(int32_t)), "memset");
-    uint8_t** cf[] = {&D.zflag, &D.sflag, &D.cflag, &D.lflag, &D.gflag};
-    for (auto p : cf) {
-        *p = h->alloc<uint8_t>(D.npatch + 1);
-        ck(cudaMemset(*p, 0, D.npatch + 1), "memset");
-    }
-    int32_t** cl[] = {&D.cand, &D.ncand, &D.gcand, &D.ngcand};
-    for (auto p : cl) {
-        *p = h->alloc<int32_t>(D.npatch + 1);
-        ck(cudaMemset(*p, 0, (D.npatch + 1) * sizeof(int32_t)), "memset");
-    }
-    for (auto p : dN) ck(cudaMemset(*p, 0, N * sizeof(R)), "memset");
-    for (auto p : dE) ck(cudaMemset(*p, 0, E * sizeof(R)), "memset");
-    ck(cudaMemset(D.q, 0, T * sizeof(R)), "memset");
-    for (auto p : bN) ck(cudaMemset(*p, 0, N16), "memset");
-    ck(cudaMemset(D.eflag, 0, E16), "memset");
-    ck(cudaMemset(D.ue, 0, coarse_E * sizeof(R)), "memset");
-    ck(cudaMemset(D.npatches, 0, LIST_COUNTS * sizeof(int32_t)), "memset");
     lvl<R>(h)[j] = D;
 }
 
@@ -1242,7 +1218,9 @@ int create_handle(const sww_config* cfg, void* stream, std::shared_ptr<Geometry>
         ck(cudaMemset(h->d_counts, 0, sizeof(int32_t) * 2 * (cfg->jmax + 1)), "memset");
         h->sig_any = h->alloc<int32_t>(cfg->jmax + 2);
         ck(cudaMemset(h->sig_any, 0, sizeof(int32_t) * (cfg->jmax + 2)), "memset");
-        ck(cudaMallocHost(&h->h_counts, sizeof(int32_t) * 2 * (cfg->jmax + 1)), "cudaMallocHost");
+        // the list sizes (two words a level, levels 0..15) and the step's record
+        ck(cudaMallocHost(&h->h_counts, sizeof(int32_t) * 32 + sizeof(BatchOut)), "cudaMallocHost");
+        h->h_out = reinterpret_cast<BatchOut*>(h->h_counts + 32);
         ck(cudaMallocHost(&h->h_dt, sizeof(double)), "cudaMallocHost");
         std::memset(h->h_counts, 0, sizeof(int32_t) * 2 * (cfg->jmax + 1));
         *h->h_dt = 0;
@@ -1273,7 +1251,6 @@ int create_handle(const sww_config* cfg, void* stream, std::shared_ptr<Geometry>
         ck(cudaMemset(h->dt, 0, sizeof(double)), "memset");
         h->jtop = cfg->jmax;
         h->out = h->alloc<BatchOut>(1);
-        ck(cudaMallocHost(&h->h_out, sizeof(BatchOut)), "cudaMallocHost");
         ck(cudaDeviceSynchronize(), "create");
         return SWW_OK;
     });
