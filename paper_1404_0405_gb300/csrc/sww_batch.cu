@@ -38,32 +38,29 @@ constexpr int MAXL = 12;
 constexpr int MAXM = 128;
 enum {
     PH_FILL = 0, PH_RESTRICT, PH_DIV, PH_UPDATE, PH_SET_DT, PH_DT, PH_DT_FINAL, PH_PARTIAL,
-    PH_DETAILS, PH_THRESH, PH_INV_A, PH_INV_B, PH_OUT
+    PH_DETAILS, PH_THRESH, PH_INV_A, PH_INV_B, PH_INV_FILL, PH_OUT
 };
 
-// items of work lists k0, k1 and k2 (< 0: none) of level L, block b of the member's bpm
-// blocks: body(0, id) for list k0, body(1, id) for list k1, body(2, id) for list k2
+// items of work lists k0 and k1 (k1 < 0: none) of level L, block b of the
+// member's bpm blocks: body(0, id) for list k0, body(1, id) for list k1
 template <class R, class Body>
-__device__ __forceinline__ void member_wl(const DevLevelT<R>& L, int k0, int k1, int k2, int b, int bpm, Body body) {
-    const int n0 = L.wl_n[k0], n1 = n0 + (k1 >= 0 ? L.wl_n[k1] : 0), n2 = n1 + (k2 >= 0 ? L.wl_n[k2] : 0);
+__device__ __forceinline__ void member_wl(const DevLevelT<R>& L, int k0, int k1, int b, int bpm, Body body) {
+    const int n0 = L.wl_n[k0], n1 = k1 >= 0 ? L.wl_n[k1] : 0;
     const int32_t* __restrict__ l0 = L.wl + wl_off(L, k0);
     const int32_t* __restrict__ l1 = k1 >= 0 ? L.wl + wl_off(L, k1) : l0;
-    const int32_t* __restrict__ l2 = k2 >= 0 ? L.wl + wl_off(L, k2) : l0;
-    for (int i = b * int(blockDim.x) + int(threadIdx.x); i < n2; i += bpm * int(blockDim.x)) {
+    for (int i = b * int(blockDim.x) + int(threadIdx.x); i < n0 + n1; i += bpm * int(blockDim.x)) {
         if (i < n0)
             body(0, int64_t(l0[i]));
-        else if (i < n1)
-            body(1, int64_t(l1[i - n0]));
         else
-            body(2, int64_t(l2[i - n1]));
+            body(1, int64_t(l1[i - n0]));
     }
 }
 
 template <int PH>
 constexpr int phase_blocks() {
-    return PH == PH_FILL || PH == PH_INV_B || PH == PH_RESTRICT || PH == PH_PARTIAL || PH == PH_DETAILS || PH == PH_INV_A || PH == PH_DIV
+    return PH == PH_FILL || PH == PH_INV_FILL || PH == PH_RESTRICT || PH == PH_PARTIAL || PH == PH_DETAILS || PH == PH_INV_A || PH == PH_DIV
                ? 4
-               : 8;
+               : PH == PH_INV_B ? 6 : 8;
 }
 
 template <class R, int PH>
@@ -103,7 +100,7 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
     }
     const int jtop = mr->jtop;
     // level-serial phases skip the members that do not reach the level
-    constexpr bool inv = PH == PH_INV_A || PH == PH_INV_B;
+    constexpr bool inv = PH == PH_INV_A || PH == PH_INV_B || PH == PH_INV_FILL;
     constexpr bool down = PH == PH_RESTRICT || PH == PH_DIV || PH == PH_PARTIAL;
     if (PH == PH_FILL && j > jtop) return;
     if (down && j > jtop - 1) return;
@@ -128,30 +125,29 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         live.init(sl, a.jmin, jtop);
         __syncthreads();
     }
-    if constexpr (PH == PH_FILL || PH == PH_INV_B) {
-        // ghost nodes and edges of level j from level j - 1; with the inverse transform's odd
-        // nodes (both read even nodes and the level below only)
-        member_wl(sl[j], WL_GN, WL_GE, PH == PH_INV_B ? WL_LN : -1, b, bpm, [&](int k, int64_t id) {
+    if constexpr (PH == PH_FILL || PH == PH_INV_FILL) {
+        // ghost nodes and edges of level j from level j - 1 (of the inverse transform: a phase
+        // behind its odd nodes, which at the rim of a proposed patch may have a parent that is
+        // not live and take its value of before)
+        member_wl(sl[j], WL_GN, WL_GE, b, bpm, [&](int k, int64_t id) {
             if (k == 0)
                 fill_node(sl[j], sl[j - 1], id);
-            else if (k == 1)
-                fill_edge(sl[j], sl[j - 1], id);
             else
-                inverse_b_item(sl[j], id);
+                fill_edge(sl[j], sl[j - 1], id);
         });
     } else if constexpr (PH == PH_RESTRICT) {
         // covered nodes and the edges with a covered end of level j
-        member_wl(sl[j], WL_CN, WL_RE, -1, b, bpm, [&](int k, int64_t id) {
+        member_wl(sl[j], WL_CN, WL_RE, b, bpm, [&](int k, int64_t id) {
             if (k == 0)
                 restrict_node(sl[j], sl[j + 1], id);
             else
                 restrict_edge(sl[j], sl[j + 1], id);
         });
     } else if constexpr (PH == PH_DIV) {
-        member_wl(sl[j], WL_DN, -1, -1, b, bpm, [&](int, int64_t id) { div_at(sl[j], id); });
+        member_wl(sl[j], WL_DN, -1, b, bpm, [&](int, int64_t id) { div_at(sl[j], id); });
     } else if constexpr (PH == PH_PARTIAL) {
         // R_h at covered nodes of level j from level j + 1 (Eq. Rh)
-        member_wl(sl[j], WL_CN, -1, -1, b, bpm, [&](int, int64_t id) { partial_node(sl[j], sl[j + 1], id); });
+        member_wl(sl[j], WL_CN, -1, b, bpm, [&](int, int64_t id) { partial_node(sl[j], sl[j + 1], id); });
     } else if constexpr (PH == PH_DT) {
         __shared__ unsigned long long sh[BATCH_TPB / 32], slev[RED_WORDS - RED_LEVEL];
         cfl_maxima(live, sl, a.jmin, jtop, first, stride, a.H, a.g, mr->red, sh, slev);   // the step in PH_DT_FINAL
@@ -159,8 +155,10 @@ __global__ void __launch_bounds__(BATCH_TPB, phase_blocks<PH>()) k_phase(const _
         __shared__ unsigned long long shm[BATCH_TPB / 32];
         details_and_maxima(live, sl, a.jmin, jtop, first, stride, mr->red, shm);
     } else if constexpr (PH == PH_INV_A) {
-        member_wl(sl[j], WL_LN, WL_LE, -1, b, bpm,
+        member_wl(sl[j], WL_LN, WL_LE, b, bpm,
                   [&](int k, int64_t id) { inverse_a_item(sl[j], sl[j - 1], k == 0 ? K_NODE : K_EDGE, id); });
+    } else if constexpr (PH == PH_INV_B) {
+        member_wl(sl[j], WL_LN, -1, b, bpm, [&](int, int64_t id) { inverse_b_item(sl[j], id); });
     } else {
         static_assert(PH == PH_UPDATE || PH == PH_SET_DT || PH == PH_DT_FINAL || PH == PH_THRESH || PH == PH_OUT, "phase");
         const R dt = to_r<R>(mr->dt ? *mr->dt : 0.0);
@@ -274,7 +272,8 @@ cudaError_t launch_batch_adapt_post(const BatchArgs<R>& a, const int64_t* level_
     for (int j = a.jmin + 1; j <= j1_max && e == cudaSuccess; ++j) {
         const int k = batch_bpm(a, level_entries[j], 4, nsm);
         e = batch_go<PH_INV_A>(a, j, k, s);
-        if (e == cudaSuccess) e = batch_go<PH_INV_B>(a, j, k, s);
+        if (e == cudaSuccess) e = batch_go<PH_INV_B>(a, j, batch_bpm(a, level_entries[j], 1, nsm), s);
+        if (e == cudaSuccess) e = batch_go<PH_INV_FILL>(a, j, k, s);
     }
     return e;
 }

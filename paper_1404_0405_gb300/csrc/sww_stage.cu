@@ -149,8 +149,8 @@ __device__ __forceinline__ int first_item() {
     return int(((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31));
 }
 
-// One level-serial phase over work lists k0 and, where given (>= 0), k1 and k2 of level L,
-// one after the other; a thread's first item is read ahead of the phase: its id and
+// One level-serial phase over work lists k0 and (k1 >= 0) k1 of level L, one after the
+// other; a thread's first item is read ahead of the phase: its id and
 // the ids it gathers through (lists, tables and flags do not change during a stage), between
 // the block's arrival at the barrier before the phase and its wait.  Then the phase is one
 // round of gathers instead of three or four rounds of dependent loads.  Items further on
@@ -158,7 +158,7 @@ __device__ __forceinline__ int first_item() {
 template <class R>
 struct ListPhase {
     const DevLevelT<R>* L = nullptr;
-    int n0 = 0, n1 = 0, n2 = 0, k0 = 0, k1 = -1, k2 = -1;
+    int n0 = 0, n1 = 0, k0 = 0, k1 = -1;
     // read ahead (by the phase's own functions below)
     int32_t id = -1, a = 0, b = 0, s[24] = {};
     uint32_t f = 0;
@@ -166,26 +166,24 @@ struct ListPhase {
     // what was read ahead before is dead (held through the trend otherwise)
     __device__ __forceinline__ void reset() { *this = ListPhase(); }
 
-    // list (0, 1, 2) of item i
-    __device__ __forceinline__ int list_of(int i) const { return i < n0 ? 0 : i < n0 + n1 ? 1 : 2; }
+    // list (0, 1) of item i
+    __device__ __forceinline__ int list_of(int i) const { return i < n0 ? 0 : 1; }
     __device__ __forceinline__ int32_t load(int i) const {
-        const int k = list_of(i);
-        return k == 0 ? L->wl[wl_off(*L, k0) + i] : k == 1 ? L->wl[wl_off(*L, k1) + (i - n0)] : L->wl[wl_off(*L, k2) + (i - n0 - n1)];
+        return i < n0 ? L->wl[wl_off(*L, k0) + i] : L->wl[wl_off(*L, k1) + (i - n0)];
     }
-    __device__ __forceinline__ int first(const DevLevelT<R>& lev, const int (&cnt)[MAXL][WL_KINDS], int j, int ka, int kb,
-                                         int kc = -1) {
+    __device__ __forceinline__ int first(const DevLevelT<R>& lev, const int (&cnt)[MAXL][WL_KINDS], int j, int ka, int kb) {
         reset();
-        L = &lev, k0 = ka, k1 = kb, k2 = kc;
-        n0 = cnt[j][ka], n1 = kb >= 0 ? cnt[j][kb] : 0, n2 = kc >= 0 ? cnt[j][kc] : 0;
+        L = &lev, k0 = ka, k1 = kb;
+        n0 = cnt[j][ka], n1 = kb >= 0 ? cnt[j][kb] : 0;
         const int i = first_item();
-        id = i < n0 + n1 + n2 ? load(i) : -1;
+        id = i < n0 + n1 ? load(i) : -1;
         return list_of(i);
     }
     // the items after the thread's first
     template <class Body>
     __device__ __forceinline__ void rest(Body body) const {
         const int stride = int(gridDim.x * blockDim.x);
-        for (int i = first_item() + stride; i < n0 + n1 + n2; i += stride) body(list_of(i), int64_t(load(i)));
+        for (int i = first_item() + stride; i < n0 + n1; i += stride) body(list_of(i), int64_t(load(i)));
     }
 
     // ---- ghosts of L (WL_GN, WL_GE) from C, as fill_node and fill_edge
@@ -194,9 +192,9 @@ struct ListPhase {
 #pragma unroll
         for (int k = 0; k < 12; ++k) s[at + k] = F.vst[k * F.E + e];
     }
-    __device__ __forceinline__ void ahead_fill(const DevLevelT<R>& F, const int (&cnt)[MAXL][WL_KINDS], int j, int kc = -1) {
-        const int k = first(F, cnt, j, WL_GN, WL_GE, kc);
-        if (id < 0 || k == 2) return;
+    __device__ __forceinline__ void ahead_fill(const DevLevelT<R>& F, const int (&cnt)[MAXL][WL_KINDS], int j) {
+        const int k = first(F, cnt, j, WL_GN, WL_GE);
+        if (id < 0) return;
         if (k == 0) {
             a = F.f2c[id];
             if (a >= 0) return;
@@ -244,16 +242,12 @@ struct ListPhase {
                     if (f & GHOST) F.u[a] = half_value(Po, P, uc);
                 }
             }
-        } else if (id >= 0 && k == 2) {
-            inverse_b_item(F, id);   // inverse transform only
         }
         rest([&](int k, int64_t x) {
             if (k == 0)
                 fill_node(F, C, x);
-            else if (k == 1)
-                fill_edge(F, C, x);
             else
-                inverse_b_item(F, x);
+                fill_edge(F, C, x);
         });
     }
 
@@ -321,6 +315,15 @@ struct ListPhase {
             }
         }
         rest([&](int k, int64_t x) { inverse_a_item(F, C, k == 0 ? K_NODE : K_EDGE, x); });
+    }
+
+    // ---- its odd nodes from the even ones (WL_LN), as inverse_b_item
+    __device__ __forceinline__ void ahead_odd(const DevLevelT<R>& F, const int (&cnt)[MAXL][WL_KINDS], int j) {
+        first(F, cnt, j, WL_LN, -1);
+    }
+    __device__ __forceinline__ void run_odd(const DevLevelT<R>& F) {
+        if (id >= 0) inverse_b_item(F, id);
+        rest([&](int, int64_t x) { inverse_b_item(F, x); });
     }
 
     // ---- restriction to L (WL_CN, WL_RE) from F, as restrict_node and restrict_edge
@@ -580,9 +583,10 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_stage(const __grid_constant__ 
 }
 
 // The inverse transform of the retained coefficients over the new lists, levels jmin + 1 up
-// to a.jtop, with the ghosts: per level the even nodes and the edges from the level below;
-// then the odd nodes from the even ones and the ghosts (which read the even nodes and the
-// level below only).
+// to a.jtop, with the ghosts: per level the even nodes and the edges from the level below,
+// then the odd nodes from the even ones, then the ghosts.  The ghosts stay behind the odd
+// nodes: at the rim of a proposed patch an odd node may have a parent that is not live, and
+// takes the parent's value of before.
 template <class R>
 __global__ void __launch_bounds__(STAGE_TPB, 1) k_inverse(const __grid_constant__ StageArgs<R> a) {
     __shared__ BlockState<R> bs;
@@ -595,7 +599,11 @@ __global__ void __launch_bounds__(STAGE_TPB, 1) k_inverse(const __grid_constant_
         const DevLevelT<R>& C = bs.sl[j - 1];
         ph.run_inverse(F, C);
         gb.arrive();
-        ph.ahead_fill(F, bs.cnt, j, WL_LN);
+        ph.ahead_odd(F, bs.cnt, j);
+        if (!gb.wait()) return;
+        ph.run_odd(F);
+        gb.arrive();
+        ph.ahead_fill(F, bs.cnt, j);
         if (!gb.wait()) return;
         ph.run_fill(F, C);
         if (j == a.jtop) break;
