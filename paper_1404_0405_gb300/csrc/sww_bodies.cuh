@@ -720,13 +720,14 @@ __device__ __forceinline__ uint8_t live_node(const DevLevelT<R>& L, int64_t i, b
 }
 
 // An edge is live when an end node is: from the closure marks (every node when `all`), not
-// from the node flags, so that nodes and edges take their flags in one pass.  A mark is
-// 0 at a node outside the mask's candidates (a marked node was live and its patch
-// active, a seed of the next mask).
-template <class R>
-__device__ __forceinline__ void live_edge(const DevLevelT<R>& L, int64_t e, bool all) {
+// from the node flags, so that nodes and edges take their flags in one pass.  counts(x):
+// whether the mark of node x makes it live (asked at marked ends only).
+template <class R, class Counts>
+__device__ __forceinline__ void live_edge(const DevLevelT<R>& L, int64_t e, bool all, Counts counts) {
     const uint8_t was = (L.eflag[e] & LIVE) ? WASLIVE : 0;
-    const bool lv = all || (L.tmask[L.en[e]] | L.tmask[L.en[L.E + e]]);
+    const int32_t a = L.en[e], b = L.en[L.E + e];
+    const uint8_t ma = L.tmask[a], mb = L.tmask[b];
+    const bool lv = all || (ma && counts(a)) || (mb && counts(b));
     L.eflag[e] = uint8_t((lv ? LIVE : 0) | was);
 }
 

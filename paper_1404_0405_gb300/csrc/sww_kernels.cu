@@ -262,7 +262,7 @@ __global__ void k_live(const DevLevelT<R>* __restrict__ lvs, Span sp, int all_le
         const DevLevelT<R>& L = lvs[j];
         const bool all = all_level == -2 || j == all_level;
         if (i < L.N) live_node(L, i, all);
-        live_edge(L, i, all);
+        live_edge(L, i, all, [](int64_t) { return true; });   // every mark is a live node here
     });
 }
 

@@ -5,10 +5,14 @@
 // with a node within p hops; two rings for p = 4) of the seeds -- the active patches
 // of level j, the patches over those of level j-1 that hold a significant
 // coefficient, and the patches under the candidates of level j+1 (built from the
-// top level down).  Every point the rules can add lies within five hops of a seed:
+// top level down).  Every point the exact rules can add lies within five hops of a seed:
 // a significant point is within one hop of a live coefficient, its neighbours and
 // children within two more, the closure's parents within two more, and a point
 // the closure brings down from level j+1 sits under a candidate of level j+1.
+// A patch the learned proposal names is not active and no seed; as a rule it is one of the
+// outermost candidates, and the closure of its nodes marks parents in patches that are
+// not candidates.  Those keep the flags they had (not live): a mark counts in a
+// candidate patch only.
 // Candidates of the ghost band: one ring (two for p = 4) around the patches that
 // hold a live node, since the band reaches five hops.  Scratch bytes are zero
 // outside the candidates when a mask starts: band0/band1 are cleared after use,
@@ -437,10 +441,18 @@ __global__ void k_live_list(const __grid_constant__ MaskBatch<R, CAP> B) {
     STAGE_LEVELS;
     DevLevelT<R> none{};
     ITEMS(K_NODE | K_EDGE, lvs, none, M.cand, M.cand_count, B.P) {
-        if (kind == K_EDGE)
-            live_edge(L, id, L.J == B.ja);
-        else if (live_node(L, id, L.J == B.ja))
+        if (kind == K_EDGE) {
+            // A mark makes its node live in a candidate patch only: the closure of a proposed
+            // patch at the rim of the candidates marks parents beyond them.  The edge's own
+            // patch is one.
+            const int64_t own = patch_of(L, el);
+            live_edge(L, id, L.J == B.ja, [&](int64_t x) {
+                const int64_t P = patch_of(L, x);
+                return P == own || L.cflag[P] != 0;
+            });
+        } else if (live_node(L, id, L.J == B.ja)) {
             L.lflag[patch_of(L, id)] = 1;
+        }
     });
 }
 
