@@ -101,7 +101,12 @@ typedef struct {
                           always.  Falls back to -1 where the cooperative launch
                           cannot run.  Other values give SWW_E_ARG.                  */
     int mask;          /* 0: mask passes over candidate patches (near the active grid);
-                          1: dense passes over every point of the levels (same mask)    */
+                          1: dense passes over every point of the levels.  The same mask,
+                          but for the perceptron's proposals (sww_set_learned mode 2):
+                          the candidate passes end with the ring around the active grid, so
+                          they leave out what the graded closure of a proposed patch
+                          adds beyond it, and a live point there may be rebuilt from
+                          values stored before the adaptation.  1 keeps it all.        */
     double nu;         /* viscosity (m^2/s) of the viscous form (Sec. 3.1): nu div grad dh
                           on the height, nu (grad div u - grad^perp curl u) on the velocity;
                           0: inviscid.  The time step rule has no viscous bound.      */
@@ -383,8 +388,8 @@ enum { SWW_P_FEATURES = 0, SWW_P_EXACT = 1, SWW_P_PROPOSAL = 2, SWW_P_ACTIVE = 3
 int sww_set_learned(sww_handle* h, int mode, const float* params, float tau);
 
 /* Explicit proposal for the next adaptation only: flags[n_patches + 1] (host; the
- * last entry is the two poles) of level j > Jmin.  A learned proposal (mode 2)
- * replaces it on the levels the perceptron covers. */
+ * last entry is the two poles) of level j > Jmin, anywhere on the level.  A learned
+ * proposal (mode 2) replaces it on the levels the perceptron covers. */
 int sww_propose(sww_handle* h, int level, const uint8_t* flags);
 
 /* Per-patch data of level j into host memory:

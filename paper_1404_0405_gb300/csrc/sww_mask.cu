@@ -9,10 +9,11 @@
 // a significant point is within one hop of a live coefficient, its neighbours and
 // children within two more, the closure's parents within two more, and a point
 // the closure brings down from level j+1 sits under a candidate of level j+1.
-// A patch the learned proposal names is not active and no seed; as a rule it is one of the
-// outermost candidates, and the closure of its nodes marks parents in patches that are
-// not candidates.  Those keep the flags they had (not live): a mark counts in a
-// candidate patch only.
+// A patch the caller proposes (sww_propose) may lie anywhere and is a seed too, so that the
+// mask is the dense one's.  The perceptron's proposals are no seeds: they lie in the ring
+// around the active grid, as a rule among the outermost candidates, where the closure of
+// their nodes marks parents in patches that are not candidates.  Those keep the flags they
+// had (not live): a mark counts in a candidate patch only.
 // Candidates of the ghost band: one ring (two for p = 4) around the patches that
 // hold a live node, since the band reaches five hops.  Scratch bytes are zero
 // outside the candidates when a mask starts: band0/band1 are cleared after use,
@@ -254,7 +255,8 @@ __global__ void k_propose(const __grid_constant__ MaskBatch<R, CAP> B) {
 
 // ------------------------------------------------------------------ mask passes
 
-// all candidate flags of the member's levels ja..jb to zero (a thread a patch), and the
+// all candidate flags of the member's levels ja..jb to zero (a thread a patch) but the seeds,
+// which start as the patches named by the caller (sww_propose), and the
 // significance bytes of the previous mask, over its candidates (they stay readable
 // until the next mask)
 template <class R, int CAP>
@@ -265,7 +267,7 @@ __global__ void k_clear(const __grid_constant__ MaskBatch<R, CAP> B) {
     int64_t P;
     if (span_find(B.patches, int64_t(blockIdx.x) * blockDim.x + threadIdx.x, j, P) && j <= M.jb) {
         const DevLevelT<R>& L = lvs[j];
-        L.zflag[P] = 0, L.sflag[P] = 0, L.cflag[P] = 0, L.lflag[P] = 0, L.gflag[P] = 0;
+        L.zflag[P] = j > B.ja && M.learn < 2 ? L.prop[P] : 0, L.sflag[P] = 0, L.cflag[P] = 0, L.lflag[P] = 0, L.gflag[P] = 0;
         L.kflag[P] = 0;
     }
     DevLevelT<R> none{};
