@@ -802,8 +802,8 @@ MaskMember<R> mask_member(const sww_handle* h) {
     return m;
 }
 
-// The shared part of a mask batch over members whose largest jb and jmax are
-// given (their grids are the same as h's).
+// The shared part of a mask batch over nm members whose largest jb and jmax are given; h:
+// a member whose grid has every level up to jmax_max.
 template <class R, int CAP>
 void mask_batch_head(MaskBatch<R, CAP>& b, const sww_handle* h, int nm, int jb_max, int jmax_max) {
     const int j0 = h->cfg.jmin;
@@ -1082,13 +1082,16 @@ void ensemble_phased(sww_handle* const* hs, int n, double dt, bool do_adapt) {
             // every member's mask in the same launches on the lead's stream
             Trace tm(lead, SWW_K_MASK);
             auto b = std::make_unique<MaskBatch<R, MASK_BATCH_MAX>>();
-            int jb_max = lead->cfg.jmin, jmax_max = lead->cfg.jmin;
+            // the spans need a grid with every level of the batch (members may have grids of
+            // their own; a level's size follows from Jmin, the patch side and the level)
+            int jb_max = lead->cfg.jmin;
+            const sww_handle* finest = lead;
             for (int i = 0; i < n; ++i) {
                 b->m[i] = mask_member<R>(hs[i]);
                 jb_max = std::max(jb_max, b->m[i].jb);
-                jmax_max = std::max(jmax_max, hs[i]->cfg.jmax);
+                if (hs[i]->cfg.jmax > finest->cfg.jmax) finest = hs[i];
             }
-            mask_batch_head(*b, lead, n, jb_max, jmax_max);
+            mask_batch_head(*b, finest, n, jb_max, finest->cfg.jmax);
             b->chain = a.chain;
             // blocks per member of the list passes: two waves of 8 blocks of 256 per SM
             // over all members (measured 8 % faster than one wave on the 64-member jet)
