@@ -1382,6 +1382,8 @@ static int set_state_at(sww_handle* h, const double* dh, const double* u, int J,
             for (int j = j0; j <= j1; ++j) {
                 ck(cudaMemsetAsync(lv[j].band0, 0, lv[j].N, s), "memset band");
                 ck(cudaMemsetAsync(lv[j].band1, 0, lv[j].N, s), "memset band");
+                // the new state's first mask follows no proposal
+                ck(cudaMemsetAsync(lv[j].prop_prev, 0, lv[j].npatch + 1, s), "memset proposal");
             }
             if (J > j0) launch_covered_all(dlv<R>(h), a.nodes_c, s);
             MaskArgsT<R> b = mask_args<R>(h, j0, j1, false);
