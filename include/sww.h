@@ -177,7 +177,11 @@ int sww_set_state(sww_handle* h, const double* dh, const double* u, int device_p
  * velocity (advect) J must be Jmax (SWW_E_ARG otherwise).  Host fields with a
  * non-finite value are refused (SWW_E_NUMERIC) before the handle's state
  * changes (they are copied into the handle's FP64 staging buffer and checked
- * there); device fields are taken as given. */
+ * there); device fields are taken as given.  The staging buffer holds N + E doubles of
+ * Jmax (84 MB at Jmax 9, on top of the state arrays), is allocated by the first call that
+ * needs it (host fields; device fields of an FP32 handle) and kept: that call can run
+ * out of memory (SWW_E_CUDA).  Reads and writes of FP32 fields use it where it is
+ * there and allocate nothing otherwise. */
 int sww_set_state_level(sww_handle* h, int level, const double* dh, const double* u, int device_ptrs);
 
 /* Adapt the grid (Sec. 2.3): wavelet coefficients at live points, thresholds

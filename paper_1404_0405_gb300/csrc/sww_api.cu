@@ -517,7 +517,8 @@ void alloc_state(sww_handle* h, int j) {
 
 void check_launch() { ck(cudaGetLastError(), "kernel launch"); }
 
-// the handle's FP64 staging buffer (N + E values of Jmax; allocated on first use)
+// the handle's FP64 staging buffer (N + E values of Jmax; allocated by its first sww_set_state of
+// host fields, or of any fields in FP32)
 double* staging(sww_handle* h) {
     if (!h->stage) h->stage = h->alloc<double>(meta(h, h->cfg.jmax).N + meta(h, h->cfg.jmax).E);
     return h->stage;
@@ -525,18 +526,22 @@ double* staging(sww_handle* h) {
 
 // host FP64 values -> device array of the working precision (on the handle's
 // stream; the caller synchronises before the host data goes away).  FP32: rounded on the
-// device from the staging buffer, in parts of at most its size.
+// device from the staging buffer, in parts of at most its size; by a handle that has none
+// (no sww_set_state yet) on the host, as a write takes no device memory of its own.
 template <class R>
 void to_device(sww_handle* h, R* dst, const double* src, int64_t n) {
     if constexpr (std::is_same<R, double>::value) {
         ck(cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyHostToDevice, h->stream), "to_device");
+    } else if (!h->stage) {
+        std::vector<R> tmp(src, src + n);
+        ck(cudaMemcpyAsync(dst, tmp.data(), n * sizeof(R), cudaMemcpyHostToDevice, h->stream), "to_device");
+        ck(cudaStreamSynchronize(h->stream), "to_device");   // tmp lives on this frame
     } else {
-        double* st = staging(h);
         const int64_t most = meta(h, h->cfg.jmax).N + meta(h, h->cfg.jmax).E;
         for (int64_t i = 0; i < n; i += most) {
             const int64_t m = std::min(most, n - i);
-            ck(cudaMemcpyAsync(st, src + i, m * sizeof(double), cudaMemcpyHostToDevice, h->stream), "to_device");
-            launch_convert(st, dst + i, m, h->stream);
+            ck(cudaMemcpyAsync(h->stage, src + i, m * sizeof(double), cudaMemcpyHostToDevice, h->stream), "to_device");
+            launch_convert(h->stage, dst + i, m, h->stream);
         }
     }
 }
@@ -544,17 +549,22 @@ void to_device(sww_handle* h, R* dst, const double* src, int64_t n) {
 // Device arrays of the working precision -> host FP64 values, queued on the handle's
 // stream (the caller joins and synchronises).  FP32 is widened on the device into the
 // staging buffer from `at` on and copied from there: widening on one host core took ten
-// times as long as the copy (2.6 million values: 0.8 ms, of 0.06 ms for the copy).
+// times as long as the copy (2.6 million values: 0.8 ms, of 0.06 ms for the copy).  A
+// handle without the buffer (its state came from sww_load) widens on the host all the same,
+// so that a read takes no device memory and cannot run out of it.
 template <class R>
 void read_values(sww_handle* h, double* dst, const R* src, int64_t n, int64_t at = 0) {
-    const double* from;
     if constexpr (std::is_same<R, double>::value) {
-        from = src;
+        ck(cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream), "from_device");
+    } else if (!h->stage) {
+        std::vector<R> tmp(n);
+        ck(cudaMemcpyAsync(tmp.data(), src, n * sizeof(R), cudaMemcpyDeviceToHost, h->stream), "from_device");
+        ck(cudaStreamSynchronize(h->stream), "from_device");
+        for (int64_t i = 0; i < n; ++i) dst[i] = double(tmp[i]);
     } else {
-        launch_convert(src, staging(h) + at, n, h->stream);
-        from = h->stage + at;
+        launch_convert(src, h->stage + at, n, h->stream);
+        ck(cudaMemcpyAsync(dst, h->stage + at, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream), "from_device");
     }
-    ck(cudaMemcpyAsync(dst, from, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream), "from_device");
 }
 
 // the same for one array (synchronous)
