@@ -683,9 +683,25 @@ template <class R>
 void stage_phases(sww_handle* h, const RKStage& st) {
     Self<R> w(h);
     w.a.st = st;
-    for (int part = 0; part < 5; ++part) {
+    auto run = [&](int part) {
         Trace t(h, STAGE_PART_CLASS[part]);
         ck(launch_stage_batch_part(w.a, w.entries, h->irr_bound, h->nsm, part, h->stream), "stage");
+    };
+    for (int part = 0; part < 3; ++part) run(part);
+    for (int j = h->jtop - 1; j >= h->cfg.jmin; --j) {
+        { Trace t(h, SWW_K_RESTRICT); ck(launch_batch_restrict(w.a, w.entries, j, h->nsm, h->stream), "restriction"); }
+        { Trace t(h, SWW_K_NODE); ck(launch_batch_div(w.a, w.entries, j, h->nsm, h->stream), "divergence"); }
+    }
+    run(4);
+}
+
+// the inverse transform of the coefficients of live points, coarse to fine up to level j1,
+// the ghosts of a level behind it
+template <class R>
+void inverse_phases(sww_handle* h, const Self<R>& w, int j1) {
+    for (int j = h->cfg.jmin + 1; j <= j1; ++j) {
+        { Trace t(h, SWW_K_INVERSE); ck(launch_batch_inverse(w.a, w.entries, j, h->nsm, h->stream), "inverse"); }
+        { Trace t(h, SWW_K_FILL); ck(launch_batch_inverse_fill(w.a, w.entries, j, h->nsm, h->stream), "inverse"); }
     }
 }
 
@@ -863,15 +879,14 @@ void mask_only(sww_handle* h) {
 template <class R>
 void mask_and_inverse(sww_handle* h, bool persistent = false) {
     mask_only<R>(h);
-    Trace t(h, SWW_K_INVERSE);
     Self<R> w(h);
-    if (persistent) {
+    if (persistent) {   // never while being profiled
         StageArgs<R> a = stage_args<R>(h);
         a.jtop = w.a.one.j1;
         ck(launch_inverse(a, h->stage_blocks, h->stream), "persistent inverse launch");
         return;
     }
-    ck(launch_batch_adapt_post(w.a, w.entries, w.a.one.j1, h->nsm, h->stream), "inverse");
+    inverse_phases(h, w, w.a.one.j1);
 }
 
 // relative coefficient tolerance: eps, or eps^{3/2} when eps is read as the trend
@@ -880,12 +895,10 @@ double eps_coeff(const sww_config& c) { return c.regime == 1 ? c.eps * std::sqrt
 
 template <class R>
 void adapt(sww_handle* h, double eh, double eu) {
-    {
-        Trace t(h, SWW_K_COEFF);
-        Self<R> w(h);
-        w.a.eps_h = eh, w.a.eps_u = eu;
-        ck(launch_batch_adapt_pre(w.a, w.entries, h->nsm, h->stream), "adapt");
-    }
+    Self<R> w(h);
+    w.a.eps_h = eh, w.a.eps_u = eu;
+    { Trace t(h, SWW_K_COEFF); ck(launch_batch_details(w.a, w.entries, h->nsm, h->stream), "coefficients"); }
+    { Trace t(h, SWW_K_MASK); ck(launch_batch_thresholds(w.a, h->stream), "thresholds"); }
     mask_and_inverse<R>(h);
 }
 
@@ -936,10 +949,8 @@ void one_step(sww_handle* h, double dt, bool do_adapt, int part = 0) {
             ck(launch_batch_pre(w.a, w.entries, h->nsm, dt, h->stream), "time step");
         }
         for (int k = 0; k < ns; ++k) stage<R>(h, st[k]);
-        {
-            Trace t(h, SWW_K_PARTIAL);
-            ck(launch_batch_post(w.a, w.entries, h->nsm, h->stream), "partial transform");
-        }
+        { Trace t(h, SWW_K_PARTIAL); ck(launch_batch_partial(w.a, w.entries, h->nsm, h->stream), "partial transform"); }
+        { Trace t(h, SWW_K_FILL); ck(launch_batch_fill(w.a, w.entries, h->nsm, h->stream), "ghosts"); }
         if (do_adapt) adapt<R>(h, -1.0, -1.0);
     }
     ck(launch_batch_out(w.a, h->stream), "read-back");
@@ -1079,12 +1090,14 @@ void ensemble_phased(sww_handle* const* hs, int n, double dt, bool do_adapt) {
     }
     {
         Trace t(lead, SWW_K_PARTIAL);
-        ck(launch_batch_post(a, entries.data(), lead->nsm, s), "batched ensemble step");
+        ck(launch_batch_partial(a, entries.data(), lead->nsm, s), "batched ensemble step");
+        ck(launch_batch_fill(a, entries.data(), lead->nsm, s), "batched ensemble step");
     }
     if (do_adapt) {
         {
             Trace t(lead, SWW_K_COEFF);
-            ck(launch_batch_adapt_pre(a, entries.data(), lead->nsm, s), "batched ensemble step");
+            ck(launch_batch_details(a, entries.data(), lead->nsm, s), "batched ensemble step");
+            ck(launch_batch_thresholds(a, s), "batched ensemble step");
         }
         bool lists = true;
         for (int i = 0; i < n; ++i) lists = lists && list_mask(hs[i]);
@@ -1121,7 +1134,10 @@ void ensemble_phased(sww_handle* const* hs, int n, double dt, bool do_adapt) {
             }
         }
         Trace t(lead, SWW_K_INVERSE);
-        ck(launch_batch_adapt_post(a, entries.data(), j1_max, lead->nsm, s), "batched ensemble step");
+        for (int j = lead->cfg.jmin + 1; j <= j1_max; ++j) {
+            ck(launch_batch_inverse(a, entries.data(), j, lead->nsm, s), "batched ensemble step");
+            ck(launch_batch_inverse_fill(a, entries.data(), j, lead->nsm, s), "batched ensemble step");
+        }
     }
     ck(launch_batch_out(a, s), "batched ensemble step");
     ck(cudaMemcpyAsync(E.h_out, E.out, sizeof(BatchOut) * n, cudaMemcpyDeviceToHost, s), "read-back");
@@ -1706,10 +1722,9 @@ int sww_inverse(sww_handle* h) {
             using R = decltype(r);
             Join jn(h);
             launch_mark_support(work_all<R>(h), h->stream);
-            Trace t(h, SWW_K_INVERSE);
             Self<R> w(h);
             w.a.one.j1 = h->jtop;
-            ck(launch_batch_adapt_post(w.a, w.entries, h->jtop, h->nsm, h->stream), "inverse");
+            inverse_phases(h, w, h->jtop);
             check_launch();
             return 0;
         });

@@ -201,6 +201,18 @@ int64_t entries_to(const BatchArgs<R>& a, const int64_t* level_entries) {
 }  // namespace
 
 template <class R>
+cudaError_t launch_batch_restrict(const BatchArgs<R>& a, const int64_t* level_entries, int j, int nsm, cudaStream_t s) {
+    if (!batch_ok(a, j + 1)) return cudaErrorInvalidValue;
+    return batch_go<PH_RESTRICT>(a, j, batch_bpm(a, level_entries[j], 4, nsm), s);
+}
+
+template <class R>
+cudaError_t launch_batch_div(const BatchArgs<R>& a, const int64_t* level_entries, int j, int nsm, cudaStream_t s) {
+    if (!batch_ok(a, j)) return cudaErrorInvalidValue;
+    return batch_go<PH_DIV>(a, j, batch_bpm(a, level_entries[j], 1, nsm), s);
+}
+
+template <class R>
 cudaError_t launch_stage_batch_part(const BatchArgs<R>& a, const int64_t* level_entries, int64_t irr_entries, int nsm,
                                     int part, cudaStream_t s) {
     if (!batch_ok(a, a.jtop_max)) return cudaErrorInvalidValue;
@@ -217,8 +229,8 @@ cudaError_t launch_stage_batch_part(const BatchArgs<R>& a, const int64_t* level_
             break;
         case 3:
             for (int j = a.jtop_max - 1; j >= a.jmin && e == cudaSuccess; --j) {
-                e = batch_go<PH_RESTRICT>(a, j, batch_bpm(a, level_entries[j], 4, nsm), s);
-                if (e == cudaSuccess) e = batch_go<PH_DIV>(a, j, batch_bpm(a, level_entries[j], 1, nsm), s);
+                e = launch_batch_restrict(a, level_entries, j, nsm, s);
+                if (e == cudaSuccess) e = launch_batch_div(a, level_entries, j, nsm, s);
             }
             break;
         default:
@@ -244,12 +256,12 @@ cudaError_t launch_batch_fill(const BatchArgs<R>& a, const int64_t* level_entrie
 }
 
 template <class R>
-cudaError_t launch_batch_post(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s) {
+cudaError_t launch_batch_partial(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s) {
     if (!batch_ok(a, a.jtop_max)) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
     for (int j = a.jtop_max - 1; j >= a.jmin && e == cudaSuccess; --j)
         e = batch_go<PH_PARTIAL>(a, j, batch_bpm(a, level_entries[j], 1, nsm), s);
-    return e == cudaSuccess ? launch_batch_fill(a, level_entries, nsm, s) : e;
+    return e;
 }
 
 template <class R>
@@ -259,23 +271,22 @@ cudaError_t launch_batch_details(const BatchArgs<R>& a, const int64_t* level_ent
 }
 
 template <class R>
-cudaError_t launch_batch_adapt_pre(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s) {
-    cudaError_t e = launch_batch_details(a, level_entries, nsm, s);
-    return e == cudaSuccess ? batch_go<PH_THRESH>(a, 0, 1, s) : e;
+cudaError_t launch_batch_thresholds(const BatchArgs<R>& a, cudaStream_t s) {
+    if (!batch_ok(a, 0)) return cudaErrorInvalidValue;
+    return batch_go<PH_THRESH>(a, 0, 1, s);
 }
 
 template <class R>
-cudaError_t launch_batch_adapt_post(const BatchArgs<R>& a, const int64_t* level_entries, int j1_max, int nsm,
-                                    cudaStream_t s) {
-    if (!batch_ok(a, j1_max)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaSuccess;
-    for (int j = a.jmin + 1; j <= j1_max && e == cudaSuccess; ++j) {
-        const int k = batch_bpm(a, level_entries[j], 4, nsm);
-        e = batch_go<PH_INV_A>(a, j, k, s);
-        if (e == cudaSuccess) e = batch_go<PH_INV_B>(a, j, batch_bpm(a, level_entries[j], 1, nsm), s);
-        if (e == cudaSuccess) e = batch_go<PH_INV_FILL>(a, j, k, s);
-    }
-    return e;
+cudaError_t launch_batch_inverse(const BatchArgs<R>& a, const int64_t* level_entries, int j, int nsm, cudaStream_t s) {
+    if (!batch_ok(a, j)) return cudaErrorInvalidValue;
+    cudaError_t e = batch_go<PH_INV_A>(a, j, batch_bpm(a, level_entries[j], 4, nsm), s);
+    return e == cudaSuccess ? batch_go<PH_INV_B>(a, j, batch_bpm(a, level_entries[j], 1, nsm), s) : e;
+}
+
+template <class R>
+cudaError_t launch_batch_inverse_fill(const BatchArgs<R>& a, const int64_t* level_entries, int j, int nsm, cudaStream_t s) {
+    if (!batch_ok(a, j)) return cudaErrorInvalidValue;
+    return batch_go<PH_INV_FILL>(a, j, batch_bpm(a, level_entries[j], 4, nsm), s);
 }
 
 template <class R>
@@ -285,12 +296,15 @@ cudaError_t launch_batch_out(const BatchArgs<R>& a, cudaStream_t s) {
 }
 
 #define BATCH_INST(R)                                                                                          \
+    template cudaError_t launch_batch_restrict<R>(const BatchArgs<R>&, const int64_t*, int, int, cudaStream_t); \
+    template cudaError_t launch_batch_div<R>(const BatchArgs<R>&, const int64_t*, int, int, cudaStream_t);     \
     template cudaError_t launch_batch_pre<R>(const BatchArgs<R>&, const int64_t*, int, double, cudaStream_t);  \
     template cudaError_t launch_batch_fill<R>(const BatchArgs<R>&, const int64_t*, int, cudaStream_t);         \
-    template cudaError_t launch_batch_post<R>(const BatchArgs<R>&, const int64_t*, int, cudaStream_t);         \
+    template cudaError_t launch_batch_partial<R>(const BatchArgs<R>&, const int64_t*, int, cudaStream_t);      \
     template cudaError_t launch_batch_details<R>(const BatchArgs<R>&, const int64_t*, int, cudaStream_t);      \
-    template cudaError_t launch_batch_adapt_pre<R>(const BatchArgs<R>&, const int64_t*, int, cudaStream_t);    \
-    template cudaError_t launch_batch_adapt_post<R>(const BatchArgs<R>&, const int64_t*, int, int, cudaStream_t); \
+    template cudaError_t launch_batch_thresholds<R>(const BatchArgs<R>&, cudaStream_t);                        \
+    template cudaError_t launch_batch_inverse<R>(const BatchArgs<R>&, const int64_t*, int, int, cudaStream_t); \
+    template cudaError_t launch_batch_inverse_fill<R>(const BatchArgs<R>&, const int64_t*, int, int, cudaStream_t); \
     template cudaError_t launch_batch_out<R>(const BatchArgs<R>&, cudaStream_t);                               \
     template cudaError_t launch_stage_batch_part<R>(const BatchArgs<R>&, const int64_t*, int64_t, int, int, cudaStream_t);
 BATCH_INST(double)

@@ -124,28 +124,33 @@ cudaError_t launch_tile_trend(const BatchArgs<R>& a, int64_t entries, int64_t ir
 template <class R>
 cudaError_t launch_stage_batch_part(const BatchArgs<R>& a, const int64_t* level_entries, int64_t irr_entries, int nsm,
                                     int part, cudaStream_t s);
+// Part 3's two launches of level j: the restriction to it, and the divergence there.
+template <class R>
+cudaError_t launch_batch_restrict(const BatchArgs<R>& a, const int64_t* level_entries, int j, int nsm, cudaStream_t s);
+template <class R>
+cudaError_t launch_batch_div(const BatchArgs<R>& a, const int64_t* level_entries, int j, int nsm, cudaStream_t s);
 // Before the stages of a step, over all members: the time step (dt > 0 for every
 // member, else each member's CFL step).
 template <class R>
 cudaError_t launch_batch_pre(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, double dt, cudaStream_t s);
-// After the stages: the partial height transform (top-1 down to Jmin) and the
+// After the stages: the partial height transform (top-1 down to Jmin), then the
 // ghosts (Jmin+1 up to the top) of every member.
 template <class R>
-cudaError_t launch_batch_post(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);
-// Every member's ghosts, Jmin+1 up to the top.
+cudaError_t launch_batch_partial(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);
 template <class R>
 cudaError_t launch_batch_fill(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);
-// The wavelet coefficients of every live point and the live maxima.
+// Before the members' masks: the wavelet coefficients of every live point and the live
+// maxima, then the thresholds.
 template <class R>
 cudaError_t launch_batch_details(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);
-// Before the members' masks: wavelet coefficients, live maxima and thresholds.
 template <class R>
-cudaError_t launch_batch_adapt_pre(const BatchArgs<R>& a, const int64_t* level_entries, int nsm, cudaStream_t s);
-// After them: the inverse transform and ghosts, level by level up to each
-// member's j1 (level_entries up to the largest j1).
+cudaError_t launch_batch_thresholds(const BatchArgs<R>& a, cudaStream_t s);
+// After them, level by level from Jmin + 1 up to the largest j1: the inverse transform onto
+// level j, then its ghosts (members whose j1 is below j take no part).
 template <class R>
-cudaError_t launch_batch_adapt_post(const BatchArgs<R>& a, const int64_t* level_entries, int j1_max, int nsm,
-                                    cudaStream_t s);
+cudaError_t launch_batch_inverse(const BatchArgs<R>& a, const int64_t* level_entries, int j, int nsm, cudaStream_t s);
+template <class R>
+cudaError_t launch_batch_inverse_fill(const BatchArgs<R>& a, const int64_t* level_entries, int j, int nsm, cudaStream_t s);
 // The read-back records (BatchOut) of every member into a.out.
 template <class R>
 cudaError_t launch_batch_out(const BatchArgs<R>& a, cudaStream_t s);
