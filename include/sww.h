@@ -96,10 +96,9 @@ typedef struct {
                           per phase on larger grids and inside
                           sww_step_ensemble (the members' steps then overlap); 3:
                           inside sww_step_ensemble, one regular launch per phase of
-                          the step over all members, each member's mask on its own
-                          stream (see sww_step_ensemble); -1: one launch per phase
-                          always.  Falls back to -1 where the cooperative launch
-                          cannot run.  Other values give SWW_E_ARG.                  */
+                          the step over all members (see sww_step_ensemble); -1: one
+                          launch per phase always.  Falls back to -1 where the
+                          cooperative launch cannot run.  Other values give SWW_E_ARG. */
     int mask;          /* 0: mask passes over candidate patches (near the active grid);
                           1: dense passes over every point of the levels.  The same mask,
                           but for the perceptron's proposals (sww_set_learned mode 2):
@@ -215,10 +214,10 @@ int sww_step(sww_handle* h, double dt, int nsteps, int adapt);
  * member the RK stages then run as one launch per phase (cooperative launches of
  * different streams do not overlap).  When every member has persistent = 3 and
  * they share precision, Jmin, patch, H, g and scheme (at most 128 members),
- * every phase of the step but the mask (time step, RK base, stage phases,
- * partial transform, ghosts, coefficients, thresholds, inverse transform,
- * read-back) is one regular launch over all members on the first member's
- * stream; each member's mask runs on its own stream in between.
+ * every phase of the step (time step, stage phases, partial transform, ghosts,
+ * coefficients, thresholds, mask, inverse transform, read-back) is one regular
+ * launch over all members on the first member's stream; when a member's mask is
+ * dense (mask = 1), each member's mask runs on its own stream in between.
  * On entry each member's work is ordered after its caller stream, and on return
  * each caller stream waits for its member.  Returns the first error; members
  * then stand at different step counts (sww_stats_get tells which). */
@@ -314,7 +313,7 @@ enum {
  * any class is traced, sww_step runs its kernels directly instead of replaying
  * the captured graph.  In sww_step_ensemble with batched stages (persistent 3)
  * the first member's records cover the batched launches of all members
- * (SWW_K_STAGE per RK stage, SWW_K_DT for the time step and RK base,
+ * (SWW_K_STAGE per RK stage, SWW_K_DT for the time step,
  * SWW_K_PARTIAL for the partial transform and ghosts after the stages). */
 int sww_profile(sww_handle* h, uint32_t class_mask);
 

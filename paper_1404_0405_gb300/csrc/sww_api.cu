@@ -244,7 +244,6 @@ struct sww_handle {
     double* h_dt = nullptr;         // pinned: time step of the last step
     int S = 64, jtop = 0, nsm = 152;
     unsigned grid_all = 1;
-    std::vector<unsigned> grid_lv;
     double t = 0, last_dt = 0;
     int64_t steps = 0;
     bool has_state = false;
@@ -1206,7 +1205,6 @@ int create_handle(const sww_config* cfg, void* stream, std::shared_ptr<Geometry>
         }
         h->lv.assign(fp32 ? 0 : cfg->jmax + 1, DevLevelT<double>{});
         h->lvf.assign(fp32 ? cfg->jmax + 1 : 0, DevLevelT<float>{});
-        h->grid_lv.assign(cfg->jmax + 1, 1);
         h->S = cfg->patch * cfg->patch;
         int64_t total = 0;
         // grid-stride launches: blocks_per_sm blocks of 256 per SM
@@ -1216,8 +1214,6 @@ int create_handle(const sww_config* cfg, void* stream, std::shared_ptr<Geometry>
                 alloc_state<float>(h, j);
             else
                 alloc_state<double>(h, j);
-            int64_t items = (meta(h, j).npatch + 1) * h->S;
-            h->grid_lv[j] = unsigned(std::min<int64_t>(blocks_for(items, 256), cap));
             total += meta(h, j).npatch + 1;
         }
         h->grid_all = unsigned(std::min<int64_t>(blocks_for(total * h->S, 256), cap));

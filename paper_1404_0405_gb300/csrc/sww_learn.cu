@@ -22,8 +22,6 @@ namespace {
 
 __device__ __forceinline__ int64_t lgid() { return int64_t(blockIdx.x) * blockDim.x + threadIdx.x; }
 
-
-
 __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
 // ------------------------------------------------------------------ training
@@ -363,7 +361,3 @@ extern "C" int sww_mlp_predict(const float* X, int64_t n, const float* params, f
     if (cudaGetLastError() != cudaSuccess) return learn_fail(SWW_E_CUDA, "sww_mlp_predict: launch failed");
     return SWW_OK;
 }
-
-namespace sww {
-
-}  // namespace sww

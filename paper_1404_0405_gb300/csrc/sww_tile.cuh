@@ -78,8 +78,10 @@ struct Tile {
     // fields (patch i of a block's sweep uses buffers i mod 2), F and q, the
     // buffers' mbarriers
     static constexpr size_t OFF_GEO = 0;   // R[2][G::WORDS]
-    // staged: dh[NN], u[3 NN] (local direction), and the validity words: of edge and
-    // triangle slots at ST_NFW, of own nodes and edges at ST_EFW
+    // staged: dh[NN], u[3 NN] (local direction), and the patch's validity block from ST_NFW
+    // on (one bulk copy): its words of edge and triangle slots, then at ST_EFW those of own
+    // nodes and edges.  ST_EF is the field copies' last array, whose end the layout check
+    // (tests/tile_layout_check.cu) holds against STAGED, as it does ST_EFW's alignment.
     static constexpr size_t ST_DH = 0, ST_U = sizeof(R) * NN, ST_EF = ST_U, ST_NFW = up16(sizeof(R) * 4 * NN),
                             ST_EFW = ST_NFW + 4 * V::N;
     static constexpr size_t STAGED = ST_NFW + V::BYTES;
@@ -130,13 +132,6 @@ struct TilePlan {
         }
     }
 };
-
-// position (a, b) of tile slot x = (a + 1) W + (b + 1)
-template <int W>
-__device__ __forceinline__ void tpos(int x, int& a, int& b) {
-    a = x / W - 1;
-    b = x % W - 1;
-}
 
 // Tile offsets, relative to node slot x, of the ring of a node: ring edge k (edge
 // slot: 0..2 the node's own edges o = k, 3..5 the edges coming in from (a-1, b),
