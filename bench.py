@@ -329,31 +329,18 @@ def combine_ranks(seconds, cells, device, world):
 # both forms) -- 232 B in FP64, 184 B in FP32.
 STAGE_BYTES_PER_CELL = {"fp64": 232, "fp32": 184}
 
-# Algorithmic bytes per available cell (live or ghost node, with its three edges
-# and two triangles) of the structured trend kernel k_tile_trend: dh and u read
-# (4 words), the flags (4 B), the 17 FP64 geometry words (136 B), and F, q, div F,
-# B and q F^perp written (8 words) -- 12 words + 140 B: 188 B in FP32, 236 B in FP64.
-TREND_BYTES_PER_CELL = {"fp64": 236, "fp32": 188}
-
-# DRAM bytes (read + write) of k_tile_trend per available cell, from an ncu
-# full-set capture of the same jet at Jmin=4..Jmax=8 with 16 members (42.6 MB for
-# 495 961 cells), scaled to a launch by the cells it processes.  The geometry
-# share falls as more members read the same blocks, so at 64 members this
-# overstates the traffic.  Remove the entry when the kernel changes.
-TREND_TRAFFIC_PER_CELL = {"fp32": 85.9}
+# Algorithmic bytes per live cell (its node, three edges and two triangles) of the
+# structured trend kernel k_tile_trend: dh and u read (4 words), the patch's geometry
+# block read (cell area, 3 d_e, 3 l_e, 6 kite areas, 2 dual areas, Coriolis at the 2
+# dual cells: 17 words), and F, q, div F, B and q F^perp written (10 words): 31 words of
+# the working precision.  The kernel runs over the core of the active grid and also
+# writes the ghost cells near live ones; they are not counted, nor are the halos.
+TREND_BYTES_PER_CELL = {"fp64": 248, "fp32": 124}
 
 
 def _live(m):
     # the count the last set_state, adapt or step brought back (no device work)
     return m.live_nodes()
-
-
-def _avail_st(st):
-    return sum(st["live_nodes"].values()) + sum(st["ghost_nodes"].values())
-
-
-def _avail(m):
-    return _avail_st(m.stats())
 
 
 _SAMPLINGS = {}
@@ -520,11 +507,9 @@ def _turbulence(sww, workloads, a, steps, flush, peak, prec_bytes):
         m.load(ck)
         m.set_learned(0)
         m.profile(["trend"])
-        tb_bytes = tb_patches = 0.0
+        tb_bytes = 0.0
         for _ in range(steps):
-            st = m.stats()
-            tb_bytes += prec_bytes * _avail_st(st) * 4
-            tb_patches += sum(st["active_patches"].values()) * 4
+            tb_bytes += prec_bytes * _live(m) * 4
             flush.zero_()
             m.step(-1.0, 1, True)
         t_ms, t_n = m.profile_read()["trend"]
@@ -534,9 +519,7 @@ def _turbulence(sww, workloads, a, steps, flush, peak, prec_bytes):
             out["roofline_trend"] = {"kernel": "k_tile_trend", "achieved": ach, "peak": peak, "unit": "GB/s",
                                      "frac": ach / peak, "avg_launch_us": t_ms * 1e3 / t_n, "launches": t_n,
                                      "algorithmic_bytes_per_launch": tb_bytes / t_n,
-                                     "available_cells_per_launch": tb_bytes / prec_bytes / t_n,
-                                     "patches_per_launch": tb_patches / t_n,
-                                     "patch_fill": tb_bytes / prec_bytes / max(tb_patches, 1.0) / m.cfg.patch ** 2}
+                                     "live_cells_per_launch": tb_bytes / prec_bytes / t_n}
     m.close()
     base.close()
     tb.close()
@@ -698,31 +681,25 @@ def run_ours(a, rank, world):
         classes = ["trend", "irregular", "fill", "restrict", "update", "stage", "dt", "partial", "coeff", "mask",
                    "inverse"]
         m0.profile(classes)
-        tbytes = sbytes = tpatches = 0.0
+        pcells = 0.0
         for _ in range(a.steps):
-            sts = [m.stats() for m in ms]
-            tbytes += TREND_BYTES_PER_CELL[prec] * sum(_avail_st(st) for st in sts) * 4
-            sbytes += STAGE_BYTES_PER_CELL[prec] * sum(sum(st["live_nodes"].values()) for st in sts) * 4
-            tpatches += sum(sum(st["active_patches"].values()) for st in sts) * 4
+            pcells += 4 * sum(_live(m) for m in ms)
             flush.zero_()
             sww.step_ensemble(ms, -1.0, 1, True)
         prof = m0.profile_read()
         m0.profile([])
+        tbytes, sbytes = TREND_BYTES_PER_CELL[prec] * pcells, STAGE_BYTES_PER_CELL[prec] * pcells
         t_ms, t_n = prof["trend"]
         s_ms, s_n = prof["stage"]
         if t_n > 0:
             achieved = tbytes / (t_ms / 1e3) / 1e9
-            roofline = {"bound": "hbm", "kernel": "k_tile_trend (structured trend of every active patch, all members)",
+            roofline = {"bound": "hbm", "kernel": "k_tile_trend (structured trend of the core patches, all members)",
                         "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                         "peak_source": f"{peak_src} (burst copy)",
-                        "traffic": (TREND_TRAFFIC_PER_CELL[prec] * tbytes / TREND_BYTES_PER_CELL[prec] / t_n
-                                    if prec in TREND_TRAFFIC_PER_CELL else None),
                         "avg_launch_us": t_ms * 1e3 / t_n, "launches": t_n,
                         "algorithmic_bytes_per_launch": tbytes / t_n,
-                        "available_cells_per_launch": tbytes / TREND_BYTES_PER_CELL[prec] / t_n,
-                        "patches_per_launch": tpatches / t_n,
-                        "patch_fill": tbytes / TREND_BYTES_PER_CELL[prec] / max(tpatches, 1.0) / cpatch ** 2,
-                        "bytes_per_available_cell": TREND_BYTES_PER_CELL[prec],
+                        "live_cells_per_launch": pcells / t_n,
+                        "bytes_per_live_cell": TREND_BYTES_PER_CELL[prec],
                         "share_of_step": (t_ms / 1e3) / max(sum(times), 1e-30)}
         if s_n > 0:
             nst = 4 * a.steps
