@@ -12,9 +12,9 @@
 //   then the partial transform top-1 down to Jmin, the ghosts, the coefficients with the
 //   live maxima, the thresholds.
 //
-// A trend evaluation alone is one stage of the same kernel.  With a launch per stage and the
-// rest as a launch per phase a step of the jet below took 764 us (FP64) and 566 us (FP32);
-// 700 and 518 now.
+// A trend evaluation alone is one stage of the same kernel.  A step of the jet with 21 550
+// live cells on five levels takes 950 us (FP64) and 577 us (FP32) as a launch per phase,
+// 720 and 504 so.
 //
 // One block of 512 threads per SM, up to 128 registers a thread (with 1024 threads of 64
 // the ids read ahead spill: 75 us a stage instead of 69 on the jet below in FP32, 118
